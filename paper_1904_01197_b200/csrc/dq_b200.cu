@@ -278,6 +278,26 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
     return DQ_OK;
 }
 
+dq::f32x2 twice(float v)
+{
+    uint32_t u;
+    std::memcpy(&u, &v, sizeof(u));
+    return ((dq::f32x2)u << 32) | u;
+}
+
+// Elements per lane of the decoder.  Up to one wave of 8-element lanes (1.2 M elements on 148 SMs) the GPU is not
+// full and the shortest chain per lane wins (W = 8: n = 266,610 6.6 us with 8, 8.5 with 16, 12.8 with 32).  Beyond it
+// 16 and then 32 elements amortise what a worker costs per lane; 32 pays from about two and a half of its own waves
+// (W = 8: n = 4.2 M 38.1 us with 16, 40.5 with 32; n = 11.7 M 79.0 and 75.7), and not for one or two workers, where
+// memory latency matters more and 16 has more warps to hide it (W = 1, n = 25.6 M: 33.8 us with 16, 38.5 with 32).
+int decode_group_size(uint64_t n, uint32_t W, int sms)
+{
+    const uint64_t lanes = (uint64_t)sms * dq::kDecThreads;
+    if (n <= 8u * lanes * dq::dec_ctas_per_sm(8)) return 8;
+    if (W <= 2u || 2u * n < 5u * 32u * lanes * dq::dec_ctas_per_sm(32)) return 16;
+    return 32;
+}
+
 dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t step, const float* side_info,
                         float* out_avg, uint32_t* status_word, bool allow_nested, cudaStream_t st,
                         bool running = false, bool half_dithered = false, uint64_t first_element = 0u,
@@ -300,27 +320,25 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
         // addresses of the (virtual) whole-gradient buffers: see DecodeArgs
         d.packed = virtual_base(m.packed, first_element / 32u * m.p.bits);
         d.scale = virtual_base(m.scale, first_element / m.p.bucket);
-        d.unit_lines = m.p.bits;
         fill_philox(d.ps, m.seed, m.worker, step);
-        d.bits = m.p.bits;
         uint32_t kind;
         if (m.kind == DQ_KIND_DQSG) {
             kind = dq::kDecDqsg;
             d.s = (float)(L - 1u) / 2.0f;
-            d.cconst = 4194304.0f + d.s - 1.5f;
+            d.neg_c = twice(-(4194304.0f + d.s - 1.5f));
             d.step_mul = is_pow2(L - 1u) && L >= 3u ? 2.0f / (float)(L - 1u) : (L == 2u ? 2.0f : 0.0f);
         } else {
             any_nested = true;
-            if (!is_pow2(m.p.coarse_K)) kind = dq::kDecNdqsgAnyK;
-            else kind = (alpha == 1.0f) ? dq::kDecNdqsgPow2 : dq::kDecNdqsgPow2Shrink;
-            d.cconst = 4194304.0f - 1.5f;
+            if (is_pow2(m.p.coarse_K)) kind = (alpha == 1.0f) ? dq::kDecNdqsgPow2 : dq::kDecNdqsgPow2Shrink;
+            else kind = (alpha == 1.0f) ? dq::kDecNdqsgAnyK : dq::kDecNdqsgAnyKShrink;
+            d.neg_c = twice(-(4194304.0f - 1.5f));
             d.A = alpha * m.p.fine_M;
             d.M1 = m.p.fine_M;
             d.alpha = alpha;
             const float a2 = alpha * alpha;
             d.one_m_alpha2 = 1.0f - a2;
-            d.Kf = (float)m.p.coarse_K;
-            d.invK = 1.0f / d.Kf;
+            d.neg_K = twice(-(float)m.p.coarse_K);
+            d.inv_K = twice(1.0f / (float)m.p.coarse_K);
             d.step_mul = float_is_pow2(m.p.fine_M) ? 1.0f / m.p.fine_M : 0.0f;
             if (running) {
                 if (w == 0u) return DQ_ERR_INVALID_ARG;      // nothing decoded yet to serve as side information
@@ -350,44 +368,29 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     a.out = virtual_base(out_avg, first_element);
     a.status = status_word;
     a.n = first_element + n;
-    a.rows = (uint32_t)((first_element + n + 31u) / 32u);
     a.first_row = (uint32_t)(first_element / 32u);
-    a.full_rows = (uint32_t)((first_element + n) / 32u);
-    a.num_units = (a.rows - a.first_row + 31u) / 32u;
     a.W = W;
     a.rows_per_bucket = msgs[0].p.bucket / 32u;
-    a.rpb_shift = 0xFFFFFFFFu;
-    if (is_pow2(a.rows_per_bucket)) {
-        a.rpb_shift = 0u;
-        while ((1u << a.rpb_shift) < a.rows_per_bucket) ++a.rpb_shift;
-    }
+    dq::set_bucket_division(a);
     a.has_side = reads_side ? 1u : 0u;
+    a.out_align32 = (reinterpret_cast<uintptr_t>(out_avg) & 31u) == 0u ? 1u : 0u;
     a.half_bias_bits = 0x4A800000u;
+    a.neg_zero = twice(-0.0f);
+    a.magic = twice(dq::kMagic);
+    a.neg_magic = twice(-dq::kMagic);
     a.Wf = (float)W;
     a.invW = is_pow2(W) ? 1.0f / (float)W : 0.0f;
-    a.error_flags = error_flags_address();
-    if (!a.error_flags) return DQ_ERR_CUDA;
-    // tile views of the caller's buffers: whole rows only (a ragged last row is handled with plain accesses)
-    CUtensorMap side_map, out_map;
-    std::memset(&side_map, 0, sizeof(side_map));
-    std::memset(&out_map, 0, sizeof(out_map));
-    const uint32_t whole_rows = a.full_rows - a.first_row;
-    a.use_tiles = whole_rows != 0u ? 1u : 0u;
-    if (whole_rows != 0u) {
-        if (!make_row_map(&out_map, out_avg, whole_rows, 32u)) return DQ_ERR_CUDA;
-        if (reads_side && !make_row_map(&side_map, side_info, whole_rows, 32u)) return DQ_ERR_CUDA;
-    }
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
     const bool d16 = (msgs[0].p.dither_bits == 16u);
+    const int E = decode_group_size(n, W, sms);
+    a.num_groups = (n + (uint32_t)E - 1u) / (uint32_t)E;
+    a.early_launch = a.num_groups <= (uint64_t)sms * dq::kDecThreads ? 1u : 0u;
     cudaError_t le;
-    if (half_dithered) le = dq::launch_decode_d0_r0(side_map, out_map, a, sms, st);
-    else if (running && any_nested) le = d16 ? dq::launch_decode_d16_r1(side_map, out_map, a, sms, st)
-                                             : dq::launch_decode_d32_r1(side_map, out_map, a, sms, st);
-    else if (from_first) le = d16 ? dq::launch_decode_d16_r2(side_map, out_map, a, sms, st)
-                                  : dq::launch_decode_d32_r2(side_map, out_map, a, sms, st);
-    else le = d16 ? dq::launch_decode_d16_r0(side_map, out_map, a, sms, st)
-                  : dq::launch_decode_d32_r0(side_map, out_map, a, sms, st);
+    if (half_dithered) le = dq::launch_decode_d0_r0(a, E, st);
+    else if (running && any_nested) le = d16 ? dq::launch_decode_d16_r1(a, E, st) : dq::launch_decode_d32_r1(a, E, st);
+    else if (from_first) le = d16 ? dq::launch_decode_d16_r2(a, E, st) : dq::launch_decode_d32_r2(a, E, st);
+    else le = d16 ? dq::launch_decode_d16_r0(a, E, st) : dq::launch_decode_d32_r0(a, E, st);
     if (le != cudaSuccess) return DQ_ERR_CUDA;
     g_launches.fetch_add(1);
     return DQ_OK;

@@ -2,26 +2,18 @@
 // server loop with the side information given as a vector, taken as the running mean, or taken as the
 // reconstruction of message 0).
 //
-// One lane owns one row = 32 consecutive elements: 32 fp32 accumulators in registers, and per worker exactly
-// `bits` packed words.  A warp owns a unit of 32 rows.  One persistent CTA of sixteen warps runs per SM; its
-// warps form teams of four that take four adjacent units at a time from the CTA's share of the gradient.  The
-// share is fixed (CTA c owns every gridDim.x-th group of four units), the order inside it is not: teams draw the
-// next group from a counter in shared memory, because the warp schedulers favour some warps by a fifth and a
-// fixed split would leave the favoured ones idle at the end.
-//   * The side information of a unit arrives in the warp's shared memory by one 2-D tile copy (32 rows x 128
-//     bytes, 128-byte swizzle, so that "lane r reads row r" is free of bank conflicts), issued one unit ahead.
-//   * Every worker's packed words of the next unit are requested into the L2 one unit ahead (one prefetch
-//     instruction per unit: lane w asks for worker w's lines); each lane then loads exactly its `bits` words with
-//     the widest vector loads their alignment allows, and the Philox work that follows hides the L2 latency.
-//   * For every worker (in array order) the lane regenerates the 32 dithers (Philox blocks four at a time),
-//     reconstructs and accumulates; the bucket scale is loaded one step ahead.
-//   * The mean goes back through the tile buffer and leaves with one tile store per unit: full 128-byte lines,
-//     issued by one lane.
-// The packed streams, the side information and the output are each touched once in HBM.
+// One lane owns E consecutive elements (a group): E fp32 accumulators in registers, and per worker exactly E * bits
+// packed bits.  A group never straddles a bucket (buckets are multiples of 32 elements), so a lane needs one scale
+// per worker.  For every worker, in array order, the lane regenerates its E dithers (E / 4 Philox blocks, E / 8 with
+// the 16-bit stream), reconstructs and accumulates; the packed words are requested before the Philox work (or one
+// worker ahead), which hides their latency, the scale one worker ahead.  Side information is read once into the
+// lane's own shared-memory slots, and so are the first Philox products, which are the same for every worker; the
+// mean is written once in full 32-byte sectors.  Nothing is shared between lanes: there is no barrier, and the
+// hardware's block scheduler balances the load.
 //
-// The path is bound by instruction issue, not by HBM: each (element, worker) pair needs a quarter of a
-// Philox block (4.5 wide multiplies, which occupy the multiplier pipe for four cycles each) before any
-// reconstruction arithmetic.
+// What bounds it: the multiplier pipe and instruction issue.  Each (element, worker) pair needs a quarter of a
+// Philox block, 4.25 wide multiplies of four cycles each, before any reconstruction arithmetic; that arithmetic runs
+// on packed pairs of fp32 values (half the instructions).
 #pragma once
 
 #include "dq_device.cuh"
@@ -32,24 +24,24 @@ namespace dq {
 // DQSG messages), the running mean of the messages decoded so far, or the reconstruction of message 0.
 enum DecSide : int { kSideGiven = 0, kSideRunning = 1, kSideFirst = 2 };
 
-enum DecKind : uint32_t { kDecDqsg = 0, kDecNdqsgPow2 = 1, kDecNdqsgPow2Shrink = 2, kDecNdqsgAnyK = 3 };
+enum DecKind : uint32_t {
+    kDecDqsg = 0, kDecNdqsgPow2 = 1, kDecNdqsgPow2Shrink = 2, kDecNdqsgAnyK = 3, kDecNdqsgAnyKShrink = 4
+};
 
 struct DecWorker {
     const uint32_t* packed;   // } addresses of the (virtual) whole-gradient buffers, see DecodeArgs
     const float* scale;       // }
-    uint32_t unit_lines;      // 128-byte lines of one unit's packed words (= bits)
-    uint32_t group_end;       // index after the last worker of the run of equal variants that this worker belongs to
     PhiloxStream ps;
     uint32_t variant;     // DecKind * 8 + bits - 1: one jump selects the routine
-    uint32_t bits;
+    uint32_t group_end;   // index after the last worker of the run of equal variants that this worker belongs to
     float s;              // DQSG (L-1)/2
-    float cconst;         // DQSG: 4194304 + s - 1.5 ; NDQSG: 4194304 - 1.5   (see unpack_half_biased)
+    f32x2 neg_c;          // } pairs of equal values (one 64-bit load each): minus (DQSG: 4194304 + s - 1.5,
+    f32x2 neg_K;          // } NDQSG: 4194304 - 1.5; see unpack_half_biased), -K, and 1/K rounded to nearest (exact
+    f32x2 inv_K;          // } when K is a power of two)
     float A;              // NDQSG alpha * M1
     float M1;
     float alpha;
     float one_m_alpha2;   // 1 - alpha*alpha
-    float Kf;             // (float)K
-    float invK;           // 1/K (exact when K is a power of two)
     float rcp_count;      // running-mean mode: 1 / (number of workers before this one)
     float step_mul;       // DQSG: 1/s, NDQSG: 1/M1, when that divisor is a power of two (the division is then an
                           // exact multiplication); 0 otherwise
@@ -60,52 +52,50 @@ struct DecodeArgs {
     float* out;
     uint32_t* status;
     // A call may cover the elements [first, n) of a longer gradient (first a multiple of the bucket size, 0 for a
-    // whole gradient).  Rows, elements and buckets are then numbered as in the whole gradient -- which is what the
+    // whole gradient).  Groups, elements and buckets are then numbered as in the whole gradient -- which is what the
     // dither counters need -- and every pointer above and in w[] is the buffer's address minus the range's offset,
-    // so that "pointer + global index" lands in the caller's buffer.  The tile maps cover the caller's buffers
-    // themselves (row 0 of a map = row first_row of the gradient) and only whole rows.
+    // so that "pointer + global index" lands in the caller's buffer.
     uint64_t n;               // end of the range (element index)
-    uint32_t rows;            // ceil(n / 32): end of the range (row index); below 2^29
     uint32_t first_row;       // first / 32
-    uint32_t full_rows;       // floor(n / 32): rows below this index have 32 elements
-    uint32_t num_units;       // ceil((rows - first_row) / 32): units of 32 rows
     uint32_t W;
+    uint64_t num_groups;      // groups of E elements in the range (E = the launched instantiation's)
     uint32_t rows_per_bucket; // B / 32
-    uint32_t rpb_shift;       // log2(rows_per_bucket) when that is a power of two, else 0xFFFFFFFF
-    uint32_t has_side;        // the side information vector is read (some message is NDQSG, not running-mean mode)
-    uint32_t use_tiles;       // the range holds at least one whole row: the tile maps are valid
+    uint32_t bucket_shift;    // row -> bucket: (row * bucket_magic) >> 32 >> bucket_shift, or row >> bucket_shift
+    uint32_t bucket_magic;    // when bucket_magic is 0 (power-of-two buckets); see set_bucket_division
+    uint32_t has_side;        // the side information vector is read
+    uint32_t early_launch;    // the grid has at most one CTA per SM (see the kernel)
+    uint32_t out_align32;     // out is 32-byte aligned: whole groups leave in 32-byte stores
     uint32_t half_bias_bits;  // 0x4A800000 (bit pattern of 2^22), passed in so that it lives in a register
     float Wf;
+    f32x2 neg_zero;           // -0.0 twice (see f32x2)           } constants that would otherwise be assembled from
+    f32x2 magic, neg_magic;   // +-1.5 * 2^23 twice               } immediates again and again
     float invW;               // 1/W when W is a power of two, else 0
-    unsigned int* error_flags;    // the library's per-device error word
     DecWorker w[64];
 };
 
-#ifndef DQ_DEC_THREADS
-#define DQ_DEC_THREADS 512
-#endif
-constexpr int kDecThreads = DQ_DEC_THREADS;
-constexpr int kDecWarps = kDecThreads / 32;
-#ifndef DQ_DEC_MINBLOCKS
-#define DQ_DEC_MINBLOCKS (512 / DQ_DEC_THREADS)
-#endif
-constexpr int kDecMinBlocks = DQ_DEC_MINBLOCKS;     // resident CTAs per SM the register budget is set for
-#ifndef DQ_DEC_TEAM
-#define DQ_DEC_TEAM 4
-#endif
-constexpr int kDecTeamWarps = DQ_DEC_TEAM;          // warps that take adjacent units and meet before each
-constexpr int kDecTeams = kDecWarps / kDecTeamWarps;
-static_assert(kDecWarps % kDecTeamWarps == 0 && kDecTeams >= 1 && (kDecTeamWarps == 1 || kDecTeams <= 15),
-              "teams of several warps use named barriers 1..15");
-constexpr int kDecTileBytes = 32 * 128;         // one unit of side information or output
-constexpr int kDecTileBuffers = 3;              // per warp: side in flight / side in use, then output leaving
-// Dynamic shared memory of a CTA: the warps' tile buffers (plus room to align to 1024 bytes).
-constexpr uint32_t kDecSmemBytes = (uint32_t)(kDecWarps * kDecTileBuffers * kDecTileBytes) + 1024u;
+// Division of a row index below 2^29 by rows_per_bucket as a multiplication: with s = floor(log2 d) and
+// m = ceil(2^(32+s) / d), m d - 2^(32+s) < d < 2^(s+1) <= 2^(32+s) / 2^29, which is what makes
+// floor(row m / 2^(32+s)) exact.
+inline void set_bucket_division(DecodeArgs& a)
+{
+    const uint32_t d = a.rows_per_bucket;
+    uint32_t s = 0u;
+    while ((2u << s) <= d) ++s;
+    a.bucket_shift = s;
+    a.bucket_magic = (d & (d - 1u)) == 0u ? 0u : (uint32_t)(((1ull << (32u + s)) + d - 1u) / d);
+}
 
-// Code of element `idx` of a row as the float 2^22 + code: the bit pattern of 2^22 with the code in mantissa
+constexpr int kDecThreads = 128;
+// Resident CTAs per SM that the register budget is set for.  E = 32 with 96 registers and 20 warps per SM is the
+// fastest form for many workers: what a worker costs per lane (scale, gain, constants, loop: about 65 instructions) is
+// spread over the most elements, and 16 warps (128 registers) are 7 % slower, 24 (80 registers, spilling) 3 %.
+// E = 16 and 8 take 64 registers (32 warps).
+constexpr int dec_ctas_per_sm(int E) { return E == 32 ? 5 : 8; }
+
+// Code of element `idx` of a group as the float 2^22 + code: the bit pattern of 2^22 with the code in mantissa
 // bits 1.. (floats in [2^22, 2^23) step by 1/2).  Subtracting a constant then gives code - c exactly.
-template <int BITS>
-__device__ __forceinline__ float unpack_half_biased(const uint32_t (&words)[BITS], int idx, uint32_t bias_bits)
+template <int BITS, int NF>
+__device__ __forceinline__ float unpack_half_biased(const uint32_t (&f)[NF], int idx, uint32_t bias_bits)
 {
     const int bit = idx * BITS;
     const int wi = bit >> 5;
@@ -113,393 +103,354 @@ __device__ __forceinline__ float unpack_half_biased(const uint32_t (&words)[BITS
     constexpr uint32_t mask2 = ((1u << BITS) - 1u) << 1;
     uint32_t v;
     if (sh + BITS <= 32) {
-        v = (sh == 0) ? (words[wi] << 1) : (words[wi] >> (sh - 1));
+        v = (sh == 0) ? (f[wi] << 1) : (f[wi] >> (sh - 1));
     } else {
-        v = __funnelshift_r(words[wi], words[(wi + 1) % BITS], sh - 1);
+        v = __funnelshift_r(f[wi], f[(wi + 1) % NF], sh - 1);
     }
     return __uint_as_float((v & mask2) | bias_bits);          // one logic op: (v & immediate) | register
 }
 
-// The lane's BITS words (p = address of the first one; a row of BITS words starts at a multiple of 4 * BITS
-// bytes), with the widest loads that alignment allows.
-template <int BITS>
-__device__ __forceinline__ void load_words(const uint32_t* p, uint32_t (&w)[BITS])
-{
-    if constexpr (BITS % 4 == 0) {
-#pragma unroll
-        for (int j = 0; j < BITS; j += 4) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(p + j));
-            w[j] = v.x; w[j + 1] = v.y; w[j + 2] = v.z; w[j + 3] = v.w;
-        }
-    } else if constexpr (BITS % 2 == 0) {
-#pragma unroll
-        for (int j = 0; j < BITS; j += 2) {
-            const uint2 v = __ldg(reinterpret_cast<const uint2*>(p + j));
-            w[j] = v.x; w[j + 1] = v.y;
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < BITS; ++j) w[j] = __ldg(p + j);
-    }
-}
+constexpr int gcd_of(int a, int b) { return b == 0 ? a : gcd_of(b, a % b); }
 
-// One worker's contribution to the 32 accumulators of a row.
-//   DQSG:  g~ = (kappa/s) ((k - s) - delta); (k - s + 1.5) - f rounds once to the same value.
-//   NDQSG: r = (m - delta) - y a;  jj = rint(r / K);  q1^ = m - K jj;  g~ = beta (q1^ - delta) [+ (1-alpha^2) y]
-// load_row: the row whose words the lane loads (its own row, or the last whole row for lanes past the end, whose
-// results are never stored); side_addr: shared-memory address of
-// the lane's row of side information with the swizzle term already OR-ed in (piece p is at side_addr ^ (p << 4)).
-template <int BITS, uint32_t KIND, int DITH, bool RUN>
-__device__ __forceinline__ void decode_row(const DecWorker& wk, uint32_t row, uint32_t load_row, float kappa,
-                                           uint32_t side_addr, float (&acc)[32], uint32_t bias_bits)
-{
-    uint32_t words[BITS];
-    load_words<BITS>(wk.packed + (uint64_t)load_row * (uint32_t)BITS, words);
+// The E * BITS bits of group `g`, aligned to bit 0 of f[0].  With `careful` (the last groups of the gradient) every
+// word is checked against the end of the stream.
+template <int BITS, int E>
+struct Field {
+    static constexpr int kBits = E * BITS;
+    static constexpr int kWords = (kBits + 31) / 32;
+    static constexpr int kAlign = gcd_of(kBits, 32);                       // a field starts at a multiple of this
+    static constexpr int kLoads = (32 - kAlign + kBits + 31) / 32;         // words that a field can touch
+    uint32_t w[kLoads];
 
-    // kappa / s and alpha kappa / M1: a division by a power of two is an exact multiplication
-    float c, a = 0.0f;
-    if (KIND == kDecDqsg) {
-        c = (wk.step_mul != 0.0f) ? __fmul_rn(kappa, wk.step_mul) : __fdiv_rn(kappa, wk.s);
-    } else {
-        a = (kappa >= 0x1p-100f) ? __fdiv_rn(wk.A, kappa) : 0.0f;
-        const float ak = __fmul_rn(wk.alpha, kappa);
-        c = (wk.step_mul != 0.0f) ? __fmul_rn(ak, wk.step_mul) : __fdiv_rn(ak, wk.M1);            // beta
-    }
-    constexpr int EPB = (DITH == 16) ? 8 : 4;       // elements per Philox block
-    constexpr int PASS = 4 * EPB;                   // elements per group of four blocks
+    __device__ __forceinline__ void load(const uint32_t* packed, uint32_t g, bool careful, uint64_t n)
+    {
+        const uint64_t wi = ((uint64_t)g * (uint32_t)kBits) >> 5;
+        const uint32_t* p = packed + wi;
+        if (careful) {
+            const uint64_t num_words = (n * (uint32_t)BITS + 31u) >> 5;
 #pragma unroll
-    for (int h = 0; h < 32 / PASS; ++h) {
-        uint32_t rnd[4][4];
-        if (DITH != 0) philox4x32_10_row<4>(row * (32u / EPB), 4 * h, wk.ps, rnd);
+            for (int j = 0; j < kLoads; ++j) w[j] = (wi + j < num_words) ? __ldg(p + j) : 0u;
+            return;
+        }
+        if constexpr (kAlign == 32 && kLoads % 4 == 0) {
 #pragma unroll
-        for (int q = 0; q < PASS / 4; ++q) {        // four elements at a time (one 16-byte piece of y)
-            float y[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            if (KIND != kDecDqsg && !RUN) {
-                asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
-                             : "=f"(y[0]), "=f"(y[1]), "=f"(y[2]), "=f"(y[3])
-                             : "r"(side_addr ^ (uint32_t)(((PASS / 4) * h + q) << 4))
-                             : "memory");
+            for (int j = 0; j < kLoads; j += 4) {
+                const uint4 v = __ldg(reinterpret_cast<const uint4*>(p + j));
+                w[j] = v.x; w[j + 1] = v.y; w[j + 2] = v.z; w[j + 3] = v.w;
             }
+        } else if constexpr (kAlign == 32 && kLoads % 2 == 0) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int t = 4 * q + e;
-                const int idx = PASS * h + t;
-                const float f = dither_of<DITH>(rnd, t);
-                const float X = __fadd_rn(unpack_half_biased<BITS>(words, idx, bias_bits), -wk.cconst);
-                float gt;
-                if (KIND == kDecDqsg) {
-                    const float d = __fadd_rn(X, -f);                      // (k - s) - delta
-                    gt = __fmul_rn(c, d);
-                } else {
-                    // side information: the given vector, or (Algorithm 2 as written) the mean of the
-                    // reconstructions accumulated so far
-                    const float yy = RUN ? __fmul_rn(acc[idx], wk.rcp_count) : y[e];
-                    const float r1 = __fadd_rn(X, -f);                     // m - delta
-                    const float r = __fmaf_rn(-yy, a, r1);
-                    float jj;
-                    if (KIND == kDecNdqsgAnyK) {
-                        jj = __fadd_rn(__fadd_rn(__fdiv_rn(r, wk.Kf), kMagic), -kMagic);
-                    } else {
-                        // K is a power of two: r * (1/K) is exact, so one rounding gives rint(r / K)
-                        jj = __fadd_rn(__fmaf_rn(r, wk.invK, kMagic), -kMagic);
-                    }
-                    const float Y = __fmaf_rn(-wk.Kf, jj, X);              // q1^ + 1.5, exact
-                    const float d = __fadd_rn(Y, -f);                      // q1^ - delta
-                    if (KIND == kDecNdqsgPow2) gt = __fmul_rn(c, d);                          // alpha == 1
-                    else if (KIND == kDecNdqsgPow2Shrink) gt = __fmaf_rn(c, d, __fmul_rn(wk.one_m_alpha2, yy));
-                    else if (wk.alpha == 1.0f) gt = __fmul_rn(c, d);
-                    else gt = __fmaf_rn(c, d, __fmul_rn(wk.one_m_alpha2, yy));
-                }
-                acc[idx] = __fadd_rn(acc[idx], gt);
+            for (int j = 0; j < kLoads; j += 2) {
+                const uint2 v = __ldg(reinterpret_cast<const uint2*>(p + j));
+                w[j] = v.x; w[j + 1] = v.y;
             }
+        } else {
+#pragma unroll
+            for (int j = 0; j < kLoads; ++j) w[j] = __ldg(p + j);
         }
     }
-}
 
-// State of a lane while it walks over the workers of a unit.
-struct DecLane {
-    uint32_t row, load_row, bucket, bucket_next, row_addr, kappa_bits_max;
-    float kappa_next;
+    __device__ __forceinline__ void align(uint32_t g, uint32_t (&f)[kWords]) const
+    {
+        const uint32_t sh = (kAlign == 32) ? 0u : ((g * (uint32_t)kBits) & 31u);
+#pragma unroll
+        for (int j = 0; j < kWords; ++j) {
+            if (kAlign == 32) f[j] = w[j];
+            else if (j + 1 < kLoads) f[j] = __funnelshift_r(w[j], w[j + 1], sh);
+            else f[j] = w[j] >> sh;
+        }
+    }
 };
 
-// The workers [w, w_end) of one run of equal variants: the same routine for each, so the jump on the variant is taken
-// once per run and not once per worker (Algorithm 2's groups P1 and P2 are two runs).
-template <int BITS, uint32_t KIND, int DITH, int SIDE>
-__device__ __forceinline__ void decode_run(const DecodeArgs& args, uint32_t w, uint32_t w_end, DecLane& ln, float (&acc)[32])
+// State of a lane while it walks over the workers.
+struct DecLane {
+    uint32_t group, bucket, kappa_bits_max;
+    uint32_t slot;              // shared-memory address of the lane's first 16-byte slot (slots are kDecThreads apart)
+    uint32_t first[2];          // first Philox product (hi, lo) of a lane with one block
+    float kappa_next;
+    bool careful;
+};
+
+// The contributions of the workers [w, w_end), a run of equal variants: the same routine for each, so the jump on the
+// variant is taken once per run and not once per worker (Algorithm 2's groups P1 and P2 are two runs).
+//   DQSG:  g~ = (kappa/s) ((k - s) - delta); (k - s + 1.5) - f rounds once to the same value.
+//   NDQSG: r = (m - delta) - y a;  jj = rint(r / K);  q1^ = m - K jj;  g~ = beta (q1^ - delta) [+ (1-alpha^2) y]
+// AHEAD: the packed words are requested one worker ahead (worth its registers with 20 warps per SM, i.e. E = 32: 4 %;
+// with 32 warps it costs as much).
+template <int BITS, uint32_t KIND, int DITH, int SIDE, int E, bool AHEAD>
+__device__ __forceinline__ void decode_run(const DecodeArgs& args, uint32_t w, uint32_t w_end, DecLane& ln,
+                                           f32x2 (&acc)[E / 2])
 {
+    constexpr bool RUN = SIDE == kSideRunning;
+    constexpr bool ANY_K = KIND == kDecNdqsgAnyK || KIND == kDecNdqsgAnyKShrink;
+    constexpr bool SHRINK = KIND == kDecNdqsgPow2Shrink || KIND == kDecNdqsgAnyKShrink;
+    constexpr int EPB = (DITH == 16) ? 8 : 4;       // elements per Philox block
+    constexpr int N = E / EPB;                      // blocks of the group
+    constexpr int P = N < 2 ? N : 2;                // blocks in flight
+    Field<BITS, E> field;
+    if constexpr (AHEAD) field.load(args.w[w].packed, ln.group, ln.careful, args.n);
 #pragma unroll 1
     for (; w < w_end; ++w) {
-        const float kappa = ln.kappa_next;
-        // the next step's scale: the next worker's for this bucket, or the first worker's for the next unit
-        ln.kappa_next = (w + 1u < args.W) ? __ldg(args.w[w + 1u].scale + ln.bucket)
-                                          : __ldg(args.w[0].scale + ln.bucket_next);
-        decode_row<BITS, KIND, DITH, SIDE == kSideRunning>(args.w[w], ln.row, ln.load_row, kappa, ln.row_addr, acc,
-                                                            args.half_bias_bits);
-        if (SIDE == kSideFirst && w == 0u) {
-            // the accumulators are now the reconstruction of message 0: it is the side information of the nested
-            // messages that follow, which read it from the lane's row of the tile buffer
+        const DecWorker& wk = args.w[w];
+        if constexpr (!AHEAD) field.load(wk.packed, ln.group, ln.careful, args.n);
+        uint32_t f[Field<BITS, E>::kWords];
+        f32x2 cc, na = 0ull;
+        const f32x2 nz = args.neg_zero;
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};"
-                             ::"r"(ln.row_addr ^ (uint32_t)(c << 4)), "f"(acc[4 * c]), "f"(acc[4 * c + 1]),
-                               "f"(acc[4 * c + 2]), "f"(acc[4 * c + 3])
+        for (int h = 0; h < N / P; ++h) {
+            uint32_t rnd[P][4];
+            if constexpr (DITH != 0) {
+                uint32_t hi[P], lo[P];
+                if constexpr (N == 1) {
+                    hi[0] = ln.first[0];
+                    lo[0] = ln.first[1];
+                } else {
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(hi[0]), "=r"(lo[0]), "=r"(hi[1]), "=r"(lo[1])
+                                 : "r"(ln.slot + (uint32_t)((E / 4 + h) * kDecThreads * 16)));
+                }
+                philox4x32_10_after_first<P>(hi, lo, wk.ps, rnd);
+            }
+            if (h == 0) {
+                // the Philox work above hides the latency of the words; the scale was requested a worker ago
+                field.align(ln.group, f);
+                if constexpr (AHEAD) {
+                    if (w + 1u < w_end) field.load(args.w[w + 1u].packed, ln.group, ln.careful, args.n);
+                }
+                const float kappa = ln.kappa_next;
+                if (w + 1u < args.W) ln.kappa_next = __ldg(args.w[w + 1u].scale + ln.bucket);
+                // kappa / s and alpha kappa / M1: a division by a power of two is an exact multiplication
+                float c;
+                if constexpr (KIND == kDecDqsg) {
+                    c = (wk.step_mul != 0.0f) ? __fmul_rn(kappa, wk.step_mul) : __fdiv_rn(kappa, wk.s);
+                } else {
+                    na = both((kappa >= 0x1p-100f) ? -__fdiv_rn(wk.A, kappa) : -0.0f);
+                    const float ak = __fmul_rn(wk.alpha, kappa);
+                    c = (wk.step_mul != 0.0f) ? __fmul_rn(ak, wk.step_mul) : __fdiv_rn(ak, wk.M1);        // beta
+                }
+                cc = both(c);
+                const uint32_t kb = __float_as_uint(kappa) & 0x7FFFFFFFu;
+                ln.kappa_bits_max = (kb > ln.kappa_bits_max) ? kb : ln.kappa_bits_max;
+            }
+#pragma unroll
+            for (int qq = 0; qq < P * EPB / 4; ++qq) {      // four elements at a time (one 16-byte slot of y)
+                const int q = h * (P * EPB / 4) + qq;
+                f32x2 y[2] = {0ull, 0ull};
+                if constexpr (KIND != kDecDqsg && !RUN)
+                    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
+                                 : "=l"(y[0]), "=l"(y[1])
+                                 : "r"(ln.slot + (uint32_t)(q * kDecThreads * 16))
+                                 : "memory");
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int t = 4 * q + 2 * e;                           // element of the group
+                    const int tr = 4 * qq + 2 * e;                         // ... of the blocks in rnd
+                    f32x2 nf;                                              // -f, f = delta + 1.5
+                    if constexpr (DITH == 0) nf = both(-1.5f);
+                    else if constexpr (DITH == 16) nf = fma2(dither_bits2<16>(rnd, tr), both(-kTwo125), both(-kF16Offset));
+                    else nf = fma2(dither_bits2<32>(rnd, tr), both(-kTwo127), both(-kF32Offset));
+                    const f32x2 X = add2(pack2(unpack_half_biased<BITS>(f, t, args.half_bias_bits),
+                                               unpack_half_biased<BITS>(f, t + 1, args.half_bias_bits)), wk.neg_c);
+                    f32x2 gt;
+                    if constexpr (KIND == kDecDqsg) {
+                        gt = fma2(cc, add2(X, nf), nz);                    // c ((k - s) - delta)
+                    } else {
+                        // side information: the given vector, the reconstruction of message 0, or (Algorithm 2 as
+                        // written) the mean of the reconstructions accumulated so far
+                        const f32x2 yy = RUN ? fma2(acc[t >> 1], both(wk.rcp_count), nz) : y[e];
+                        const f32x2 r1 = add2(X, nf);                      // m - delta
+                        const f32x2 r = fma2(yy, na, r1);
+                        f32x2 jj;
+                        if constexpr (ANY_K) {
+                            // r / K rounded to nearest from the correctly rounded 1/K: one residual correction leaves
+                            // a relative error below 2^-46 before the last rounding, while r / K (24-bit r, 8-bit K)
+                            // is either representable or at least 2^-33 away from every rounding boundary
+                            const f32x2 q0 = fma2(r, wk.inv_K, nz);
+                            const f32x2 rem = fma2(wk.neg_K, q0, r);
+                            jj = add2(add2(fma2(rem, wk.inv_K, q0), args.magic), args.neg_magic);
+                        } else {
+                            // K is a power of two: r * (1/K) is exact, so one rounding gives rint(r / K)
+                            jj = add2(fma2(r, wk.inv_K, args.magic), args.neg_magic);
+                        }
+                        const f32x2 d = add2(fma2(wk.neg_K, jj, X), nf);   // q1^ - delta  (q1^ + 1.5 is exact)
+                        gt = fma2(cc, d, SHRINK ? fma2(both(wk.one_m_alpha2), yy, nz) : nz);
+                    }
+                    acc[t >> 1] = add2(acc[t >> 1], gt);
+                }
+            }
+        }
+        if (SIDE == kSideFirst && w == 0u) {
+            // the accumulators are now the reconstruction of message 0: the side information of the nested messages
+#pragma unroll
+            for (int q = 0; q < E / 4; ++q)
+                asm volatile("st.shared.v2.b64 [%0], {%1, %2};"
+                             ::"r"(ln.slot + (uint32_t)(q * kDecThreads * 16)), "l"(acc[2 * q]), "l"(acc[2 * q + 1])
                              : "memory");
         }
-        const uint32_t kb = __float_as_uint(kappa) & 0x7FFFFFFFu;
-        ln.kappa_bits_max = (kb > ln.kappa_bits_max) ? kb : ln.kappa_bits_max;
     }
 }
 
-// All W workers of a unit, run by run; dispatch on (kind, bits) with one jump per run.
-template <int DITH, int SIDE>
-__device__ __forceinline__ void decode_workers(const DecodeArgs& args, DecLane& ln, float (&acc)[32])
+// The variants that nearly every caller uses: DQSG, and NDQSG with a power-of-two K and no shrinkage, up to 4 bits.
+// They have kernels of their own: with all forty routines in one kernel the compiler's register allocation costs every
+// routine 1 to 5 % (W = 16, 3 bits, n = 124.4 M: 1973 us against 1920).
+inline bool is_usual_variant(uint32_t variant) { return (variant >> 3) <= kDecNdqsgPow2 && (variant & 7u) < 4u; }
+
+// All W workers, run by run; dispatch on (kind, bits) with one jump per run.  ALL: every variant, else the usual ones.
+template <int DITH, int SIDE, int E, bool ALL>
+__device__ __forceinline__ void decode_workers(const DecodeArgs& args, DecLane& ln, f32x2 (&acc)[E / 2])
 {
 #define DQ_DEC_CASE(KIND, BITS)                                                                                    \
-    case (KIND) * 8u + (BITS) - 1u: decode_run<BITS, KIND, DITH, SIDE>(args, w, w_end, ln, acc); break;
+    case (KIND) * 8u + (BITS) - 1u:                                                                                \
+        decode_run<BITS, KIND, DITH, SIDE, E, E == 32 && !ALL>(args, w, w_end, ln, acc);                           \
+        break;
+#define DQ_DEC_LOW(KIND)                                                                                           \
+    DQ_DEC_CASE(KIND, 1) DQ_DEC_CASE(KIND, 2) DQ_DEC_CASE(KIND, 3) DQ_DEC_CASE(KIND, 4)
 #define DQ_DEC_KIND(KIND)                                                                                          \
-    DQ_DEC_CASE(KIND, 1) DQ_DEC_CASE(KIND, 2) DQ_DEC_CASE(KIND, 3) DQ_DEC_CASE(KIND, 4)                            \
+    DQ_DEC_LOW(KIND)                                                                                               \
     DQ_DEC_CASE(KIND, 5) DQ_DEC_CASE(KIND, 6) DQ_DEC_CASE(KIND, 7) DQ_DEC_CASE(KIND, 8)
 #pragma unroll 1
     for (uint32_t w = 0; w < args.W;) {
         const uint32_t w_end = args.w[w].group_end;
-        switch (args.w[w].variant) {
-            DQ_DEC_KIND(kDecDqsg)
-            DQ_DEC_KIND(kDecNdqsgPow2)
-            DQ_DEC_KIND(kDecNdqsgPow2Shrink)
-            DQ_DEC_KIND(kDecNdqsgAnyK)
-            default: break;
+        if constexpr (ALL) {
+            switch (args.w[w].variant) {
+                DQ_DEC_KIND(kDecDqsg)
+                DQ_DEC_KIND(kDecNdqsgPow2)
+                DQ_DEC_KIND(kDecNdqsgPow2Shrink)
+                DQ_DEC_KIND(kDecNdqsgAnyK)
+                DQ_DEC_KIND(kDecNdqsgAnyKShrink)
+                default: break;
+            }
+        } else {
+            switch (args.w[w].variant) {
+                DQ_DEC_LOW(kDecDqsg)
+                DQ_DEC_LOW(kDecNdqsgPow2)
+                default: break;
+            }
         }
         w = w_end;
     }
 #undef DQ_DEC_KIND
+#undef DQ_DEC_LOW
 #undef DQ_DEC_CASE
 }
 
-// The last row of a gradient whose length is not a multiple of 32: one element per lane (`e` = the lane, of a
-// whole warp), everything at run time, straight from and to global memory.  Same arithmetic, in the same order,
-// as decode_row.  Each element is a chain of dependent loads and divisions, about a microsecond per worker.
-template <int DITH, int SIDE>
-__device__ __noinline__ void decode_partial_row(const DecodeArgs& args, uint32_t row, uint32_t bucket, uint32_t nvalid,
-                                                uint32_t e)
+__device__ __forceinline__ void store8(float* p, const f32x2 (&v)[4], bool align32)
 {
-    constexpr bool RUN = (SIDE == kSideRunning);
-    if (e < nvalid) {
-        const uint64_t i = (uint64_t)row * 32u + e;
-        float yside = (!RUN && args.has_side) ? __ldg(args.side + i) : 0.0f;
-        float acc = 0.0f;
-        for (uint32_t w = 0; w < args.W; ++w) {
-            if (SIDE == kSideFirst && w == 1u) yside = acc;      // the reconstruction of message 0
-            const DecWorker& wk = args.w[w];
-            const uint32_t kind = wk.variant >> 3;
-            const uint32_t bits = wk.bits;
-            const uint64_t bit = i * bits;
-            const uint64_t num_words = (args.n * bits + 31u) >> 5;
-            uint32_t lo = __ldg(wk.packed + (bit >> 5));
-            const uint32_t sh = (uint32_t)(bit & 31u);
-            uint32_t code = lo >> sh;
-            if (sh + bits > 32u && (bit >> 5) + 1u < num_words) code |= __ldg(wk.packed + (bit >> 5) + 1u) << (32u - sh);
-            code &= (1u << bits) - 1u;
-            uint32_t ctr[1], rnd[1][4];
-            float f;
-            if (DITH == 0) {
-                f = 1.5f;
-            } else if (DITH == 16) {
-                ctr[0] = (uint32_t)(i >> 3);
-                philox4x32_10_xN<1>(ctr, wk.ps, rnd);
-                f = dither16_f12(rnd[0][(i & 7u) >> 1], (int)(i & 1u));
-            } else {
-                ctr[0] = (uint32_t)(i >> 2);
-                philox4x32_10_xN<1>(ctr, wk.ps, rnd);
-                f = dither_f12(rnd[0][i & 3u]);
-            }
-            const float kappa = __ldg(wk.scale + bucket);
-            if (args.status != nullptr && !(fabsf(kappa) <= 3.402823466e38f)) atomicOr(args.status, 0x1u);
-            const float X = __fadd_rn(__uint_as_float((code << 1) | 0x4A800000u), -wk.cconst);
-            float gt;
-            if (kind == kDecDqsg) {
-                gt = __fmul_rn(__fdiv_rn(kappa, wk.s), __fadd_rn(X, -f));
-            } else {
-                const float yy = RUN ? __fmul_rn(acc, wk.rcp_count) : yside;
-                const float a = (kappa >= 0x1p-100f) ? __fdiv_rn(wk.A, kappa) : 0.0f;
-                const float c = __fdiv_rn(__fmul_rn(wk.alpha, kappa), wk.M1);
-                const float r = __fmaf_rn(-yy, a, __fadd_rn(X, -f));
-                const float t = (kind == kDecNdqsgAnyK) ? __fdiv_rn(r, wk.Kf) : __fmul_rn(r, wk.invK);
-                const float jj = __fadd_rn(__fadd_rn(t, kMagic), -kMagic);
-                const float d = __fadd_rn(__fmaf_rn(-wk.Kf, jj, X), -f);
-                gt = (wk.alpha == 1.0f) ? __fmul_rn(c, d) : __fmaf_rn(c, d, __fmul_rn(wk.one_m_alpha2, yy));
-            }
-            acc = __fadd_rn(acc, gt);
-        }
-        args.out[i] = (args.invW != 0.0f) ? __fmul_rn(acc, args.invW) : __fdiv_rn(acc, args.Wf);
+    if (align32) {
+        asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(p), "l"(v[0]), "l"(v[1]), "l"(v[2]), "l"(v[3])
+                     : "memory");
+    } else {
+        asm volatile("st.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(v[0]), "l"(v[1]) : "memory");
+        asm volatile("st.global.v2.b64 [%0], {%1, %2};" ::"l"(p + 4), "l"(v[2]), "l"(v[3]) : "memory");
     }
 }
 
 // ---------------------------------------------------------------------------------------------------
-// The decode kernel.  Grid = persistent CTAs (one per SM) of teams of four warps; dynamic shared memory =
-// kDecSmemBytes.
-// side_map / out_map: [whole rows x 32 floats] views of the caller's side information and output (valid when
-// args.use_tiles; side_map only when args.has_side).
+// The decode kernel: one group of E elements per lane.
 // ---------------------------------------------------------------------------------------------------
-template <int DITH, int SIDE>
-__global__ void __launch_bounds__(kDecThreads, kDecMinBlocks)
-decode_aggregate_kernel(const __grid_constant__ CUtensorMap side_map, const __grid_constant__ CUtensorMap out_map,
-                        const __grid_constant__ DecodeArgs args)
+template <int DITH, int SIDE, int E, bool ALL>
+__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(E))
+decode_aggregate_kernel(const __grid_constant__ DecodeArgs args)
 {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bar_side_mem[kDecWarps][kDecTileBuffers];
+    // per lane: E / 4 slots of side information, then the first Philox products (two blocks per slot)
+    constexpr int N = (DITH == 16) ? E / 8 : E / 4;
+    constexpr int kSlots = E / 4 + (DITH != 0 && N > 1 ? N / 2 : 0);
+    __shared__ __align__(16) float4 slots[kSlots][kDecThreads];
 
-    const uint32_t warp = threadIdx.x >> 5;
-    const uint32_t lane = threadIdx.x & 31u;
-    grid_dependency_launch_next();
-
-    const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t tiles = smem_base + warp * (uint32_t)(kDecTileBuffers * kDecTileBytes);
-    const uint32_t bar_side = smem_u32(&bar_side_mem[warp][0]);
-    const bool side_tiles = SIDE == kSideGiven && args.has_side != 0u && args.use_tiles != 0u;
-
-    if (lane == 0) {
+    const uint64_t local = (uint64_t)blockIdx.x * (uint32_t)kDecThreads + threadIdx.x;
+    if (local >= args.num_groups) return;                       // no barrier below
+    DecLane ln;
+    ln.group = args.first_row * (32u / E) + (uint32_t)local;
+    const uint64_t i0 = (uint64_t)ln.group * (uint32_t)E;
+    const uint32_t row = ln.group / (32u / E);
+    ln.bucket = (args.bucket_magic != 0u) ? (__umulhi(row, args.bucket_magic) >> args.bucket_shift)
+                                          : (row >> args.bucket_shift);
+    ln.slot = smem_u32(&slots[0][threadIdx.x]);
+    ln.kappa_bits_max = 0u;
+    ln.careful = i0 + 64u > args.n;             // the words of a field may reach past the stream's end
+    const bool whole = i0 + (uint32_t)E <= args.n;
+    ln.first[0] = ln.first[1] = 0u;
+    if constexpr (DITH != 0) {
+        uint32_t p[2 * N];
 #pragma unroll
-        for (int i = 0; i < kDecTileBuffers; ++i) mbar_init(bar_side + 8u * i, 1u);
-        fence_mbar_init();
-        if (args.use_tiles) asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&out_map) : "memory");
-        if (side_tiles) asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&side_map) : "memory");
+        for (int j = 0; j < N; ++j) {
+            const uint64_t p0 = (uint64_t)kPhiloxM0 * (ln.group * (uint32_t)N + (uint32_t)j);
+            p[2 * j] = (uint32_t)(p0 >> 32);
+            p[2 * j + 1] = (uint32_t)p0;
+        }
+        ln.first[0] = p[0];
+        ln.first[1] = p[1];
+        if constexpr (N > 1) {
+#pragma unroll
+            for (int j = 0; j < N / 2; ++j)
+                slots[E / 4 + j][threadIdx.x] = make_float4(__uint_as_float(p[4 * j]), __uint_as_float(p[4 * j + 1]),
+                                                            __uint_as_float(p[4 * j + 2]), __uint_as_float(p[4 * j + 3]));
+        }
     }
+    // The next kernel may become resident once every CTA of this one is past its wait, so that at most one kernel
+    // waits beside the running one.  Letting it in at once would let kernel after kernel of a short-call loop pile up,
+    // and the CTAs of one kernel would then be placed wherever slots happen to fall free, several on one SM and none
+    // on others (W = 8, n = 266,610: 11.9 us per call instead of 6.6).  A grid of at most one CTA per SM has nothing to
+    // balance, and gains 0.8 us per call by overlapping two launches.
+    if (args.early_launch != 0u) grid_dependency_launch_next();
     // the messages (and the side information) may be the previous kernel's output
     grid_dependency_wait();
+    if (args.early_launch == 0u) grid_dependency_launch_next();
+    ln.kappa_next = __ldg(args.w[0].scale + ln.bucket);
 
-    // Work: a team-unit is kDecTeamWarps adjacent units (32 rows each), one per warp of a team.  CTA c owns the
-    // team-units c, c + gridDim.x, ...; its teams draw them from a counter in shared memory, one ahead of the
-    // one they work on, so a team that the schedulers favour simply takes more of them and all teams of an SM
-    // finish within one unit of each other.  The warps of a team meet before each unit, so that they run through
-    // the same code at about the same time (teams of one to four warps measure alike, larger ones are slower).
-    __shared__ uint32_t draw_count;
-    __shared__ uint32_t drawn[kDecTeams][2];
-    const uint32_t team = warp / (uint32_t)kDecTeamWarps;
-    const uint32_t tw = warp % (uint32_t)kDecTeamWarps;
-    const uint32_t num_tunits = (args.num_units + (uint32_t)kDecTeamWarps - 1u) / (uint32_t)kDecTeamWarps;
-    const uint32_t cta_tunits = (blockIdx.x < num_tunits) ? (num_tunits - blockIdx.x - 1u) / gridDim.x + 1u : 0u;
-    auto team_meet = [&]() {
-        if constexpr (kDecTeams == 1) __syncthreads();
-        else if constexpr (kDecTeamWarps == 1) __syncwarp();
-        else asm volatile("bar.sync %0, %1;" ::"r"(team + 1u), "n"(kDecTeamWarps * 32) : "memory");
-    };
-    // unit of this warp in the CTA's j-th team-unit (>= num_units: none)
-    auto unit_of = [&](uint32_t j) {
-        return (j < cta_tunits) ? (blockIdx.x + j * gridDim.x) * (uint32_t)kDecTeamWarps + tw : 0xFFFFFFFFu;
-    };
-    if (threadIdx.x == 0) draw_count = 0u;
-    __syncthreads();
-    if (tw == 0u && lane == 0u) drawn[team][0] = atomicAdd(&draw_count, 1u);
-    team_meet();
-    uint32_t unit = unit_of(drawn[team][0]);
-    const uint32_t whole_rows = args.full_rows - args.first_row;       // rows of the tile maps
-
-    // side information of unit `u` -> tile buffer `b` (lane 0)
-    auto issue_side = [&](uint32_t u, uint32_t b) {
-        if (u * 32u >= whole_rows) return;                              // a unit that is only the ragged last row
-        mbar_expect_tx(bar_side + 8u * b, (uint32_t)kDecTileBytes);
-        tma_load_rows(tiles + b * (uint32_t)kDecTileBytes, &side_map, bar_side + 8u * b, (int32_t)(u * 32u));
-    };
-    // Ask the L2 for every worker's packed words of the unit that starts at row `row0`: lane w (and w + 32)
-    // requests the 128-byte lines of worker w, whose words of a unit are 128 * bits contiguous bytes.
-    auto prefetch_words = [&](uint32_t row0) {
-        if (row0 >= args.full_rows) return;
-        for (uint32_t w = lane; w < args.W; w += 32u) {
-            const uint32_t* p = args.w[w].packed + (uint64_t)row0 * args.w[w].bits;
-            const uint32_t rows_left = args.full_rows - row0;
-            const uint32_t lines = (rows_left >= 32u) ? args.w[w].bits : (rows_left * args.w[w].bits + 31u) / 32u;
-            for (uint32_t l = 0; l < lines; ++l) prefetch_l2(p + 32u * l);
-        }
-    };
-    if (lane == 0 && side_tiles && unit < args.num_units) issue_side(unit, 0u);
-    __syncwarp();
-
-    // bucket of a row (rows past the end take the last row's bucket: their results are never stored)
-    auto bucket_of = [&](uint32_t r) {
-        const uint32_t rc = (r < args.rows) ? r : args.rows - 1u;
-        return (args.rpb_shift != 0xFFFFFFFFu) ? (rc >> args.rpb_shift) : (rc / args.rows_per_bucket);
-    };
-
-    // The ragged last row goes first, on the warp that tends to have the least to do: left to the end of the
-    // unit that contains it, its serial chains would be what the whole grid waits for.
-    if (args.full_rows < args.rows && blockIdx.x == gridDim.x - 1u && warp == (uint32_t)kDecWarps - 1u)
-        decode_partial_row<DITH, SIDE>(args, args.full_rows, bucket_of(args.full_rows),
-                                       (uint32_t)(args.n - (uint64_t)args.full_rows * 32u), lane);
-
-    const uint32_t swz16 = (lane & 7u) << 4;
-    bool gave_up = false;
-    uint32_t bucket = bucket_of(args.first_row + (unit < args.num_units ? unit : 0u) * 32u + lane);
-    float kappa_next = __ldg(args.w[0].scale + bucket);
-
-#pragma unroll 1
-    for (uint32_t it = 0; unit != 0xFFFFFFFFu; ++it) {
-        // draw the next team-unit, then meet: everyone has read the previous draw before the one after this
-        if (tw == 0u && lane == 0u) drawn[team][(it + 1u) & 1u] = atomicAdd(&draw_count, 1u);
-        team_meet();
-        const uint32_t unit_next = unit_of(drawn[team][(it + 1u) & 1u]);
-        if (unit >= args.num_units) { unit = unit_next; continue; }    // past the end (last team-unit only)
-        const uint32_t row = args.first_row + unit * 32u + lane;
-        const uint32_t b = it % (uint32_t)kDecTileBuffers;
-        const uint32_t tile = tiles + b * (uint32_t)kDecTileBytes;
-        const bool more = unit_next < args.num_units;
-        const uint32_t bucket_next = more ? bucket_of(args.first_row + unit_next * 32u + lane) : bucket;
-        if (more) prefetch_words(args.first_row + unit_next * 32u);
-        if (lane == 0) {
-            // the store issued two units ago has read its buffer: that buffer takes the next unit's side
-            // information now and this unit's output later
-            bulk_wait_group_read<1>();
-            if (side_tiles && more) issue_side(unit_next, (it + 1u) % (uint32_t)kDecTileBuffers);
-        }
-        __syncwarp();
-        const bool unit_has_tile = unit * 32u < whole_rows;
-        if (side_tiles && unit_has_tile &&
-            !mbar_wait_bounded(bar_side + 8u * b, (it / (uint32_t)kDecTileBuffers) & 1u, gave_up)) {
-            gave_up = true;
-            if (lane == 0) atomicOr(args.error_flags, 0x2u);
-        }
-        const uint32_t row_addr = (tile + lane * 128u) | swz16;
-        // lanes past the last whole row compute on the last whole row's words (in bounds) and are never stored
-        const uint32_t load_row = (row < args.full_rows) ? row : args.full_rows - 1u;
-
-        float acc[32];
+    if (SIDE == kSideGiven && args.has_side != 0u) {
+        const float* s = args.side + i0;
 #pragma unroll
-        for (int e = 0; e < 32; ++e) acc[e] = 0.0f;
-        DecLane ln;
-        ln.row = row; ln.load_row = load_row; ln.bucket = bucket; ln.bucket_next = bucket_next;
-        ln.row_addr = row_addr; ln.kappa_bits_max = 0u; ln.kappa_next = kappa_next;
-        if (unit_has_tile) {
-            decode_workers<DITH, SIDE>(args, ln, acc);
-            kappa_next = ln.kappa_next;
-        } else {
-            kappa_next = __ldg(args.w[0].scale + bucket_next);
+        for (int q = 0; q < E / 4; ++q) {
+            float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (whole) {
+                v = __ldg(reinterpret_cast<const float4*>(s) + q);
+            } else {
+                if (i0 + 4 * q < args.n) v.x = __ldg(s + 4 * q);
+                if (i0 + 4 * q + 1 < args.n) v.y = __ldg(s + 4 * q + 1);
+                if (i0 + 4 * q + 2 < args.n) v.z = __ldg(s + 4 * q + 2);
+                if (i0 + 4 * q + 3 < args.n) v.w = __ldg(s + 4 * q + 3);
+            }
+            slots[q][threadIdx.x] = v;
         }
-        const uint32_t kappa_bits_max = ln.kappa_bits_max;
-        bucket = bucket_next;
-
-        // the mean leaves through the tile buffer: the lane writes its row where it read its side information
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            float v[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                v[e] = (args.W == 1u)        ? acc[4 * c + e]                       // the mean of one message is itself
-                       : (args.invW != 0.0f) ? __fmul_rn(acc[4 * c + e], args.invW)
-                                             : __fdiv_rn(acc[4 * c + e], args.Wf);
-            asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};"
-                         ::"r"(row_addr ^ (uint32_t)(c << 4)), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
-                         : "memory");
-        }
-        fence_proxy_async_shared();
-        __syncwarp();
-        if (lane == 0 && unit_has_tile) {
-            tma_store_rows(&out_map, tile, (int32_t)(unit * 32u));
-            bulk_commit_group();
-        }
-        if (args.status != nullptr && kappa_bits_max >= 0x7F800000u && row < args.full_rows) atomicOr(args.status, 0x1u);
-        unit = unit_next;
     }
-    // shared memory must stay valid until the last stores have read it
-    if (lane == 0) bulk_wait_group_read<0>();
+
+    f32x2 acc[E / 2];
+#pragma unroll
+    for (int e = 0; e < E / 2; ++e) acc[e] = 0ull;
+    decode_workers<DITH, SIDE, E, ALL>(args, ln, acc);
+
+    // the mean (of one message: the message itself)
+    if (args.W > 1u) {
+        const f32x2 nz = args.neg_zero;
+#pragma unroll
+        for (int e = 0; e < E / 2; ++e) {
+            if (args.invW != 0.0f) {
+                acc[e] = fma2(acc[e], both(args.invW), nz);
+            } else {
+                float u, v;
+                unpack2(acc[e], u, v);
+                acc[e] = pack2(__fdiv_rn(u, args.Wf), __fdiv_rn(v, args.Wf));
+            }
+        }
+    }
+    float* o = args.out + i0;
+    if (whole) {
+#pragma unroll
+        for (int k = 0; k < E / 8; ++k) {
+            const f32x2 v[4] = {acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]};
+            store8(o + 8 * k, v, args.out_align32 != 0u);
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < E / 2; ++e) {
+            float u, v;
+            unpack2(acc[e], u, v);
+            if (i0 + 2 * e < args.n) o[2 * e] = u;
+            if (i0 + 2 * e + 1 < args.n) o[2 * e + 1] = v;
+        }
+    }
+    if (args.status != nullptr && ln.kappa_bits_max >= 0x7F800000u) atomicOr(args.status, 0x1u);
 }
 
 }  // namespace dq

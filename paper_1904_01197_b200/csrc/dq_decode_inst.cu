@@ -1,7 +1,5 @@
-// Instantiation of decode_aggregate_kernel for one dither width and one side-information mode (DQ_INST_DITH,
-// DQ_INST_RUN = a DecSide value, given on the compiler's command line).
-#include <atomic>
-
+// Instantiations of decode_aggregate_kernel for one dither width and one side-information mode (DQ_INST_DITH,
+// DQ_INST_RUN = a DecSide value, given on the compiler's command line), all group sizes and both sets of variants.
 #include "dq_decode.cuh"
 #include "dq_launch.h"
 
@@ -14,31 +12,26 @@ namespace dq {
 #define DQ_NAME2(D, R) launch_decode_d##D##_r##R
 #define DQ_NAME(D, R) DQ_NAME2(D, R)
 
-cudaError_t DQ_NAME(DQ_INST_DITH, DQ_INST_RUN)(const CUtensorMap& side_map, const CUtensorMap& out_map,
-                                               const DecodeArgs& a, int sm_count, cudaStream_t st)
+namespace {
+
+template <int E>
+cudaError_t launch_groups_of(const DecodeArgs& a, cudaStream_t st)
 {
-    auto k = decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN>;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    // per device: the shared-memory attribute and the resident CTAs per SM
-    static std::atomic<uint64_t> configured{0};
-    static std::atomic<int> per_sm[64];
-    if (!(configured.load(std::memory_order_acquire) & (1ull << dev))) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDecSmemBytes);
-        if (e != cudaSuccess) return e;
-        int blocks = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, k, kDecThreads, kDecSmemBytes);
-        if (e != cudaSuccess) return e;
-        if (blocks < 1) return cudaErrorLaunchOutOfResources;
-        per_sm[dev].store(blocks);
-        configured.fetch_or(1ull << dev, std::memory_order_release);
-    }
-    const uint32_t smem = kDecSmemBytes;
-    const int blocks = per_sm[dev].load();
-    const uint64_t want = ((uint64_t)a.num_units + kDecTeamWarps - 1u) / kDecTeamWarps;   // one team-unit each at least
-    const uint64_t room = (uint64_t)blocks * (uint64_t)sm_count;
-    const uint32_t grid = (uint32_t)(want < room ? want : room);
-    return launch_overlapped(k, grid, (uint32_t)kDecThreads, smem, st, side_map, out_map, a);
+    const uint32_t grid = (uint32_t)((a.num_groups + kDecThreads - 1u) / kDecThreads);
+    bool usual = true;
+    for (uint32_t w = 0; w < a.W; ++w) usual = usual && is_usual_variant(a.w[w].variant);
+    auto k = usual ? decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, false>
+                   : decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, true>;
+    return launch_overlapped(k, grid, (uint32_t)kDecThreads, 0, st, a);
+}
+
+}  // namespace
+
+cudaError_t DQ_NAME(DQ_INST_DITH, DQ_INST_RUN)(const DecodeArgs& a, int group_size, cudaStream_t st)
+{
+    if (group_size == 32) return launch_groups_of<32>(a, st);
+    if (group_size == 16) return launch_groups_of<16>(a, st);
+    return launch_groups_of<8>(a, st);
 }
 
 }  // namespace dq

@@ -36,29 +36,20 @@ static __constant__ uint64_t c_philox_m0j[8] = {
     0ull * kPhiloxM0, 1ull * kPhiloxM0, 2ull * kPhiloxM0, 3ull * kPhiloxM0,
     4ull * kPhiloxM0, 5ull * kPhiloxM0, 6ull * kPhiloxM0, 7ull * kPhiloxM0};
 
-// N blocks at once, rounds outermost, so N independent dependency chains are in flight.
-// Counter word 0 of block j is c0[j] = index of its 4-element chunk (element index / 4).
+// Rounds 1..9 for N blocks whose first products M0 * c0 (all that round 0 computes per block, and independent of the
+// worker) are given as hi / lo words.
 template <int N>
-__device__ __forceinline__ void philox4x32_10_xN(const uint32_t (&c0in)[N], const PhiloxStream& ps,
-                                                 uint32_t (&out)[N][4])
+__device__ __forceinline__ void philox4x32_10_after_first(const uint32_t (&p0hi)[N], const uint32_t (&p0lo)[N],
+                                                          const PhiloxStream& ps, uint32_t (&out)[N][4])
 {
     uint32_t c0[N], c1[N], c2[N], c3[N];
-    // round 0: only M0*c0 depends on the block
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-        const uint64_t p0 = (uint64_t)kPhiloxM0 * (uint64_t)c0in[j];
-        c2[j] = (uint32_t)(p0 >> 32) ^ ps.v0;
-        c3[j] = (uint32_t)p0;
-    }
-    // round 1: c0, c1 are still block-independent
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint64_t)c2[j];
+        const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint64_t)(p0hi[j] ^ ps.v0);
         c0[j] = (uint32_t)(p1 >> 32) ^ ps.v1;
         c1[j] = (uint32_t)p1;
-        c2[j] = c3[j] ^ ps.v2;
+        c2[j] = p0lo[j] ^ ps.v2;
     }
-    // round 2: c3 is block-independent (folded into v3)
 #pragma unroll
     for (int j = 0; j < N; ++j) {
         const uint64_t p0 = (uint64_t)kPhiloxM0 * (uint64_t)c0[j];
@@ -84,58 +75,20 @@ __device__ __forceinline__ void philox4x32_10_xN(const uint32_t (&c0in)[N], cons
     for (int j = 0; j < N; ++j) { out[j][0] = c0[j]; out[j][1] = c1[j]; out[j][2] = c2[j]; out[j][3] = c3[j]; }
 }
 
-// The same for the N consecutive blocks base + first, ..., base + first + N - 1 of a row (first + N <= 8 and
-// base + 7 < 2^32): see c_philox_m0j.
+// The N consecutive blocks base + first, ..., base + first + N - 1 of a row (first + N <= 8 and base + 7 < 2^32): see
+// c_philox_m0j.
 template <int N>
 __device__ __forceinline__ void philox4x32_10_row(uint32_t base, int first, const PhiloxStream& ps,
                                                   uint32_t (&out)[N][4])
 {
-    uint32_t c0[N], c1[N], c2[N], c3[N];
+    uint32_t hi[N], lo[N];
 #pragma unroll
     for (int j = 0; j < N; ++j) {
         const uint64_t p0 = (uint64_t)kPhiloxM0 * (uint64_t)base + c_philox_m0j[first + j];
-        c2[j] = (uint32_t)(p0 >> 32) ^ ps.v0;
-        c3[j] = (uint32_t)p0;
+        hi[j] = (uint32_t)(p0 >> 32);
+        lo[j] = (uint32_t)p0;
     }
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint64_t)c2[j];
-        c0[j] = (uint32_t)(p1 >> 32) ^ ps.v1;
-        c1[j] = (uint32_t)p1;
-        c2[j] = c3[j] ^ ps.v2;
-    }
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-        const uint64_t p0 = (uint64_t)kPhiloxM0 * (uint64_t)c0[j];
-        const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint64_t)c2[j];
-        c0[j] = (uint32_t)(p1 >> 32) ^ c1[j] ^ ps.rk[2][0];
-        c1[j] = (uint32_t)p1;
-        c2[j] = (uint32_t)(p0 >> 32) ^ ps.v3;
-        c3[j] = (uint32_t)p0;
-    }
-#pragma unroll
-    for (int r = 3; r < 10; ++r) {
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            const uint64_t p0 = (uint64_t)kPhiloxM0 * (uint64_t)c0[j];
-            const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint64_t)c2[j];
-            c0[j] = (uint32_t)(p1 >> 32) ^ c1[j] ^ ps.rk[r][0];
-            c1[j] = (uint32_t)p1;
-            c2[j] = (uint32_t)(p0 >> 32) ^ c3[j] ^ ps.rk[r][1];
-            c3[j] = (uint32_t)p0;
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < N; ++j) { out[j][0] = c0[j]; out[j][1] = c1[j]; out[j][2] = c2[j]; out[j][3] = c3[j]; }
-}
-
-// One block (reference form, all ten rounds written out).
-__device__ __forceinline__ void philox4x32_10(uint32_t c0, const PhiloxStream& ps, uint32_t (&out)[4])
-{
-    const uint32_t in[1] = {c0};
-    uint32_t o[1][4];
-    philox4x32_10_xN<1>(in, ps, o);
-    out[0] = o[0][0]; out[1] = o[0][1]; out[2] = o[0][2]; out[3] = o[0][3];
+    philox4x32_10_after_first<N>(hi, lo, ps, out);
 }
 
 // Dither values without an integer-to-float conversion and with a single integer instruction: the 22 random
@@ -146,11 +99,8 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, const PhiloxStream& p
 //   delta = (2j+1) 2^-23 - 1/2            the dither itself
 constexpr float kTwo127 = 1.7014118346046923e38f;      // 2^127
 constexpr float kTwo125 = 4.2535295865117308e37f;      // 2^125
-
-__device__ __forceinline__ float dither_f12(uint32_t x)
-{
-    return __fmaf_rn(__uint_as_float(x >> 10), kTwo127, 1.00000011920928955078125f);      // 1 + 2^-23
-}
+constexpr float kF32Offset = 1.00000011920928955078125f;   // 1 + 2^-23
+constexpr float kF16Offset = 1.00000762939453125f;         // 1 + 2^-17
 
 __device__ __forceinline__ float dither_delta(uint32_t x)
 {
@@ -164,23 +114,9 @@ __device__ __forceinline__ float half_word_as_small_float(uint32_t word, int hig
     return __uint_as_float(__byte_perm(word, 0u, high ? 0x4324u : 0x4104u));
 }
 
-__device__ __forceinline__ float dither16_f12(uint32_t word, int high)
-{
-    return __fmaf_rn(half_word_as_small_float(word, high), kTwo125, 1.00000762939453125f);   // 1 + 2^-17
-}
-
 __device__ __forceinline__ float dither16_delta(uint32_t word, int high)
 {
     return __fmaf_rn(half_word_as_small_float(word, high), kTwo125, -0.49999237060546875f);  // -(1/2 - 2^-17)
-}
-
-// f of element t (0 .. 4*EPB-1) of a group of four Philox blocks; EPB = elements per block (4 or 8).
-template <int DITH>
-__device__ __forceinline__ float dither_of(const uint32_t (&rnd)[4][4], int t)
-{
-    if (DITH == 0) return 1.5f;                      // no dither at the receiver (half-dithered decoding)
-    if (DITH == 16) return dither16_f12(rnd[t >> 3][(t & 7) >> 1], t & 1);
-    return dither_f12(rnd[t >> 2][t & 3]);
 }
 
 // The dither itself (encoder side).
@@ -189,6 +125,53 @@ __device__ __forceinline__ float dither_delta_of(const uint32_t (&rnd)[4][4], in
 {
     if (DITH == 16) return dither16_delta(rnd[t >> 3][(t & 7) >> 1], t & 1);
     return dither_delta(rnd[t >> 2][t & 3]);
+}
+
+// Pairs of fp32 values in one 64-bit register: one instruction of the packed fp32 unit works on both.  Each half
+// rounds exactly as the scalar operation does (subnormals included).
+//
+// There is no packed multiply here: ptxas contracts mul.rn.f32x2 followed by add.rn.f32x2 into one fused
+// multiply-add, which rounds once where the method's definition rounds twice.  A product is therefore written as
+// fma2(a, b, nz) with nz = a pair of -0.0 whose value the compiler cannot see (it arrives as a kernel argument):
+// x + (-0.0) is x for every x, signed zeros included.
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
+}
+__device__ __forceinline__ f32x2 both(float a) { return pack2(a, a); }
+__device__ __forceinline__ void unpack2(f32x2 d, float& a, float& b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(d));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
+// Random bits of elements t and t + 1 (t even) of a group of Philox blocks as the small floats that one
+// multiply-add turns into the dither: x >> 10 for the 32-bit stream (scale 2^127), the half-words for the 16-bit
+// stream (scale 2^125).
+template <int DITH, int N>
+__device__ __forceinline__ f32x2 dither_bits2(const uint32_t (&rnd)[N][4], int t)
+{
+    if constexpr (DITH == 16) {
+        const uint32_t w = rnd[t >> 3][(t & 7) >> 1];
+        return pack2(half_word_as_small_float(w, 0), half_word_as_small_float(w, 1));
+    } else {
+        return pack2(__uint_as_float(rnd[t >> 2][t & 3] >> 10), __uint_as_float(rnd[t >> 2][(t & 3) + 1] >> 10));
+    }
 }
 
 // Round-to-nearest-even of |w| < 2^22 by adding 1.5 * 2^23: the integer lands in the low mantissa bits.
