@@ -1,13 +1,15 @@
-"""ctypes binding of ``libdq_b200.so``.  Argument marshalling only.
+"""Binding of ``libdq_b200.so``.  Argument marshalling only.
 
 Tensors are ``torch`` CUDA tensors (device entry points) or CPU tensors / numpy arrays (``*_host`` entry
 points); the binding passes their addresses and the current CUDA stream to the C ABI and raises
-``DqError`` on a non-zero status.  There is no fallback: if the shared library is missing the import of
-``lib()`` fails.
+``DqError`` on a non-zero status.  The device entry points go through the native calls of ``dq_calls.so``
+(a small gradient's kernel takes less time than a ctypes call), the rest through ctypes.  There is no
+fallback: if a shared library is missing the first call fails.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 from pathlib import Path
 from typing import Optional, Sequence
 
@@ -23,6 +25,7 @@ DQ_FLAG_OUTPUT_FREE = 0x2
 DQ_FLAG_TEST_DROP_COPY = 0x80000000
 
 _LIB_PATH = Path(__file__).resolve().parent / "lib" / "libdq_b200.so"
+_CALLS_PATH = _LIB_PATH.with_name("dq_calls.so")
 
 
 class DqError(RuntimeError):
@@ -99,6 +102,23 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_calls_module = None
+
+
+def _calls():
+    """The native calls of the device entry points (csrc/dq_calls.cpp)."""
+    global _calls_module
+    if _calls_module is None:
+        lib()
+        if not _CALLS_PATH.exists():
+            raise ImportError(f"{_CALLS_PATH} is missing: run `python -m paper_1904_01197_b200.build`")
+        spec = importlib.util.spec_from_file_location("dq_calls", _CALLS_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _calls_module = module
+    return _calls_module
+
+
 def packed_words(n: int, bits: int) -> int:
     return int(lib().dq_packed_words(n, bits))
 
@@ -150,7 +170,7 @@ def make_params(bucket: int, bits: int, levels: int = 0, coarse_K: int = 0, fine
 
 
 class Message:
-    """A worker's message on the device plus what the decoder must know about it."""
+    """A worker's message plus what the decoder must know about it."""
 
     def __init__(self, packed: torch.Tensor, scale: torch.Tensor, seed: int, worker: int, kind: int,
                  params: DqParams):
@@ -158,13 +178,9 @@ class Message:
         self.seed, self.worker, self.kind, self.params = seed, worker, kind, params
 
     def as_struct(self, host: bool = False) -> DqMsg:
-        if host:
-            pk = _host_ptr(self.packed, torch.int32, "packed")
-            sc = _host_ptr(self.scale, torch.float32, "scale")
-        else:
-            pk = _dev_ptr(self.packed, torch.int32, "packed")
-            sc = _dev_ptr(self.scale, torch.float32, "scale")
-        return DqMsg(pk, sc, self.seed, self.worker, self.kind, self.params)
+        ptr = _host_ptr if host else _dev_ptr
+        return DqMsg(ptr(self.packed, torch.int32, "packed"), ptr(self.scale, torch.float32, "scale"), self.seed,
+                     self.worker, self.kind, self.params)
 
 
 def new_output(numel: int, dtype, device) -> torch.Tensor:
@@ -180,28 +196,28 @@ def alloc_message(n: int, params: DqParams, device="cuda"):
     return packed, scale
 
 
-def _encode(fn, what, grad, seed, worker, step, params, out_packed, out_scale, stream):
-    n = grad.numel()
+def _encode(kind, what, grad, first_element, seed, worker, step, params, out_packed, out_scale, stream):
     if out_packed is None or out_scale is None:
-        out_packed, out_scale = alloc_message(n, params, grad.device)
-    if out_packed.numel() < packed_words(n, params.bits) or out_scale.numel() < num_buckets(n, params.bucket):
-        raise ValueError(f"{what}: output buffers too small")
-    _check(fn(_dev_ptr(grad, torch.float32, "grad"), n, seed, worker, step, C.byref(params),
-              _dev_ptr(out_packed, torch.int32, "out_packed"), _dev_ptr(out_scale, torch.float32, "out_scale"),
-              _stream_ptr(stream)), what)
+        out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
+    status = (_calls_module or _calls()).encode(kind, grad, first_element, seed, worker, step, params, out_packed,
+                                                out_scale, stream)
+    if status != 0:
+        if status < 0:
+            raise ValueError(f"{what}: output buffers too small")
+        raise DqError(status, what)
     return out_packed, out_scale
 
 
 def dqsg_encode(grad: torch.Tensor, seed: int, worker: int, step: int, params: DqParams,
                 out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                 stream=None):
-    return _encode(lib().dqsg_encode, "dqsg_encode", grad, seed, worker, step, params, out_packed, out_scale, stream)
+    return _encode(DQ_KIND_DQSG, "dqsg_encode", grad, 0, seed, worker, step, params, out_packed, out_scale, stream)
 
 
 def ndqsg_encode(grad: torch.Tensor, seed: int, worker: int, step: int, params: DqParams,
                  out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                  stream=None):
-    return _encode(lib().ndqsg_encode, "ndqsg_encode", grad, seed, worker, step, params, out_packed, out_scale, stream)
+    return _encode(DQ_KIND_NDQSG, "ndqsg_encode", grad, 0, seed, worker, step, params, out_packed, out_scale, stream)
 
 
 def bucket_ranges(n: int, bucket: int, parts: int):
@@ -222,31 +238,19 @@ def bucket_ranges(n: int, bucket: int, parts: int):
     return out
 
 
-def _encode_range(fn, what, grad, first_element, seed, worker, step, params, out_packed, out_scale, stream):
-    n = grad.numel()
-    if out_packed is None or out_scale is None:
-        out_packed, out_scale = alloc_message(n, params, grad.device)
-    if out_packed.numel() < packed_words(n, params.bits) or out_scale.numel() < num_buckets(n, params.bucket):
-        raise ValueError(f"{what}: output buffers too small")
-    _check(fn(_dev_ptr(grad, torch.float32, "grad"), n, first_element, seed, worker, step, C.byref(params),
-              _dev_ptr(out_packed, torch.int32, "out_packed"), _dev_ptr(out_scale, torch.float32, "out_scale"),
-              _stream_ptr(stream)), what)
-    return out_packed, out_scale
-
-
 def dqsg_encode_range(grad: torch.Tensor, first_element: int, seed: int, worker: int, step: int, params: DqParams,
                       out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                       stream=None):
     """DQSG encode of the elements [first_element, first_element + grad.numel()) of a longer gradient."""
-    return _encode_range(lib().dqsg_encode_range, "dqsg_encode_range", grad, first_element, seed, worker, step,
-                         params, out_packed, out_scale, stream)
+    return _encode(DQ_KIND_DQSG, "dqsg_encode_range", grad, first_element, seed, worker, step, params, out_packed,
+                   out_scale, stream)
 
 
 def ndqsg_encode_range(grad: torch.Tensor, first_element: int, seed: int, worker: int, step: int, params: DqParams,
                        out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                        stream=None):
-    return _encode_range(lib().ndqsg_encode_range, "ndqsg_encode_range", grad, first_element, seed, worker, step,
-                         params, out_packed, out_scale, stream)
+    return _encode(DQ_KIND_NDQSG, "ndqsg_encode_range", grad, first_element, seed, worker, step, params, out_packed,
+                   out_scale, stream)
 
 
 def _msg_array(msgs: Sequence[Message], host: bool = False):
@@ -256,78 +260,58 @@ def _msg_array(msgs: Sequence[Message], host: bool = False):
     return arr
 
 
-def dqsg_decode_aggregate(msgs: Sequence[Message], n: int, step: int, out_avg: Optional[torch.Tensor] = None,
-                          stream=None) -> torch.Tensor:
+# Which decoder dq_calls.decode runs.
+_DQSG, _NDQSG, _RANGE, _HALF_DITHERED, _RUNNING, _SIDE_FIRST = range(6)
+
+
+def _decode(how, what, msgs, n, first_element, step, side_info, out_avg, status_word, stream):
     if out_avg is None:
         out_avg = new_output(max(1, n), torch.float32, msgs[0].packed.device)
-    _check(lib().dqsg_decode_aggregate(_msg_array(msgs), len(msgs), n, step,
-                                       _dev_ptr(out_avg, torch.float32, "out_avg"), _stream_ptr(stream)),
-           "dqsg_decode_aggregate")
+    status = (_calls_module or _calls()).decode(how, msgs, n, first_element, step, side_info, out_avg, status_word,
+                                                stream)
+    if status != 0:
+        raise DqError(status, what)
     return out_avg
+
+
+def dqsg_decode_aggregate(msgs: Sequence[Message], n: int, step: int, out_avg: Optional[torch.Tensor] = None,
+                          stream=None) -> torch.Tensor:
+    return _decode(_DQSG, "dqsg_decode_aggregate", msgs, n, 0, step, None, out_avg, None, stream)
 
 
 def ndqsg_decode_aggregate(msgs: Sequence[Message], n: int, step: int, side_info: Optional[torch.Tensor],
                            out_avg: Optional[torch.Tensor] = None, status_word: Optional[torch.Tensor] = None,
                            stream=None) -> torch.Tensor:
-    if out_avg is None:
-        out_avg = new_output(max(1, n), torch.float32, msgs[0].packed.device)
-    _check(lib().ndqsg_decode_aggregate(_msg_array(msgs), len(msgs), n, step,
-                                        _dev_ptr(side_info, torch.float32, "side_info"),
-                                        _dev_ptr(out_avg, torch.float32, "out_avg"),
-                                        _dev_ptr(status_word, torch.int32, "status_word"), _stream_ptr(stream)),
-           "ndqsg_decode_aggregate")
-    return out_avg
+    return _decode(_NDQSG, "ndqsg_decode_aggregate", msgs, n, 0, step, side_info, out_avg, status_word, stream)
 
 
 def ndqsg_decode_aggregate_range(msgs: Sequence[Message], n: int, first_element: int, step: int,
                                  side_info: Optional[torch.Tensor], out_avg: Optional[torch.Tensor] = None,
                                  status_word: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Fused decode-and-average of a bucket range: every buffer holds the range's data only."""
-    if out_avg is None:
-        out_avg = new_output(max(1, n), torch.float32, msgs[0].packed.device)
-    _check(lib().ndqsg_decode_aggregate_range(_msg_array(msgs), len(msgs), n, first_element, step,
-                                              _dev_ptr(side_info, torch.float32, "side_info"),
-                                              _dev_ptr(out_avg, torch.float32, "out_avg"),
-                                              _dev_ptr(status_word, torch.int32, "status_word"),
-                                              _stream_ptr(stream)), "ndqsg_decode_aggregate_range")
-    return out_avg
+    return _decode(_RANGE, "ndqsg_decode_aggregate_range", msgs, n, first_element, step, side_info, out_avg, status_word,
+                   stream)
 
 
 def dqsg_decode_aggregate_half_dithered(msgs: Sequence[Message], n: int, out_avg: Optional[torch.Tensor] = None,
                                         stream=None) -> torch.Tensor:
     """Mean of the DQSG messages reconstructed without subtracting the dither (Section 2.1, Lemma 1)."""
-    if out_avg is None:
-        out_avg = new_output(max(1, n), torch.float32, msgs[0].packed.device)
-    _check(lib().dqsg_decode_aggregate_half_dithered(_msg_array(msgs), len(msgs), n,
-                                                     _dev_ptr(out_avg, torch.float32, "out_avg"),
-                                                     _stream_ptr(stream)), "dqsg_decode_aggregate_half_dithered")
-    return out_avg
+    return _decode(_HALF_DITHERED, "dqsg_decode_aggregate_half_dithered", msgs, n, 0, 0, None, out_avg, None, stream)
 
 
 def ndqsg_decode_aggregate_running(msgs: Sequence[Message], n: int, step: int,
                                    out_avg: Optional[torch.Tensor] = None,
                                    status_word: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Algorithm 2's server loop: NDQSG messages are decoded against the mean of the messages before them."""
-    if out_avg is None:
-        out_avg = new_output(max(1, n), torch.float32, msgs[0].packed.device)
-    _check(lib().ndqsg_decode_aggregate_running(_msg_array(msgs), len(msgs), n, step,
-                                                _dev_ptr(out_avg, torch.float32, "out_avg"),
-                                                _dev_ptr(status_word, torch.int32, "status_word"),
-                                                _stream_ptr(stream)), "ndqsg_decode_aggregate_running")
-    return out_avg
+    return _decode(_RUNNING, "ndqsg_decode_aggregate_running", msgs, n, 0, step, None, out_avg, status_word, stream)
 
 
 def ndqsg_decode_aggregate_side_first(msgs: Sequence[Message], n: int, step: int,
                                       out_avg: Optional[torch.Tensor] = None,
                                       status_word: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Algorithm 2 with one P1 worker: the reconstruction of message 0 is the side information of the rest."""
-    if out_avg is None:
-        out_avg = new_output(max(1, n), torch.float32, msgs[0].packed.device)
-    _check(lib().ndqsg_decode_aggregate_side_first(_msg_array(msgs), len(msgs), n, step,
-                                                   _dev_ptr(out_avg, torch.float32, "out_avg"),
-                                                   _dev_ptr(status_word, torch.int32, "status_word"),
-                                                   _stream_ptr(stream)), "ndqsg_decode_aggregate_side_first")
-    return out_avg
+    return _decode(_SIDE_FIRST, "ndqsg_decode_aggregate_side_first", msgs, n, 0, step, None, out_avg, status_word,
+                   stream)
 
 
 def code_histogram(packed: torch.Tensor, n: int, bits: int, hist: Optional[torch.Tensor] = None,
@@ -335,8 +319,7 @@ def code_histogram(packed: torch.Tensor, n: int, bits: int, hist: Optional[torch
     """hist[c] = number of elements of the packed message whose code is c (int64[2^bits] on the device)."""
     if hist is None:
         hist = new_output(1 << bits, torch.int64, packed.device)
-    _check(lib().dq_code_histogram(_dev_ptr(packed, torch.int32, "packed"), n, bits,
-                                   _dev_ptr(hist, torch.int64, "hist"), _stream_ptr(stream)), "dq_code_histogram")
+    _check((_calls_module or _calls()).code_histogram(packed, n, bits, hist, stream), "dq_code_histogram")
     return hist
 
 
@@ -360,9 +343,7 @@ def ternary_pack(packed: torch.Tensor, n: int, out: Optional[torch.Tensor] = Non
     """2-bit stream of a three-level message -> five codes per byte (uint8[ternary_bytes(n)] on the device)."""
     if out is None:
         out = new_output(max(1, ternary_bytes(n)), torch.uint8, packed.device)
-    _check(lib().dq_ternary_pack(_dev_ptr(packed, torch.int32, "packed"), n, _dev_ptr(out, torch.uint8, "out"),
-                                 _dev_ptr(status_word, torch.int32, "status_word"), _stream_ptr(stream)),
-           "dq_ternary_pack")
+    _check((_calls_module or _calls()).ternary_pack(packed, n, out, status_word, stream), "dq_ternary_pack")
     return out
 
 
@@ -370,8 +351,7 @@ def ternary_unpack(data: torch.Tensor, n: int, out: Optional[torch.Tensor] = Non
     """Five codes per byte -> the 2-bit stream (int32[packed_words(n, 2)] on the device)."""
     if out is None:
         out = new_output(max(1, packed_words(n, 2)), torch.int32, data.device)
-    _check(lib().dq_ternary_unpack(_dev_ptr(data, torch.uint8, "data"), n, _dev_ptr(out, torch.int32, "out"),
-                                   _stream_ptr(stream)), "dq_ternary_unpack")
+    _check((_calls_module or _calls()).ternary_unpack(data, n, out, stream), "dq_ternary_unpack")
     return out
 
 

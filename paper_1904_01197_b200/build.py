@@ -2,6 +2,7 @@
 
 The kernels are templates with many instantiations; they are spread over translation units (one per encoder
 mode and dither width, one per decoder variant) that are compiled in parallel and linked into one shared library.
+The Python calls (csrc/dq_calls.cpp) are a second, small library, linked against the first.
 """
 from __future__ import annotations
 
@@ -9,6 +10,7 @@ import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
@@ -16,8 +18,9 @@ PKG = Path(__file__).resolve().parent
 ROOT = PKG.parent
 CSRC = PKG / "csrc"
 LIB = PKG / "lib" / "libdq_b200.so"
+CALLS = PKG / "lib" / "dq_calls.so"
 OBJ = PKG / "lib" / "obj"
-DEPS = sorted(CSRC.glob("*.cu*")) + sorted(CSRC.glob("*.h")) + [ROOT / "include" / "dq.h"]
+DEPS = sorted(CSRC.glob("*.cu*")) + sorted(CSRC.glob("*.h")) + sorted(CSRC.glob("*.cpp")) + [ROOT / "include" / "dq.h"]
 
 NVCC_FLAGS = [
     "-std=c++17", "-O3",
@@ -51,9 +54,9 @@ def source_hash() -> str:
 
 
 def stale() -> bool:
-    if not LIB.exists():
+    if not LIB.exists() or not CALLS.exists():
         return True
-    t = LIB.stat().st_mtime
+    t = min(LIB.stat().st_mtime, CALLS.stat().st_mtime)
     return any(d.stat().st_mtime > t for d in DEPS)
 
 
@@ -75,7 +78,34 @@ def build(force: bool = False, verbose: bool = False, out: Path | None = None, e
         return _build_to(Path(out), list(extra_flags), verbose)
     if not force and not stale():
         return LIB
-    return _build_to(LIB, [], verbose)
+    with ThreadPoolExecutor(max_workers=1) as pool:
+        calls = pool.submit(_compile_calls)
+        lib = _build_to(LIB, [], verbose)
+        _link_calls(calls.result())
+    return lib
+
+
+def _compile_calls() -> Path:
+    import torch
+    from torch.utils.cpp_extension import include_paths
+    OBJ.mkdir(parents=True, exist_ok=True)
+    obj = OBJ / "dq_calls.o"
+    inc = [*include_paths(), sysconfig.get_paths()["include"], str(Path(nvcc_path()).resolve().parents[1] / "include"),
+           str(ROOT / "include")]
+    abi = f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}"
+    subprocess.run([os.environ.get("CXX", "g++"), "-std=c++20", "-O2", "-fPIC", "-fvisibility=hidden", abi,
+                    *[f"-isystem{i}" for i in inc], "-c", "-o", str(obj), str(CSRC / "dq_calls.cpp")], check=True)
+    return obj
+
+
+def _link_calls(obj: Path) -> None:
+    from torch.utils.cpp_extension import library_paths
+    tmp = CALLS.with_suffix(f".{os.getpid()}.tmp")
+    # torch's libraries are in the process before this one is loaded; libdq_b200.so lies beside it
+    subprocess.run([os.environ.get("CXX", "g++"), "-shared", "-o", str(tmp), str(obj),
+                    *[f"-L{d}" for d in library_paths()], "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10_cuda",
+                    "-lc10", f"-L{LIB.parent}", f"-l:{LIB.name}", "-Wl,-rpath,$ORIGIN"], check=True)
+    os.replace(tmp, CALLS)
 
 
 def _build_to(lib: Path, extra_flags, verbose: bool) -> Path:
