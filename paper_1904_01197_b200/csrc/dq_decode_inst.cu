@@ -22,7 +22,7 @@ cudaError_t launch_groups_of(const DecodeArgs& a, cudaStream_t st)
     for (uint32_t w = 0; w < a.W; ++w) usual = usual && is_usual_variant(a.w[w].variant);
     auto k = usual ? decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, false>
                    : decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, true>;
-    return launch_overlapped(k, grid, (uint32_t)kDecThreads, 0, st, a);
+    return launch_overlapped(k, grid, (uint32_t)kDecThreads, 0, st, 1u, a);
 }
 
 }  // namespace

@@ -101,6 +101,8 @@ constexpr float kTwo127 = 1.7014118346046923e38f;      // 2^127
 constexpr float kTwo125 = 4.2535295865117308e37f;      // 2^125
 constexpr float kF32Offset = 1.00000011920928955078125f;   // 1 + 2^-23
 constexpr float kF16Offset = 1.00000762939453125f;         // 1 + 2^-17
+constexpr float kD32Offset = 0.49999988079071044921875f;   // 1/2 - 2^-23
+constexpr float kD16Offset = 0.49999237060546875f;         // 1/2 - 2^-17
 
 __device__ __forceinline__ float dither_delta(uint32_t x)
 {

@@ -69,9 +69,11 @@ struct EncodeArgs {
                                 // time; warps_per_bucket = B / 2048 warps share a bucket (units are buckets)
     float gain_num;          // DQSG: s = (L-1)/2;  NDQSG: A = alpha * M1
     float shift;             // DQSG: s
-    float kmax;              // DQSG: L - 1
+    int32_t kmax;            // DQSG: L - 1
+    f32x2 shift2, magic, two, off;  // pairs of equal values: DQSG s; 1.5 * 2^23; scale and offset of the dither
     uint32_t K;              // NDQSG: coarse ratio
     uint32_t K_offset;       // NDQSG any K: multiple of K that is >= 2^22
+    uint32_t K_magic;        // NDQSG any K: ceil(2^32 / K)
     uint32_t row_offset;     // index of grad[0]'s row in the whole gradient (0 unless a bucket range is encoded):
                              // only the dither counters see it
     uint32_t sm_count;       // SMs of the device            } spacing of the first tile requests,
@@ -95,12 +97,19 @@ __device__ __forceinline__ float max3_abs(float m, float a, float b)
     return d;
 }
 
+__device__ __forceinline__ float max_pair(float m, f32x2 x)
+{
+    float u, v;
+    unpack2(x, u, v);
+    return max3_abs(m, u, v);
+}
+
 // Appends the low BITS bits of `tb` to the row's bit stream.  `sr` is a 32-bit shift register whose top bits are
 // the most recent part of the stream: one funnel shift moves the older codes down and drops the bits of `tb` above
 // the code, so no masking and no shift of the code itself is needed.  `idx` (the element's position in the row) is
 // a compile-time constant after unrolling; a second funnel shift is only needed where a code straddles two words.
-template <int BITS>
-__device__ __forceinline__ void push_code(uint32_t& sr, uint32_t tb, int idx, uint32_t (&out)[BITS])
+template <int BITS, int NW>
+__device__ __forceinline__ void push_code(uint32_t& sr, uint32_t tb, int idx, uint32_t (&out)[NW])
 {
     const int end = (idx + 1) * BITS;                       // stream position after this code
     const int over = end & 31;                              // bits of this code that belong to the next word
@@ -110,53 +119,55 @@ __device__ __forceinline__ void push_code(uint32_t& sr, uint32_t tb, int idx, ui
     if (completes && over == 0) out[(end >> 5) - 1] = sr;
 }
 
-// DQSG: bit pattern kMagicBits + k of one element, k the rounded, clamped index (0 .. L-1).
-//   v = fma(g, a, delta);  w = v + s;  k = clamp(rint(w), 0, L-1)   (clamping before rounding gives the same k)
-__device__ __forceinline__ uint32_t dqsg_index_bits(float x, float a, float delta, const EncodeArgs& args)
+// Code of one element from the bit pattern of 1.5 * 2^23 + (rounded value): the low mantissa bits hold the rounded
+// index (DQSG: before the clamp to 0 .. L-1; NDQSG: two's complement).  Only the low BITS bits of the result count.
+template <int MODE, typename Args>
+__device__ __forceinline__ uint32_t code_of(float t, const Args& args)
 {
-    const float v = __fmaf_rn(x, a, delta);
-    float w = __fadd_rn(v, args.shift);
-    w = fminf(fmaxf(w, 0.0f), args.kmax);
-    return __float_as_uint(__fadd_rn(w, kMagic));                         // rint for 0 <= w < 2^22
+    const uint32_t tb = __float_as_uint(t);
+    if constexpr (MODE == kEncDqsg) {
+        // clamp to [0, L - 1] in one instruction: max(min(tb - bits of 1.5 * 2^23, L - 1), 0)
+        return (uint32_t)__viaddmin_s32_relu((int)tb, -(int)kMagicBits, args.kmax);
+    } else if constexpr (MODE == kEncNdqsgPow2Mask) {
+        return tb & (args.K - 1u);
+    } else if constexpr (MODE == kEncNdqsgAnyK) {
+        // v = q1 + a positive multiple of K, below 2^23 + 2^8; v mod K with the quotient from one high multiply, which
+        // is exact because v (K_magic K - 2^32) < v K < 2^32
+        const uint32_t v = tb - kMagicBits + args.K_offset;
+        return v - args.K * __umulhi(v, args.K_magic);
+    } else {
+        return tb;
+    }
 }
 
-// NDQSG: bit pattern kMagicBits + q1 (two's complement in the low bits) of one element.
-__device__ __forceinline__ uint32_t ndqsg_index_bits(float x, float a, float delta)
-{
-    const float v = __fmaf_rn(x, a, delta);
-    return __float_as_uint(__fadd_rn(v, kMagic));
-}
-
-// Quantize and pack one row.  x: the 32 elements; row: index of the row in the whole gradient (the Philox
+// Quantize and pack one row.  x: the 32 elements as pairs; row: index of the row in the whole gradient (the Philox
 // counters follow from it; it differs from the row's position in this call's buffers when a bucket range is
 // encoded); a: the bucket's gain.  out: the row's BITS words.  DITH: 32 or 16 random bits per dither value.
 //
-// Adding 1.5 * 2^23 leaves the rounded index in the low mantissa bits of a float, so a code costs one fp32 add and
+// Adding 1.5 * 2^23 leaves the rounded index in the low mantissa bits of a float, so a code costs half a packed add and
 // one funnel shift (push_code); only a coarse ratio below 2^BITS needs an extra mask or modulo.
 template <int BITS, int MODE, int DITH>
-__device__ __forceinline__ void encode_row(const float (&x)[32], uint32_t row, float a,
+__device__ __forceinline__ void encode_row(const f32x2 (&x)[16], uint32_t row, float a,
                                            const EncodeArgs& args, uint32_t (&out)[BITS])
 {
     constexpr int EPB = (DITH == 16) ? 8 : 4;       // elements per Philox block
     constexpr int PASS = 4 * EPB;                   // elements per group of four blocks
+    const f32x2 aa = both(a);
     uint32_t sr = 0u;
 #pragma unroll
     for (int h = 0; h < 32 / PASS; ++h) {           // four Philox blocks in flight at a time
         uint32_t rnd[4][4];
         philox4x32_10_row<4>(row * (32u / EPB), 4 * h, args.ps, rnd);
 #pragma unroll
-        for (int t = 0; t < PASS; ++t) {
+        for (int t = 0; t < PASS; t += 2) {
             const int idx = PASS * h + t;
-            const float delta = dither_delta_of<DITH>(rnd, t);
-            uint32_t tb;
-            if (MODE == kEncDqsg) {
-                tb = dqsg_index_bits(x[idx], a, delta, args);
-            } else {
-                tb = ndqsg_index_bits(x[idx], a, delta);
-                if (MODE == kEncNdqsgPow2Mask) tb &= args.K - 1u;
-                if (MODE == kEncNdqsgAnyK) tb = (tb - kMagicBits + args.K_offset) % args.K;   // q1 + positive multiple of K
-            }
-            push_code<BITS>(sr, tb, idx, out);
+            // v = fma(g, a, delta); DQSG: w = v + s; then round to nearest even
+            f32x2 v = fma2(x[idx / 2], aa, fma2(dither_bits2<DITH>(rnd, t), args.two, args.off));
+            if constexpr (MODE == kEncDqsg) v = add2(v, args.shift2);
+            float t0, t1;
+            unpack2(add2(v, args.magic), t0, t1);
+            push_code<BITS>(sr, code_of<MODE>(t0, args), idx, out);
+            push_code<BITS>(sr, code_of<MODE>(t1, args), idx + 1, out);
         }
     }
 }
@@ -188,24 +199,25 @@ __device__ __forceinline__ float bucket_gain(float num, float kappa)
 // ---------------------------------------------------------------------------------------------------
 
 // The `nvalid` (1..32) elements of row `grow` of the gradient, zero-filled.
-__device__ __forceinline__ void load_row_plain(const EncodeArgs& args, uint64_t grow, uint32_t nvalid, float (&x)[32])
+__device__ __forceinline__ void load_row_plain(const EncodeArgs& args, uint64_t grow, uint32_t nvalid, f32x2 (&x)[16])
 {
     const float* g = args.grad + grow * 32u;
     if (nvalid == 32u) {
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const float4 v = reinterpret_cast<const float4*>(g)[c];
-            x[4 * c] = v.x; x[4 * c + 1] = v.y; x[4 * c + 2] = v.z; x[4 * c + 3] = v.w;
+            x[2 * c] = pack2(v.x, v.y); x[2 * c + 1] = pack2(v.z, v.w);
         }
     } else {
 #pragma unroll
-        for (int e = 0; e < 32; ++e) x[e] = ((uint32_t)e < nvalid) ? g[e] : 0.0f;
+        for (int e = 0; e < 32; e += 2)
+            x[e / 2] = pack2(((uint32_t)e < nvalid) ? g[e] : 0.0f, ((uint32_t)e + 1u < nvalid) ? g[e + 1] : 0.0f);
     }
 }
 
 // Quantizes and stores row `grow` (already in registers) with the bucket's gain `a`.
 template <int BITS, int MODE, int DITH>
-__device__ __forceinline__ void encode_store_row_plain(const EncodeArgs& args, const float (&x)[32], uint64_t grow,
+__device__ __forceinline__ void encode_store_row_plain(const EncodeArgs& args, const f32x2 (&x)[16], uint64_t grow,
                                                        uint32_t nvalid, float a)
 {
     uint32_t out[BITS];
@@ -237,12 +249,12 @@ __device__ __forceinline__ void encode_window_plain(const EncodeArgs& args, uint
     const uint64_t grow = (args.first_bucket * rpb) + window * rows_per_window + lane;
     const bool active = lane < rows_per_window && grow < total_rows;
     const uint32_t nvalid = !active ? 0u : (args.n - grow * 32u < 32u) ? (uint32_t)(args.n - grow * 32u) : 32u;
-    float x[32];
+    f32x2 x[16];
     float mx = 0.0f;
     if (active) {
         load_row_plain(args, grow, nvalid, x);
 #pragma unroll
-        for (int e = 0; e < 32; e += 2) mx = max3_abs(mx, x[e], x[e + 1]);
+        for (int e = 0; e < 16; ++e) mx = max_pair(mx, x[e]);
     }
     // lanes of one bucket are adjacent: take the neighbour's maximum while it belongs to the same bucket
     const uint32_t seg = lane / rpb;
@@ -280,7 +292,7 @@ __device__ __forceinline__ void encode_bucket_warp_plain(const EncodeArgs& args,
     for (uint32_t r = lane; r < rows; r += 32u) {
         const uint32_t nvalid = (len - r * 32u < 32u) ? (len - r * 32u) : 32u;
         const uint64_t grow = (lo >> 5) + r;
-        float x[32];
+        f32x2 x[16];
         load_row_plain(args, grow, nvalid, x);
         encode_store_row_plain<BITS, MODE, DITH>(args, x, grow, nvalid, a);
     }
@@ -317,7 +329,7 @@ __device__ __forceinline__ void encode_bucket_cta_plain(const EncodeArgs& args, 
     for (uint32_t r = threadIdx.x; r < rows; r += (uint32_t)kEncThreads) {
         const uint32_t nvalid = (len - r * 32u < 32u) ? (len - r * 32u) : 32u;
         const uint64_t grow = (lo >> 5) + r;
-        float x[32];
+        f32x2 x[16];
         load_row_plain(args, grow, nvalid, x);
         encode_store_row_plain<BITS, MODE, DITH>(args, x, grow, nvalid, a);
     }
@@ -432,7 +444,7 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
         for (uint32_t pair = first_tile; pair < args.num_units; pair += stride, ++k) {
             const uint32_t par = k & 1u;
             const uint32_t part = pair * wpb + sub;      // index of this warp's 2048 elements in the gradient
-            float x[32];
+            f32x2 x[16];
             float mx = 0.0f;
 #pragma unroll 1
             for (uint32_t half = 0; half < 2u; ++half) {
@@ -457,14 +469,14 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
                 }
 #pragma unroll
                 for (uint32_t c = 0; c < 8; ++c) {
-                    asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
-                                 : "=f"(x[4 * c]), "=f"(x[4 * c + 1]), "=f"(x[4 * c + 2]), "=f"(x[4 * c + 3])
+                    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
+                                 : "=l"(x[2 * c]), "=l"(x[2 * c + 1])
                                  : "r"(stage_addr ^ (c << 4))
                                  : "memory");
                 }
                 if (half == 0u) {
 #pragma unroll
-                    for (int e = 0; e < 32; e += 2) mx = max3_abs(mx, x[e], x[e + 1]);
+                    for (int e = 0; e < 16; ++e) mx = max_pair(mx, x[e]);
 #pragma unroll
                     for (uint32_t off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, off));
                     if (wpb > 1u) {
@@ -479,7 +491,7 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
                 } else {
                     uint32_t sink = 0u;                 // all loads of this half have completed after this
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) sink ^= __float_as_uint(x[4 * c]);
+                    for (int c = 0; c < 8; ++c) sink ^= (uint32_t)x[2 * c];
                     asm volatile("" ::"r"(sink));
                 }
                 __syncwarp();
@@ -516,12 +528,12 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
             if (lane == 0) atomicOr(args.error_flags, 0x2u);
         }
         // the lane's row -> registers
-        float x[32];
+        f32x2 x[16];
         const uint32_t row_addr = (my_smem + s * kWarpTileBytes + lane * 128u) | swz16;
 #pragma unroll
         for (uint32_t c = 0; c < 8; ++c) {
-            asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];"
-                         : "=f"(x[4 * c]), "=f"(x[4 * c + 1]), "=f"(x[4 * c + 2]), "=f"(x[4 * c + 3])
+            asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];"
+                         : "=l"(x[2 * c]), "=l"(x[2 * c + 1])
                          : "r"(row_addr ^ (c << 4))
                          : "memory");
         }
@@ -529,7 +541,7 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
         // __syncwarp below, so after it the stage can be overwritten by the next copy.
         float mx = 0.0f;
 #pragma unroll
-        for (int e = 0; e < 32; e += 2) mx = max3_abs(mx, x[e], x[e + 1]);
+        for (int e = 0; e < 16; ++e) mx = max_pair(mx, x[e]);
 #pragma unroll
         for (uint32_t off = 16; off > 0; off >>= 1) {
             const float o = __shfl_xor_sync(0xFFFFFFFFu, mx, off);

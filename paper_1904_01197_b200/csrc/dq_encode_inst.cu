@@ -3,6 +3,7 @@
 #include <atomic>
 
 #include "dq_encode.cuh"
+#include "dq_encode_direct.cuh"
 #include "dq_launch.h"
 
 #ifndef DQ_INST_MODE
@@ -25,7 +26,15 @@ cudaError_t launch_one(const CUtensorMap& map, const EncodeArgs& a, uint32_t gri
         if (e != cudaSuccess) return e;
         configured.fetch_or(1ull << dev, std::memory_order_release);
     }
-    return launch_overlapped(k, grid, (uint32_t)kEncThreads, kEncSmemBytes, st, map, a);
+    return launch_overlapped(k, grid, (uint32_t)kEncThreads, kEncSmemBytes, st, 1u, map, a);
+}
+
+template <int BITS>
+cudaError_t launch_direct_one(int R, const DirectArgs& a, uint32_t grid, uint32_t threads, cudaStream_t st)
+{
+    auto k = R == 1 ? encode_direct_kernel<BITS, DQ_INST_MODE, DQ_INST_DITH, 1>
+                    : encode_direct_kernel<BITS, DQ_INST_MODE, DQ_INST_DITH, 4>;
+    return launch_overlapped(k, grid, threads, 0, st, a.cluster, a);
 }
 
 }  // namespace
@@ -45,6 +54,24 @@ cudaError_t DQ_NAME(DQ_INST_MODE, DQ_INST_DITH)(uint32_t bits, const CUtensorMap
         case 6: return launch_one<6>(map, a, grid, st);
         case 7: return launch_one<7>(map, a, grid, st);
         default: return launch_one<8>(map, a, grid, st);
+    }
+}
+
+#define DQ_DNAME2(M, D) launch_direct_m##M##_d##D
+#define DQ_DNAME(M, D) DQ_DNAME2(M, D)
+
+cudaError_t DQ_DNAME(DQ_INST_MODE, DQ_INST_DITH)(uint32_t bits, int R, const DirectArgs& a, uint32_t grid,
+                                                  uint32_t threads, cudaStream_t st)
+{
+    switch (bits) {
+        case 1: return launch_direct_one<1>(R, a, grid, threads, st);
+        case 2: return launch_direct_one<2>(R, a, grid, threads, st);
+        case 3: return launch_direct_one<3>(R, a, grid, threads, st);
+        case 4: return launch_direct_one<4>(R, a, grid, threads, st);
+        case 5: return launch_direct_one<5>(R, a, grid, threads, st);
+        case 6: return launch_direct_one<6>(R, a, grid, threads, st);
+        case 7: return launch_direct_one<7>(R, a, grid, threads, st);
+        default: return launch_direct_one<8>(R, a, grid, threads, st);
     }
 }
 

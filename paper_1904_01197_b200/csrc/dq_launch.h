@@ -13,6 +13,7 @@
 namespace dq {
 
 struct EncodeArgs;
+struct DirectArgs;
 struct DecodeArgs;
 
 // Launch with programmatic stream serialization allowed: every kernel of this library executes
@@ -21,18 +22,25 @@ struct DecodeArgs;
 // latency.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_overlapped(void (*kernel)(KArgs...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t st,
-                              Args&&... args)
+                              uint32_t cluster, Args&&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (cluster > 1u) {
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = cluster;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+    }
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
@@ -43,6 +51,14 @@ cudaError_t launch_overlapped(void (*kernel)(KArgs...), uint32_t grid, uint32_t 
 DQ_DECLARE_ENCODE(0, 32) DQ_DECLARE_ENCODE(1, 32) DQ_DECLARE_ENCODE(2, 32) DQ_DECLARE_ENCODE(3, 32)
 DQ_DECLARE_ENCODE(0, 16) DQ_DECLARE_ENCODE(1, 16) DQ_DECLARE_ENCODE(2, 16) DQ_DECLARE_ENCODE(3, 16)
 #undef DQ_DECLARE_ENCODE
+
+// The same for the direct encoder; R = groups per lane, 1 or 4.
+#define DQ_DECLARE_DIRECT(MODE, DITH)                                                                              \
+    cudaError_t launch_direct_m##MODE##_d##DITH(uint32_t bits, int R, const DirectArgs& a, uint32_t grid,          \
+                                                uint32_t threads, cudaStream_t st);
+DQ_DECLARE_DIRECT(0, 32) DQ_DECLARE_DIRECT(1, 32) DQ_DECLARE_DIRECT(2, 32) DQ_DECLARE_DIRECT(3, 32)
+DQ_DECLARE_DIRECT(0, 16) DQ_DECLARE_DIRECT(1, 16) DQ_DECLARE_DIRECT(2, 16) DQ_DECLARE_DIRECT(3, 16)
+#undef DQ_DECLARE_DIRECT
 
 // Decoder: dith = 32, 16 or 0 (no dither at the receiver); run = DecSide (0 given vector or none, 1 running mean,
 // 2 reconstruction of message 0).
