@@ -474,6 +474,42 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     return DQ_OK;
 }
 
+// CTAs in the histogram's cluster: 16 (which needs an attribute per kernel and device) where one can be resident, else
+// the portable 8; 0 on a CUDA error.
+uint32_t hist_cluster_size()
+{
+    static std::mutex mu;
+    static uint32_t size[kMaxDevices] = {};
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0u;
+    std::lock_guard<std::mutex> lock(mu);
+    if (size[dev] == 0u) {
+        uint32_t s = 8u;
+        bool ok = true;
+        for (auto k : {dq::code_histogram_cluster_kernel<1>, dq::code_histogram_cluster_kernel<2>})
+            ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        if (ok) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(dq::kHistCluster);
+            cfg.blockDim = dim3(dq::kHistClusterThreads);
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = dq::kHistCluster;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            int clusters = 0;
+            if (cudaOccupancyMaxActiveClusters(&clusters, dq::code_histogram_cluster_kernel<2>, &cfg) == cudaSuccess &&
+                clusters > 0)
+                s = (uint32_t)dq::kHistCluster;
+        }
+        cudaGetLastError();
+        size[dev] = s;
+    }
+    return size[dev];
+}
+
 uint64_t align_up(uint64_t v, uint64_t a) { return (v + a - 1u) / a * a; }
 
 }  // namespace
@@ -576,19 +612,34 @@ dq_status dq_code_histogram(const uint32_t* packed, uint64_t n, uint32_t bits, u
     if (!hist) return DQ_ERR_INVALID_ARG;
     if (n >= (1ull << 34)) return DQ_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    if (n != 0 && !packed) return DQ_ERR_INVALID_ARG;
+    if (n != 0 && (!aligned16(packed) || (reinterpret_cast<uintptr_t>(hist) & 7u) != 0u)) return DQ_ERR_ALIGNMENT;
+    static_assert(sizeof(unsigned long long) == sizeof(uint64_t), "histogram counters are 64-bit");
+    unsigned long long* h = reinterpret_cast<unsigned long long*>(hist);
+    if (n != 0 && bits <= 2u && n * bits <= 8u * dq::kHistClusterBytes) {
+        const uint32_t cluster = hist_cluster_size();
+        if (cluster == 0u) return DQ_ERR_CUDA;
+        // no CTA without at least two 16-byte pieces per warp
+        uint32_t ctas = 1u;
+        while (ctas < cluster && n * bits > 128u * 64u * ctas) ctas *= 2u;
+        auto k = bits == 1u ? dq::code_histogram_cluster_kernel<1> : dq::code_histogram_cluster_kernel<2>;
+        if (launch_overlapped(k, ctas, (uint32_t)dq::kHistClusterThreads, 0, st, ctas, packed, n, h) != cudaSuccess)
+            return DQ_ERR_CUDA;
+        g_launches.fetch_add(1);
+        return DQ_OK;
+    }
     if (cudaMemsetAsync(hist, 0, sizeof(uint64_t) << bits, st) != cudaSuccess) return DQ_ERR_CUDA;
     if (n == 0) return DQ_OK;
-    if (!packed) return DQ_ERR_INVALID_ARG;
-    if (!aligned16(packed) || (reinterpret_cast<uintptr_t>(hist) & 7u) != 0u) return DQ_ERR_ALIGNMENT;
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
     const uint64_t rows = (n + 31u) / 32u;
     uint64_t grid = (rows + dq::kHistThreads - 1u) / dq::kHistThreads;
-    if (grid > (uint64_t)sms * 8u) grid = (uint64_t)sms * 8u;
-    static_assert(sizeof(unsigned long long) == sizeof(uint64_t), "histogram counters are 64-bit");
-    if (launch_overlapped(dq::code_histogram_kernel, (uint32_t)grid, (uint32_t)dq::kHistThreads, 0, st, 1u, packed, n,
-                          bits, reinterpret_cast<unsigned long long*>(hist)) != cudaSuccess)
-        return DQ_ERR_CUDA;
+    if (grid > (uint64_t)sms * 6u) grid = (uint64_t)sms * 6u;
+    const uint32_t g = (uint32_t)grid, t = (uint32_t)dq::kHistThreads;
+    const cudaError_t e = bits == 1u   ? launch_overlapped(dq::code_histogram_words_kernel<1>, g, t, 0, st, 1u, packed, n, h)
+                          : bits == 2u ? launch_overlapped(dq::code_histogram_words_kernel<2>, g, t, 0, st, 1u, packed, n, h)
+                                       : launch_overlapped(dq::code_histogram_kernel, g, t, 0, st, 1u, packed, n, bits, h);
+    if (e != cudaSuccess) return DQ_ERR_CUDA;
     g_launches.fetch_add(1);
     return DQ_OK;
 }

@@ -1,5 +1,11 @@
 // Histogram of the codes of a packed message: the input of the paper's rate accounting (entropy of the index
-// stream, Section 4, tables of raw and entropy-coded bits).  Not on the hot path; one pass over the packed words.
+// stream, Section 4, tables of raw and entropy-coded bits).  One pass over the packed words.
+//
+// One and two bits are counted by population counts of whole words; wider codes one by one into shared memory.
+// Messages of one- and two-bit codes up to kHistClusterBytes are counted by a single cluster of CTAs, whose partial
+// counts meet in the first CTA's shared memory: the counters are written once, so they need not be cleared first.  A
+// second launch (or a memset, which the next kernel cannot overlap) costs more than the cluster's fewer SMs do
+// (2 bits: n = 65,536 6.2 us for memset and count, HIST_SMALL us for the cluster).
 #pragma once
 
 #include "dq_device.cuh"
@@ -7,18 +13,129 @@
 namespace dq {
 
 constexpr int kHistThreads = 256;
+constexpr int kHistClusterThreads = 1024;
+constexpr int kHistCluster = 16;                       // 8 where a cluster of 16 cannot be resident
+constexpr uint64_t kHistClusterBytes = 4ull << 20;
 
-// Each warp counts into its own 256-bin histogram in shared memory (no contention between warps); the CTA's
-// histograms are added to the global one at the end.  A thread handles one row (32 codes, `bits` words) at a time.
+// Counts of the codes 1, 2 and 3 (of the code 1 with one bit) in a stretch of words.
+struct FewCounts { uint32_t c1, c2, c3; };
+
+// Two words of 2-bit codes: three population counts, the codes of the second word beside those of the first.
+__device__ __forceinline__ void count2(uint32_t a, uint32_t b, FewCounts& f)
+{
+    const uint32_t m = 0x55555555u;
+    const uint32_t lo = (a & m) | ((b & m) << 1), hi = ((a >> 1) & m) | (b & ~m);
+    f.c1 += __popc(lo & ~hi);
+    f.c2 += __popc(hi & ~lo);
+    f.c3 += __popc(lo & hi);
+}
+
+template <int BITS>
+__device__ __forceinline__ void count_words(const uint32_t* __restrict__ packed, uint64_t n, uint64_t first, uint64_t stride,
+                                            FewCounts& f)
+{
+    const uint64_t quads = (n * BITS) >> 7;            // 16-byte pieces without pad bits
+    auto count = [&](const uint4& v) {
+        if constexpr (BITS == 1) {
+            f.c1 += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+        } else {
+            count2(v.x, v.y, f);
+            count2(v.z, v.w, f);
+        }
+    };
+    const uint4* p = reinterpret_cast<const uint4*>(packed);
+    uint64_t i = first;
+    for (; i + 3u * stride < quads; i += 4u * stride) {        // four loads in flight
+        uint4 v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = __ldg(p + i + (uint64_t)j * stride);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) count(v[j]);
+    }
+    for (; i < quads; i += stride) count(__ldg(p + i));
+    if (first == 0u) {                                 // what is left: at most four words, the last one partly pad
+        for (uint64_t w = quads * 4u; w * 32u < n * BITS; ++w) {
+            const uint64_t left = n * BITS - w * 32u;
+            uint4 v = make_uint4(__ldg(packed + w) & (left >= 32u ? 0xFFFFFFFFu : (1u << (uint32_t)left) - 1u), 0u, 0u, 0u);
+            count(v);
+        }
+    }
+}
+
+// Adds every thread's counts into sums[0..2] (shared memory, zero on entry; the caller synchronises before and after).
+__device__ __forceinline__ void add_counts(const FewCounts& f, uint32_t* sums)
+{
+    const uint32_t a = __reduce_add_sync(0xFFFFFFFFu, f.c1), b = __reduce_add_sync(0xFFFFFFFFu, f.c2),
+                   c = __reduce_add_sync(0xFFFFFFFFu, f.c3);
+    if ((threadIdx.x & 31u) == 0u) {
+        atomicAdd(sums, a);
+        atomicAdd(sums + 1, b);
+        atomicAdd(sums + 2, c);
+    }
+}
+
+// One cluster counts everything and writes the counters (fewer than 2^32 codes).
+template <int BITS>
+__global__ void __launch_bounds__(kHistClusterThreads)
+code_histogram_cluster_kernel(const uint32_t* __restrict__ packed, uint64_t n, unsigned long long* hist)
+{
+    __shared__ uint32_t sums[3], total[3];
+    if (threadIdx.x < 3u) sums[threadIdx.x] = total[threadIdx.x] = 0u;
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    grid_dependency_launch_next();
+    grid_dependency_wait();
+    FewCounts f = {0u, 0u, 0u};
+    count_words<BITS>(packed, n, (uint64_t)blockIdx.x * kHistClusterThreads + threadIdx.x,
+                      (uint64_t)gridDim.x * kHistClusterThreads, f);
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");        // total[] of CTA 0 is zero
+    add_counts(f, sums);
+    __syncthreads();
+    if (threadIdx.x < 3u) {
+        uint32_t remote;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(smem_u32(total + threadIdx.x)));
+        asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(remote), "r"(sums[threadIdx.x]) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (blockIdx.x == 0u && threadIdx.x < (1u << BITS))
+        hist[threadIdx.x] = threadIdx.x == 0u ? n - total[0] - total[1] - total[2] : total[threadIdx.x - 1u];
+}
+
+// Longer messages of one- and two-bit codes; hist has been cleared.
+template <int BITS>
+__global__ void __launch_bounds__(kHistThreads)
+code_histogram_words_kernel(const uint32_t* __restrict__ packed, uint64_t n, unsigned long long* hist)
+{
+    __shared__ uint32_t sums[3];
+    if (threadIdx.x < 3u) sums[threadIdx.x] = 0u;
+    grid_dependency_wait();
+    grid_dependency_launch_next();
+    FewCounts f = {0u, 0u, 0u};
+    count_words<BITS>(packed, n, (uint64_t)blockIdx.x * kHistThreads + threadIdx.x, (uint64_t)gridDim.x * kHistThreads, f);
+    __syncthreads();
+    add_counts(f, sums);
+    __syncthreads();
+    if (threadIdx.x < (1u << BITS) - 1u) {
+        atomicAdd(hist + 1 + threadIdx.x, (unsigned long long)sums[threadIdx.x]);
+        atomicAdd(hist, 0ull - (unsigned long long)sums[threadIdx.x]);          // (modulo 2^64)
+    }
+    if (blockIdx.x == 0u && threadIdx.x == 31u) atomicAdd(hist, (unsigned long long)n);
+}
+
+// Wider codes; hist has been cleared.  Up to five bits every thread has counters of its own (no two lanes of a warp meet
+// in a shared-memory bank); beyond that each warp has 256.  A thread handles one row (32 codes, `bits` words) at a time.
 __global__ void __launch_bounds__(kHistThreads)
 code_histogram_kernel(const uint32_t* __restrict__ packed, uint64_t n, uint32_t bits, unsigned long long* hist)
 {
-    __shared__ uint32_t bins[kHistThreads / 32][256];
+    __shared__ uint32_t bins[32 * kHistThreads];
     grid_dependency_wait();
     grid_dependency_launch_next();
-    const uint32_t warp = threadIdx.x >> 5;
-    for (uint32_t i = threadIdx.x; i < (kHistThreads / 32) * 256u; i += kHistThreads) (&bins[0][0])[i] = 0u;
+    const bool own = bits <= 5u;
+    const uint32_t used = own ? (1u << bits) * kHistThreads : (kHistThreads / 32) * 256u;
+    for (uint32_t i = threadIdx.x; i < used; i += kHistThreads) bins[i] = 0u;
     __syncthreads();
+    const uint32_t base = own ? threadIdx.x : (threadIdx.x >> 5) * 256u;
+    const uint32_t step = own ? (uint32_t)kHistThreads : 1u;
 
     const uint64_t rows = (n + 31u) >> 5;
     const uint64_t num_words = (n * bits + 31u) >> 5;
@@ -39,18 +156,28 @@ code_histogram_kernel(const uint32_t* __restrict__ packed, uint64_t n, uint32_t 
                 lo = hi >> (bits - have);
                 have += 32u - bits;
             } else {
-                lo = (bits < 32u) ? (lo >> bits) : 0u;
+                lo >>= bits;
                 have -= bits;
             }
-            atomicAdd(&bins[warp][code & mask], 1u);
+            atomicAdd(&bins[base + (code & mask) * step], 1u);
         }
     }
     __syncthreads();
-    for (uint32_t b = threadIdx.x; b <= mask; b += kHistThreads) {
-        unsigned long long s = 0ull;
+    if (own) {
+        // a warp adds up the counters of one code at a time
+        for (uint32_t b = threadIdx.x >> 5; b <= mask; b += kHistThreads / 32) {
+            uint32_t s = 0u;
+            for (uint32_t t = threadIdx.x & 31u; t < (uint32_t)kHistThreads; t += 32u) s += bins[b * kHistThreads + t];
+            s = __reduce_add_sync(0xFFFFFFFFu, s);
+            if ((threadIdx.x & 31u) == 0u && s != 0u) atomicAdd(hist + b, (unsigned long long)s);
+        }
+    } else {
+        for (uint32_t b = threadIdx.x; b <= mask; b += kHistThreads) {
+            unsigned long long s = 0ull;
 #pragma unroll
-        for (int w = 0; w < kHistThreads / 32; ++w) s += bins[w][b];
-        if (s) atomicAdd(hist + b, s);
+            for (int w = 0; w < kHistThreads / 32; ++w) s += bins[w * 256 + b];
+            if (s) atomicAdd(hist + b, s);
+        }
     }
 }
 

@@ -71,6 +71,20 @@ ternary_pack_kernel(const uint32_t* __restrict__ packed, uint64_t n, uint8_t* __
 __global__ void __launch_bounds__(kTernaryThreads)
 ternary_unpack_kernel(const uint8_t* __restrict__ data, uint64_t n, uint32_t* __restrict__ packed)
 {
+    // the five base-3 digits of every byte value as five 2-bit codes, filled in while the previous kernel drains: a look-up
+    // per byte instead of five divisions by three
+    __shared__ uint16_t digits[256];
+    static_assert(kTernaryThreads == 256, "a thread per table entry");
+    {
+        uint32_t v = threadIdx.x, g = 0u;
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {                          // code q of the byte = digit q of v in base 3
+            g |= (v % 3u) << (2 * q);
+            v /= 3u;
+        }
+        digits[threadIdx.x] = (uint16_t)g;
+    }
+    __syncthreads();
     grid_dependency_wait();
     grid_dependency_launch_next();
     const uint64_t unit = (uint64_t)blockIdx.x * kTernaryThreads + threadIdx.x;
@@ -91,13 +105,7 @@ ternary_unpack_kernel(const uint8_t* __restrict__ data, uint64_t n, uint32_t* __
     uint32_t w[5] = {0u, 0u, 0u, 0u, 0u};
 #pragma unroll
     for (int b = 0; b < 16; ++b) {
-        uint32_t v = (in[b >> 2] >> (8 * (b & 3))) & 0xFFu;
-        uint32_t g = 0u;
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {                          // code q of the byte = digit q of v in base 3
-            g |= (v % 3u) << (2 * q);
-            v /= 3u;
-        }
+        const uint32_t g = digits[(in[b >> 2] >> (8 * (b & 3))) & 0xFFu];
         const int bit = 10 * b, wi = bit >> 5, sh = bit & 31;
         w[wi] |= g << sh;
         if (sh + 10 > 32) w[wi + 1] |= g >> (32 - sh);
