@@ -196,28 +196,32 @@ def alloc_message(n: int, params: DqParams, device="cuda"):
     return packed, scale
 
 
-def _encode(kind, what, grad, first_element, seed, worker, step, params, out_packed, out_scale, stream):
-    if out_packed is None or out_scale is None:
-        out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
-    status = (_calls_module or _calls()).encode(kind, grad, first_element, seed, worker, step, params, out_packed,
-                                                out_scale, stream)
-    if status != 0:
-        if status < 0:
-            raise ValueError(f"{what}: output buffers too small")
-        raise DqError(status, what)
-    return out_packed, out_scale
+def _encode_failed(status, what):
+    if status < 0:
+        raise ValueError(f"{what}: output buffers too small")
+    raise DqError(status, what)
 
 
 def dqsg_encode(grad: torch.Tensor, seed: int, worker: int, step: int, params: DqParams,
                 out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                 stream=None):
-    return _encode(DQ_KIND_DQSG, "dqsg_encode", grad, 0, seed, worker, step, params, out_packed, out_scale, stream)
+    if out_packed is None or out_scale is None:
+        out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
+    status = (_calls_module or _calls()).encode(DQ_KIND_DQSG, grad, 0, seed, worker, step, params, out_packed, out_scale, stream)
+    if status:
+        _encode_failed(status, "dqsg_encode")
+    return out_packed, out_scale
 
 
 def ndqsg_encode(grad: torch.Tensor, seed: int, worker: int, step: int, params: DqParams,
                  out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                  stream=None):
-    return _encode(DQ_KIND_NDQSG, "ndqsg_encode", grad, 0, seed, worker, step, params, out_packed, out_scale, stream)
+    if out_packed is None or out_scale is None:
+        out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
+    status = (_calls_module or _calls()).encode(DQ_KIND_NDQSG, grad, 0, seed, worker, step, params, out_packed, out_scale, stream)
+    if status:
+        _encode_failed(status, "ndqsg_encode")
+    return out_packed, out_scale
 
 
 def bucket_ranges(n: int, bucket: int, parts: int):
@@ -238,19 +242,29 @@ def bucket_ranges(n: int, bucket: int, parts: int):
     return out
 
 
+def _encode_range(kind, what, grad, first_element, seed, worker, step, params, out_packed, out_scale, stream):
+    if out_packed is None or out_scale is None:
+        out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
+    status = (_calls_module or _calls()).encode(kind, grad, first_element, seed, worker, step, params, out_packed,
+                                                out_scale, stream)
+    if status:
+        _encode_failed(status, what)
+    return out_packed, out_scale
+
+
 def dqsg_encode_range(grad: torch.Tensor, first_element: int, seed: int, worker: int, step: int, params: DqParams,
                       out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                       stream=None):
     """DQSG encode of the elements [first_element, first_element + grad.numel()) of a longer gradient."""
-    return _encode(DQ_KIND_DQSG, "dqsg_encode_range", grad, first_element, seed, worker, step, params, out_packed,
-                   out_scale, stream)
+    return _encode_range(DQ_KIND_DQSG, "dqsg_encode_range", grad, first_element, seed, worker, step, params, out_packed,
+                         out_scale, stream)
 
 
 def ndqsg_encode_range(grad: torch.Tensor, first_element: int, seed: int, worker: int, step: int, params: DqParams,
                        out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                        stream=None):
-    return _encode(DQ_KIND_NDQSG, "ndqsg_encode_range", grad, first_element, seed, worker, step, params, out_packed,
-                   out_scale, stream)
+    return _encode_range(DQ_KIND_NDQSG, "ndqsg_encode_range", grad, first_element, seed, worker, step, params, out_packed,
+                         out_scale, stream)
 
 
 def _msg_array(msgs: Sequence[Message], host: bool = False):

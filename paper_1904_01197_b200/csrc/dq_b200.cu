@@ -382,8 +382,8 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
                         bool side_first = false)
 {
     if (!msgs || W == 0u || W > DQ_MAX_WORKERS) return DQ_ERR_INVALID_ARG;
-    static thread_local dq::DecodeArgs a;    // ~10 KB: keep it off the stack
-    std::memset(&a, 0, sizeof(a));
+    static thread_local dq::DecodeArgs a;    // ~13 KB: keep it off the stack; the first W entries of a.w are filled
+    std::memset(static_cast<dq::DecodeHead*>(&a), 0, sizeof(dq::DecodeHead));
     bool any_nested = false;
     for (uint32_t w = 0; w < W; ++w) {
         const dq_msg& m = msgs[w];
@@ -395,6 +395,7 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
         if (m.p.bucket != msgs[0].p.bucket) return DQ_ERR_UNSUPPORTED;
         if (!half_dithered && (m.p.dither_bits == 16u) != (msgs[0].p.dither_bits == 16u)) return DQ_ERR_UNSUPPORTED;
         dq::DecWorker& d = a.w[w];
+        std::memset(&d, 0, sizeof(d));
         // addresses of the (virtual) whole-gradient buffers: see DecodeArgs
         d.packed = virtual_base(m.packed, first_element / 32u * m.p.bits);
         d.scale = virtual_base(m.scale, first_element / m.p.bucket);
@@ -634,11 +635,19 @@ dq_status dq_code_histogram(const uint32_t* packed, uint64_t n, uint32_t bits, u
     if (sms <= 0) return DQ_ERR_CUDA;
     const uint64_t rows = (n + 31u) / 32u;
     uint64_t grid = (rows + dq::kHistThreads - 1u) / dq::kHistThreads;
-    if (grid > (uint64_t)sms * 6u) grid = (uint64_t)sms * 6u;
+    if (grid > (uint64_t)sms * 4u) grid = (uint64_t)sms * 4u;
     const uint32_t g = (uint32_t)grid, t = (uint32_t)dq::kHistThreads;
-    const cudaError_t e = bits == 1u   ? launch_overlapped(dq::code_histogram_words_kernel<1>, g, t, 0, st, 1u, packed, n, h)
-                          : bits == 2u ? launch_overlapped(dq::code_histogram_words_kernel<2>, g, t, 0, st, 1u, packed, n, h)
-                                       : launch_overlapped(dq::code_histogram_kernel, g, t, 0, st, 1u, packed, n, bits, h);
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (bits) {
+        case 1: e = launch_overlapped(dq::code_histogram_words_kernel<1>, g, t, 0, st, 1u, packed, n, h); break;
+        case 2: e = launch_overlapped(dq::code_histogram_words_kernel<2>, g, t, 0, st, 1u, packed, n, h); break;
+        case 3: e = launch_overlapped(dq::code_histogram_kernel<3>, g, t, 0, st, 1u, packed, n, h); break;
+        case 4: e = launch_overlapped(dq::code_histogram_kernel<4>, g, t, 0, st, 1u, packed, n, h); break;
+        case 5: e = launch_overlapped(dq::code_histogram_kernel<5>, g, t, 0, st, 1u, packed, n, h); break;
+        case 6: e = launch_overlapped(dq::code_histogram_kernel<6>, g, t, 0, st, 1u, packed, n, h); break;
+        case 7: e = launch_overlapped(dq::code_histogram_kernel<7>, g, t, 0, st, 1u, packed, n, h); break;
+        default: e = launch_overlapped(dq::code_histogram_kernel<8>, g, t, 0, st, 1u, packed, n, h); break;
+    }
     if (e != cudaSuccess) return DQ_ERR_CUDA;
     g_launches.fetch_add(1);
     return DQ_OK;

@@ -47,7 +47,7 @@ struct DecWorker {
                           // exact multiplication); 0 otherwise
 };
 
-struct DecodeArgs {
+struct DecodeHead {
     const float* side;
     float* out;
     uint32_t* status;
@@ -70,13 +70,21 @@ struct DecodeArgs {
     f32x2 neg_zero;           // -0.0 twice (see f32x2)           } constants that would otherwise be assembled from
     f32x2 magic, neg_magic;   // +-1.5 * 2^23 twice               } immediates again and again
     float invW;               // 1/W when W is a power of two, else 0
-    DecWorker w[64];
 };
+
+// Kernel parameters for up to MAXW workers.  A launch copies all of them: 0.8 us more for 64 workers (13 KB) than for 8,
+// which counts for short gradients (kDecFewWorkers).
+template <int MAXW>
+struct DecodeArgsOf : DecodeHead {
+    DecWorker w[MAXW];
+};
+using DecodeArgs = DecodeArgsOf<64>;
+constexpr int kDecFewWorkers = 8;
 
 // Division of a row index below 2^29 by rows_per_bucket as a multiplication: with s = floor(log2 d) and
 // m = ceil(2^(32+s) / d), m d - 2^(32+s) < d < 2^(s+1) <= 2^(32+s) / 2^29, which is what makes
 // floor(row m / 2^(32+s)) exact.
-inline void set_bucket_division(DecodeArgs& a)
+inline void set_bucket_division(DecodeHead& a)
 {
     const uint32_t d = a.rows_per_bucket;
     uint32_t s = 0u;
@@ -177,8 +185,8 @@ struct DecLane {
 //   NDQSG: r = (m - delta) - y a;  jj = rint(r / K);  q1^ = m - K jj;  g~ = beta (q1^ - delta) [+ (1-alpha^2) y]
 // AHEAD: the packed words are requested one worker ahead (worth its registers with 20 warps per SM, i.e. E = 32: 4 %;
 // with 32 warps it costs as much).
-template <int BITS, uint32_t KIND, int DITH, int SIDE, int E, bool AHEAD>
-__device__ __forceinline__ void decode_run(const DecodeArgs& args, uint32_t w, uint32_t w_end, DecLane& ln,
+template <int BITS, uint32_t KIND, int DITH, int SIDE, int E, bool AHEAD, typename Args>
+__device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_t w_end, DecLane& ln,
                                            f32x2 (&acc)[E / 2])
 {
     constexpr bool RUN = SIDE == kSideRunning;
@@ -296,8 +304,8 @@ __device__ __forceinline__ void decode_run(const DecodeArgs& args, uint32_t w, u
 inline bool is_usual_variant(uint32_t variant) { return (variant >> 3) <= kDecNdqsgPow2 && (variant & 7u) < 4u; }
 
 // All W workers, run by run; dispatch on (kind, bits) with one jump per run.  ALL: every variant, else the usual ones.
-template <int DITH, int SIDE, int E, bool ALL>
-__device__ __forceinline__ void decode_workers(const DecodeArgs& args, DecLane& ln, f32x2 (&acc)[E / 2])
+template <int DITH, int SIDE, int E, bool ALL, typename Args>
+__device__ __forceinline__ void decode_workers(const Args& args, DecLane& ln, f32x2 (&acc)[E / 2])
 {
 #define DQ_DEC_CASE(KIND, BITS)                                                                                    \
     case (KIND) * 8u + (BITS) - 1u:                                                                                \
@@ -348,9 +356,9 @@ __device__ __forceinline__ void store8(float* p, const f32x2 (&v)[4], bool align
 // ---------------------------------------------------------------------------------------------------
 // The decode kernel: one group of E elements per lane.
 // ---------------------------------------------------------------------------------------------------
-template <int DITH, int SIDE, int E, bool ALL>
+template <int DITH, int SIDE, int E, bool ALL, int MAXW>
 __global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(E))
-decode_aggregate_kernel(const __grid_constant__ DecodeArgs args)
+decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
 {
     // per lane: E / 4 slots of side information, then the first Philox products (two blocks per slot)
     constexpr int N = (DITH == 16) ? E / 8 : E / 4;

@@ -14,7 +14,8 @@ namespace dq {
 
 struct EncodeArgs;
 struct DirectArgs;
-struct DecodeArgs;
+template <int MAXW> struct DecodeArgsOf;
+using DecodeArgs = DecodeArgsOf<64>;
 
 // Launch with programmatic stream serialization allowed: every kernel of this library executes
 // griddepcontrol.wait before it writes anything, and before it reads anything that the previous kernel of the

@@ -44,15 +44,15 @@ __device__ __forceinline__ void count_words(const uint32_t* __restrict__ packed,
         }
     };
     const uint4* p = reinterpret_cast<const uint4*>(packed);
-    uint64_t i = first;
-    for (; i + 3u * stride < quads; i += 4u * stride) {        // four loads in flight
-        uint4 v[4];
+    constexpr int kFlight = 8;                         // loads in flight: a short message is two or three latencies
+    for (uint64_t i = first; i < quads; i += kFlight * stride) {
+        uint4 v[kFlight];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) v[j] = __ldg(p + i + (uint64_t)j * stride);
+        for (int j = 0; j < kFlight; ++j)
+            v[j] = i + (uint64_t)j * stride < quads ? __ldg(p + i + (uint64_t)j * stride) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) count(v[j]);
+        for (int j = 0; j < kFlight; ++j) count(v[j]);
     }
-    for (; i < quads; i += stride) count(__ldg(p + i));
     if (first == 0u) {                                 // what is left: at most four words, the last one partly pad
         for (uint64_t w = quads * 4u; w * 32u < n * BITS; ++w) {
             const uint64_t left = n * BITS - w * 32u;
@@ -123,59 +123,51 @@ code_histogram_words_kernel(const uint32_t* __restrict__ packed, uint64_t n, uns
 }
 
 // Wider codes; hist has been cleared.  Up to five bits every thread has counters of its own (no two lanes of a warp meet
-// in a shared-memory bank); beyond that each warp has 256.  A thread handles one row (32 codes, `bits` words) at a time.
+// in a shared-memory bank); beyond that each warp has 256.  A thread handles one row (32 codes, BITS words) at a time.
+template <int BITS>
 __global__ void __launch_bounds__(kHistThreads)
-code_histogram_kernel(const uint32_t* __restrict__ packed, uint64_t n, uint32_t bits, unsigned long long* hist)
+code_histogram_kernel(const uint32_t* __restrict__ packed, uint64_t n, unsigned long long* hist)
 {
-    __shared__ uint32_t bins[32 * kHistThreads];
+    constexpr bool kOwn = BITS <= 5;
+    constexpr uint32_t kBins = 1u << BITS, kWarps = kHistThreads / 32;
+    constexpr uint32_t kStep = kOwn ? (uint32_t)kHistThreads : 1u;
+    __shared__ uint32_t bins[kOwn ? kBins * kHistThreads : kBins * kWarps];
+    for (uint32_t i = threadIdx.x; i < sizeof(bins) / 4u; i += kHistThreads) bins[i] = 0u;
+    __syncthreads();
     grid_dependency_wait();
     grid_dependency_launch_next();
-    const bool own = bits <= 5u;
-    const uint32_t used = own ? (1u << bits) * kHistThreads : (kHistThreads / 32) * 256u;
-    for (uint32_t i = threadIdx.x; i < used; i += kHistThreads) bins[i] = 0u;
-    __syncthreads();
-    const uint32_t base = own ? threadIdx.x : (threadIdx.x >> 5) * 256u;
-    const uint32_t step = own ? (uint32_t)kHistThreads : 1u;
+    uint32_t* mine = bins + (kOwn ? threadIdx.x : (threadIdx.x >> 5) * kBins);
 
     const uint64_t rows = (n + 31u) >> 5;
-    const uint64_t num_words = (n * bits + 31u) >> 5;
-    const uint32_t mask = (1u << bits) - 1u;
+    const uint64_t num_words = (n * BITS + 31u) >> 5;
     for (uint64_t row = (uint64_t)blockIdx.x * kHistThreads + threadIdx.x; row < rows;
          row += (uint64_t)gridDim.x * kHistThreads) {
         const uint32_t valid = (row * 32u + 32u <= n) ? 32u : (uint32_t)(n - row * 32u);
-        const uint64_t w0 = row * bits;
-        uint32_t lo = __ldg(packed + w0);
-        uint32_t next_word = 1u;
-        uint32_t have = 32u;                                     // unread bits left in `lo`
-        for (uint32_t e = 0; e < valid; ++e) {
-            uint32_t code = lo;
-            if (have < bits) {                                   // the code straddles into the next word
-                const uint32_t hi = (w0 + next_word < num_words) ? __ldg(packed + w0 + next_word) : 0u;
-                ++next_word;
-                code |= hi << have;
-                lo = hi >> (bits - have);
-                have += 32u - bits;
-            } else {
-                lo >>= bits;
-                have -= bits;
-            }
-            atomicAdd(&bins[base + (code & mask) * step], 1u);
+        uint32_t w[BITS];
+#pragma unroll
+        for (int j = 0; j < BITS; ++j) w[j] = (row * BITS + j < num_words) ? __ldg(packed + row * BITS + j) : 0u;
+#pragma unroll
+        for (int e = 0; e < 32; ++e) {
+            const int bit = e * BITS, wi = bit >> 5, sh = bit & 31;
+            const uint32_t v = (sh + BITS <= 32) ? (w[wi] >> sh) : __funnelshift_r(w[wi], w[(wi + 1) % BITS], sh);
+            if ((uint32_t)e < valid) atomicAdd(mine + (v & (kBins - 1u)) * kStep, 1u);
         }
     }
     __syncthreads();
-    if (own) {
+    if constexpr (kOwn) {
         // a warp adds up the counters of one code at a time
-        for (uint32_t b = threadIdx.x >> 5; b <= mask; b += kHistThreads / 32) {
+        for (uint32_t b = threadIdx.x >> 5; b < kBins; b += kWarps) {
             uint32_t s = 0u;
-            for (uint32_t t = threadIdx.x & 31u; t < (uint32_t)kHistThreads; t += 32u) s += bins[b * kHistThreads + t];
+#pragma unroll
+            for (uint32_t t = 0; t < (uint32_t)kHistThreads; t += 32u) s += bins[b * kHistThreads + t + (threadIdx.x & 31u)];
             s = __reduce_add_sync(0xFFFFFFFFu, s);
             if ((threadIdx.x & 31u) == 0u && s != 0u) atomicAdd(hist + b, (unsigned long long)s);
         }
     } else {
-        for (uint32_t b = threadIdx.x; b <= mask; b += kHistThreads) {
+        for (uint32_t b = threadIdx.x; b < kBins; b += kHistThreads) {
             unsigned long long s = 0ull;
 #pragma unroll
-            for (int w = 0; w < kHistThreads / 32; ++w) s += bins[w * 256 + b];
+            for (uint32_t w = 0; w < kWarps; ++w) s += bins[w * kBins + b];
             if (s) atomicAdd(hist + b, s);
         }
     }
