@@ -207,7 +207,8 @@ def dqsg_encode(grad: torch.Tensor, seed: int, worker: int, step: int, params: D
                 stream=None):
     if out_packed is None or out_scale is None:
         out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
-    status = (_calls_module or _calls()).encode(DQ_KIND_DQSG, grad, 0, seed, worker, step, params, out_packed, out_scale, stream)
+    status = (_calls_module or _calls()).encode(DQ_KIND_DQSG, grad, 0, seed, worker, step, params, out_packed, out_scale,
+                                                stream)
     if status:
         _encode_failed(status, "dqsg_encode")
     return out_packed, out_scale
@@ -218,7 +219,8 @@ def ndqsg_encode(grad: torch.Tensor, seed: int, worker: int, step: int, params: 
                  stream=None):
     if out_packed is None or out_scale is None:
         out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
-    status = (_calls_module or _calls()).encode(DQ_KIND_NDQSG, grad, 0, seed, worker, step, params, out_packed, out_scale, stream)
+    status = (_calls_module or _calls()).encode(DQ_KIND_NDQSG, grad, 0, seed, worker, step, params, out_packed, out_scale,
+                                                stream)
     if status:
         _encode_failed(status, "ndqsg_encode")
     return out_packed, out_scale

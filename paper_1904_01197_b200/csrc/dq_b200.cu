@@ -629,8 +629,9 @@ dq_status dq_code_histogram(const uint32_t* packed, uint64_t n, uint32_t bits, u
         g_launches.fetch_add(1);
         return DQ_OK;
     }
-    if (cudaMemsetAsync(hist, 0, sizeof(uint64_t) << bits, st) != cudaSuccess) return DQ_ERR_CUDA;
-    if (n == 0) return DQ_OK;
+    if (n == 0) return cudaMemsetAsync(hist, 0, sizeof(uint64_t) << bits, st) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+    if (launch_overlapped(dq::clear_histogram_kernel, 1u, 1u << bits, 0, st, 1u, h) != cudaSuccess) return DQ_ERR_CUDA;
+    g_launches.fetch_add(1);
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
     const uint64_t rows = (n + 31u) / 32u;

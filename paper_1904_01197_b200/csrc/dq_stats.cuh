@@ -3,9 +3,10 @@
 //
 // One and two bits are counted by population counts of whole words; wider codes one by one into shared memory.
 // Messages of one- and two-bit codes up to kHistClusterBytes are counted by a single cluster of CTAs, whose partial
-// counts meet in the first CTA's shared memory: the counters are written once, so they need not be cleared first.  A
-// second launch (or a memset, which the next kernel cannot overlap) costs more than the cluster's fewer SMs do
-// (2 bits: n = 65,536 6.2 us for memset and count, HIST_SMALL us for the cluster).
+// counts meet in the first CTA's shared memory: the counters are written once, so they need not be cleared first, and
+// one launch is all (2 bits, n = 65,536: 6.2 us with a memset, 2.4 us).  Longer messages take the whole GPU and a small
+// kernel before it that clears the counters: the count can begin to launch while it runs, which it cannot behind a
+// memset.
 #pragma once
 
 #include "dq_device.cuh"
@@ -15,7 +16,14 @@ namespace dq {
 constexpr int kHistThreads = 256;
 constexpr int kHistClusterThreads = 1024;
 constexpr int kHistCluster = 16;                       // 8 where a cluster of 16 cannot be resident
-constexpr uint64_t kHistClusterBytes = 4ull << 20;
+constexpr uint64_t kHistClusterBytes = 3ull << 19;
+
+__global__ void __launch_bounds__(kHistThreads) clear_histogram_kernel(unsigned long long* hist)
+{
+    grid_dependency_launch_next();
+    grid_dependency_wait();
+    hist[threadIdx.x] = 0ull;
+}
 
 // Counts of the codes 1, 2 and 3 (of the code 1 with one bit) in a stretch of words.
 struct FewCounts { uint32_t c1, c2, c3; };
@@ -44,14 +52,15 @@ __device__ __forceinline__ void count_words(const uint32_t* __restrict__ packed,
         }
     };
     const uint4* p = reinterpret_cast<const uint4*>(packed);
-    constexpr int kFlight = 8;                         // loads in flight: a short message is two or three latencies
+    constexpr int kFlight = 4;                         // loads in flight: a short message is two or three latencies
     for (uint64_t i = first; i < quads; i += kFlight * stride) {
         uint4 v[kFlight];
 #pragma unroll
         for (int j = 0; j < kFlight; ++j)
-            v[j] = i + (uint64_t)j * stride < quads ? __ldg(p + i + (uint64_t)j * stride) : make_uint4(0u, 0u, 0u, 0u);
+            if (i + (uint64_t)j * stride < quads) v[j] = __ldg(p + i + (uint64_t)j * stride);
 #pragma unroll
-        for (int j = 0; j < kFlight; ++j) count(v[j]);
+        for (int j = 0; j < kFlight; ++j)
+            if (i + (uint64_t)j * stride < quads) count(v[j]);
     }
     if (first == 0u) {                                 // what is left: at most four words, the last one partly pad
         for (uint64_t w = quads * 4u; w * 32u < n * BITS; ++w) {

@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 
 from test_gpu_parity import dq  # noqa: E402,F401
 
-CLUSTER_BITS = 8 * (4 << 20)            # longest message that one cluster counts
+CLUSTER_BITS = 8 * (3 << 19)            # longest message that one cluster counts
 
 
 @pytest.mark.parametrize("bits", range(1, 9))
