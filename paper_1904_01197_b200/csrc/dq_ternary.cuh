@@ -16,13 +16,19 @@ namespace dq {
 constexpr int kTernaryThreads = 256;
 constexpr uint32_t kWarnCodeRange = 0x4u;      // DQ_WARN_CODE_RANGE
 
-// The ten bits (five 2-bit codes) that start at bit 10*b of a unit's 160-bit string.
-__device__ __forceinline__ uint32_t ten_bits(const uint32_t (&w)[5], int b)
+// Two container bytes (the second one 8 bits up) from the ten codes that start at bit 20*k of a unit's 160-bit string.
+// 4^i turns into 3^i by subtraction: a pair of codes x = c0 + 4 c1 is worth x - c1, and c0 + 4 c1 + 64 (...) likewise, so
+// a byte costs six integer instructions instead of twelve (n = 30 M: 6.8 -> 4.8 us per call).
+__device__ __forceinline__ uint32_t two_bytes(const uint32_t (&w)[5], int k)
 {
-    const int bit = 10 * b, wi = bit >> 5, sh = bit & 31;
-    uint32_t v = w[wi] >> sh;
-    if (sh + 10 > 32) v |= w[wi + 1] << (32 - sh);
-    return v & 0x3FFu;
+    const int bit = 20 * k, wi = bit >> 5, sh = bit & 31;
+    const uint32_t f = (sh + 20 > 32) ? __funnelshift_r(w[wi], w[wi + 1], sh) : (w[wi] >> sh);
+    // codes 0 1 | 2 3 | 4, 5 | 6 7 | 8 9: the four whole pairs become nibbles 0..8, codes 4 and 5 stay as they are
+    const uint32_t y = f - ((f >> 2) & 0x33033u);
+    const uint32_t lo = y & 0xFFu, mid = (y >> 8) & 3u, z = (y >> 10) & 0x3FFu;
+    const uint32_t b0 = lo - 7u * (lo >> 4) + 81u * mid;                        // N0 + 9 N1 + 81 c4
+    const uint32_t b1 = z - ((z >> 2) & 15u) - 37u * (z >> 6);                  // c5 + 3 N3 + 27 N4
+    return b0 + (b1 << 8);
 }
 
 __global__ void __launch_bounds__(kTernaryThreads)
@@ -35,13 +41,14 @@ ternary_pack_kernel(const uint32_t* __restrict__ packed, uint64_t n, uint8_t* __
     const uint64_t num_words = (n + 15u) >> 4;
     const uint64_t num_bytes = (n + 4u) / 5u;
     const uint64_t left = n - unit * 80u;                      // codes from the start of this unit to the end
+    const bool whole = left >= 80u;
     uint32_t w[5];
     uint32_t bad = 0u;
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
         const uint64_t wi = unit * 5u + j;
-        uint32_t v = (wi < num_words) ? __ldg(packed + wi) : 0u;
-        if (left < 16u * (j + 1)) {                            // codes past the end count as 0
+        uint32_t v = (whole || wi < num_words) ? __ldg(packed + wi) : 0u;
+        if (!whole && left < 16u * (j + 1)) {                  // codes past the end count as 0
             const uint32_t keep = (left > 16u * j) ? (uint32_t)(left - 16u * j) : 0u;
             v = keep ? (v & (0xFFFFFFFFu >> (32u - 2u * keep))) : 0u;
         }
@@ -52,12 +59,7 @@ ternary_pack_kernel(const uint32_t* __restrict__ packed, uint64_t n, uint8_t* __
     if (bad != 0u && status != nullptr) atomicOr(status, kWarnCodeRange);
     uint32_t o[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-    for (int b = 0; b < 16; ++b) {
-        const uint32_t g = ten_bits(w, b);
-        const uint32_t byte = (g & 3u) + 3u * ((g >> 2) & 3u) + 9u * ((g >> 4) & 3u) + 27u * ((g >> 6) & 3u) +
-                              81u * (g >> 8);
-        o[b >> 2] |= byte << (8 * (b & 3));
-    }
+    for (int k = 0; k < 8; ++k) o[k >> 1] |= two_bytes(w, k) << (16 * (k & 1));
     const uint64_t byte0 = unit * 16u;
     if (byte0 + 16u <= num_bytes) {
         reinterpret_cast<uint4*>(out)[unit] = make_uint4(o[0], o[1], o[2], o[3]);
@@ -92,6 +94,7 @@ ternary_unpack_kernel(const uint8_t* __restrict__ data, uint64_t n, uint32_t* __
     const uint64_t num_words = (n + 15u) >> 4;
     const uint64_t num_bytes = (n + 4u) / 5u;
     const uint64_t left = n - unit * 80u;
+    const bool whole = left >= 80u;
     const uint64_t byte0 = unit * 16u;
     uint32_t in[4] = {0u, 0u, 0u, 0u};
     if (byte0 + 16u <= num_bytes) {
@@ -113,9 +116,9 @@ ternary_unpack_kernel(const uint8_t* __restrict__ data, uint64_t n, uint32_t* __
 #pragma unroll
     for (int j = 0; j < 5; ++j) {
         const uint64_t wi = unit * 5u + j;
-        if (wi >= num_words) break;
+        if (!whole && wi >= num_words) break;
         uint32_t v = w[j];
-        if (left < 16u * (j + 1)) {                            // pad bits of the last word are written as 0
+        if (!whole && left < 16u * (j + 1)) {                          // pad bits of the last word are written as 0
             const uint32_t keep = (uint32_t)(left - 16u * j);  // >= 1 because wi < num_words
             v &= 0xFFFFFFFFu >> (32u - 2u * keep);
         }
