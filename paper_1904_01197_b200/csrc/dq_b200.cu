@@ -727,6 +727,68 @@ uint64_t dq_decode_workspace_bytes(const dq_msg* msgs, uint32_t W, uint64_t n, i
     return total;
 }
 
+namespace {
+
+// The *_host calls move their data in one of three ways:
+//   - short gradients in pinned memory: no copies at all, the kernels read and write the host buffers over the bus (a
+//     copy costs 4 us of set-up, and a decode has two per message);
+//   - long ones: in pieces, so that the copies of one direction, the kernels and the copies of the other direction run
+//     side by side (the bus moves 55 GB/s in each direction at once);
+//   - everything else: copy in, kernel, copy out.
+constexpr uint64_t kHostDirectElements = 1ull << 20;       // up to here without copies
+constexpr uint64_t kHostPieceElements = 1ull << 21;        // from here in pieces
+constexpr int kHostPieces = 4;
+
+// Device address of pinned host memory, null for any other (or for one that is not 16-byte aligned).
+template <typename T>
+T* pinned_view(T* host)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (at.type != cudaMemoryTypeHost || !at.devicePointer || !aligned16(at.devicePointer)) return nullptr;
+    return static_cast<T*>(const_cast<void*>(static_cast<const void*>(at.devicePointer)));
+}
+
+// A second stream and the events that tie it to the caller's: one set per host thread and device, made at the thread's
+// first long *_host call on the device and given back when the thread ends.
+struct HostPipe {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t arrived[kHostPieces] = {};
+    bool make()
+    {
+        if (stream) return true;
+        for (cudaEvent_t& e : arrived)
+            if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
+        return cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) == cudaSuccess;
+    }
+    ~HostPipe()
+    {
+        for (cudaEvent_t e : arrived)
+            if (e) cudaEventDestroy(e);
+        if (stream) cudaStreamDestroy(stream);
+    }
+};
+
+HostPipe* host_pipe()
+{
+    static thread_local HostPipe pipes[kMaxDevices];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    return pipes[dev].make() ? &pipes[dev] : nullptr;
+}
+
+// Start of piece i when n elements are cut at `sixteenths[i]` sixteenths: a multiple of four buckets, so that every
+// buffer's piece is 16-byte aligned.
+uint64_t piece_start(uint64_t n, uint32_t bucket, uint32_t sixteenths)
+{
+    return sixteenths >= 16u ? n : n / 16u * sixteenths / (4u * bucket) * (4u * bucket);
+}
+
+}  // namespace
+
 static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64_t seed, uint32_t worker,
                              uint64_t step, const dq_params* p, uint32_t* out_packed, float* out_scale,
                              void* workspace, uint64_t workspace_bytes, void* cuda_stream)
@@ -741,6 +803,17 @@ static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0u) return DQ_ERR_ALIGNMENT;
     if (workspace_bytes < dq_encode_workspace_bytes(n, p)) return DQ_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    const bool plain = (p->flags & DQ_FLAG_TEST_DROP_COPY) != 0u;        // (the hook is about one launch)
+    if (!plain && n <= kHostDirectElements) {
+        const float* h_grad = pinned_view(grad);
+        uint32_t* h_packed = h_grad ? pinned_view(out_packed) : nullptr;
+        float* h_scale = h_packed ? pinned_view(out_scale) : nullptr;
+        if (h_scale) {
+            s = encode_common(kind, h_grad, n, seed, worker, step, p, h_packed, h_scale, st);
+            if (s != DQ_OK) return s;
+            return cudaStreamSynchronize(st) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+        }
+    }
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     float* d_grad = reinterpret_cast<float*>(ws);
     ws += align_up(n * 4u, 256u);
@@ -749,6 +822,31 @@ static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64
     ws += align_up(pbytes, 256u);
     float* d_scale = reinterpret_cast<float*>(ws);
     const uint64_t sbytes = dq_num_buckets(n, p->bucket) * 4u;
+    HostPipe* pipe = (!plain && n >= kHostPieceElements) ? host_pipe() : nullptr;
+    if (pipe) {
+        // The gradient is what takes long: pieces of falling size, so that little is left to do when the last arrives.
+        static constexpr uint32_t cuts[kHostPieces + 1] = {0u, 8u, 12u, 14u, 16u};
+        bool ok = true;
+        s = DQ_OK;
+        for (int i = 0; i < kHostPieces && ok && s == DQ_OK; ++i) {
+            const uint64_t lo = piece_start(n, p->bucket, cuts[i]), hi = piece_start(n, p->bucket, cuts[i + 1]);
+            if (lo == hi) continue;
+            ok = cudaMemcpyAsync(d_grad + lo, grad + lo, (hi - lo) * 4u, cudaMemcpyHostToDevice, st) == cudaSuccess &&
+                 cudaEventRecord(pipe->arrived[i], st) == cudaSuccess &&
+                 cudaStreamWaitEvent(pipe->stream, pipe->arrived[i], 0) == cudaSuccess;
+            if (!ok) break;
+            const uint64_t w0 = lo / 32u * p->bits, w1 = hi == n ? pbytes / 4u : hi / 32u * p->bits;
+            s = encode_common(kind, d_grad + lo, hi - lo, seed, worker, step, p, d_packed + w0, d_scale + lo / p->bucket,
+                              pipe->stream, lo);
+            ok = s != DQ_OK || cudaMemcpyAsync(out_packed + w0, d_packed + w0, (w1 - w0) * 4u, cudaMemcpyDeviceToHost,
+                                               pipe->stream) == cudaSuccess;
+        }
+        if (ok && s == DQ_OK)
+            ok = cudaMemcpyAsync(out_scale, d_scale, sbytes, cudaMemcpyDeviceToHost, pipe->stream) == cudaSuccess;
+        // both streams, also after an error: copies that are queued use the caller's buffers
+        const bool done = cudaStreamSynchronize(st) == cudaSuccess && cudaStreamSynchronize(pipe->stream) == cudaSuccess;
+        return s != DQ_OK ? s : (ok && done) ? DQ_OK : DQ_ERR_CUDA;
+    }
     if (cudaMemcpyAsync(d_grad, grad, n * 4u, cudaMemcpyHostToDevice, st) != cudaSuccess) return DQ_ERR_CUDA;
     s = encode_common(kind, d_grad, n, seed, worker, step, p, d_packed, d_scale, st);
     if (s != DQ_OK) {
@@ -800,6 +898,24 @@ static dq_status decode_host(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0u) return DQ_ERR_ALIGNMENT;
     if (workspace_bytes < dq_decode_workspace_bytes(msgs, W, n, side_info != nullptr)) return DQ_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    dq_msg dev_msgs[DQ_MAX_WORKERS];
+    if (n <= kHostDirectElements) {
+        float* h_out = pinned_view(out_avg);
+        const float* h_side = (h_out && side_info) ? pinned_view(side_info) : nullptr;
+        bool direct = h_out != nullptr && (!side_info || h_side);
+        for (uint32_t w = 0; w < W && direct; ++w) {
+            dev_msgs[w] = msgs[w];
+            dev_msgs[w].packed = pinned_view(msgs[w].packed);
+            dev_msgs[w].scale = pinned_view(msgs[w].scale);
+            direct = dev_msgs[w].packed && dev_msgs[w].scale;
+        }
+        if (direct) {
+            const dq_status s = decode_common(dev_msgs, W, n, step, h_side, h_out, nullptr, true, st, false, false, 0u,
+                                              side_first);
+            if (s != DQ_OK) return s;
+            return cudaStreamSynchronize(st) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+        }
+    }
     uint8_t* ws = static_cast<uint8_t*>(workspace);
     float* d_out = reinterpret_cast<float*>(ws);
     ws += align_up(n * 4u, 256u);
@@ -807,30 +923,54 @@ static dq_status decode_host(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_
     if (side_info) {
         d_side = reinterpret_cast<float*>(ws);
         ws += align_up(n * 4u, 256u);
-        if (cudaMemcpyAsync(d_side, side_info, n * 4u, cudaMemcpyHostToDevice, st) != cudaSuccess) return DQ_ERR_CUDA;
     }
-    dq_msg dev_msgs[DQ_MAX_WORKERS];
+    uint32_t* d_packed[DQ_MAX_WORKERS];
+    float* d_scale[DQ_MAX_WORKERS];
     for (uint32_t w = 0; w < W; ++w) {
         dev_msgs[w] = msgs[w];
-        const uint64_t pbytes = dq_packed_words(n, msgs[w].p.bits) * 4u;
-        const uint64_t sbytes = dq_num_buckets(n, msgs[w].p.bucket) * 4u;
-        uint32_t* d_p = reinterpret_cast<uint32_t*>(ws);
-        ws += align_up(pbytes, 256u);
-        float* d_s = reinterpret_cast<float*>(ws);
-        ws += align_up(sbytes, 256u);
-        if (cudaMemcpyAsync(d_p, msgs[w].packed, pbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return DQ_ERR_CUDA;
-        if (cudaMemcpyAsync(d_s, msgs[w].scale, sbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return DQ_ERR_CUDA;
-        dev_msgs[w].packed = d_p;
-        dev_msgs[w].scale = d_s;
+        d_packed[w] = reinterpret_cast<uint32_t*>(ws);
+        ws += align_up(dq_packed_words(n, msgs[w].p.bits) * 4u, 256u);
+        d_scale[w] = reinterpret_cast<float*>(ws);
+        ws += align_up(dq_num_buckets(n, msgs[w].p.bucket) * 4u, 256u);
     }
-    dq_status s = decode_common(dev_msgs, W, n, step, d_side, d_out, nullptr, true, st, false, false, 0u, side_first);
-    if (s != DQ_OK) {
-        cudaStreamSynchronize(st);          // copies queued above may still be reading the caller's buffers
-        return s;
+    const uint32_t bucket = msgs[0].p.bucket;
+    HostPipe* pipe = n >= kHostPieceElements ? host_pipe() : nullptr;
+    // The mean is what takes long (a long side information vector as long): pieces of rising size, so that the first
+    // part of it starts early.  Without the second stream there is one piece.
+    static constexpr uint32_t rising[kHostPieces + 1] = {0u, 1u, 4u, 8u, 16u}, one[2] = {0u, 16u};
+    const uint32_t* cuts = pipe ? rising : one;
+    const int pieces = pipe ? kHostPieces : 1;
+    cudaStream_t out_st = pipe ? pipe->stream : st;
+    bool ok = true;
+    dq_status s = DQ_OK;
+    for (uint32_t w = 0; w < W && ok; ++w)
+        ok = cudaMemcpyAsync(d_scale[w], msgs[w].scale, dq_num_buckets(n, bucket) * 4u, cudaMemcpyHostToDevice, st) ==
+             cudaSuccess;
+    for (int i = 0; i < pieces && ok && s == DQ_OK; ++i) {
+        const uint64_t lo = piece_start(n, bucket, cuts[i]), hi = piece_start(n, bucket, cuts[i + 1]);
+        if (lo == hi) continue;
+        if (side_info)
+            ok = cudaMemcpyAsync(d_side + lo, side_info + lo, (hi - lo) * 4u, cudaMemcpyHostToDevice, st) == cudaSuccess;
+        for (uint32_t w = 0; w < W && ok; ++w) {
+            const uint32_t bits = msgs[w].p.bits;
+            const uint64_t w0 = lo / 32u * bits, w1 = hi == n ? dq_packed_words(n, bits) : hi / 32u * bits;
+            ok = cudaMemcpyAsync(d_packed[w] + w0, msgs[w].packed + w0, (w1 - w0) * 4u, cudaMemcpyHostToDevice, st) ==
+                 cudaSuccess;
+            dev_msgs[w].packed = d_packed[w] + w0;
+            dev_msgs[w].scale = d_scale[w] + lo / bucket;
+        }
+        if (ok && pipe)
+            ok = cudaEventRecord(pipe->arrived[i], st) == cudaSuccess &&
+                 cudaStreamWaitEvent(out_st, pipe->arrived[i], 0) == cudaSuccess;
+        if (!ok) break;
+        s = decode_common(dev_msgs, W, hi - lo, step, side_info ? d_side + lo : nullptr, d_out + lo, nullptr, true, out_st,
+                          false, false, lo, side_first);
+        ok = s != DQ_OK ||
+             cudaMemcpyAsync(out_avg + lo, d_out + lo, (hi - lo) * 4u, cudaMemcpyDeviceToHost, out_st) == cudaSuccess;
     }
-    if (cudaMemcpyAsync(out_avg, d_out, n * 4u, cudaMemcpyDeviceToHost, st) != cudaSuccess) return DQ_ERR_CUDA;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return DQ_ERR_CUDA;
-    return DQ_OK;
+    // both streams, also after an error: copies that are queued use the caller's buffers
+    const bool done = cudaStreamSynchronize(st) == cudaSuccess && (!pipe || cudaStreamSynchronize(out_st) == cudaSuccess);
+    return s != DQ_OK ? s : (ok && done) ? DQ_OK : DQ_ERR_CUDA;
 }
 
 dq_status ndqsg_decode_aggregate_host(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t step,
