@@ -515,6 +515,68 @@ uint64_t align_up(uint64_t v, uint64_t a) { return (v + a - 1u) / a * a; }
 
 }  // namespace
 
+namespace {
+
+// The *_host calls move their data in one of three ways:
+//   - short gradients in pinned memory: no copies at all, the kernels read and write the host buffers over the bus (a
+//     copy costs 4 us of set-up, and a decode has two per message);
+//   - long ones: in pieces, so that the copies of one direction, the kernels and the copies of the other direction run
+//     side by side (the bus moves 55 GB/s in each direction at once);
+//   - everything else: copy in, kernel, copy out.
+constexpr uint64_t kHostDirectElements = 1ull << 20;       // up to here without copies
+constexpr uint64_t kHostPieceElements = 1ull << 21;        // from here in pieces
+constexpr int kHostPieces = 4;
+
+// Device address of pinned host memory, null for any other (or for one that is not 16-byte aligned).
+template <typename T>
+T* pinned_view(T* host)
+{
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (at.type != cudaMemoryTypeHost || !at.devicePointer || !aligned16(at.devicePointer)) return nullptr;
+    return static_cast<T*>(const_cast<void*>(static_cast<const void*>(at.devicePointer)));
+}
+
+// A second stream and the events that tie it to the caller's: one set per host thread and device, made at the thread's
+// first long *_host call on the device and given back when the thread ends.
+struct HostPipe {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t arrived[kHostPieces] = {};
+    bool make()
+    {
+        if (stream) return true;
+        for (cudaEvent_t& e : arrived)
+            if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
+        return cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) == cudaSuccess;
+    }
+    ~HostPipe()
+    {
+        for (cudaEvent_t e : arrived)
+            if (e) cudaEventDestroy(e);
+        if (stream) cudaStreamDestroy(stream);
+    }
+};
+
+HostPipe* host_pipe()
+{
+    static thread_local HostPipe pipes[kMaxDevices];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    return pipes[dev].make() ? &pipes[dev] : nullptr;
+}
+
+// Start of piece i when n elements are cut at `sixteenths[i]` sixteenths: a multiple of four buckets, so that every
+// buffer's piece is 16-byte aligned.
+uint64_t piece_start(uint64_t n, uint32_t bucket, uint32_t sixteenths)
+{
+    return sixteenths >= 16u ? n : n / 16u * sixteenths / (4u * bucket) * (4u * bucket);
+}
+
+}  // namespace
+
 extern "C" {
 
 uint64_t dq_packed_words(uint64_t n, uint32_t bits) { return (n * (uint64_t)bits + 31u) / 32u; }
@@ -726,68 +788,6 @@ uint64_t dq_decode_workspace_bytes(const dq_msg* msgs, uint32_t W, uint64_t n, i
     }
     return total;
 }
-
-namespace {
-
-// The *_host calls move their data in one of three ways:
-//   - short gradients in pinned memory: no copies at all, the kernels read and write the host buffers over the bus (a
-//     copy costs 4 us of set-up, and a decode has two per message);
-//   - long ones: in pieces, so that the copies of one direction, the kernels and the copies of the other direction run
-//     side by side (the bus moves 55 GB/s in each direction at once);
-//   - everything else: copy in, kernel, copy out.
-constexpr uint64_t kHostDirectElements = 1ull << 20;       // up to here without copies
-constexpr uint64_t kHostPieceElements = 1ull << 21;        // from here in pieces
-constexpr int kHostPieces = 4;
-
-// Device address of pinned host memory, null for any other (or for one that is not 16-byte aligned).
-template <typename T>
-T* pinned_view(T* host)
-{
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    if (at.type != cudaMemoryTypeHost || !at.devicePointer || !aligned16(at.devicePointer)) return nullptr;
-    return static_cast<T*>(const_cast<void*>(static_cast<const void*>(at.devicePointer)));
-}
-
-// A second stream and the events that tie it to the caller's: one set per host thread and device, made at the thread's
-// first long *_host call on the device and given back when the thread ends.
-struct HostPipe {
-    cudaStream_t stream = nullptr;
-    cudaEvent_t arrived[kHostPieces] = {};
-    bool make()
-    {
-        if (stream) return true;
-        for (cudaEvent_t& e : arrived)
-            if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) return false;
-        return cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking) == cudaSuccess;
-    }
-    ~HostPipe()
-    {
-        for (cudaEvent_t e : arrived)
-            if (e) cudaEventDestroy(e);
-        if (stream) cudaStreamDestroy(stream);
-    }
-};
-
-HostPipe* host_pipe()
-{
-    static thread_local HostPipe pipes[kMaxDevices];
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-    return pipes[dev].make() ? &pipes[dev] : nullptr;
-}
-
-// Start of piece i when n elements are cut at `sixteenths[i]` sixteenths: a multiple of four buckets, so that every
-// buffer's piece is 16-byte aligned.
-uint64_t piece_start(uint64_t n, uint32_t bucket, uint32_t sixteenths)
-{
-    return sixteenths >= 16u ? n : n / 16u * sixteenths / (4u * bucket) * (4u * bucket);
-}
-
-}  // namespace
 
 static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64_t seed, uint32_t worker,
                              uint64_t step, const dq_params* p, uint32_t* out_packed, float* out_scale,
