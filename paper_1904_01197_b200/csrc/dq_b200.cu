@@ -544,7 +544,7 @@ T* pinned_view(T* host)
 // first long *_host call on the device and given back when the thread ends.
 struct HostPipe {
     cudaStream_t stream = nullptr;
-    cudaEvent_t arrived[kHostPieces] = {};
+    cudaEvent_t arrived[kHostPieces] = {};       // (piece i is ready for the second stream)
     bool make()
     {
         if (stream) return true;
@@ -825,7 +825,7 @@ static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64
     HostPipe* pipe = (!plain && n >= kHostPieceElements) ? host_pipe() : nullptr;
     if (pipe) {
         // The gradient is what takes long: pieces of falling size, so that little is left to do when the last arrives.
-        static constexpr uint32_t cuts[kHostPieces + 1] = {0u, 8u, 12u, 14u, 16u};
+        static constexpr uint32_t cuts[kHostPieces + 1] = {0u, 8u, 12u, 15u, 16u};
         bool ok = true;
         s = DQ_OK;
         for (int i = 0; i < kHostPieces && ok && s == DQ_OK; ++i) {
@@ -959,14 +959,15 @@ static dq_status decode_host(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_
             dev_msgs[w].packed = d_packed[w] + w0;
             dev_msgs[w].scale = d_scale[w] + lo / bucket;
         }
-        if (ok && pipe)
+        if (!ok) break;
+        // the kernel runs between two copies in: those have time, while the copies out follow each other without a gap
+        s = decode_common(dev_msgs, W, hi - lo, step, side_info ? d_side + lo : nullptr, d_out + lo, nullptr, true, st,
+                          false, false, lo, side_first);
+        if (s != DQ_OK) break;
+        if (pipe)
             ok = cudaEventRecord(pipe->arrived[i], st) == cudaSuccess &&
                  cudaStreamWaitEvent(out_st, pipe->arrived[i], 0) == cudaSuccess;
-        if (!ok) break;
-        s = decode_common(dev_msgs, W, hi - lo, step, side_info ? d_side + lo : nullptr, d_out + lo, nullptr, true, out_st,
-                          false, false, lo, side_first);
-        ok = s != DQ_OK ||
-             cudaMemcpyAsync(out_avg + lo, d_out + lo, (hi - lo) * 4u, cudaMemcpyDeviceToHost, out_st) == cudaSuccess;
+        ok = ok && cudaMemcpyAsync(out_avg + lo, d_out + lo, (hi - lo) * 4u, cudaMemcpyDeviceToHost, out_st) == cudaSuccess;
     }
     // both streams, also after an error: copies that are queued use the caller's buffers
     const bool done = cudaStreamSynchronize(st) == cudaSuccess && (!pipe || cudaStreamSynchronize(out_st) == cudaSuccess);
