@@ -520,12 +520,14 @@ namespace {
 // The *_host calls move their data in one of three ways:
 //   - short gradients in pinned memory: no copies at all, the kernels read and write the host buffers over the bus (a
 //     copy costs 4 us of set-up, and a decode has two per message);
-//   - long ones: in pieces, so that the copies of one direction, the kernels and the copies of the other direction run
-//     side by side (the bus moves 55 GB/s in each direction at once);
+//   - long ones: in two pieces, so that the copies of one direction run beside the kernel and the copies of the other.
+//     The bus moves 55 GB/s in each direction at once, but a change between copies, events and kernels costs some 20 us,
+//     so more pieces than two gain nothing (n = 11.7 M: encode 942 us in one piece, 893 in two, 892 in three; decode of
+//     four messages 1183, 1102 and 1115);
 //   - everything else: copy in, kernel, copy out.
 constexpr uint64_t kHostDirectElements = 1ull << 20;       // up to here without copies
-constexpr uint64_t kHostPieceElements = 1ull << 21;        // from here in pieces
-constexpr int kHostPieces = 4;
+constexpr uint64_t kHostPieceElements = 1ull << 22;        // from here in pieces
+constexpr int kHostPieces = 2;
 
 // Device address of pinned host memory, null for any other (or for one that is not 16-byte aligned).
 template <typename T>
@@ -824,8 +826,8 @@ static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64
     const uint64_t sbytes = dq_num_buckets(n, p->bucket) * 4u;
     HostPipe* pipe = (!plain && n >= kHostPieceElements) ? host_pipe() : nullptr;
     if (pipe) {
-        // The gradient is what takes long: pieces of falling size, so that little is left to do when the last arrives.
-        static constexpr uint32_t cuts[kHostPieces + 1] = {0u, 8u, 12u, 15u, 16u};
+        // The gradient is what takes long: a small last piece, so that little is left to do when it arrives.
+        static constexpr uint32_t cuts[kHostPieces + 1] = {0u, 14u, 16u};
         bool ok = true;
         s = DQ_OK;
         for (int i = 0; i < kHostPieces && ok && s == DQ_OK; ++i) {
@@ -935,10 +937,10 @@ static dq_status decode_host(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_
     }
     const uint32_t bucket = msgs[0].p.bucket;
     HostPipe* pipe = n >= kHostPieceElements ? host_pipe() : nullptr;
-    // The mean is what takes long (a long side information vector as long): pieces of rising size, so that the first
-    // part of it starts early.  Without the second stream there is one piece.
-    static constexpr uint32_t rising[kHostPieces + 1] = {0u, 1u, 4u, 8u, 16u}, one[2] = {0u, 16u};
-    const uint32_t* cuts = pipe ? rising : one;
+    // The mean is what takes long (a side information vector as long): a small first piece, so that it starts early.
+    // Without the second stream there is one piece.
+    static constexpr uint32_t two[kHostPieces + 1] = {0u, 5u, 16u}, one[2] = {0u, 16u};
+    const uint32_t* cuts = pipe ? two : one;
     const int pieces = pipe ? kHostPieces : 1;
     cudaStream_t out_st = pipe ? pipe->stream : st;
     bool ok = true;

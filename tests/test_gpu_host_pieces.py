@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 
 from test_gpu_parity import dq  # noqa: E402,F401
 
-DIRECT, PIECES = 1 << 20, 1 << 21
+DIRECT, PIECES = 1 << 20, 1 << 22
 
 
 def _host(t, how):
