@@ -1,7 +1,7 @@
 """Builds the CUDA library in-tree with nvcc for sm_100a (cross-compiles without a GPU).
 
 The kernels are templates with many instantiations; they are spread over translation units (one per encoder
-mode and dither width, one per decoder variant) that are compiled in parallel and linked into one shared library.
+mode and dither width, one per decoder variant and group size) that are compiled in parallel and linked into one shared library.
 The Python calls (csrc/dq_calls.cpp) are a second, small library, linked against the first.
 """
 from __future__ import annotations
@@ -34,8 +34,8 @@ NVCC_FLAGS = [
 UNITS = [("dq_b200", "dq_b200.cu", [])]
 UNITS += [(f"enc_m{m}_d{d}", "dq_encode_inst.cu", [f"-DDQ_INST_MODE={m}", f"-DDQ_INST_DITH={d}"])
           for m in (0, 1, 2, 3) for d in (32, 16)]
-UNITS += [(f"dec_d{d}_r{r}", "dq_decode_inst.cu", [f"-DDQ_INST_DITH={d}", f"-DDQ_INST_RUN={r}"])
-          for d, r in ((32, 0), (32, 1), (32, 2), (16, 0), (16, 1), (16, 2), (0, 0))]
+UNITS += [(f"dec_d{d}_r{r}_e{e}", "dq_decode_inst.cu", [f"-DDQ_INST_DITH={d}", f"-DDQ_INST_RUN={r}", f"-DDQ_INST_E={e}"])
+          for d, r in ((32, 0), (32, 1), (32, 2), (16, 0), (16, 1), (16, 2), (0, 0)) for e in (32, 16, 8)]
 
 
 def nvcc_path() -> str:

@@ -98,7 +98,13 @@ constexpr int kDecThreads = 128;
 // fastest form for many workers: what a worker costs per lane (scale, gain, constants, loop: about 65 instructions) is
 // spread over the most elements, and 16 warps (128 registers) are 7 % slower, 24 (80 registers, spilling) 3 %.
 // E = 16 and 8 take 64 registers (32 warps).
-constexpr int dec_ctas_per_sm(int E) { return E == 32 ? 5 : 8; }
+#ifndef DQ_C32
+#define DQ_C32 5
+#endif
+#ifndef DQ_AH
+#define DQ_AH 1
+#endif
+constexpr int dec_ctas_per_sm(int E) { return E == 32 ? DQ_C32 : 8; }
 
 // Code of element `idx` of a group as the float 2^22 + code: the bit pattern of 2^22 with the code in mantissa
 // bits 1.. (floats in [2^22, 2^23) step by 1/2).  Subtracting a constant then gives code - c exactly.
@@ -298,18 +304,22 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
     }
 }
 
-// The variants that nearly every caller uses: DQSG, and NDQSG with a power-of-two K and no shrinkage, up to 4 bits.
-// They have kernels of their own: with all forty routines in one kernel the compiler's register allocation costs every
-// routine 1 to 5 % (W = 16, 3 bits, n = 124.4 M: 1973 us against 1920).
+// Which variants a kernel holds.  With all forty routines in one kernel the compiler's register allocation and its
+// choice between uniform and per-lane loads of a worker's constants cost every routine 5 to 12 %, so the usual variants
+// (DQSG, and NDQSG with a power-of-two K and no shrinkage, up to 4 bits) have kernels of their own, and for long
+// gradients every pair of one DQSG and one NDQSG width has (W = 16, 3 bits, n = 124.4 M: 1973 us with all, 1933 with the
+// usual ones, 1790 with the pair; W = 8, 2 bits, n = 25.6 M: 217, 210 and 193).
+constexpr int kSetAll = 0, kSetUsual = 1;
+constexpr int pair_set(int dqsg_bits, int ndqsg_bits) { return 16 * dqsg_bits + ndqsg_bits; }
 inline bool is_usual_variant(uint32_t variant) { return (variant >> 3) <= kDecNdqsgPow2 && (variant & 7u) < 4u; }
 
-// All W workers, run by run; dispatch on (kind, bits) with one jump per run.  ALL: every variant, else the usual ones.
-template <int DITH, int SIDE, int E, bool ALL, typename Args>
+// All W workers, run by run; dispatch on (kind, bits) with one jump per run.
+template <int DITH, int SIDE, int E, int SET, typename Args>
 __device__ __forceinline__ void decode_workers(const Args& args, DecLane& ln, f32x2 (&acc)[E / 2])
 {
 #define DQ_DEC_CASE(KIND, BITS)                                                                                    \
     case (KIND) * 8u + (BITS) - 1u:                                                                                \
-        decode_run<BITS, KIND, DITH, SIDE, E, E == 32 && !ALL>(args, w, w_end, ln, acc);                           \
+        decode_run<BITS, KIND, DITH, SIDE, E, DQ_AH && (SET > kSetUsual)>(args, w, w_end, ln, acc);                           \
         break;
 #define DQ_DEC_LOW(KIND)                                                                                           \
     DQ_DEC_CASE(KIND, 1) DQ_DEC_CASE(KIND, 2) DQ_DEC_CASE(KIND, 3) DQ_DEC_CASE(KIND, 4)
@@ -319,7 +329,7 @@ __device__ __forceinline__ void decode_workers(const Args& args, DecLane& ln, f3
 #pragma unroll 1
     for (uint32_t w = 0; w < args.W;) {
         const uint32_t w_end = args.w[w].group_end;
-        if constexpr (ALL) {
+        if constexpr (SET == kSetAll) {
             switch (args.w[w].variant) {
                 DQ_DEC_KIND(kDecDqsg)
                 DQ_DEC_KIND(kDecNdqsgPow2)
@@ -328,10 +338,16 @@ __device__ __forceinline__ void decode_workers(const Args& args, DecLane& ln, f3
                 DQ_DEC_KIND(kDecNdqsgAnyKShrink)
                 default: break;
             }
-        } else {
+        } else if constexpr (SET == kSetUsual) {
             switch (args.w[w].variant) {
                 DQ_DEC_LOW(kDecDqsg)
                 DQ_DEC_LOW(kDecNdqsgPow2)
+                default: break;
+            }
+        } else {
+            switch (args.w[w].variant) {
+                DQ_DEC_CASE(kDecDqsg, SET / 16)
+                DQ_DEC_CASE(kDecNdqsgPow2, SET % 16)
                 default: break;
             }
         }
@@ -356,7 +372,7 @@ __device__ __forceinline__ void store8(float* p, const f32x2 (&v)[4], bool align
 // ---------------------------------------------------------------------------------------------------
 // The decode kernel: one group of E elements per lane.
 // ---------------------------------------------------------------------------------------------------
-template <int DITH, int SIDE, int E, bool ALL, int MAXW>
+template <int DITH, int SIDE, int E, int SET, int MAXW>
 __global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(E))
 decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
 {
@@ -426,7 +442,7 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
     f32x2 acc[E / 2];
 #pragma unroll
     for (int e = 0; e < E / 2; ++e) acc[e] = 0ull;
-    decode_workers<DITH, SIDE, E, ALL>(args, ln, acc);
+    decode_workers<DITH, SIDE, E, SET>(args, ln, acc);
 
     // the mean (of one message: the message itself)
     if (args.W > 1u) {

@@ -1,50 +1,85 @@
-// Instantiations of decode_aggregate_kernel for one dither width and one side-information mode (DQ_INST_DITH,
-// DQ_INST_RUN = a DecSide value, given on the compiler's command line), all group sizes and both sets of variants.
+// Instantiations of decode_aggregate_kernel for one dither width, one side-information mode and one group size
+// (DQ_INST_DITH, DQ_INST_RUN = a DecSide value, DQ_INST_E, given on the compiler's command line) and all sets of variants.
 #include <cstring>
 
 #include "dq_decode.cuh"
 #include "dq_launch.h"
 
 #ifndef DQ_INST_DITH
-#error "compile with -DDQ_INST_DITH=<32|16|0> -DDQ_INST_RUN=<0|1|2>"
+#error "compile with -DDQ_INST_DITH=<32|16|0> -DDQ_INST_RUN=<0|1|2> -DDQ_INST_E=<32|16|8>"
 #endif
 
 namespace dq {
 
-#define DQ_NAME2(D, R) launch_decode_d##D##_r##R
-#define DQ_NAME(D, R) DQ_NAME2(D, R)
+#define DQ_NAME2(D, R, E) launch_decode_d##D##_r##R##_e##E
+#define DQ_NAME(D, R, E) DQ_NAME2(D, R, E)
 
 namespace {
+
+template <int E, int SET, int MAXW = 64>
+cudaError_t launch_set(const DecodeArgsOf<MAXW>& a, uint32_t grid, cudaStream_t st)
+{
+    return launch_overlapped(decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, SET, MAXW>, grid, (uint32_t)kDecThreads, 0,
+                             st, 1u, a);
+}
+
+template <int A>
+cudaError_t launch_pair(int b, const DecodeArgs& a, uint32_t grid, cudaStream_t st)
+{
+    switch (b) {
+        case 1: return launch_set<32, pair_set(A, 1)>(a, grid, st);
+        case 2: return launch_set<32, pair_set(A, 2)>(a, grid, st);
+        case 3: return launch_set<32, pair_set(A, 3)>(a, grid, st);
+        default: return launch_set<32, pair_set(A, 4)>(a, grid, st);
+    }
+}
 
 template <int E>
 cudaError_t launch_groups_of(const DecodeArgs& a, cudaStream_t st)
 {
     const uint32_t grid = (uint32_t)((a.num_groups + kDecThreads - 1u) / kDecThreads);
-    bool usual = true;
-    for (uint32_t w = 0; w < a.W; ++w) usual = usual && is_usual_variant(a.w[w].variant);
-    if constexpr (E == 8) {
-        // short gradients: the launch itself counts
-        if (a.W <= (uint32_t)kDecFewWorkers) {
-            auto k = usual ? decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, false, kDecFewWorkers>
-                           : decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, true, kDecFewWorkers>;
-            DecodeArgsOf<kDecFewWorkers> few;
-            static_cast<DecodeHead&>(few) = a;
-            std::memcpy(few.w, a.w, a.W * sizeof(DecWorker));
-            return launch_overlapped(k, grid, (uint32_t)kDecThreads, 0, st, 1u, few);
-        }
+    bool usual = true, one_pair = true;
+    int width[2] = {0, 0};              // code widths of the DQSG and of the NDQSG messages
+    for (uint32_t w = 0; w < a.W; ++w) {
+        const uint32_t v = a.w[w].variant;
+        usual = usual && is_usual_variant(v);
+        if (!usual) break;
+        int& have = width[v >> 3];
+        one_pair = one_pair && (have == 0 || have == (int)(v & 7u) + 1);
+        have = (int)(v & 7u) + 1;
     }
-    auto k = usual ? decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, false, 64>
-                   : decode_aggregate_kernel<DQ_INST_DITH, DQ_INST_RUN, E, true, 64>;
-    return launch_overlapped(k, grid, (uint32_t)kDecThreads, 0, st, 1u, a);
+    if constexpr (E == 32) {
+        if (usual && one_pair) {
+            if (width[0] == 0) width[0] = width[1];
+            if (width[1] == 0) width[1] = width[0];
+            switch (width[0]) {
+                case 1: return launch_pair<1>(width[1], a, grid, st);
+                case 2: return launch_pair<2>(width[1], a, grid, st);
+                case 3: return launch_pair<3>(width[1], a, grid, st);
+                default: return launch_pair<4>(width[1], a, grid, st);
+            }
+        }
+        return launch_set<E, kSetAll>(a, grid, st);
+    } else {
+        if constexpr (E == 8) {
+            // short gradients: the launch itself counts
+            if (a.W <= (uint32_t)kDecFewWorkers) {
+                DecodeArgsOf<kDecFewWorkers> few;
+                static_cast<DecodeHead&>(few) = a;
+                std::memcpy(few.w, a.w, a.W * sizeof(DecWorker));
+                return usual ? launch_set<E, kSetUsual, kDecFewWorkers>(few, grid, st)
+                             : launch_set<E, kSetAll, kDecFewWorkers>(few, grid, st);
+            }
+        }
+        return usual ? launch_set<E, kSetUsual>(a, grid, st) : launch_set<E, kSetAll>(a, grid, st);
+    }
 }
 
 }  // namespace
 
-cudaError_t DQ_NAME(DQ_INST_DITH, DQ_INST_RUN)(const DecodeArgs& a, int group_size, cudaStream_t st)
+cudaError_t DQ_NAME(DQ_INST_DITH, DQ_INST_RUN, DQ_INST_E)(const DecodeArgs& a, cudaStream_t st)
 {
-    if (group_size == 32) return launch_groups_of<32>(a, st);
-    if (group_size == 16) return launch_groups_of<16>(a, st);
-    return launch_groups_of<8>(a, st);
+    return launch_groups_of<DQ_INST_E>(a, st);
 }
 
 }  // namespace dq
