@@ -371,8 +371,8 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 int decode_group_size(uint64_t n, uint32_t W, int sms)
 {
     const uint64_t lanes = (uint64_t)sms * dq::kDecThreads;
-    if (n <= 8u * lanes * dq::dec_ctas_per_sm(8)) return 8;
-    if (W <= 2u || 2u * n < 5u * 32u * lanes * dq::dec_ctas_per_sm(32)) return 16;
+    if (n <= 8u * lanes * dq::dec_ctas_per_sm(8, dq::kSetUsual)) return 8;
+    if (W <= 2u || 2u * n < 5u * 32u * lanes * dq::dec_ctas_per_sm(32, dq::kSetAll)) return 16;
     return 32;
 }
 

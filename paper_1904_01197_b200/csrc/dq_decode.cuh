@@ -94,17 +94,20 @@ inline void set_bucket_division(DecodeHead& a)
 }
 
 constexpr int kDecThreads = 128;
-// Resident CTAs per SM that the register budget is set for.  E = 32 with 96 registers and 20 warps per SM is the
-// fastest form for many workers: what a worker costs per lane (scale, gain, constants, loop: about 65 instructions) is
-// spread over the most elements, and 16 warps (128 registers) are 7 % slower, 24 (80 registers, spilling) 3 %.
+// Which variants a kernel holds.  With all forty routines in one kernel the compiler's register allocation and its
+// choice between uniform and per-lane loads of a worker's constants cost every routine 5 to 12 %, so the usual variants
+// (DQSG, and NDQSG with a power-of-two K and no shrinkage, up to 4 bits) have kernels of their own, and for long
+// gradients every pair of one DQSG and one NDQSG width has (W = 16, 3 bits, n = 124.4 M: 1973 us with all, 1933 with the
+// usual ones, 1782 with the pair; W = 8, 2 bits, n = 25.6 M: 217, 210 and 197).
+constexpr int kSetAll = 0, kSetUsual = 1;
+constexpr int pair_set(int dqsg_bits, int ndqsg_bits) { return 16 * dqsg_bits + ndqsg_bits; }
+
+// Resident CTAs per SM that the register budget is set for.  E = 32 takes 80 registers (24 warps per SM) in the pair
+// kernels: what a worker costs per lane (scale, gain, constants, loop: about 65 instructions) is spread over the most
+// elements.  96 registers are 3 % faster for a given side information vector but 2 to 8 % slower otherwise (the compiler
+// then loads a worker's constants lane by lane), 128 registers 7 % slower; the kernel with all routines wants 96.
 // E = 16 and 8 take 64 registers (32 warps).
-#ifndef DQ_C32
-#define DQ_C32 5
-#endif
-#ifndef DQ_AH
-#define DQ_AH 1
-#endif
-constexpr int dec_ctas_per_sm(int E) { return E == 32 ? DQ_C32 : 8; }
+constexpr int dec_ctas_per_sm(int E, int set) { return E == 32 ? (set == kSetAll ? 5 : 6) : 8; }
 
 // Code of element `idx` of a group as the float 2^22 + code: the bit pattern of 2^22 with the code in mantissa
 // bits 1.. (floats in [2^22, 2^23) step by 1/2).  Subtracting a constant then gives code - c exactly.
@@ -189,8 +192,15 @@ struct DecLane {
 // variant is taken once per run and not once per worker (Algorithm 2's groups P1 and P2 are two runs).
 //   DQSG:  g~ = (kappa/s) ((k - s) - delta); (k - s + 1.5) - f rounds once to the same value.
 //   NDQSG: r = (m - delta) - y a;  jj = rint(r / K);  q1^ = m - K jj;  g~ = beta (q1^ - delta) [+ (1-alpha^2) y]
-// AHEAD: the packed words are requested one worker ahead (worth its registers with 20 warps per SM, i.e. E = 32: 4 %;
-// with 32 warps it costs as much).
+// AHEAD: the packed words are requested one worker ahead (see words_ahead).
+//
+// Requesting the words a worker ahead costs registers and pays only where a worker is done soonest: the 16-bit stream's
+// DQSG messages (W = 8, n = 11.7 M: 54.9 -> 52.4 us); elsewhere the Philox work hides the latency.
+constexpr bool words_ahead(int dith, uint32_t kind, int E, int set)
+{
+    return dith == 16 && kind == kDecDqsg && E == 32 && set != kSetAll;
+}
+
 template <int BITS, uint32_t KIND, int DITH, int SIDE, int E, bool AHEAD, typename Args>
 __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_t w_end, DecLane& ln,
                                            f32x2 (&acc)[E / 2])
@@ -304,13 +314,6 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
     }
 }
 
-// Which variants a kernel holds.  With all forty routines in one kernel the compiler's register allocation and its
-// choice between uniform and per-lane loads of a worker's constants cost every routine 5 to 12 %, so the usual variants
-// (DQSG, and NDQSG with a power-of-two K and no shrinkage, up to 4 bits) have kernels of their own, and for long
-// gradients every pair of one DQSG and one NDQSG width has (W = 16, 3 bits, n = 124.4 M: 1973 us with all, 1933 with the
-// usual ones, 1790 with the pair; W = 8, 2 bits, n = 25.6 M: 217, 210 and 193).
-constexpr int kSetAll = 0, kSetUsual = 1;
-constexpr int pair_set(int dqsg_bits, int ndqsg_bits) { return 16 * dqsg_bits + ndqsg_bits; }
 inline bool is_usual_variant(uint32_t variant) { return (variant >> 3) <= kDecNdqsgPow2 && (variant & 7u) < 4u; }
 
 // All W workers, run by run; dispatch on (kind, bits) with one jump per run.
@@ -319,7 +322,7 @@ __device__ __forceinline__ void decode_workers(const Args& args, DecLane& ln, f3
 {
 #define DQ_DEC_CASE(KIND, BITS)                                                                                    \
     case (KIND) * 8u + (BITS) - 1u:                                                                                \
-        decode_run<BITS, KIND, DITH, SIDE, E, DQ_AH && (SET > kSetUsual)>(args, w, w_end, ln, acc);                           \
+        decode_run<BITS, KIND, DITH, SIDE, E, words_ahead(DITH, KIND, E, SET)>(args, w, w_end, ln, acc);          \
         break;
 #define DQ_DEC_LOW(KIND)                                                                                           \
     DQ_DEC_CASE(KIND, 1) DQ_DEC_CASE(KIND, 2) DQ_DEC_CASE(KIND, 3) DQ_DEC_CASE(KIND, 4)
@@ -373,7 +376,7 @@ __device__ __forceinline__ void store8(float* p, const f32x2 (&v)[4], bool align
 // The decode kernel: one group of E elements per lane.
 // ---------------------------------------------------------------------------------------------------
 template <int DITH, int SIDE, int E, int SET, int MAXW>
-__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(E))
+__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(E, SET))
 decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
 {
     // per lane: E / 4 slots of side information, then the first Philox products (two blocks per slot)
