@@ -192,14 +192,12 @@ struct DecLane {
 // variant is taken once per run and not once per worker (Algorithm 2's groups P1 and P2 are two runs).
 //   DQSG:  g~ = (kappa/s) ((k - s) - delta); (k - s + 1.5) - f rounds once to the same value.
 //   NDQSG: r = (m - delta) - y a;  jj = rint(r / K);  q1^ = m - K jj;  g~ = beta (q1^ - delta) [+ (1-alpha^2) y]
-// AHEAD: the packed words are requested one worker ahead (see words_ahead).
+// AHEAD: the packed words are requested one worker ahead (see kWordsAhead).
 //
 // Requesting the words a worker ahead costs registers and pays only where a worker is done soonest: the 16-bit stream's
 // DQSG messages (W = 8, n = 11.7 M: 54.9 -> 52.4 us); elsewhere the Philox work hides the latency.
-constexpr bool words_ahead(int dith, uint32_t kind, int E, int set)
-{
-    return dith == 16 && kind == kDecDqsg && E == 32 && set != kSetAll;
-}
+template <int DITH, uint32_t KIND, int E, int SET>
+constexpr bool kWordsAhead = DITH == 16 && KIND == kDecDqsg && E == 32 && SET != kSetAll;
 
 template <int BITS, uint32_t KIND, int DITH, int SIDE, int E, bool AHEAD, typename Args>
 __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_t w_end, DecLane& ln,
@@ -322,7 +320,7 @@ __device__ __forceinline__ void decode_workers(const Args& args, DecLane& ln, f3
 {
 #define DQ_DEC_CASE(KIND, BITS)                                                                                    \
     case (KIND) * 8u + (BITS) - 1u:                                                                                \
-        decode_run<BITS, KIND, DITH, SIDE, E, words_ahead(DITH, KIND, E, SET)>(args, w, w_end, ln, acc);          \
+        decode_run<BITS, KIND, DITH, SIDE, E, kWordsAhead<DITH, KIND, E, SET>>(args, w, w_end, ln, acc);        \
         break;
 #define DQ_DEC_LOW(KIND)                                                                                           \
     DQ_DEC_CASE(KIND, 1) DQ_DEC_CASE(KIND, 2) DQ_DEC_CASE(KIND, 3) DQ_DEC_CASE(KIND, 4)
