@@ -383,9 +383,16 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
     __shared__ __align__(16) float4 slots[kSlots][kDecThreads];
 
     const uint64_t local = (uint64_t)blockIdx.x * (uint32_t)kDecThreads + threadIdx.x;
-    if (local >= args.num_groups) return;                       // no barrier below
+    // Lanes past the end either leave (there is no barrier below), or repeat the last group and store nothing: then the
+    // control flow stays uniform for the compiler and a worker's constants take the uniform data path, which gains 1 to 2 %
+    // with long chains per lane and loses as much in the shorter ones.
+    constexpr bool kClamp = E == 32 || (E == 16 && SET <= kSetUsual);
+    const bool live = local < args.num_groups;
+    if constexpr (!kClamp) {
+        if (!live) return;
+    }
     DecLane ln;
-    ln.group = args.first_row * (32u / E) + (uint32_t)local;
+    ln.group = args.first_row * (32u / E) + (uint32_t)(!kClamp || live ? local : args.num_groups - 1u);
     const uint64_t i0 = (uint64_t)ln.group * (uint32_t)E;
     const uint32_t row = ln.group / (32u / E);
     ln.bucket = (args.bucket_magic != 0u) ? (__umulhi(row, args.bucket_magic) >> args.bucket_shift)
@@ -460,6 +467,7 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
         }
     }
     float* o = args.out + i0;
+    if (kClamp && !live) return;
     if (whole) {
 #pragma unroll
         for (int k = 0; k < E / 8; ++k) {
