@@ -21,9 +21,6 @@
 #include "dq_device.cuh"
 #include "dq_encode.cuh"
 
-#ifndef DQ_MB
-#define DQ_MB 3
-#endif
 namespace dq {
 
 template <int R> constexpr int kDirectMaxThreads = R == 1 ? 1024 : 256;
@@ -92,37 +89,33 @@ inline DirectShape direct_shape(uint32_t g, int R)
     return best;
 }
 
-// The codes of G groups, 8 * BITS bits each in ceil(BITS / 4) words.  x: the elements as pairs, four per group; p0: first
-// Philox product (M0 * counter) of the first group's first block, the next group's being `step` further; aa: the buckets'
-// gains twice.
-template <int BITS, int MODE, int DITH, int G>
-__device__ __forceinline__ void encode_groups8(const f32x2* x, uint64_t p0, uint64_t step, const f32x2* aa,
-                                               const DirectArgs& args, uint32_t (*out)[(BITS + 3) / 4])
+// The codes of a group: 8 * BITS bits in ceil(BITS / 4) words.  x: the elements as pairs; p0: first Philox product
+// (M0 * counter) of the group's first block; aa: the bucket's gain twice.
+template <int BITS, int MODE, int DITH>
+__device__ __forceinline__ void encode_group8(const f32x2* x, uint64_t p0, f32x2 aa, const DirectArgs& args,
+                                              uint32_t (&out)[(BITS + 3) / 4])
 {
     constexpr int N = (DITH == 16) ? 1 : 2;
-    uint32_t hi[G * N], lo[G * N], rnd[G * N][4];
+    uint32_t hi[N], lo[N], rnd[N][4];
 #pragma unroll
-    for (int j = 0; j < G * N; ++j) {
-        const uint64_t p = p0 + (uint64_t)(j / N) * step + (uint64_t)(j % N) * kPhiloxM0;
+    for (int j = 0; j < N; ++j) {
+        const uint64_t p = p0 + (uint64_t)j * kPhiloxM0;
         hi[j] = (uint32_t)(p >> 32);
         lo[j] = (uint32_t)p;
     }
-    philox4x32_10_after_first<G * N>(hi, lo, args.ps, rnd);
+    philox4x32_10_after_first<N>(hi, lo, args.ps, rnd);
+    uint32_t sr = 0u;
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-        uint32_t sr = 0u;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            // v = fma(g, a, delta); DQSG: w = v + s; then round to nearest even
-            f32x2 v = fma2(x[4 * g + e], aa[g], fma2(dither_bits2<DITH>(rnd, 8 * g + 2 * e), args.two, args.off));
-            if constexpr (MODE == kEncDqsg) v = add2(v, args.shift);
-            float t0, t1;
-            unpack2(add2(v, args.magic), t0, t1);
-            push_code<BITS>(sr, code_of<MODE>(t0, args), 2 * e, out[g]);
-            push_code<BITS>(sr, code_of<MODE>(t1, args), 2 * e + 1, out[g]);
-        }
-        if constexpr (BITS % 4 != 0) out[g][BITS / 4] = sr >> (32 - 8 * BITS % 32);
+    for (int e = 0; e < 4; ++e) {
+        // v = fma(g, a, delta); DQSG: w = v + s; then round to nearest even
+        f32x2 v = fma2(x[e], aa, fma2(dither_bits2<DITH>(rnd, 2 * e), args.two, args.off));
+        if constexpr (MODE == kEncDqsg) v = add2(v, args.shift);
+        float t0, t1;
+        unpack2(add2(v, args.magic), t0, t1);
+        push_code<BITS>(sr, code_of<MODE>(t0, args), 2 * e, out);
+        push_code<BITS>(sr, code_of<MODE>(t1, args), 2 * e + 1, out);
     }
+    if constexpr (BITS % 4 != 0) out[BITS / 4] = sr >> (32 - 8 * BITS % 32);
 }
 
 // The BITS bytes of a whole group.
@@ -177,7 +170,7 @@ __device__ __forceinline__ uint32_t cluster_max(uint32_t mine, uint32_t part, ui
 }
 
 template <int BITS, int MODE, int DITH, int R>
-__global__ void __launch_bounds__(kDirectMaxThreads<R>, R == 1 ? 1 : DQ_MB)
+__global__ void __launch_bounds__(kDirectMaxThreads<R>, R == 1 ? 1 : 3)
 encode_direct_kernel(const __grid_constant__ DirectArgs args)
 {
     constexpr int NW = (BITS + 3) / 4;
@@ -292,22 +285,12 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
     // M0 k + M0 j), which are cheaper than wide multiplies on the pipe that bounds the kernel
     const uint64_t p0 = (uint64_t)kPhiloxM0 * ((args.first_group + group) * kBlocks);
     uint32_t out[R][NW];
-    f32x2 aa[R];
-    aa[0] = both(bucket_gain(args.gain_num, __uint_as_float(mb[0])));
+    f32x2 aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[0])));
 #pragma unroll
-    for (int c = 1; c < R; ++c) aa[c] = aa[0];
-    if (args.reduce != kWarpInBucket) {
-#pragma unroll
-        for (int c = 1; c < R; ++c) aa[c] = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
+    for (int c = 0; c < R; ++c) {
+        if (c > 0 && args.reduce != kWarpInBucket) aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
+        encode_group8<BITS, MODE, DITH>(x + 4 * c, p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0, aa, args, out[c]);
     }
-#ifndef DQ_G
-#define DQ_G 2
-#endif
-    constexpr int G = R < DQ_G ? R : DQ_G;
-#pragma unroll
-    for (int c = 0; c < R; c += G)
-        encode_groups8<BITS, MODE, DITH, G>(x + 4 * c, p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0,
-                                            (uint64_t)(32u * kBlocks) * kPhiloxM0, aa + c, args, out + c);
     if (!waited && args.early_store == 0u) {
         grid_dependency_wait();
         waited = true;
