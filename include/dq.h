@@ -23,9 +23,10 @@
  *   - A message is `scale` (one fp32 per bucket) plus `packed`: element i's b-bit code at bit offset
  *     i*b of a little-endian stream of 32-bit words; pad bits of the last word are written as 0.
  *   - "device" pointers are CUDA device memory on the current device, 16-byte aligned, owned by the
- *     caller.  The library allocates nothing at run time and keeps no state between calls, with two
+ *     caller.  The library allocates no device memory at run time and keeps no state between calls, with two
  *     exceptions that live in its device image: one error word per GPU (dq_device_error_flags) and the
- *     fixed staging array of dqsg_encode_host_static.  It is asynchronous on the given stream (it never
+ *     fixed staging array of dqsg_encode_host_static.  (Long *_host calls also keep a stream and two events per
+ *     host thread and device, given back when the thread ends.)  It is asynchronous on the given stream (it never
  *     synchronises), except for the *_host entry points, which return after the results are in the
  *     caller's host buffers.
  *   - Outputs must not alias inputs.  Inputs are assumed finite.
@@ -275,8 +276,11 @@ dq_status dq_ternary_unpack(const uint8_t* radix, uint64_t n, uint32_t* out_pack
  * Host-buffer variants.  Every data pointer (grad, out_packed, out_scale, the packed/scale pointers
  * inside msgs, side_info, out_avg) is HOST memory (pinned memory makes the copies asynchronous);
  * `workspace` is device memory of at least the stated size, 256-byte aligned, provided by the caller.
- * Each call copies its inputs to the workspace, runs the same kernels as the device entry points,
- * copies the results back and synchronises the stream before returning.
+ * Each call runs the same kernels as the device entry points and synchronises the stream before returning.  Long
+ * gradients are copied to the workspace, processed and copied back in two pieces, with a second stream that the
+ * library keeps per host thread and device; up to 2^20 elements in pinned, 16-byte aligned buffers the kernels read
+ * and write the host memory directly and the workspace is not used; anything else is copied in, processed and copied
+ * back.  The results are the same bits in every case.
  */
 uint64_t dq_encode_workspace_bytes(uint64_t n, const dq_params* p);
 uint64_t dq_decode_workspace_bytes(const dq_msg* msgs, uint32_t W, uint64_t n, int has_side_info);

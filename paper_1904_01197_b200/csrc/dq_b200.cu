@@ -293,25 +293,24 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
     a.error_flags = error_flags_address();
     if (!a.error_flags) return DQ_ERR_CUDA;
 
-    // power-of-two buckets up to 8192: whole work units (a bucket, or 1024 elements for smaller buckets) go
-    // through the tile path of the kernel, the rest (and every other bucket size) through its plain-load part,
-    // in the same launch
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
     // The tile kernel streams back-to-back encodes of long gradients through persistent CTAs: with launches that overlap
     // by the caller's flags it is 1 to 6 % faster from 16 M elements on (n = 25.6 M, B = 2048: 22.1 us against 22.4 with
     // two bits, 23.6 against 24.9 with three).  Everything else goes through the direct kernel.
-    const bool tiles_wanted = a.test_drop_copy != 0u ||
-                              (a.early_store != 0u && is_pow2(p->bucket) && p->bucket <= 8192u && n >= (1ull << 24));
+    const bool tiles_wanted = is_pow2(p->bucket) && p->bucket <= 8192u &&
+                              (a.test_drop_copy != 0u || (a.early_store != 0u && n >= (1ull << 24)));
     if (!tiles_wanted) {
         if (encode_direct(mode, *p, a, n, sms, st) != cudaSuccess) return DQ_ERR_CUDA;
         g_launches.fetch_add(1);
         return DQ_OK;
     }
+    // whole work units (a bucket, or 1024 elements for smaller buckets) go through the tile path of the kernel, the rest
+    // through its plain-load part, in the same launch
     a.sm_count = (uint32_t)sms;
     const uint32_t B = p->bucket;
     const uint32_t U = (B < 1024u) ? 1024u : B;                     // elements per work unit
-    uint64_t tiles = (is_pow2(B) && B <= 8192u) ? n / U : 0u;       // whole units
+    const uint64_t tiles = n / U;                                   // whole units
     if (tiles > 0xFFFFFFFFull) return DQ_ERR_UNSUPPORTED;
     CUtensorMap map;
     std::memset(&map, 0, sizeof(map));

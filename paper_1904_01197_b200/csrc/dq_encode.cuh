@@ -1,13 +1,12 @@
-// Encode kernel: per-bucket scale, dither, quantize, (coset), pack -- one pass over the gradient
-// (Eq. (DQSG) and Algorithm 1, worker steps; nested encoder equation and Algorithm 2, workers in P2).
+// Tile encoder: the encode step (see dq_encode_direct.cuh, which serves every other call) for long gradients that are
+// encoded back to back with overlapping launches, in power-of-two buckets up to 8192; and what both encoders share.
 //
 // Work decomposition: a "row" is 32 consecutive elements = one 128-byte line of the gradient and exactly
 // `bits` 32-bit words of the bit stream.  One lane quantizes and packs a whole row, so no lane ever shares a
 // packed word with another lane and no shuffles are needed for packing.
 //
-// Power-of-two buckets up to 8192 take the tile path: persistent CTAs of eight warps, every warp with its own
-// two-stage shared-memory pipeline of 4 KB tiles (32 rows) filled by asynchronous 2-D tile copies (128-byte
-// swizzle, which makes "lane r reads row r" free of bank conflicts).
+// Persistent CTAs of eight warps, every warp with its own two-stage shared-memory pipeline of 4 KB tiles (32 rows)
+// filled by asynchronous 2-D tile copies (128-byte swizzle, which makes "lane r reads row r" free of bank conflicts).
 //   B <= 1024: a work unit is 1024 elements; a warp takes a stage into registers, re-arms the stage with the
 //     copy for the unit after next, reduces max|g| over each bucket with shuffles and quantizes from registers.
 //   B = 2048, 4096, 8192: a work unit is a bucket and a warp takes 2048 elements of it as two halves in time,
@@ -17,10 +16,14 @@
 //     meet once per bucket in a named barrier to exchange their maxima.
 // The units are dealt out round-robin over the warp groups of all CTAs.  The gradient is read from HBM exactly once.
 //
-// Everything else -- other bucket sizes, the part of the vector past the last whole tile, the ragged end --
-// is handled by plain-load code in extra CTAs of the same launch: buckets of at most 32 rows in warp windows of
-// whole buckets (one row per lane, segmented maximum over the lanes), buckets of up to 4096 elements one per warp,
-// larger ones one per CTA (a sweep for the maximum, then a second, cached sweep that quantizes).
+// The part of the vector past the last whole tile is handled by plain-load code in extra CTAs of the same launch:
+// buckets of at most 32 rows in warp windows of whole buckets (one row per lane, segmented maximum over the lanes),
+// buckets of up to 4096 elements one per warp, larger ones one per CTA (a sweep for the maximum, then a second, cached
+// sweep that quantizes).
+//
+// What bounds it: the multiplier pipe and instruction issue, as in the direct encoder.  On packed fp32 pairs and with
+// the clamp in one instruction the overlapped encode of n = 25.6 M takes 22.1 us (2 bits, before 22.6) and 23.6 us
+// (3 bits, before 25.5).
 #pragma once
 
 #include "dq_device.cuh"
