@@ -365,13 +365,14 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 // Elements per lane of the decoder.  Up to one wave of 8-element lanes (1.2 M elements on 148 SMs) the GPU is not
 // full and the shortest chain per lane wins (W = 8: n = 266,610 6.6 us with 8, 8.5 with 16, 12.8 with 32).  Beyond it
 // 16 and then 32 elements amortise what a worker costs per lane; 32 pays from about two and a half of its own waves
-// (W = 8: n = 4.2 M 38.1 us with 16, 40.5 with 32; n = 11.7 M 79.0 and 75.7), and not for one or two workers, where
-// memory latency matters more and 16 has more warps to hide it (W = 1, n = 25.6 M: 33.8 us with 16, 38.5 with 32).
-int decode_group_size(uint64_t n, uint32_t W, int sms)
+// (W = 8: n = 4.2 M 38.1 us with 16, 40.5 with 32; n = 11.7 M 79.0 and 75.7), and not for one worker, or two and a side
+// information vector, where memory latency matters more and 16 has more warps to hide it (n = 25.6 M: W = 1 31.1 us with
+// 16, 34.8 with 32; W = 2 with a vector 62.6 and 67.4, without 51.6 and 47.2).
+int decode_group_size(uint64_t n, uint32_t W, bool reads_side, int sms)
 {
     const uint64_t lanes = (uint64_t)sms * dq::kDecThreads;
     if (n <= 8u * lanes * dq::dec_ctas_per_sm(8, dq::kSetUsual)) return 8;
-    if (W <= 2u || 2u * n < 5u * 32u * lanes * dq::dec_ctas_per_sm(32, dq::kSetAll)) return 16;
+    if (W <= (reads_side ? 2u : 1u) || 2u * n < 5u * 32u * lanes * dq::dec_ctas_per_sm(32, dq::kSetAll)) return 16;
     return 32;
 }
 
@@ -461,7 +462,7 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
     const bool d16 = (msgs[0].p.dither_bits == 16u);
-    const int E = decode_group_size(n, W, sms);
+    const int E = decode_group_size(n, W, reads_side, sms);
     a.num_groups = (n + (uint32_t)E - 1u) / (uint32_t)E;
     a.early_launch = a.num_groups <= (uint64_t)sms * dq::kDecThreads ? 1u : 0u;
     cudaError_t le;

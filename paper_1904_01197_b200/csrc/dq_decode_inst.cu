@@ -49,7 +49,8 @@ cudaError_t launch_groups_of(const DecodeArgs& a, cudaStream_t st)
         have = (int)(v & 7u) + 1;
     }
     if constexpr (E >= 16) {
-        if (usual && one_pair && a.W > 2u) {           // (one or two messages are no faster: n = 25.6 M 31.8 and 33.9 us)
+        // (not for one or two messages in groups of 16: W = 1, n = 25.6 M 31.8 us with the usual set, 33.9 with the pair)
+        if (usual && one_pair && (a.W > 2u || E == 32)) {
             if (width[0] == 0) width[0] = width[1];
             if (width[1] == 0) width[1] = width[0];
             switch (width[0]) {
