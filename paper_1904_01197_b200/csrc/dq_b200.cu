@@ -217,7 +217,8 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     // while gpb <= 1024, and larger buckets are alone in their window
     a.bucket_magic = ((1u << 22) + gpb - 1u) / gpb;
     a.reduce = (gpb <= 32u && is_pow2(gpb))                            ? dq::kPartOfWarp
-               : (R == 4 && (gpb == 64u || gpb == 128u))               ? dq::kChunks
+               : (R == 4 && gpb == 64u)                                ? dq::kTwoChunks
+               : (R == 4 && gpb == 128u)                               ? dq::kWarpIsBucket
                : (shape.cluster > 1u || gpb % (32u * (uint32_t)R) == 0u) ? dq::kWarpInBucket
                                                                        : dq::kAnywhere;
     a.grad_align32 = (reinterpret_cast<uintptr_t>(e.grad) & 31u) == 0u ? 1u : 0u;

@@ -29,9 +29,10 @@ template <int R> constexpr int kDirectMaxCluster = 65536 / (8 * R * kDirectMaxTh
 // How the lanes' maxima meet in a bucket's scale.
 enum DirectReduce : uint32_t {
     kPartOfWarp = 0,      // a bucket is an aligned power-of-two part of a chunk of 32 groups
-    kChunks = 1,          // a bucket is 2 or 4 of a warp's chunks
-    kWarpInBucket = 2,    // a warp lies within one bucket: shared memory
-    kAnywhere = 3         // anything else: shared memory, lane by lane
+    kTwoChunks = 1,       // a bucket is two of a warp's four chunks
+    kWarpIsBucket = 2,    // a bucket is what a warp takes: no barrier, one gain
+    kWarpInBucket = 3,    // a warp lies within one bucket: shared memory, one gain
+    kAnywhere = 4         // anything else: shared memory, lane by lane
 };
 
 struct DirectArgs {
@@ -253,16 +254,20 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
 #pragma unroll
         for (int c = 0; c < R; ++c) mb[c] = m;
     } else if (args.reduce == kPartOfWarp) {
-        for (uint32_t step = 1u; step < gpb; step <<= 1) {
+        if (gpb == 32u) {
 #pragma unroll
-            for (int c = 0; c < R; ++c) mb[c] = max(mb[c], __shfl_xor_sync(0xFFFFFFFFu, mb[c], step));
+            for (int c = 0; c < R; ++c) mb[c] = warp_max(mb[c]);
+        } else {
+            for (uint32_t step = 1u; step < gpb; step <<= 1) {
+#pragma unroll
+                for (int c = 0; c < R; ++c) mb[c] = max(mb[c], __shfl_xor_sync(0xFFFFFFFFu, mb[c], step));
+            }
         }
-    } else if (args.reduce == kChunks) {
-        if constexpr (R == 4) {
-            mb[0] = mb[1] = warp_max(max(mb[0], mb[1]));
-            mb[2] = mb[3] = warp_max(max(mb[2], mb[3]));
-            if (gpb == 128u) mb[0] = mb[1] = mb[2] = mb[3] = max(mb[0], mb[2]);
-        }
+    } else if (R == 4 && args.reduce == kWarpIsBucket) {
+        mb[0] = mb[1 % R] = mb[2 % R] = mb[3 % R] = warp_max(max(max(mb[0], mb[1 % R]), max(mb[2 % R], mb[3 % R])));
+    } else if (R == 4 && args.reduce == kTwoChunks) {
+        mb[0] = mb[1 % R] = warp_max(max(mb[0], mb[1 % R]));
+        mb[2 % R] = mb[3 % R] = warp_max(max(mb[2 % R], mb[3 % R]));
     } else {
 #pragma unroll
         for (int c = 0; c < R; ++c) {
@@ -285,10 +290,12 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
     // M0 k + M0 j), which are cheaper than wide multiplies on the pipe that bounds the kernel
     const uint64_t p0 = (uint64_t)kPhiloxM0 * ((args.first_group + group) * kBlocks);
     uint32_t out[R][NW];
+    const bool one_gain = args.reduce == kWarpIsBucket || args.reduce == kWarpInBucket;
     f32x2 aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[0])));
 #pragma unroll
     for (int c = 0; c < R; ++c) {
-        if (c > 0 && args.reduce != kWarpInBucket) aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
+        if (c > 0 && !one_gain && !(c % 2 == 1 && args.reduce == kTwoChunks))
+            aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
         encode_group8<BITS, MODE, DITH>(x + 4 * c, p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0, aa, args, out[c]);
     }
     if (!waited && args.early_store == 0u) {
@@ -310,7 +317,7 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
     // the scale leaves with the first group of a bucket
 #pragma unroll
     for (int c = 0; c < R; ++c) {
-        if (c > 0 && args.reduce == kWarpInBucket) break;       // a warp's first group is the only candidate
+        if (c > 0 && one_gain) break;            // a warp's first group is the only candidate
         const uint32_t at = local + 32u * c;
         const uint32_t b = (args.cluster > 1u) ? 0u : (at * args.bucket_magic) >> 22;
         if (at == b * gpb && at < gpw && group + 32u * c < args.num_groups)
