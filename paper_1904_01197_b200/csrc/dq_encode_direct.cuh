@@ -49,6 +49,7 @@ struct DirectArgs {
     uint32_t cluster;             // CTAs per bucket, 1 unless a bucket is larger than a CTA
     uint32_t bucket_magic;        // group of the window -> bucket: (group * bucket_magic) >> 22
     uint32_t reduce;              // DirectReduce
+    uint32_t gains;               // further gains than the first chunk's: 0 none, 1 the third's, 2 every chunk's
     uint32_t grad_align32;        // grad is 32-byte aligned
     float gain_num;               // DQSG: s = (L-1)/2;  NDQSG: A = alpha * M1
     int32_t kmax;                 // DQSG: L - 1
@@ -290,12 +291,10 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
     // M0 k + M0 j), which are cheaper than wide multiplies on the pipe that bounds the kernel
     const uint64_t p0 = (uint64_t)kPhiloxM0 * ((args.first_group + group) * kBlocks);
     uint32_t out[R][NW];
-    const bool one_gain = args.reduce == kWarpIsBucket || args.reduce == kWarpInBucket;
     f32x2 aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[0])));
 #pragma unroll
     for (int c = 0; c < R; ++c) {
-        if (c > 0 && !one_gain && !(c % 2 == 1 && args.reduce == kTwoChunks))
-            aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
+        if (c > 0 && args.gains > (uint32_t)(c % 2)) aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
         encode_group8<BITS, MODE, DITH>(x + 4 * c, p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0, aa, args, out[c]);
     }
     if (!waited && args.early_store == 0u) {
@@ -317,7 +316,7 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
     // the scale leaves with the first group of a bucket
 #pragma unroll
     for (int c = 0; c < R; ++c) {
-        if (c > 0 && one_gain) break;            // a warp's first group is the only candidate
+        if (c > 0 && args.gains == 0u) break;    // a warp's first group is the only candidate
         const uint32_t at = local + 32u * c;
         const uint32_t b = (args.cluster > 1u) ? 0u : (at * args.bucket_magic) >> 22;
         if (at == b * gpb && at < gpw && group + 32u * c < args.num_groups)
