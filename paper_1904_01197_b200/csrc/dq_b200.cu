@@ -221,7 +221,9 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
                : (R == 4 && gpb == 128u)                               ? dq::kWarpIsBucket
                : (shape.cluster > 1u || gpb % (32u * (uint32_t)R) == 0u) ? dq::kWarpInBucket
                                                                        : dq::kAnywhere;
-    a.gains = (a.reduce == dq::kWarpIsBucket || a.reduce == dq::kWarpInBucket) ? 0u : a.reduce == dq::kTwoChunks ? 1u : 2u;
+    a.gains = (a.reduce == dq::kWarpIsBucket || a.reduce == dq::kWarpInBucket) ? 0u
+              : a.reduce == dq::kTwoChunks                                     ? 1u
+                                                                               : 2u;
     a.grad_align32 = (reinterpret_cast<uintptr_t>(e.grad) & 31u) == 0u ? 1u : 0u;
     a.gain_num = e.gain_num;
     a.kmax = e.kmax;
