@@ -8,6 +8,7 @@ fallback: if a shared library is missing the first call fails.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes as C
 import importlib.util
 from pathlib import Path
@@ -189,6 +190,16 @@ def new_output(numel: int, dtype, device) -> torch.Tensor:
     return torch.empty(numel, dtype=dtype, device=device)
 
 
+def _allocating_for(stream, device):
+    """Context for allocating the outputs of a call on `stream`: they belong to the stream that the kernel runs on.
+    Memory of the current stream may still be in use by what is queued there, which the kernel would not wait for."""
+    if stream is None:
+        return contextlib.nullcontext()
+    if not isinstance(stream, torch.cuda.Stream):
+        stream = torch.cuda.ExternalStream(int(stream.cuda_stream), device)
+    return torch.cuda.stream(stream)
+
+
 def alloc_message(n: int, params: DqParams, device="cuda"):
     """Uninitialised output buffers for one encode call (packed words as int32, scales as fp32)."""
     packed = new_output(max(1, packed_words(n, params.bits)), torch.int32, device)
@@ -206,7 +217,8 @@ def dqsg_encode(grad: torch.Tensor, seed: int, worker: int, step: int, params: D
                 out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                 stream=None):
     if out_packed is None or out_scale is None:
-        out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
+        with _allocating_for(stream, grad.device):
+            out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
     status = (_calls_module or _calls()).encode(DQ_KIND_DQSG, grad, 0, seed, worker, step, params, out_packed, out_scale,
                                                 stream)
     if status:
@@ -218,7 +230,8 @@ def ndqsg_encode(grad: torch.Tensor, seed: int, worker: int, step: int, params: 
                  out_packed: Optional[torch.Tensor] = None, out_scale: Optional[torch.Tensor] = None,
                  stream=None):
     if out_packed is None or out_scale is None:
-        out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
+        with _allocating_for(stream, grad.device):
+            out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
     status = (_calls_module or _calls()).encode(DQ_KIND_NDQSG, grad, 0, seed, worker, step, params, out_packed, out_scale,
                                                 stream)
     if status:
@@ -246,7 +259,8 @@ def bucket_ranges(n: int, bucket: int, parts: int):
 
 def _encode_range(kind, what, grad, first_element, seed, worker, step, params, out_packed, out_scale, stream):
     if out_packed is None or out_scale is None:
-        out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
+        with _allocating_for(stream, grad.device):
+            out_packed, out_scale = alloc_message(grad.numel(), params, grad.device)
     status = (_calls_module or _calls()).encode(kind, grad, first_element, seed, worker, step, params, out_packed,
                                                 out_scale, stream)
     if status:
@@ -282,7 +296,8 @@ _DQSG, _NDQSG, _RANGE, _HALF_DITHERED, _RUNNING, _SIDE_FIRST = range(6)
 
 def _decode(how, what, msgs, n, first_element, step, side_info, out_avg, status_word, stream):
     if out_avg is None:
-        out_avg = new_output(max(1, n), torch.float32, msgs[0].packed.device)
+        with _allocating_for(stream, msgs[0].packed.device):
+            out_avg = new_output(max(1, n), torch.float32, msgs[0].packed.device)
     status = (_calls_module or _calls()).decode(how, msgs, n, first_element, step, side_info, out_avg, status_word,
                                                 stream)
     if status != 0:
@@ -334,7 +349,8 @@ def code_histogram(packed: torch.Tensor, n: int, bits: int, hist: Optional[torch
                    stream=None) -> torch.Tensor:
     """hist[c] = number of elements of the packed message whose code is c (int64[2^bits] on the device)."""
     if hist is None:
-        hist = new_output(1 << bits, torch.int64, packed.device)
+        with _allocating_for(stream, packed.device):
+            hist = new_output(1 << bits, torch.int64, packed.device)
     _check((_calls_module or _calls()).code_histogram(packed, n, bits, hist, stream), "dq_code_histogram")
     return hist
 
@@ -358,7 +374,8 @@ def ternary_pack(packed: torch.Tensor, n: int, out: Optional[torch.Tensor] = Non
                  status_word: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """2-bit stream of a three-level message -> five codes per byte (uint8[ternary_bytes(n)] on the device)."""
     if out is None:
-        out = new_output(max(1, ternary_bytes(n)), torch.uint8, packed.device)
+        with _allocating_for(stream, packed.device):
+            out = new_output(max(1, ternary_bytes(n)), torch.uint8, packed.device)
     _check((_calls_module or _calls()).ternary_pack(packed, n, out, status_word, stream), "dq_ternary_pack")
     return out
 
@@ -366,7 +383,8 @@ def ternary_pack(packed: torch.Tensor, n: int, out: Optional[torch.Tensor] = Non
 def ternary_unpack(data: torch.Tensor, n: int, out: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Five codes per byte -> the 2-bit stream (int32[packed_words(n, 2)] on the device)."""
     if out is None:
-        out = new_output(max(1, packed_words(n, 2)), torch.int32, data.device)
+        with _allocating_for(stream, data.device):
+            out = new_output(max(1, packed_words(n, 2)), torch.int32, data.device)
     _check((_calls_module or _calls()).ternary_unpack(data, n, out, stream), "dq_ternary_unpack")
     return out
 

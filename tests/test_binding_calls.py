@@ -1,0 +1,87 @@
+"""The Python binding's own work, without a GPU: where the outputs that it allocates come from."""
+import contextlib
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def dq():
+    from paper_1904_01197_b200 import build
+    build.build()
+    import paper_1904_01197_b200 as dq
+    return dq
+
+
+def _calls_that_allocate(dq):
+    p = dq.DqParams(512, 2, 3)
+    g = torch.zeros(1000)
+    m = [dq.Message(torch.zeros(63, dtype=torch.int32), torch.zeros(2), 1, 0, dq.DQ_KIND_DQSG, p)]
+    return {
+        "dqsg_encode": lambda s: dq.dqsg_encode(g, 1, 0, 0, p, stream=s),
+        "ndqsg_encode": lambda s: dq.ndqsg_encode(g, 1, 0, 0, p, stream=s),
+        "dqsg_encode_range": lambda s: dq.dqsg_encode_range(g, 512, 1, 0, 0, p, stream=s),
+        "ndqsg_encode_range": lambda s: dq.ndqsg_encode_range(g, 512, 1, 0, 0, p, stream=s),
+        "dqsg_decode_aggregate": lambda s: dq.dqsg_decode_aggregate(m, 1000, 0, stream=s),
+        "ndqsg_decode_aggregate": lambda s: dq.ndqsg_decode_aggregate(m, 1000, 0, None, stream=s),
+        "range": lambda s: dq.ndqsg_decode_aggregate_range(m, 1000, 512, 0, None, stream=s),
+        "half": lambda s: dq.dqsg_decode_aggregate_half_dithered(m, 1000, stream=s),
+        "running": lambda s: dq.ndqsg_decode_aggregate_running(m, 1000, 0, stream=s),
+        "first": lambda s: dq.ndqsg_decode_aggregate_side_first(m, 1000, 0, stream=s),
+        "histogram": lambda s: dq.code_histogram(m[0].packed, 1000, 2, stream=s),
+        "ternary_pack": lambda s: dq.ternary_pack(m[0].packed, 1000, stream=s),
+        "ternary_unpack": lambda s: dq.ternary_unpack(torch.zeros(200, dtype=torch.uint8), 1000, stream=s),
+    }
+
+
+class _Stream:
+    cuda_stream = 0x1230
+
+
+class _FakeCalls:
+    """In the place of the native calls: every call succeeds without a GPU."""
+    encode = decode = code_histogram = ternary_pack = ternary_unpack = staticmethod(lambda *a: 0)
+
+
+@pytest.mark.parametrize("given", [True, False])
+def test_outputs_are_allocated_on_the_stream_of_the_call(dq, monkeypatch, given):
+    entered, allocated_in = [], []
+
+    @contextlib.contextmanager
+    def on(stream):
+        entered.append(stream)
+        yield
+        entered.pop()
+
+    def new_output(numel, dtype, device):
+        allocated_in.append(list(entered))
+        return torch.empty(numel, dtype=dtype)
+
+    monkeypatch.setattr(torch.cuda, "stream", on)
+    monkeypatch.setattr(torch.cuda, "ExternalStream", lambda ptr, device: ("stream", ptr))
+    monkeypatch.setattr(dq.binding, "new_output", new_output)
+    monkeypatch.setattr(dq.binding, "_calls_module", _FakeCalls)
+    for name, call in _calls_that_allocate(dq).items():
+        allocated_in.clear()
+        call(_Stream if given else None)
+        assert allocated_in, name
+        assert all(a == ([("stream", 0x1230)] if given else []) for a in allocated_in), name
+
+
+@pytest.mark.gpu
+def test_a_call_on_a_side_stream_does_not_wait_for_and_is_not_overwritten_by_the_current_one(dq):
+    """The current stream is busy while the call runs on another: what the current stream has queued (here the fill of
+    the guard words, done when an output is allocated) must not land on the results."""
+    p = dq.DqParams(512, 2, 3)
+    g = torch.randn(70_001, device="cuda")
+    want = dq.dqsg_encode(g, 1, 0, 0, p)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    torch.cuda._sleep(20_000_000)                       # about ten milliseconds
+    got = dq.dqsg_encode(g, 1, 0, 0, p, stream=side)
+    with torch.cuda.stream(side):
+        early = [t.cpu() for t in got]
+    torch.cuda.synchronize()
+    for w, e, t in zip(want, early, got):
+        assert torch.equal(w.cpu(), e) and torch.equal(w, t)
