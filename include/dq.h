@@ -87,6 +87,10 @@ typedef struct {
  * gradients are encoded back to back.  The encoder then requests and quantizes its first tiles while the
  * previous kernel is still draining; its stores to out_packed and out_scale still wait for that kernel to
  * complete, so outputs may be shared with it.  Results are identical with and without the flag.
+ * This flag and the next one speak about the previous kernel of the stream only: everything that was enqueued before
+ * that kernel is complete when the encoder starts, where that kernel is one of this library's or was launched in the
+ * ordinary way.  (A kernel of the caller's that is itself launched with programmatic stream serialization must not
+ * trigger the launch of its dependents before it has waited for its own predecessor.)
  */
 #define DQ_FLAG_INPUT_READY 0x1u
 /*

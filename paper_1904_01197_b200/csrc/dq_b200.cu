@@ -238,8 +238,9 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     a.two = e.two;
     a.off = e.off;
     a.ps = e.ps;
-    const uint64_t grid = (dq_num_buckets(n, p.bucket) + shape.buckets - 1u) / shape.buckets * shape.cluster;
-    a.early_launch = (a.early_read || grid <= (uint64_t)sms) ? 1u : 0u;
+    // (with early_read one cluster more: see the kernel)
+    const uint64_t grid = ((dq_num_buckets(n, p.bucket) + shape.buckets - 1u) / shape.buckets + (a.early_read ? 1u : 0u)) *
+                          shape.cluster;
     return launch_direct(mode, p.bits, p.dither_bits == 16u, R, a, (uint32_t)grid, shape.threads, st);
 }
 
@@ -468,7 +469,6 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     const bool d16 = (msgs[0].p.dither_bits == 16u);
     const int E = decode_group_size(n, W, reads_side, sms);
     a.num_groups = (n + (uint32_t)E - 1u) / (uint32_t)E;
-    a.early_launch = a.num_groups <= (uint64_t)sms * dq::kDecThreads ? 1u : 0u;
     cudaError_t le;
     if (half_dithered) le = dq::launch_decode_d0_r0(a, E, st);
     else if (running && any_nested) le = d16 ? dq::launch_decode_d16_r1(a, E, st) : dq::launch_decode_d32_r1(a, E, st);

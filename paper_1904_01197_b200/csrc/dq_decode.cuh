@@ -63,7 +63,6 @@ struct DecodeHead {
     uint32_t bucket_shift;    // row -> bucket: (row * bucket_magic) >> 32 >> bucket_shift, or row >> bucket_shift
     uint32_t bucket_magic;    // when bucket_magic is 0 (power-of-two buckets); see set_bucket_division
     uint32_t has_side;        // the side information vector is read
-    uint32_t early_launch;    // the grid has at most one CTA per SM (see the kernel)
     uint32_t out_align32;     // out is 32-byte aligned: whole groups leave in 32-byte stores
     uint32_t half_bias_bits;  // 0x4A800000 (bit pattern of 2^22), passed in so that it lives in a register
     float Wf;
@@ -419,15 +418,12 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
                                                             __uint_as_float(p[4 * j + 2]), __uint_as_float(p[4 * j + 3]));
         }
     }
-    // The next kernel may become resident once every CTA of this one is past its wait, so that at most one kernel
-    // waits beside the running one.  Letting it in at once would let kernel after kernel of a short-call loop pile up,
-    // and the CTAs of one kernel would then be placed wherever slots happen to fall free, several on one SM and none
-    // on others (W = 8, n = 266,610: 11.9 us per call instead of 6.6).  A grid of at most one CTA per SM has nothing to
-    // balance, and gains 0.8 us per call by overlapping two launches.
-    if (args.early_launch != 0u) grid_dependency_launch_next();
     // the messages (and the side information) may be the previous kernel's output
     grid_dependency_wait();
-    if (args.early_launch == 0u) grid_dependency_launch_next();
+    // The next kernel may become resident once every CTA of this one is past its wait: see launch_overlapped.  Letting
+    // kernel after kernel of a short-call loop pile up would also place the CTAs of one kernel wherever slots happen to
+    // fall free, several on one SM and none on others (W = 8, n = 266,610: 11.9 us per call instead of 6.6).
+    grid_dependency_launch_next();
     ln.kappa_next = __ldg(args.w[0].scale + ln.bucket);
 
     if (SIDE == kSideGiven && args.has_side != 0u) {

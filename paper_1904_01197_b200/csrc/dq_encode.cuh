@@ -357,10 +357,14 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
     const uint32_t warp = threadIdx.x >> 5;
     const uint32_t lane = threadIdx.x & 31u;
 
-    grid_dependency_launch_next();
+    // With early_read the next kernel is let in at once, but for the last CTA, which waits for the previous kernel
+    // before its first stores and lets the next one in only then: see launch_overlapped.
+    const bool last_cta = blockIdx.x == gridDim.x - 1u;
+    if (args.early_read != 0u && !last_cta) grid_dependency_launch_next();
 
     if (blockIdx.x < args.plain_ctas) {
         grid_dependency_wait();
+        grid_dependency_launch_next();
         if (args.bucket <= 1024u) {
             // windows of whole buckets (at most 32 rows), one per warp, round-robin over these CTAs
             for (uint64_t w = (uint64_t)blockIdx.x * kConsumerWarps + warp; w < args.plain_windows;
@@ -403,8 +407,11 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
     // outputs are declared free as well (early_store), it moves to the end of the warp's work, where it only keeps
     // this grid from completing before its predecessor (a later kernel that waits for this one may rely on both).
     bool waited = (args.early_read == 0u);
-    const bool wait_before_store = (args.early_store == 0u);
-    if (waited) grid_dependency_wait();
+    const bool wait_before_store = (args.early_store == 0u) || last_cta;
+    if (waited) {
+        grid_dependency_wait();
+        grid_dependency_launch_next();
+    }
     if (lane == 0) {
         // All resident warps would request their first tiles (the whole shared memory of every SM, a quarter of a
         // ResNet-50-sized gradient) at the same instant; served interleaved, every warp would then get its data
@@ -513,12 +520,17 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
                 const uint32_t row = part * 64u + half * 32u + lane;
                 uint32_t out[BITS];
                 encode_row<BITS, MODE, DITH>(x, row + args.row_offset, a, args, out);
-                if (!waited && wait_before_store) { grid_dependency_wait(); waited = true; }
+                if (!waited && wait_before_store) {
+                    grid_dependency_wait();
+                    grid_dependency_launch_next();
+                    waited = true;
+                }
                 if (half == 0u && lane == 0 && sub == 0u) args.scale[pair] = mx;
                 store_row_words<BITS>(args.packed + (uint64_t)row * BITS, out);
             }
         }
         if (!waited) grid_dependency_wait();
+        grid_dependency_launch_next();
         return;
     }
 
@@ -566,11 +578,16 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
 
         uint32_t out[BITS];
         encode_row<BITS, MODE, DITH>(x, row + args.row_offset, a, args, out);
-        if (!waited && wait_before_store) { grid_dependency_wait(); waited = true; }
+        if (!waited && wait_before_store) {
+            grid_dependency_wait();
+            grid_dependency_launch_next();
+            waited = true;
+        }
         if ((lane & (args.lanes_per_bucket - 1u)) == 0u) args.scale[row >> (args.bucket_log2 - 5u)] = mx;
         store_row_words<BITS>(args.packed + (uint64_t)row * BITS, out);
     }
     if (!waited) grid_dependency_wait();
+    grid_dependency_launch_next();
 }
 
 }  // namespace dq

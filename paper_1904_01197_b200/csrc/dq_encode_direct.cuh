@@ -61,8 +61,7 @@ struct DirectArgs {
     uint32_t K_magic;             // NDQSG any K: ceil(2^32 / K)
     uint32_t first_group;         // index of grad[0]'s group in the whole gradient (0 unless a bucket range is encoded):
                                   // only the dither counters see it
-    uint32_t early_launch;        // } see the kernel and EncodeArgs
-    uint32_t early_read;          // }
+    uint32_t early_read;          // } see the kernel and EncodeArgs
     uint32_t early_store;         // }
     f32x2 shift, magic, two, off; // pairs of equal values: DQSG s; 1.5 * 2^23; scale and offset of the dither
     PhiloxStream ps;
@@ -185,9 +184,18 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     const uint32_t gpb = args.groups_per_bucket, gpw = args.groups_per_window;
-    // One kernel waits beside the running one at most (see the decoder), unless this one has nothing to balance or
-    // overlaps with its predecessor by the caller's flags.
-    if (args.early_launch != 0u) grid_dependency_launch_next();
+    // A launch that overlaps with its predecessor by the caller's flags lets its successor in at once, but for its last
+    // cluster, which has no work: that one waits for the predecessor first.  The successor, which may store without
+    // waiting, therefore starts only when everything before this grid is complete (see launch_overlapped), and this grid
+    // does not complete before its predecessor, on which a later kernel relies.
+    if (args.early_read != 0u) {
+        if (blockIdx.x >= gridDim.x - args.cluster) {
+            grid_dependency_wait();
+            grid_dependency_launch_next();
+            return;
+        }
+        grid_dependency_launch_next();
+    }
     uint32_t window = blockIdx.x, part = 0u;
     if (args.cluster > 1u) {
         window = blockIdx.x / args.cluster;
@@ -199,10 +207,9 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
     const uint32_t warp_end = local - lane + 32u * (uint32_t)R;
     const bool whole = warp_end <= gpw && group - lane + 32u * (uint32_t)R <= args.whole_groups;     // (uniform in a warp)
 
-    bool waited = args.early_read == 0u;
-    if (waited) {
+    if (args.early_read == 0u) {
         grid_dependency_wait();
-        if (args.early_launch == 0u) grid_dependency_launch_next();
+        grid_dependency_launch_next();
     }
     f32x2 x[4 * R];
     uint32_t mb[R];
@@ -300,10 +307,7 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
         if (c > 0 && args.gains > (uint32_t)(c % 2)) aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
         encode_group8<BITS, MODE, DITH>(x + 4 * c, p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0, aa, args, out[c]);
     }
-    if (!waited && args.early_store == 0u) {
-        grid_dependency_wait();
-        waited = true;
-    }
+    if (args.early_read != 0u && args.early_store == 0u) grid_dependency_wait();
     const uint64_t byte = (uint64_t)group * (uint32_t)BITS;
     uint8_t* dst = reinterpret_cast<uint8_t*>(args.packed) + byte;
     if (whole) {
@@ -325,9 +329,6 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
         if (at == b * gpb && at < gpw && group + 32u * c < args.num_groups)
             args.scale[(uint64_t)window * args.buckets_per_window + b] = __uint_as_float(mb[c]);
     }
-    // A grid whose outputs are free of its predecessor still must not complete before it (a later kernel relies on
-    // both): it is enough that its last CTA waits.
-    if (!waited && blockIdx.x == gridDim.x - 1u) grid_dependency_wait();
 }
 
 }  // namespace dq

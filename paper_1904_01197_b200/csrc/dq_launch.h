@@ -17,10 +17,12 @@ struct DirectArgs;
 template <int MAXW> struct DecodeArgsOf;
 using DecodeArgs = DecodeArgsOf<64>;
 
-// Launch with programmatic stream serialization allowed: every kernel of this library executes
-// griddepcontrol.wait before it writes anything, and before it reads anything that the previous kernel of the
-// stream may have produced, so letting the next launch become resident while this one drains only hides launch
-// latency.
+// Launch with programmatic stream serialization allowed: a kernel may become resident while the previous one of the
+// stream drains, which hides launch latency.  Every kernel executes griddepcontrol.wait before it writes anything, and
+// before it reads anything that the previous kernel may have produced -- unless the caller's flags say that an encode
+// need not (EncodeArgs::early_read, early_store), which they say about the previous kernel only.  Therefore at least one
+// CTA of every kernel executes griddepcontrol.launch_dependents only after its own wait: a kernel then starts when
+// everything before its predecessor is complete, and no more than two kernels ever overlap.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_overlapped(void (*kernel)(KArgs...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t st,
                               uint32_t cluster, Args&&... args)

@@ -20,8 +20,8 @@ constexpr uint64_t kHistClusterBytes = 3ull << 19;
 
 __global__ void __launch_bounds__(kHistThreads) clear_histogram_kernel(unsigned long long* hist)
 {
-    grid_dependency_launch_next();
     grid_dependency_wait();
+    grid_dependency_launch_next();
     hist[threadIdx.x] = 0ull;
 }
 
@@ -91,8 +91,8 @@ code_histogram_cluster_kernel(const uint32_t* __restrict__ packed, uint64_t n, u
     __shared__ uint32_t sums[3], total[3];
     if (threadIdx.x < 3u) sums[threadIdx.x] = total[threadIdx.x] = 0u;
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    grid_dependency_launch_next();
     grid_dependency_wait();
+    grid_dependency_launch_next();
     FewCounts f = {0u, 0u, 0u};
     count_words<BITS>(packed, n, (uint64_t)blockIdx.x * kHistClusterThreads + threadIdx.x,
                       (uint64_t)gridDim.x * kHistClusterThreads, f);
