@@ -25,11 +25,12 @@ const char* type_name(at::ScalarType t)
                                                                                              : "torch.uint8";
 }
 
-// Address of a contiguous CUDA tensor of the given type; None is a null pointer.  False: an exception is set.
+// Address of a contiguous CUDA tensor of the given type; None is a null pointer, which the library judges -- but not where
+// the call's length is the tensor's (`numel` given).  False: an exception is set.
 bool device_pointer(PyObject* o, at::ScalarType type, const char* what, void** out, int64_t* numel = nullptr)
 {
     *out = nullptr;
-    if (o == Py_None) return true;
+    if (o == Py_None && !numel) return true;
     if (THPVariable_Check(o)) {
         const at::Tensor& t = THPVariable_Unpack(o);
         if (t.is_cuda() && t.is_contiguous() && t.scalar_type() == type) {

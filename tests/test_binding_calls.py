@@ -1,4 +1,4 @@
-"""The Python binding's own work, without a GPU: where the outputs that it allocates come from."""
+"""The Python binding's own work, without a GPU: where the outputs that it allocates come from, and what it refuses."""
 import contextlib
 
 import pytest
@@ -69,6 +69,17 @@ def test_outputs_are_allocated_on_the_stream_of_the_call(dq, monkeypatch, given)
         assert all(a == ([("stream", 0x1230)] if given else []) for a in allocated_in), name
 
 
+def test_an_encode_without_a_gradient_is_refused(dq):
+    p = dq.DqParams(512, 2, 3)
+    out = torch.zeros(63, dtype=torch.int32), torch.zeros(2)
+    for encode in (dq.dqsg_encode, dq.ndqsg_encode):
+        with pytest.raises(TypeError, match="grad"):
+            encode(None, 1, 0, 0, p, *out, stream=_Stream)
+    # the buffers are as necessary as the gradient
+    with pytest.raises(TypeError):
+        dq.binding._calls().encode(dq.DQ_KIND_DQSG, None, 0, 1, 0, 0, p, None, None, _Stream)
+
+
 @pytest.mark.gpu
 def test_a_call_on_a_side_stream_does_not_wait_for_and_is_not_overwritten_by_the_current_one(dq):
     """The current stream is busy while the call runs on another: what the current stream has queued (here the fill of
@@ -85,3 +96,12 @@ def test_a_call_on_a_side_stream_does_not_wait_for_and_is_not_overwritten_by_the
     torch.cuda.synchronize()
     for w, e, t in zip(want, early, got):
         assert torch.equal(w.cpu(), e) and torch.equal(w, t)
+
+
+@pytest.mark.gpu
+def test_an_encode_without_a_gradient_leaves_the_buffers_alone(dq):
+    p = dq.DqParams(512, 2, 3)
+    pk, sc = torch.full((63,), 7, dtype=torch.int32, device="cuda"), torch.full((2,), 7.0, device="cuda")
+    with pytest.raises(TypeError):
+        dq.dqsg_encode(None, 1, 0, 0, p, pk, sc)
+    assert bool((pk == 7).all()) and bool((sc == 7.0).all())
