@@ -5,10 +5,13 @@
 // the same work takes 0.4 us plus 0.2 us per message.  The GIL is released around the library call, which may block
 // while the stream's launch queue is full.
 //
-// Every function returns the dq_status; errors of the arguments' types raise TypeError, as the ctypes calls do.
+// Every function returns the dq_status; errors of the arguments' types raise TypeError, as the ctypes calls do.  What torch
+// throws while a tensor is looked at (one under vmap has no storage, for instance) is raised as the Python exception
+// that the tensor's own methods raise.
 #include <Python.h>
 
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <vector>
@@ -18,6 +21,21 @@
 namespace {
 
 PyObject *s_packed, *s_scale, *s_seed, *s_worker, *s_kind, *s_params, *s_cuda_stream;
+
+// An owned reference.
+struct Ref {
+    PyObject* v;
+    explicit Ref(PyObject* owned) : v(owned) {}
+    ~Ref() { Py_XDECREF(v); }
+    Ref(const Ref&) = delete;
+    Ref& operator=(const Ref&) = delete;
+};
+
+// The GIL is released while one of these lives.
+struct WithoutGil {
+    PyThreadState* state = PyEval_SaveThread();
+    ~WithoutGil() { PyEval_RestoreThread(state); }
+};
 
 const char* type_name(at::ScalarType t)
 {
@@ -73,44 +91,38 @@ bool as_params(PyObject* o, dq_params* out)
 bool as_stream(PyObject* o, void** out)
 {
     if (o == Py_None) {
-        try {
-            *out = c10::cuda::getCurrentCUDAStream().stream();
-        } catch (const std::exception& e) {
-            PyErr_SetString(PyExc_RuntimeError, e.what());
-            return false;
-        }
+        *out = c10::cuda::getCurrentCUDAStream().stream();
         return true;
     }
-    PyObject* a = PyObject_GetAttr(o, s_cuda_stream);
-    if (!a) return false;
+    Ref a(PyObject_GetAttr(o, s_cuda_stream));
     uint64_t v;
-    const bool ok = as_u64(a, &v);
-    Py_DECREF(a);
+    if (!a.v || !as_u64(a.v, &v)) return false;
     *out = reinterpret_cast<void*>(v);
-    return ok;
+    return true;
 }
 
 bool as_message(PyObject* o, dq_msg* m)
 {
-    struct Attr {
-        PyObject* v;
-        Attr(PyObject* obj, PyObject* name) : v(PyObject_GetAttr(obj, name)) {}
-        ~Attr() { Py_XDECREF(v); }
-    };
     void* p;
     uint32_t kind;
     {
-        Attr a(o, s_packed);
+        Ref a(PyObject_GetAttr(o, s_packed));
         if (!a.v || !device_pointer(a.v, at::kInt, "packed", &p)) return false;
         m->packed = static_cast<const uint32_t*>(p);
     }
     {
-        Attr a(o, s_scale);
+        Ref a(PyObject_GetAttr(o, s_scale));
         if (!a.v || !device_pointer(a.v, at::kFloat, "scale", &p)) return false;
         m->scale = static_cast<const float*>(p);
     }
-    Attr seed(o, s_seed), worker(o, s_worker), k(o, s_kind), params(o, s_params);
-    if (!seed.v || !worker.v || !k.v || !params.v) return false;
+    Ref seed(PyObject_GetAttr(o, s_seed));
+    if (!seed.v) return false;
+    Ref worker(PyObject_GetAttr(o, s_worker));
+    if (!worker.v) return false;
+    Ref k(PyObject_GetAttr(o, s_kind));
+    if (!k.v) return false;
+    Ref params(PyObject_GetAttr(o, s_params));
+    if (!params.v) return false;
     if (!as_u64(seed.v, &m->seed) || !as_u32(worker.v, &m->worker) || !as_u32(k.v, &kind)) return false;
     m->kind = static_cast<dq_kind>(kind);
     return as_params(params.v, &m->p);
@@ -141,11 +153,12 @@ PyObject* encode(PyObject*, PyObject* const* a, Py_ssize_t n_args)
         (uint64_t)have_scales < dq_num_buckets((uint64_t)n, p.bucket))
         return PyLong_FromLong(-1);
     dq_status s;
-    Py_BEGIN_ALLOW_THREADS
-    s = (kind == DQ_KIND_DQSG ? dqsg_encode_range : ndqsg_encode_range)(
-        static_cast<const float*>(grad), (uint64_t)n, first, seed, worker, step, &p, static_cast<uint32_t*>(packed),
-        static_cast<float*>(scale), stream);
-    Py_END_ALLOW_THREADS
+    {
+        WithoutGil released;
+        s = (kind == DQ_KIND_DQSG ? dqsg_encode_range : ndqsg_encode_range)(
+            static_cast<const float*>(grad), (uint64_t)n, first, seed, worker, step, &p, static_cast<uint32_t*>(packed),
+            static_cast<float*>(scale), stream);
+    }
     return PyLong_FromLong(s);
 }
 
@@ -162,9 +175,9 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n_args)
         !device_pointer(a[5], at::kFloat, "side_info", &side) || !device_pointer(a[6], at::kFloat, "out_avg", &out) ||
         !device_pointer(a[7], at::kInt, "status_word", &status) || !as_stream(a[8], &stream))
         return nullptr;
-    PyObject* seq = PySequence_Fast(a[1], "msgs: expected a sequence of messages");
-    if (!seq) return nullptr;
-    const Py_ssize_t W = PySequence_Fast_GET_SIZE(seq);
+    Ref seq(PySequence_Tuple(a[1]));         // (a list could change while its messages' attributes are read)
+    if (!seq.v) return nullptr;
+    const Py_ssize_t W = PyTuple_GET_SIZE(seq.v);
     dq_msg few[DQ_MAX_WORKERS];
     std::vector<dq_msg> many;
     dq_msg* m = few;
@@ -173,31 +186,28 @@ PyObject* decode(PyObject*, PyObject* const* a, Py_ssize_t n_args)
         m = many.data();
     }
     for (Py_ssize_t w = 0; w < W; ++w) {
-        if (!as_message(PySequence_Fast_GET_ITEM(seq, w), m + w)) {
-            Py_DECREF(seq);
-            return nullptr;
-        }
+        if (!as_message(PyTuple_GET_ITEM(seq.v, w), m + w)) return nullptr;
     }
-    Py_DECREF(seq);
     float* o = static_cast<float*>(out);
     uint32_t* st = static_cast<uint32_t*>(status);
     dq_status s = DQ_ERR_INVALID_ARG;
-    Py_BEGIN_ALLOW_THREADS
-    switch (how) {
-        case kDqsg: s = dqsg_decode_aggregate(m, (uint32_t)W, n, step, o, stream); break;
-        case kNdqsg:
-            s = ndqsg_decode_aggregate(m, (uint32_t)W, n, step, static_cast<const float*>(side), o, st, stream);
-            break;
-        case kRange:
-            s = ndqsg_decode_aggregate_range(m, (uint32_t)W, n, first, step, static_cast<const float*>(side), o, st,
-                                             stream);
-            break;
-        case kHalfDithered: s = dqsg_decode_aggregate_half_dithered(m, (uint32_t)W, n, o, stream); break;
-        case kRunning: s = ndqsg_decode_aggregate_running(m, (uint32_t)W, n, step, o, st, stream); break;
-        case kSideFirst: s = ndqsg_decode_aggregate_side_first(m, (uint32_t)W, n, step, o, st, stream); break;
-        default: break;
+    {
+        WithoutGil released;
+        switch (how) {
+            case kDqsg: s = dqsg_decode_aggregate(m, (uint32_t)W, n, step, o, stream); break;
+            case kNdqsg:
+                s = ndqsg_decode_aggregate(m, (uint32_t)W, n, step, static_cast<const float*>(side), o, st, stream);
+                break;
+            case kRange:
+                s = ndqsg_decode_aggregate_range(m, (uint32_t)W, n, first, step, static_cast<const float*>(side), o, st,
+                                                 stream);
+                break;
+            case kHalfDithered: s = dqsg_decode_aggregate_half_dithered(m, (uint32_t)W, n, o, stream); break;
+            case kRunning: s = ndqsg_decode_aggregate_running(m, (uint32_t)W, n, step, o, st, stream); break;
+            case kSideFirst: s = ndqsg_decode_aggregate_side_first(m, (uint32_t)W, n, step, o, st, stream); break;
+            default: break;
+        }
     }
-    Py_END_ALLOW_THREADS
     return PyLong_FromLong(s);
 }
 
@@ -212,9 +222,10 @@ PyObject* code_histogram(PyObject*, PyObject* const* a, Py_ssize_t n_args)
         !device_pointer(a[3], at::kLong, "hist", &hist) || !as_stream(a[4], &stream))
         return nullptr;
     dq_status s;
-    Py_BEGIN_ALLOW_THREADS
-    s = dq_code_histogram(static_cast<const uint32_t*>(packed), n, bits, static_cast<uint64_t*>(hist), stream);
-    Py_END_ALLOW_THREADS
+    {
+        WithoutGil released;
+        s = dq_code_histogram(static_cast<const uint32_t*>(packed), n, bits, static_cast<uint64_t*>(hist), stream);
+    }
     return PyLong_FromLong(s);
 }
 
@@ -229,10 +240,11 @@ PyObject* ternary_pack(PyObject*, PyObject* const* a, Py_ssize_t n_args)
         !as_stream(a[4], &stream))
         return nullptr;
     dq_status s;
-    Py_BEGIN_ALLOW_THREADS
-    s = dq_ternary_pack(static_cast<const uint32_t*>(packed), n, static_cast<uint8_t*>(out),
-                        static_cast<uint32_t*>(status), stream);
-    Py_END_ALLOW_THREADS
+    {
+        WithoutGil released;
+        s = dq_ternary_pack(static_cast<const uint32_t*>(packed), n, static_cast<uint8_t*>(out),
+                            static_cast<uint32_t*>(status), stream);
+    }
     return PyLong_FromLong(s);
 }
 
@@ -246,13 +258,23 @@ PyObject* ternary_unpack(PyObject*, PyObject* const* a, Py_ssize_t n_args)
         !device_pointer(a[2], at::kInt, "out", &out) || !as_stream(a[3], &stream))
         return nullptr;
     dq_status s;
-    Py_BEGIN_ALLOW_THREADS
-    s = dq_ternary_unpack(static_cast<const uint8_t*>(data), n, static_cast<uint32_t*>(out), stream);
-    Py_END_ALLOW_THREADS
+    {
+        WithoutGil released;
+        s = dq_ternary_unpack(static_cast<const uint8_t*>(data), n, static_cast<uint32_t*>(out), stream);
+    }
     return PyLong_FromLong(s);
 }
 
-#define DQ_METHOD(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(f)), METH_FASTCALL, nullptr}
+// No C++ exception may leave through the interpreter's C frames.
+template <PyObject* (*F)(PyObject*, PyObject* const*, Py_ssize_t)>
+PyObject* guarded(PyObject* self, PyObject* const* a, Py_ssize_t n_args)
+{
+    HANDLE_TH_ERRORS
+    return F(self, a, n_args);
+    END_HANDLE_TH_ERRORS
+}
+
+#define DQ_METHOD(f) {#f, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(guarded<f>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {DQ_METHOD(encode),       DQ_METHOD(decode),         DQ_METHOD(code_histogram),
                          DQ_METHOD(ternary_pack), DQ_METHOD(ternary_unpack), {nullptr, nullptr, 0, nullptr}};
 #undef DQ_METHOD

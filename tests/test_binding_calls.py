@@ -1,5 +1,8 @@
 """The Python binding's own work, without a GPU: where the outputs that it allocates come from, and what it refuses."""
 import contextlib
+import subprocess
+import sys
+from pathlib import Path
 
 import pytest
 
@@ -78,6 +81,45 @@ def test_an_encode_without_a_gradient_is_refused(dq):
     # the buffers are as necessary as the gradient
     with pytest.raises(TypeError):
         dq.binding._calls().encode(dq.DQ_KIND_DQSG, None, 0, 1, 0, 0, p, None, None, _Stream)
+
+
+# Tensors under vmap have no storage: torch throws when their address is asked for.
+_VMAPPED = """
+import sys
+sys.path.insert(0, sys.argv[1])
+import torch
+from torch._subclasses.fake_tensor import FakeTensorMode
+import paper_1904_01197_b200 as dq
+
+class Stream:
+    cuda_stream = 0
+
+p = dq.DqParams(512, 2, 3)
+with FakeTensorMode(allow_non_fake_inputs=True):
+    f32, i32, u8 = (torch.empty(3, 1024, dtype=t, device="cuda:0") for t in (torch.float32, torch.int32, torch.uint8))
+    pk, sc, out = i32[0], f32[0], f32[1]
+    for name, x, call in (
+            ("encode", f32, lambda x: dq.dqsg_encode(x, 1, 0, 0, p, pk, sc, stream=Stream)),
+            ("decode", i32, lambda x: dq.dqsg_decode_aggregate([dq.Message(x, sc, 1, 0, 0, p)], 1024, 0, out, stream=Stream)),
+            ("histogram", i32, lambda x: dq.code_histogram(x, 1024, 2, torch.empty(4, dtype=torch.int64, device="cuda:0"),
+                                                           stream=Stream)),
+            ("pack", i32, lambda x: dq.ternary_pack(x, 1024, u8[0], stream=Stream)),
+            ("unpack", u8, lambda x: dq.ternary_unpack(x, 1024, pk, stream=Stream))):
+        def body(t):
+            try:
+                call(t)
+            except RuntimeError as e:
+                print(name, "raised", "storage" in str(e))
+            return t
+        torch.vmap(body)(x)
+"""
+
+
+def test_a_tensor_without_storage_raises_and_does_not_end_the_process(dq):
+    r = subprocess.run([sys.executable, "-c", _VMAPPED, str(Path(__file__).resolve().parent.parent)], capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout.split("\n")[:5] == [f"{c} raised True" for c in ("encode", "decode", "histogram", "pack", "unpack")]
 
 
 @pytest.mark.gpu
