@@ -11,6 +11,7 @@
 #include "dq_decode.cuh"
 #include "dq_encode.cuh"
 #include "dq_encode_direct.cuh"
+#include "dq_host_memory.h"
 #include "dq_launch.h"
 #include "dq_stats.cuh"
 #include "dq_ternary.cuh"
@@ -533,17 +534,55 @@ constexpr uint64_t kHostDirectElements = 1ull << 20;       // up to here without
 constexpr uint64_t kHostPieceElements = 1ull << 22;        // from here in pieces
 constexpr int kHostPieces = 2;
 
-// Device address of pinned host memory, null for any other (or for one that is not 16-byte aligned).
-template <typename T>
-T* pinned_view(T* host)
+// cuPointerGetAttributes, looked up like cuTensorMapEncodeTiled.
+typedef CUresult (*pointer_attributes_fn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+
+pointer_attributes_fn get_pointer_attributes()
 {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    static pointer_attributes_fn fn = []() -> pointer_attributes_fn {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult qres;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &p, cudaEnableDefault, &qres) != cudaSuccess ||
+            qres != cudaDriverEntryPointSuccess)
+            return nullptr;
+        return reinterpret_cast<pointer_attributes_fn>(p);
+    }();
+    return fn;
+}
+
+// The page-locked range that `host` lies in; false when it is not page-locked (or managed memory).
+bool pinned_range(const void* host, dq::PinnedRange* out)
+{
+    pointer_attributes_fn fn = get_pointer_attributes();
+    if (!fn) return false;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_POINTER, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    unsigned int type = 0u;
+    int managed = 0;
+    CUdeviceptr device = 0u, start = 0u;
+    size_t size = 0u;
+    void* values[] = {&type, &managed, &device, &start, &size};
+    const CUdeviceptr p = static_cast<CUdeviceptr>(reinterpret_cast<uintptr_t>(host));
+    if (fn(5u, what, values, p) != CUDA_SUCCESS) {
+        // a host thread that has no context yet gets the runtime's by this call
+        cudaPointerAttributes at;
+        if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (fn(5u, what, values, p) != CUDA_SUCCESS) return false;
     }
-    if (at.type != cudaMemoryTypeHost || !at.devicePointer || !aligned16(at.devicePointer)) return nullptr;
-    return static_cast<T*>(const_cast<void*>(static_cast<const void*>(at.devicePointer)));
+    if (type != (unsigned int)CU_MEMORYTYPE_HOST || managed || device == 0u) return false;
+    *out = {(uint64_t)device, (uint64_t)start, (uint64_t)size};
+    return true;
+}
+
+// Device address of `count` values in page-locked host memory, null where the kernels cannot work on them.
+template <typename T>
+T* pinned_view(T* host, uint64_t count)
+{
+    return reinterpret_cast<T*>(static_cast<uintptr_t>(dq::pinned_device_address(host, count * sizeof(T), pinned_range)));
 }
 
 // A second stream and the events that tie it to the caller's: one set per host thread and device, made at the thread's
@@ -811,9 +850,9 @@ static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const bool plain = (p->flags & DQ_FLAG_TEST_DROP_COPY) != 0u;        // (the hook is about one launch)
     if (!plain && n <= kHostDirectElements) {
-        const float* h_grad = pinned_view(grad);
-        uint32_t* h_packed = h_grad ? pinned_view(out_packed) : nullptr;
-        float* h_scale = h_packed ? pinned_view(out_scale) : nullptr;
+        const float* h_grad = pinned_view(grad, n);
+        uint32_t* h_packed = h_grad ? pinned_view(out_packed, dq_packed_words(n, p->bits)) : nullptr;
+        float* h_scale = h_packed ? pinned_view(out_scale, dq_num_buckets(n, p->bucket)) : nullptr;
         if (h_scale) {
             s = encode_common(kind, h_grad, n, seed, worker, step, p, h_packed, h_scale, st);
             if (s != DQ_OK) return s;
@@ -906,13 +945,13 @@ static dq_status decode_host(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     dq_msg dev_msgs[DQ_MAX_WORKERS];
     if (n <= kHostDirectElements) {
-        float* h_out = pinned_view(out_avg);
-        const float* h_side = (h_out && side_info) ? pinned_view(side_info) : nullptr;
+        float* h_out = pinned_view(out_avg, n);
+        const float* h_side = (h_out && side_info) ? pinned_view(side_info, n) : nullptr;
         bool direct = h_out != nullptr && (!side_info || h_side);
         for (uint32_t w = 0; w < W && direct; ++w) {
             dev_msgs[w] = msgs[w];
-            dev_msgs[w].packed = pinned_view(msgs[w].packed);
-            dev_msgs[w].scale = pinned_view(msgs[w].scale);
+            dev_msgs[w].packed = pinned_view(msgs[w].packed, dq_packed_words(n, msgs[w].p.bits));
+            dev_msgs[w].scale = pinned_view(msgs[w].scale, dq_num_buckets(n, msgs[w].p.bucket));
             direct = dev_msgs[w].packed && dev_msgs[w].scale;
         }
         if (direct) {

@@ -48,3 +48,42 @@ def test_host_calls_give_the_bits_of_the_device_calls(dq, n, bucket, how):
     out.zero_()
     dq.ndqsg_decode_aggregate_host(host, n, 2, _host(common, how), out, ws)
     assert torch.equal(out, dq.ndqsg_decode_aggregate(dev, n, 2, common)[:n].cpu())
+
+
+@pytest.mark.parametrize("how,in_place", [("pinned", True), ("end of a block", True), ("registered", True), ("pageable", False),
+                                          ("misaligned", False)])
+def test_the_workspace_stays_untouched_where_the_buffers_are_used_in_place(dq, how, in_place):
+    """... and nowhere else.  `registered`: page-locked by registration of exactly the buffer's pages."""
+    n, p = 8192, dq.DqParams(512, 2, 3, 0, 0, 0, 32, 0)
+    g = torch.randn(n, device="cuda")
+    want = dq.dqsg_encode(g, 3, 0, 1, p)
+    registered = []
+
+    def host(t):
+        if how == "end of a block":                       # nothing behind the buffer in its page-locked block
+            h = torch.empty((1 << 20) // t.element_size(), dtype=t.dtype).pin_memory()[-t.numel():]
+        elif how == "registered":
+            page = torch.empty(4096 * 17, dtype=torch.uint8)
+            at = -page.data_ptr() % 4096
+            size = -(-t.numel() * t.element_size() // 4096) * 4096
+            h = page[at:at + size].view(t.dtype)[-t.numel():]
+            assert int(torch.cuda.cudart().cudaHostRegister(page.data_ptr() + at, size, 0)) == 0
+            registered.append((page.data_ptr() + at, page))       # (the pages live until they are unregistered)
+        else:
+            h = _host(t, how)
+        return h.copy_(t)
+
+    ws = torch.full((1 << 20,), 0x5A, dtype=torch.uint8, device="cuda")
+    pk, sc = host(torch.zeros(n // 16, dtype=torch.int32)), host(torch.zeros(16))
+    try:
+        dq.dqsg_encode_host(host(g.cpu()), 3, 0, 1, p, pk, sc, ws)
+        assert torch.equal(pk, want[0].cpu()) and torch.equal(sc, want[1].cpu())
+        assert bool((ws == 0x5A).all()) == in_place
+        out = host(torch.zeros(n))
+        ws.fill_(0x5A)
+        dq.ndqsg_decode_aggregate_host([dq.Message(pk, sc, 3, 0, 0, p)], n, 1, None, out, ws)
+        assert torch.equal(out, dq.dqsg_decode_aggregate([dq.Message(*want, 3, 0, 0, p)], n, 1)[:n].cpu())
+        assert bool((ws == 0x5A).all()) == in_place
+    finally:
+        for address, _ in registered:
+            torch.cuda.cudart().cudaHostUnregister(address)
