@@ -284,7 +284,8 @@ dq_status dq_ternary_unpack(const uint8_t* radix, uint64_t n, uint32_t* out_pack
  * gradients are copied to the workspace, processed and copied back in two pieces, with a second stream that the
  * library keeps per host thread and device; up to 2^20 elements in 16-byte aligned buffers that each lie completely in
  * one page-locked allocation or registration, the kernels read and write the host memory directly and the workspace is
- * not used; anything else is copied in, processed and copied back.  The results are the same bits in every case.
+ * not used (but for the codes that an encoder of 3, 5, 6 or 7 bits writes); anything else is copied in, processed and
+ * copied back.  The results are the same bits in every case.
  */
 uint64_t dq_encode_workspace_bytes(uint64_t n, const dq_params* p);
 uint64_t dq_decode_workspace_bytes(const dq_msg* msgs, uint32_t W, uint64_t n, int has_side_info);

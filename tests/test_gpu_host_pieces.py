@@ -87,3 +87,17 @@ def test_the_workspace_stays_untouched_where_the_buffers_are_used_in_place(dq, h
     finally:
         for address, _ in registered:
             torch.cuda.cudart().cudaHostUnregister(address)
+
+
+@pytest.mark.parametrize("bits", range(1, 9))
+def test_codes_that_would_cross_the_bus_in_small_pieces_go_through_the_workspace(dq, bits):
+    n, p = 70_001, dq.DqParams(512, bits, 0, 0, 0, 0, 32, 0)
+    g = torch.randn(n, device="cuda")
+    pk, sc = dq.dqsg_encode(g, 3, 0, 1, p)
+    ws = torch.full((1 << 20,), 0x5A, dtype=torch.uint8, device="cuda")
+    hpk, hsc = _host(torch.zeros_like(pk), "pinned"), _host(torch.zeros_like(sc), "pinned")
+    dq.dqsg_encode_host(_host(g, "pinned"), 3, 0, 1, p, hpk, hsc, ws)
+    assert torch.equal(hpk, pk.cpu()) and torch.equal(hsc, sc.cpu())
+    used = ws.cpu() != 0x5A
+    assert bool(used.any()) == (bits in (3, 5, 6, 7))
+    assert not bool(used[4 * pk.numel():].any())
