@@ -131,21 +131,21 @@ code_histogram_words_kernel(const uint32_t* __restrict__ packed, uint64_t n, uns
     if (blockIdx.x == 0u && threadIdx.x == 31u) atomicAdd(hist, (unsigned long long)n);
 }
 
-// Wider codes; hist has been cleared.  Up to five bits every thread has counters of its own (no two lanes of a warp meet
-// in a shared-memory bank); beyond that each warp has 256.  A thread handles one row (32 codes, BITS words) at a time.
-template <int BITS>
+// Wider codes; hist has been cleared.  A thread handles one row (32 codes, BITS words) at a time.  Each warp has counters
+// of its own; with OWN (four and five bits, very long messages: see dq_code_histogram) each thread has, so that no two
+// lanes of a warp meet in a shared-memory bank, but 32 KB have to be cleared and added up per CTA.
+template <int BITS, bool OWN>
 __global__ void __launch_bounds__(kHistThreads)
 code_histogram_kernel(const uint32_t* __restrict__ packed, uint64_t n, unsigned long long* hist)
 {
-    constexpr bool kOwn = BITS <= 5;
     constexpr uint32_t kBins = 1u << BITS, kWarps = kHistThreads / 32;
-    constexpr uint32_t kStep = kOwn ? (uint32_t)kHistThreads : 1u;
-    __shared__ uint32_t bins[kOwn ? kBins * kHistThreads : kBins * kWarps];
+    constexpr uint32_t kStep = OWN ? (uint32_t)kHistThreads : 1u;
+    __shared__ uint32_t bins[OWN ? kBins * kHistThreads : kBins * kWarps];
     for (uint32_t i = threadIdx.x; i < sizeof(bins) / 4u; i += kHistThreads) bins[i] = 0u;
     __syncthreads();
     grid_dependency_wait();
     grid_dependency_launch_next();
-    uint32_t* mine = bins + (kOwn ? threadIdx.x : (threadIdx.x >> 5) * kBins);
+    uint32_t* mine = bins + (OWN ? threadIdx.x : (threadIdx.x >> 5) * kBins);
 
     const uint64_t rows = (n + 31u) >> 5;
     const uint64_t num_words = (n * BITS + 31u) >> 5;
@@ -163,7 +163,7 @@ code_histogram_kernel(const uint32_t* __restrict__ packed, uint64_t n, unsigned 
         }
     }
     __syncthreads();
-    if constexpr (kOwn) {
+    if constexpr (OWN) {
         // a warp adds up the counters of one code at a time
         for (uint32_t b = threadIdx.x >> 5; b < kBins; b += kWarps) {
             uint32_t s = 0u;
