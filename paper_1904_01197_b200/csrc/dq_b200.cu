@@ -239,6 +239,11 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     a.two = e.two;
     a.off = e.off;
     a.ps = e.ps;
+    // A grid of up to two waves lets the next kernel in late: beside it, the CTAs of the next one would be placed unevenly
+    // (see the decoder; n = 2.4 M, B = 2048: 5.5 us per call, late 4.2; 1.9 M, B = 16384: 5.6 and 4.7; 1.2 M, B = 2048: 3.4
+    // and 2.7).  With more waves it does not matter and the early launch hides a little more (11.7 M: 13.8 us, late 14.0), and
+    // so it does where clusters of one-group lanes leave the GPU half empty (0.6 M, B = 16384: 3.65 us, late 3.86).
+    a.late_launch = (R == 4 ? n <= (uint64_t)sms * 768u * 32u * 2u : shape.cluster == 1u) ? 1u : 0u;
     // (with early_read one cluster more: see the kernel)
     const uint64_t grid = ((dq_num_buckets(n, p.bucket) + shape.buckets - 1u) / shape.buckets + (a.early_read ? 1u : 0u)) *
                           shape.cluster;
@@ -373,11 +378,15 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 // 16 and then 32 elements amortise what a worker costs per lane; 32 pays from about two and a half of its own waves
 // (W = 8: n = 4.2 M 38.1 us with 16, 40.5 with 32; n = 11.7 M 79.0 and 75.7), and not for one worker, or two and a side
 // information vector, where memory latency matters more and 16 has more warps to hide it (n = 25.6 M: W = 1 31.1 us with
-// 16, 34.8 with 32; W = 2 with a vector 62.6 and 67.4, without 51.6 and 47.2).
-int decode_group_size(uint64_t n, uint32_t W, bool reads_side, int sms)
+// 16, 34.8 with 32; W = 2 with a vector 62.6 and 67.4, without 51.6 and 47.2).  In the kernel with all routines, whose
+// routines are longer, 32 pays from one wave of 16-element lanes on if there are eight messages (`usual` false; six bits,
+// W = 8: n = 2.4 M 24.1 us with 16, 24.2 with 32; 3 M 29.2 and 26.1; 4.2 M 39.4 and 35.0; W = 32, 4.2 M 151 and 133; but
+// W = 3 and a vector, 4.2 M 19.5 and 22.5).
+int decode_group_size(uint64_t n, uint32_t W, bool reads_side, bool usual, int sms)
 {
     const uint64_t lanes = (uint64_t)sms * dq::kDecThreads;
     if (n <= 8u * lanes * dq::dec_ctas_per_sm(8, dq::kSetUsual)) return 8;
+    if (!usual && W >= 8u && n > 16u * lanes * dq::dec_ctas_per_sm(16, dq::kSetAll)) return 32;
     if (W <= (reads_side ? 2u : 1u) || 2u * n < 5u * 32u * lanes * dq::dec_ctas_per_sm(32, dq::kSetAll)) return 16;
     return 32;
 }
@@ -468,7 +477,9 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
     const bool d16 = (msgs[0].p.dither_bits == 16u);
-    const int E = decode_group_size(n, W, reads_side, sms);
+    bool usual = true;
+    for (uint32_t w = 0; w < W; ++w) usual = usual && dq::is_usual_variant(a.w[w].variant);
+    const int E = decode_group_size(n, W, reads_side, usual, sms);
     a.num_groups = (n + (uint32_t)E - 1u) / (uint32_t)E;
     cudaError_t le;
     if (half_dithered) le = dq::launch_decode_d0_r0(a, E, st);

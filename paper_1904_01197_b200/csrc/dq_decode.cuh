@@ -420,10 +420,6 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
     }
     // the messages (and the side information) may be the previous kernel's output
     grid_dependency_wait();
-    // The next kernel may become resident once every CTA of this one is past its wait: see launch_overlapped.  Letting
-    // kernel after kernel of a short-call loop pile up would also place the CTAs of one kernel wherever slots happen to
-    // fall free, several on one SM and none on others (W = 8, n = 266,610: 11.9 us per call instead of 6.6).
-    grid_dependency_launch_next();
     ln.kappa_next = __ldg(args.w[0].scale + ln.bucket);
 
     if (SIDE == kSideGiven && args.has_side != 0u) {
@@ -448,6 +444,11 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
     for (int e = 0; e < E / 2; ++e) acc[e] = 0ull;
     decode_workers<DITH, SIDE, E, SET>(args, ln, acc);
 
+    // The next kernel may become resident when every CTA of this one is about to store.  Let in right after the wait, its
+    // CTAs would take the slots that this kernel leaves free, and what does not fit would be placed when these end,
+    // several CTAs on one SM and none on others, as soon as a grid takes more than half the slots (W = 8: n = 1.3 M 20.3 us
+    // per call, now 14.7; 1.6 M 20.6 and 16.9; 266,610 6.8 and 6.5; from a few waves on there is no difference).
+    grid_dependency_launch_next();
     // the mean (of one message: the message itself)
     if (args.W > 1u) {
         const f32x2 nz = args.neg_zero;

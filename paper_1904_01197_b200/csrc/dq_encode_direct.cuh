@@ -61,6 +61,7 @@ struct DirectArgs {
     uint32_t K_magic;             // NDQSG any K: ceil(2^32 / K)
     uint32_t first_group;         // index of grad[0]'s group in the whole gradient (0 unless a bucket range is encoded):
                                   // only the dither counters see it
+    uint32_t late_launch;         // the next kernel is let in at the end of this one and not right after the wait
     uint32_t early_read;          // } see the kernel and EncodeArgs
     uint32_t early_store;         // }
     f32x2 shift, magic, two, off; // pairs of equal values: DQSG s; 1.5 * 2^23; scale and offset of the dither
@@ -209,7 +210,7 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
 
     if (args.early_read == 0u) {
         grid_dependency_wait();
-        grid_dependency_launch_next();
+        if (args.late_launch == 0u) grid_dependency_launch_next();
     }
     f32x2 x[4 * R];
     uint32_t mb[R];
@@ -307,7 +308,8 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
         if (c > 0 && args.gains > (uint32_t)(c % 2)) aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
         encode_group8<BITS, MODE, DITH>(x + 4 * c, p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0, aa, args, out[c]);
     }
-    if (args.early_read != 0u && args.early_store == 0u) grid_dependency_wait();
+    if (args.early_read == 0u) grid_dependency_launch_next();
+    else if (args.early_store == 0u) grid_dependency_wait();
     const uint64_t byte = (uint64_t)group * (uint32_t)BITS;
     uint8_t* dst = reinterpret_cast<uint8_t*>(args.packed) + byte;
     if (whole) {

@@ -17,17 +17,20 @@ def _edges():
     sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
     wave8 = sms * 128 * 8 * 8                    # longest call of 8-element lanes
     two_and_a_half32 = sms * 128 * 32 * 5 * 5 // 2
-    return {"8 last": wave8, "16 first": wave8 + 1, "16 last": two_and_a_half32 - 1, "32 first": two_and_a_half32 + 9}
+    return {"8 last": wave8, "16 first": wave8 + 1, "16 last": two_and_a_half32 - 1, "32 first": two_and_a_half32 + 9,
+            "16 last of all routines": 2 * wave8, "32 first of all routines": 2 * wave8 + 33}
 
 
-@pytest.mark.parametrize("edge", ["8 last", "16 first", "16 last", "32 first"])
+@pytest.mark.parametrize("edge", ["8 last", "16 first", "16 last", "32 first", "16 last of all routines",
+                                  "32 first of all routines"])
 @pytest.mark.parametrize("bits,K,alpha,dither,bucket", [(1, 2, 1.0, 32, 96), (3, 8, 1.0, 16, 2048), (5, 21, 0.75, 32, 1248),
                                                         (7, 100, 1.0, 16, 32), (8, 128, 0.5, 32, 65536)])
 def test_group_sizes_at_their_edges(dq, oracle, edge, bits, K, alpha, dither, bucket):
     n, step = _edges()[edge], 5
     rng = np.random.default_rng(bits)
-    specs = [WorkerSpec(DQSG, bits, 0, 0, 0.0, 1.0, 11, dither), WorkerSpec(NDQSG, bits, 0, K, float(K), alpha, 12, dither),
-             WorkerSpec(NDQSG, bits, 0, K, float(K), alpha, 13, dither)]
+    nested = 7 if "all routines" in edge else 2
+    specs = [WorkerSpec(DQSG, bits, 0, 0, 0.0, 1.0, 11, dither),
+             *[WorkerSpec(NDQSG, bits, 0, K, float(K), alpha, 12 + w, dither) for w in range(nested)]]
     side = (0.01 * rng.standard_normal(n)).astype(np.float32)
     gmsgs, sent = [], []
     for w, sp in enumerate(specs):
