@@ -25,8 +25,8 @@
  *   - "device" pointers are CUDA device memory on the current device, 16-byte aligned, owned by the
  *     caller.  The library allocates no device memory at run time and keeps no state between calls, with two
  *     exceptions that live in its device image: one error word per GPU (dq_device_error_flags) and the
- *     fixed staging array of dqsg_encode_host_static.  (Long *_host calls also keep a stream and two events per
- *     host thread and device, given back when the thread ends.)  It is asynchronous on the given stream (it never
+ *     fixed staging array of dqsg_encode_host_static.  (Long *_host calls, but not that one, also keep a stream and two
+ *     events per host thread and device, given back when the thread ends.)  It is asynchronous on the given stream (it never
  *     synchronises), except for the *_host entry points, which return after the results are in the
  *     caller's host buffers.
  *   - Outputs must not alias inputs.  Inputs are assumed finite.
@@ -320,16 +320,18 @@ dq_status ndqsg_decode_aggregate_side_first_host(const dq_msg* msgs, uint32_t W,
  *   returns DQ_ERR_TOO_LARGE      when dq_encode_workspace_bytes(n, p) > DQ_STATIC_SCRATCH_BYTES
  *                                 (about 7.8 million elements at 2 bits); nothing is copied or launched
  *
- * The call performs no cudaMalloc / cudaFree and calls no allocating library routine.  The array is part of
- * the library's device image: the driver reserves it when that image is loaded on a device, which with lazy
- * loading is the first use of ANY entry point there; if the memory cannot be reserved, every entry point fails
- * with DQ_ERR_CUDA.  The first call of this function on each device additionally looks up the array's device
- * address (once per device, with that device current); make one warm-up call per device at start-up, outside
- * any stream capture and outside the latency-critical loop.  The address is cached for the life of the
- * process: cudaDeviceReset is not supported once it has been looked up.  The array is shared by all calls and keeps whatever the last call
- * left in it.  Nothing in it has to start at zero: the gradient is copied over its input region and the
- * kernel writes every packed word and every scale before they are copied back.  Two calls that overlap in
- * time on one device (different host threads or streams) use the same bytes and race; serialise them.
+ * The call performs no cudaMalloc / cudaFree, creates no stream or event and calls no allocating library routine:
+ * it copies, launches one kernel and copies back on the caller's stream, whatever the length (short gradients in
+ * page-locked buffers are used in place, as in dqsg_encode_host).  The array is part of the library's device image:
+ * the driver reserves it when that image is loaded on a device, which with lazy loading is the first use of ANY
+ * entry point there; if the memory cannot be reserved, every entry point fails with DQ_ERR_CUDA.  The first call of
+ * this function on each device additionally looks up the array's device address (once per device, with that device
+ * current); make one warm-up call per device at start-up, outside any stream capture and outside the
+ * latency-critical loop.  The address is cached for the life of the process: cudaDeviceReset is not supported once
+ * it has been looked up.  The array is shared by all calls and keeps whatever the last call left in it.  Nothing in
+ * it has to start at zero: whatever part of it a call uses, the gradient is copied over its input region and the
+ * kernel writes every packed word and every scale before they are copied back.  Two calls that overlap in time on
+ * one device (different host threads or streams) use the same bytes and race; serialise them.
  */
 #define DQ_STATIC_SCRATCH_BYTES (32u * 1024u * 1024u)
 dq_status dqsg_encode_host_static(const float* grad, uint64_t n, uint64_t seed, uint32_t worker, uint64_t step,

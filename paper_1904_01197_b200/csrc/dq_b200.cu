@@ -850,9 +850,10 @@ uint64_t dq_decode_workspace_bytes(const dq_msg* msgs, uint32_t W, uint64_t n, i
     return total;
 }
 
+// may_pipe: long gradients may go in pieces over the host thread's second stream, which the first such call creates.
 static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64_t seed, uint32_t worker,
                              uint64_t step, const dq_params* p, uint32_t* out_packed, float* out_scale,
-                             void* workspace, uint64_t workspace_bytes, void* cuda_stream)
+                             void* workspace, uint64_t workspace_bytes, void* cuda_stream, bool may_pipe = true)
 {
     uint32_t L;
     float alpha;
@@ -890,7 +891,7 @@ static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64
     ws += align_up(pbytes, 256u);
     float* d_scale = reinterpret_cast<float*>(ws);
     const uint64_t sbytes = dq_num_buckets(n, p->bucket) * 4u;
-    HostPipe* pipe = (!plain && n >= kHostPieceElements) ? host_pipe() : nullptr;
+    HostPipe* pipe = (may_pipe && !plain && n >= kHostPieceElements) ? host_pipe() : nullptr;
     if (pipe) {
         // The gradient is what takes long: a small last piece, so that little is left to do when it arrives.
         static constexpr uint32_t cuts[kHostPieces + 1] = {0u, 14u, 16u};
@@ -1095,8 +1096,9 @@ dq_status dqsg_encode_host_static(const float* grad, uint64_t n, uint64_t seed, 
     void* scratch = nullptr;
     s = static_scratch_address(&scratch);
     if (s != DQ_OK) return s;
+    // (no second stream: this call creates nothing, on whichever thread)
     return encode_host(DQ_KIND_DQSG, grad, n, seed, worker, step, p, out_packed, out_scale, scratch,
-                       (uint64_t)DQ_STATIC_SCRATCH_BYTES, cuda_stream);
+                       (uint64_t)DQ_STATIC_SCRATCH_BYTES, cuda_stream, false);
 }
 
 dq_status dq_device_error_flags(uint32_t* out_flags)

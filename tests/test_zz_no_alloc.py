@@ -90,3 +90,27 @@ def test_static_scratch_rejects_inputs_beyond_its_size(dq):
     assert rc == 5 and "scratch" in dq.status_string(rc)
     # the largest vector that fits is accepted by the size check (n = 0 needs no buffers at all)
     assert dq.lib().dqsg_encode_host_static(fake, 0, 1, 0, 0, C.byref(params), fake, fake, None) == 0
+
+
+@pytest.mark.parametrize("n,bits,pinned", [((1 << 22) - 1, 2, False), (1 << 22, 2, False), (5_000_011, 3, False),
+                                           (7_700_000, 2, False), (1 << 22, 2, True), (200_003, 2, True), (200_003, 3, True)])
+def test_static_scratch_encode_is_one_launch_of_any_length(dq, n, bits, pinned):
+    """dqsg_encode_host cuts long gradients in pieces, with a stream and events that the first such call of a host thread
+    creates; the call for callers that must not allocate has one kernel on the caller's stream, also where the buffers are
+    page-locked, and also on a host thread whose first call it is."""
+    from concurrent.futures import ThreadPoolExecutor
+    params = dq.binding.make_params(2048, bits, 3)
+    assert dq.encode_workspace_bytes(n, params) <= dq.STATIC_SCRATCH_BYTES
+    g = (np.random.default_rng(n).standard_normal(n) * 0.01).astype(np.float32)
+    if pinned:
+        host = (torch.from_numpy(g).pin_memory(), torch.empty(dq.packed_words(n, bits), dtype=torch.int32).pin_memory(),
+                torch.empty(dq.num_buckets(n, 2048)).pin_memory())
+        run = lambda: dq.dqsg_encode_host_static(host[0], 5, 2, 9, params, host[1], host[2])       # noqa: E731
+    else:
+        run = lambda: _static(dq, g, 5, 2, 9, params)                                              # noqa: E731
+    before = dq.launch_count()
+    with ThreadPoolExecutor(max_workers=1) as pool:
+        pk, sc = pool.submit(run).result()
+    assert dq.launch_count() == before + 1
+    ref_pk, ref_sc = _reference(dq, g, 5, 2, 9, params)
+    assert np.array_equal(np.asarray(pk), ref_pk) and np.array_equal(np.asarray(sc).view(np.uint32), ref_sc.view(np.uint32))
