@@ -80,7 +80,7 @@ typedef struct {
 } dq_params;
 
 /*
- * DQ_FLAG_INPUT_READY (encoders only; ignored elsewhere).  By default an encode kernel touches no memory
+ * DQ_FLAG_INPUT_READY (encoders from device memory only; ignored elsewhere, also by the *_host calls).  By default an encode kernel touches no memory
  * before the previous kernel of its stream has completed.  With this flag the caller declares that `grad`
  * was completely written before that previous kernel was launched and is not written by it -- the usual case
  * when a gradient produced by the backward pass is encoded after some unrelated kernel, or when several

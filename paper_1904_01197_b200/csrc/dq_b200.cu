@@ -866,6 +866,10 @@ static dq_status encode_host(dq_kind kind, const float* grad, uint64_t n, uint64
     if (workspace_bytes < dq_encode_workspace_bytes(n, p)) return DQ_ERR_INVALID_ARG;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const bool plain = (p->flags & DQ_FLAG_TEST_DROP_COPY) != 0u;        // (the hook is about one launch)
+    // The launch flags say nothing about host buffers and the workspace, which the caller's previous kernel may use.
+    dq_params unflagged = *p;
+    unflagged.flags &= ~(DQ_FLAG_INPUT_READY | DQ_FLAG_OUTPUT_FREE);
+    p = &unflagged;
     if (!plain && n <= kHostDirectElements) {
         const float* h_grad = pinned_view(grad, n);
         uint32_t* h_packed = h_grad ? pinned_view(out_packed, dq_packed_words(n, p->bits)) : nullptr;

@@ -89,6 +89,24 @@ def test_the_workspace_stays_untouched_where_the_buffers_are_used_in_place(dq, h
             torch.cuda.cudart().cudaHostUnregister(address)
 
 
+@pytest.mark.parametrize("n,bits", [(70_001, 2), (70_001, 3), (5_000_011, 2), (18_000_000, 2)])
+def test_the_launch_flags_mean_nothing_to_host_calls(dq, n, bits):
+    """A short call in place directly follows the caller's previous kernel, which may still use the workspace: here it
+    copies from it, and must find what was there."""
+    flags = dq.DQ_FLAG_INPUT_READY | dq.DQ_FLAG_OUTPUT_FREE
+    p, pf = dq.DqParams(2048, bits, 3, 0, 0, 0, 32, 0), dq.DqParams(2048, bits, 3, 0, 0, 0, 32, flags)
+    g = torch.randn(n, device="cuda")
+    pk, sc = dq.dqsg_encode(g, 3, 0, 1, p)
+    host = _host(g, "pinned"), _host(torch.zeros_like(pk), "pinned"), _host(torch.zeros_like(sc), "pinned")
+    ws = torch.empty(dq.encode_workspace_bytes(n, p), dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        ws.fill_(0x5A)
+        hist = dq.code_histogram(ws.view(torch.int32), ws.numel() // 4, 8)
+        dq.dqsg_encode_host(host[0], 3, 0, 1, pf, host[1], host[2], ws)
+        assert torch.equal(host[1], pk.cpu()) and torch.equal(host[2], sc.cpu())
+        assert int(hist[0x5A]) == ws.numel() // 4
+
+
 @pytest.mark.parametrize("bits", range(1, 9))
 def test_codes_that_would_cross_the_bus_in_small_pieces_go_through_the_workspace(dq, bits):
     n, p = 70_001, dq.DqParams(512, bits, 0, 0, 0, 0, 32, 0)
