@@ -283,7 +283,7 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
         a.kmax = (int32_t)(L - 1u);
     } else {
         // K = 2^bits: the coset is the low `bits` bits of the fine index; a smaller power of two: one mask more;
-        // any other K: a modulo
+        // any other K: the remainder
         mode = (p->coarse_K == (1u << p->bits)) ? dq::kEncNdqsgPow2
                : is_pow2(p->coarse_K)           ? dq::kEncNdqsgPow2Mask
                                                 : dq::kEncNdqsgAnyK;
@@ -318,7 +318,6 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
     }
     // whole work units (a bucket, or 1024 elements for smaller buckets) go through the tile path of the kernel, the rest
     // through its plain-load part, in the same launch
-    a.sm_count = (uint32_t)sms;
     const uint32_t B = p->bucket;
     const uint32_t U = (B < 1024u) ? 1024u : B;                     // elements per work unit
     const uint64_t tiles = n / U;                                   // whole units
@@ -365,9 +364,6 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
         const uint64_t want_ctas = (tiles + groups_per_cta - 1u) / groups_per_cta;
         tile_ctas = (uint32_t)(want_ctas < room ? want_ctas : room);
     }
-    // the spacing only pays when the first requests of all resident warps saturate HBM
-    // (a launch that reads early gets its CTAs one by one, as the previous kernel's CTAs leave: nothing to space)
-    a.request_spacing_ns = a.early_read ? 0u : (uint32_t)((uint64_t)dq::kFirstRequestSpacingNs * tile_ctas / slots);
     if (launch_encode(mode, p->bits, d16, map, a, plain + tile_ctas, st) != cudaSuccess) return DQ_ERR_CUDA;
     g_launches.fetch_add(1);
     return DQ_OK;

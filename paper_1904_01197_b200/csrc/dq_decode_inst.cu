@@ -26,11 +26,15 @@ cudaError_t launch_set(const DecodeArgsOf<MAXW>& a, uint32_t grid, cudaStream_t 
 template <int E, int A>
 cudaError_t launch_pair(int b, const DecodeArgs& a, uint32_t grid, cudaStream_t st)
 {
-    switch (b) {
-        case 1: return launch_set<E, pair_set(A, 1)>(a, grid, st);
-        case 2: return launch_set<E, pair_set(A, 2)>(a, grid, st);
-        case 3: return launch_set<E, pair_set(A, 3)>(a, grid, st);
-        default: return launch_set<E, pair_set(A, 4)>(a, grid, st);
+    if constexpr (DQ_INST_DITH == 0) {        // (the receiver without the dither takes DQSG messages only)
+        return launch_set<E, pair_set(A, A)>(a, grid, st);
+    } else {
+        switch (b) {
+            case 1: return launch_set<E, pair_set(A, 1)>(a, grid, st);
+            case 2: return launch_set<E, pair_set(A, 2)>(a, grid, st);
+            case 3: return launch_set<E, pair_set(A, 3)>(a, grid, st);
+            default: return launch_set<E, pair_set(A, 4)>(a, grid, st);
+        }
     }
 }
 

@@ -104,29 +104,11 @@ constexpr float kF16Offset = 1.00000762939453125f;         // 1 + 2^-17
 constexpr float kD32Offset = 0.49999988079071044921875f;   // 1/2 - 2^-23
 constexpr float kD16Offset = 0.49999237060546875f;         // 1/2 - 2^-17
 
-__device__ __forceinline__ float dither_delta(uint32_t x)
-{
-    return __fmaf_rn(__uint_as_float(x >> 10), kTwo127, -0.49999988079071044921875f);     // -(1/2 - 2^-23)
-}
-
 // 16-bit stream: half-word h -> f = 1 + (2h+1) 2^-17, delta = (2h+1) 2^-17 - 1/2.  One byte permutation puts
 // h into bits 8..23 (the subnormal or small normal number h * 2^-141); the multiply-add scales by 2^125.
 __device__ __forceinline__ float half_word_as_small_float(uint32_t word, int high)
 {
     return __uint_as_float(__byte_perm(word, 0u, high ? 0x4324u : 0x4104u));
-}
-
-__device__ __forceinline__ float dither16_delta(uint32_t word, int high)
-{
-    return __fmaf_rn(half_word_as_small_float(word, high), kTwo125, -0.49999237060546875f);  // -(1/2 - 2^-17)
-}
-
-// The dither itself (encoder side).
-template <int DITH>
-__device__ __forceinline__ float dither_delta_of(const uint32_t (&rnd)[4][4], int t)
-{
-    if (DITH == 16) return dither16_delta(rnd[t >> 3][(t & 7) >> 1], t & 1);
-    return dither_delta(rnd[t >> 2][t & 3]);
 }
 
 // Pairs of fp32 values in one 64-bit register: one instruction of the packed fp32 unit works on both.  Each half
@@ -213,41 +195,6 @@ __device__ __forceinline__ void tma_load_rows(uint32_t dst, const CUtensorMap* t
         : "memory");
 }
 
-// Contiguous bulk copy global -> shared memory (both addresses 16-byte aligned, size a multiple of 16 bytes).
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
-// Store a [32 rows x 32 floats] box from shared memory (128-byte swizzle) to rows row0.. of the mapped array; rows
-// past the array's end are not written.  Completion is tracked by the issuing thread's bulk groups.
-__device__ __forceinline__ void tma_store_rows(const CUtensorMap* tmap, uint32_t src, int32_t row0)
-{
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                 ::"l"((uint64_t)tmap), "r"(src), "r"(0), "r"(row0)
-                 : "memory");
-}
-
-__device__ __forceinline__ void bulk_commit_group()
-{
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-
-// Waits until at most N of this thread's bulk groups still have to read their shared-memory source.
-template <int N>
-__device__ __forceinline__ void bulk_wait_group_read()
-{
-    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
-
-// Makes this thread's earlier shared-memory writes visible to the asynchronous copy engine.
-__device__ __forceinline__ void fence_proxy_async_shared()
-{
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
 // Upper bound, in nanoseconds, that one try may stay suspended in hardware before it reports "not yet".
 constexpr uint32_t kWaitHintNs = 2000u;
 // A copy that has not landed after this long (by the global nanosecond timer) is given up: a tile copy takes
@@ -292,16 +239,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
 __device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t threads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-__device__ __forceinline__ void prefetch_l1(const void* p)
-{
-    asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-
-__device__ __forceinline__ void prefetch_l2(const void* p)
-{
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 // Programmatic dependent launch: wait until the previous kernel of the stream has completed and its writes are

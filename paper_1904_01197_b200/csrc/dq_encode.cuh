@@ -31,7 +31,7 @@
 namespace dq {
 
 // kEncNdqsgPow2: K = 2^BITS, the coset is the low BITS bits of the fine index; kEncNdqsgPow2Mask: a smaller power
-// of two; kEncNdqsgAnyK: any K (a true modulo).
+// of two; kEncNdqsgAnyK: any K (the remainder from one high multiply).
 enum EncMode : int { kEncDqsg = 0, kEncNdqsgPow2 = 1, kEncNdqsgAnyK = 2, kEncNdqsgPow2Mask = 3 };
 
 constexpr int kTileRows = 256;                     // rows a CTA holds per pipeline stage (8 warps x 32 rows, 32 KB)
@@ -48,8 +48,6 @@ constexpr int kEncThreads = 32 * kConsumerWarps;
 constexpr int kEncStages = DQ_ENC_STAGES;
 constexpr int kEncCtasPerSm = DQ_ENC_CTAS_PER_SM;
 constexpr size_t kEncSmemBytes = (size_t)kEncStages * kTileBytes + 1024;
-// Time HBM needs to deliver one warp's pipeline stages (8 KB) to each of the 148 SMs: 148 x 8 KB / 6.5 TB/s.
-constexpr uint32_t kFirstRequestSpacingNs = 190u;
 // Plain-load part: buckets up to 1024 elements are taken in warp windows, up to this size by one warp, above by a CTA.
 constexpr uint32_t kPlainWarpBucketMax = 4096u;
 
@@ -79,8 +77,6 @@ struct EncodeArgs {
     uint32_t K_magic;        // NDQSG any K: ceil(2^32 / K)
     uint32_t row_offset;     // index of grad[0]'s row in the whole gradient (0 unless a bucket range is encoded):
                              // only the dither counters see it
-    uint32_t sm_count;       // SMs of the device            } spacing of the first tile requests,
-    uint32_t request_spacing_ns;   // see encode_kernel      } 0 when the grid does not fill the device
     uint32_t early_read;     // the caller guarantees that grad was complete before the previous kernel of the stream
                              // began: the tile path requests (and quantizes) its first tiles while that kernel
                              // drains, and only its stores wait for it
@@ -413,16 +409,6 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
         grid_dependency_launch_next();
     }
     if (lane == 0) {
-        // All resident warps would request their first tiles (the whole shared memory of every SM, a quarter of a
-        // ResNet-50-sized gradient) at the same instant; served interleaved, every warp would then get its data
-        // late and the ALUs would idle for 3-6 us.  Spacing the requests of an SM's warps at the rate at which
-        // HBM can serve them lets the first warps start after about 1 us while the memory system stays busy.
-        // (CTAs are assumed to be placed round-robin over the SMs; any other placement only changes the order.)
-        // The CTAs with the lowest indices go first; they are also the ones whose warps take one unit more when
-        // the units do not divide evenly, so the longest-running warps start earliest.
-        const uint32_t rank = ((blockIdx.x - args.plain_ctas) / args.sm_count) * (uint32_t)kConsumerWarps + warp;
-        const uint64_t until = global_timer_ns() + (uint64_t)rank * args.request_spacing_ns;
-        for (uint32_t it = 0; it < 4096u && args.request_spacing_ns != 0u && global_timer_ns() < until; ++it) { }
 #pragma unroll
         for (int s = 0; s < kEncStages; ++s) {
             // first copies: the next two units of this warp, or (pair mode) the two halves of its first bucket
