@@ -206,7 +206,8 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     a.num_groups = (uint32_t)((n + 31u) / 32u * 4u);
     a.whole_groups = (uint32_t)(n / 8u);
     // Up to one wave of one-group lanes (1.2 M elements on 148 SMs) the GPU is not full and the shortest chain per lane
-    // wins (n = 2 M: 4.2 us with one group, 3.9 with four).
+    // wins (B = 2048: n = 266,610 1.8 us with one group, 2.4 with four; 1.2 M 2.7 and 3.1).  Past it large buckets want four at
+    // once (B = 16384: 1.3 M 6.3 and 4.7 us), small ones from 2 M on (B = 2048: 1.3 M 3.0 and 3.6, 2.4 M 4.4 and 4.2).
     const int R = n <= (uint64_t)sms * 1024u * 8u ? 1 : 4;
     const uint32_t gpb = p.bucket / 8u;
     const dq::DirectShape shape = dq::direct_shape(gpb, R);
@@ -307,8 +308,10 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
     // The tile kernel streams back-to-back encodes of long gradients through persistent CTAs: with launches that overlap
-    // by the caller's flags it is 1 to 6 % faster from 16 M elements on (n = 25.6 M, B = 2048: 22.1 us against 22.4 with
-    // two bits, 23.6 against 24.9 with three).  Everything else goes through the direct kernel.
+    // by the caller's flags it is up to 8 % faster from 16 M elements on (B = 2048: n = 16.8 M 15.1 us against 15.1, 25.6 M
+    // 22.2 against 22.7 with two bits and 22.4 against 23.4 with three, 67 M 55.8 against 59.0 with three; B = 512, 67 M 57.5
+    // against 61.5) -- but not for B = 4096, where pairs of warps meet (25.6 M: 23.6 us against 22.7 with two bits, 23.7
+    // against 23.2 with three), which has no rule of its own.  Everything else goes through the direct kernel.
     const bool tiles_wanted = is_pow2(p->bucket) && p->bucket <= 8192u &&
                               (a.test_drop_copy != 0u || (a.early_store != 0u && n >= (1ull << 24)));
     if (!tiles_wanted) {
@@ -370,14 +373,15 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 }
 
 // Elements per lane of the decoder.  Up to one wave of 8-element lanes (1.2 M elements on 148 SMs) the GPU is not
-// full and the shortest chain per lane wins (W = 8: n = 266,610 6.6 us with 8, 8.5 with 16, 12.8 with 32).  Beyond it
-// 16 and then 32 elements amortise what a worker costs per lane; 32 pays from about two and a half of its own waves
-// (W = 8: n = 4.2 M 38.1 us with 16, 40.5 with 32; n = 11.7 M 79.0 and 75.7), and not for one worker, or two and a side
-// information vector, where memory latency matters more and 16 has more warps to hide it (n = 25.6 M: W = 1 31.1 us with
-// 16, 34.8 with 32; W = 2 with a vector 62.6 and 67.4, without 51.6 and 47.2).  In the kernel with all routines, whose
-// routines are longer, 32 pays from one wave of 16-element lanes on if there are eight messages (`usual` false; six bits,
-// W = 8: n = 2.4 M 24.1 us with 16, 24.2 with 32; 3 M 29.2 and 26.1; 4.2 M 39.4 and 35.0; W = 32, 4.2 M 151 and 133; but
-// W = 3 and a vector, 4.2 M 19.5 and 22.5).
+// full and the shortest chain per lane wins (W = 8: n = 266,610 6.5 us with 8, 8.0 with 16, 9.9 with 32).  Beyond it 16 and
+// then 32 elements amortise what a worker costs per lane.  32 pays from about two and a half of its own waves, a little
+// before or after with the side information (W = 8: first 3.3 M +5 %, 4.2 M -2 %, 7.4 M -2 %; running mean 0, -6, -5 %; a vector
+// +14, +5, +4 %; two widths of nested messages and the running mean +9, +3, +3 %; W = 4 and 2, 7.6 M -4 %; W = 8, 11.7 M
+// -5 %), and not for one worker, or two and a side information vector, where memory latency matters more and 16 has more
+// warps to hide it (n = 25.6 M: W = 1 30.6 us with 16, 34.0 with 32; W = 2 with a vector 62.6 and 67.4, without 56.9 and
+// 51.9).  In the kernel with all routines, whose routines are longer, 32 pays from one wave of 16-element lanes on if there
+// are eight messages (`usual` false; six bits, W = 8: n = 2.4 M 24.1 us with 16, 24.2 with 32; 3 M 29.2 and 26.1; 4.2 M
+// 39.4 and 35.0; W = 32, 4.2 M 151 and 133; but W = 3 and a vector, 4.2 M 19.5 and 22.5).
 int decode_group_size(uint64_t n, uint32_t W, bool reads_side, bool usual, int sms)
 {
     const uint64_t lanes = (uint64_t)sms * dq::kDecThreads;

@@ -22,7 +22,7 @@
 // sweep that quantizes).
 //
 // What bounds it: the multiplier pipe and instruction issue, as in the direct encoder.  On packed fp32 pairs and with
-// the clamp in one instruction the overlapped encode of n = 25.6 M takes 22.1 us (2 bits, before 22.6) and 23.6 us
+// the clamp in one instruction the overlapped encode of n = 25.6 M, B = 2048 takes 22.2 us (2 bits, before 22.6) and 22.4 us
 // (3 bits, before 25.5).
 #pragma once
 

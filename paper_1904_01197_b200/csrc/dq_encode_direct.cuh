@@ -8,7 +8,7 @@
 // over the cluster's distributed shared memory), then every lane quantizes its groups from registers.  The gradient is
 // read once, whatever the bucket size, and the hardware's block scheduler balances the load.
 //   R = 1 for gradients that do not fill the GPU: the most lanes, the shortest chain per lane.
-//   R = 4 for longer ones: what a warp costs once (indices, round keys, reduction, gain: about 130 instructions) is
+//   R = 4 for longer ones: what a warp costs once (indices, round keys, reduction, gain) is
 //     spread over 32 elements per lane.
 //
 // What bounds it at large n: the multiplier pipe (about four wide multiplies of four cycles each per dither value) and
