@@ -82,6 +82,7 @@ struct EncodeArgs {
                              // drains, and only its stores wait for it
     uint32_t early_store;    // ... and that the previous kernel neither reads nor writes this call's outputs: nothing
                              // waits for that kernel except the end of this one (see encode_kernel)
+    uint32_t all_lanes;      // 0xFFFFFFFF, see encode_kernel
     uint32_t test_drop_copy; // test hook: warp 0 of the first tile CTA arms the barrier for its last unit without
                              // issuing the copy, so that the bounded wait for it runs out (see DQ_FLAG_TEST_DROP_COPY)
     unsigned int* error_flags;     // the library's per-device error word
@@ -470,6 +471,10 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
                                  : "r"(stage_addr ^ (c << 4))
                                  : "memory");
                 }
+                // Before the stage is given back every lane's loads must have returned.  The maximum needs the first half's;
+                // nothing needs the second half's yet, so the mask of the __syncwarp does: 0xFFFFFFFF whatever it is ORed
+                // with, but the compiler does not know that.
+                uint32_t lanes = 0xFFFFFFFFu;
                 if (half == 0u) {
 #pragma unroll
                     for (int e = 0; e < 16; ++e) mx = max_pair(mx, x[e]);
@@ -485,12 +490,11 @@ encode_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ 
                         }
                     }
                 } else {
-                    uint32_t sink = 0u;                 // all loads of this half have completed after this
+                    lanes = args.all_lanes;
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) sink ^= (uint32_t)x[2 * c];
-                    asm volatile("" ::"r"(sink));
+                    for (int c = 0; c < 8; ++c) lanes |= (uint32_t)x[2 * c];
                 }
-                __syncwarp();
+                __syncwarp(lanes);
                 if (lane == 0) {
                     const uint32_t next = pair + stride;
                     if (next < args.num_units) {

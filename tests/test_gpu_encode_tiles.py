@@ -107,3 +107,22 @@ def test_a_captured_sequence_replays_bit_identically(dq, gradient):
         for (pk, sc), (wpk, wsc) in zip(bufs, want):
             assert torch.equal(pk, wpk) and torch.equal(sc, wsc)
     assert dq.device_error_flags() == 0
+
+
+@pytest.mark.parametrize("mode,bits,dither", [("mask", 8, 32), ("any", 8, 16), ("any", 8, 32), ("dqsg", 8, 32), ("mask", 7, 16),
+                                              ("pow2", 8, 16), ("any", 5, 32), ("dqsg", 3, 16)])
+@pytest.mark.parametrize("bucket", [1024, 2048, 8192])
+def test_many_launches_give_the_same_bits(dq, gradient, mode, bits, dither, bucket):
+    """A row must be in registers before its stage takes the next copy: where it was not, one launch in a few hundred had
+    codes of the wrong elements at the ends of some rows."""
+    sp, g = _spec(mode, bits, dither), gradient[:FIRST]
+    encode = dq.dqsg_encode if sp.kind == DQSG else dq.ndqsg_encode
+    make = lambda f: dq.binding.make_params(bucket, bits, sp.levels, sp.coarse_K, sp.fine_M, sp.alpha, dither, f)  # noqa: E731
+    want = encode(g, 3, 1, 2, make(0))
+    p = make(dq.DQ_FLAG_INPUT_READY | dq.DQ_FLAG_OUTPUT_FREE)
+    out = dq.binding.alloc_message(FIRST, p)
+    wrong = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(1000):
+        encode(g, 3, 1, 2, p, *out)
+        wrong += (out[0] != want[0]).sum() + (out[1] != want[1]).sum()
+    assert int(wrong) == 0
