@@ -36,10 +36,12 @@ METRIC = "encode / fused decode-aggregate GB/s and % of HBM peak on 1 B200; Gele
 L2_BYTES = 126 * 1024 * 1024
 HBM_NOMINAL_GBS = 8000.0
 SM_COUNT, ISSUE_PER_SM_CLK, LANES = 148, 4, 32           # issue ceiling: SMs x schedulers x lanes x clock
-# Algorithmic lane-instructions of the method itself: a quarter of a Philox block per dither value (4.5 wide
-# multiplies + 4.75 three-input XORs), the dither conversion (2), and for the fused decode unpacking (3) plus 5
-# (DQSG) to 9 (NDQSG) fp32 operations per (element, worker), about 10 per element for the mean and the stores;
-# for the encode 24 per element with the scale reduction and the packing.
+# Algorithmic lane-instructions of the method itself, in scalar operations (the kernels do the fp32 part on
+# packed pairs and execute 21 per (element, worker) and 20 per element, profiles/counters_*.md): a quarter of a
+# Philox block per dither value (4.5 wide multiplies + 4.75 three-input XORs), the dither conversion (2), and
+# for the fused decode unpacking (3) plus 5 (DQSG) to 9 (NDQSG) fp32 operations per (element, worker), about 10
+# per element for the mean and the stores; for the encode 24 per element with the scale reduction and the
+# packing.
 DEC_INSTR_PER_ELEM_WORKER, DEC_INSTR_PER_ELEM, ENC_INSTR_PER_ELEM = 22.0, 10.0, 24.0
 FLAG_INPUT_READY, FLAG_OUTPUT_FREE = 1, 2
 
@@ -424,7 +426,8 @@ def other_workloads(torch, hbm_peak, sm_max_mhz):
         sched_hz = SM_COUNT * ISSUE_PER_SM_CLK * sm_max_mhz * 1e6
         out["issue_probe"] = dict(
             probe, what=("scheduler cycles per group, 4 warps per scheduler: one 32x32->64 multiply; one Philox "
-                         "round; the decoder's / encoder's instruction mix for 16 elements with nothing else"),
+                         "round; the decoder's / encoder's instruction mix for 16 elements (fp32 part in scalar form; the "
+                         "kernels use packed pairs) with nothing else"),
             philox_only_gblocks_s=sched_hz * LANES / (9.0 * probe["round_cycles"]) / 1e9,
             decode_mix_ceiling_gelem_worker_s=sched_hz * LANES * 16.0 / probe["dec_coarse_cycles"] / 1e9,
             encode_mix_ceiling_gelem_s=sched_hz * LANES * 16.0 / probe["enc_coarse_cycles"] / 1e9)
@@ -740,7 +743,7 @@ def main():
                                                    "frac": 4.0 * wide_per_unit / cyc_per_unit}}
             probe = (other or {}).get("issue_probe", {})
             if dith == 32 and "decode_mix_ceiling_gelem_worker_s" in probe:
-                # what the decoder's arithmetic alone (nine rounds for four blocks, then 16 NDQSG elements) reaches
+                # what the decoder's arithmetic alone, in scalar form (nine rounds, then 16 NDQSG elements), reaches
                 # on this GPU, measured in this run by bench_tools/issue_probe
                 roofline_decode["measured_mix_ceiling"] = {
                     "gelem_worker_s": probe["decode_mix_ceiling_gelem_worker_s"],
