@@ -26,6 +26,14 @@ namespace dq {
 template <int R> constexpr int kDirectMaxThreads = R == 1 ? 1024 : 256;
 template <int R> constexpr int kDirectMaxCluster = 65536 / (8 * R * kDirectMaxThreads<R>);
 
+// Groups of a lane whose dither is made before the first use of its elements.  With none, a CTA computes nothing while it
+// waits for memory, and then for the maxima of its other warps (n = 11.7 M, B = 2048, 2 bits: 14.1 us with none, 13.4 with one,
+// 13.1 two, 12.7 three, 12.8 four; 25.6 M: 25.4, 24.5, 24.1, 23.7, 23.7; B = 8192: 27.2, 25.6, 25.0, 24.3, 24.3; n = 124.4 M,
+// 3 bits: 112.2, 109.4, 109.0, 107.8, 108.3).  All four fit beside the elements with the 16-bit stream (25.6 M: 19.7 us
+// with none, 18.8 three, 18.4 four).  Two groups per Philox pass instead of one: no difference (23.8).  One-group lanes:
+// n = 1.66 M, B = 16384, K = 3 5.0 us without, 4.7 with it; 2.4 M 4.06 and 3.8.
+template <int R, int DITH> constexpr int kDitherAhead = R == 1 ? 1 : DITH == 16 ? 4 : 3;
+
 // How the lanes' maxima meet in a bucket's scale.  Where a bucket is a power-of-two number of chunks the warp needs
 // neither a barrier nor a gain (a division) per chunk: n = 25.6 M, 2 bits: bucket 1024 28.8 -> 26.5 us, 512 29.0 -> 28.0,
 // 256 30.6 -> 28.7 (one redux per chunk instead of five shuffles).
@@ -94,11 +102,9 @@ inline DirectShape direct_shape(uint32_t g, int R)
     return best;
 }
 
-// The codes of a group: 8 * BITS bits in ceil(BITS / 4) words.  x: the elements as pairs; p0: first Philox product
-// (M0 * counter) of the group's first block; aa: the bucket's gain twice.
-template <int BITS, int MODE, int DITH>
-__device__ __forceinline__ void encode_group8(const f32x2* x, uint64_t p0, f32x2 aa, const DirectArgs& args,
-                                              uint32_t (&out)[(BITS + 3) / 4])
+// The dither values of a group as pairs.  p0: first Philox product (M0 * counter) of the group's first block.
+template <int DITH>
+__device__ __forceinline__ void dither_group8(uint64_t p0, const DirectArgs& args, f32x2 (&delta)[4])
 {
     constexpr int N = (DITH == 16) ? 1 : 2;
     uint32_t hi[N], lo[N], rnd[N][4];
@@ -109,11 +115,20 @@ __device__ __forceinline__ void encode_group8(const f32x2* x, uint64_t p0, f32x2
         lo[j] = (uint32_t)p;
     }
     philox4x32_10_after_first<N>(hi, lo, args.ps, rnd);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) delta[e] = fma2(dither_bits2<DITH>(rnd, 2 * e), args.two, args.off);
+}
+
+// The codes of a group: 8 * BITS bits in ceil(BITS / 4) words.  x: the elements as pairs; aa: the bucket's gain twice.
+template <int BITS, int MODE>
+__device__ __forceinline__ void encode_group8(const f32x2* x, const f32x2 (&delta)[4], f32x2 aa, const DirectArgs& args,
+                                              uint32_t (&out)[(BITS + 3) / 4])
+{
     uint32_t sr = 0u;
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         // v = fma(g, a, delta); DQSG: w = v + s; then round to nearest even
-        f32x2 v = fma2(x[e], aa, fma2(dither_bits2<DITH>(rnd, 2 * e), args.two, args.off));
+        f32x2 v = fma2(x[e], aa, delta[e]);
         if constexpr (MODE == kEncDqsg) v = add2(v, args.shift);
         float t0, t1;
         unpack2(add2(v, args.magic), t0, t1);
@@ -208,6 +223,15 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
     const uint32_t warp_end = local - lane + 32u * (uint32_t)R;
     const bool whole = warp_end <= gpw && group - lane + 32u * (uint32_t)R <= args.whole_groups;     // (uniform in a warp)
 
+    // first product of the lane's first block; those of its other blocks follow by 64-bit additions (M0 (k + j) is
+    // M0 k + M0 j), which are cheaper than wide multiplies on the pipe that bounds the kernel
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * ((args.first_group + group) * kBlocks);
+    // The dither does not depend on the gradient: the dithers of kAhead groups are made while the elements are on their way.
+    constexpr int kAhead = kDitherAhead<R, DITH>;
+    f32x2 delta[R][4];
+    auto dither = [&](int c) { dither_group8<DITH>(p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0, args, delta[c]); };
+    // (a value that is used here is not computed further down)
+    auto made = [&](int c) { asm volatile("" ::"l"(delta[c][0]), "l"(delta[c][1]), "l"(delta[c][2]), "l"(delta[c][3])); };
     if (args.early_read == 0u) {
         grid_dependency_wait();
         if (args.late_launch == 0u) grid_dependency_launch_next();
@@ -240,6 +264,11 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
                 x[4 * c + e] = pack2(2u * e < nvalid ? __ldg(g + 256 * c + 2u * e) : 0.0f,
                                      2u * e + 1u < nvalid ? __ldg(g + 256 * c + 2u * e + 1u) : 0.0f);
         }
+    }
+#pragma unroll
+    for (int c = 0; c < kAhead; ++c) {
+        dither(c);
+        made(c);
     }
     if (args.reduce >= kWarpInBucket) {
         for (uint32_t i = tid; i < args.buckets_per_window; i += blockDim.x) slot[i] = 0u;
@@ -298,15 +327,13 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
             mb[c] = at < gpw ? slot[(at * args.bucket_magic) >> 22] : 0u;
         }
     }
-    // first product of the lane's first block; those of its other blocks follow by 64-bit additions (M0 (k + j) is
-    // M0 k + M0 j), which are cheaper than wide multiplies on the pipe that bounds the kernel
-    const uint64_t p0 = (uint64_t)kPhiloxM0 * ((args.first_group + group) * kBlocks);
     uint32_t out[R][NW];
     f32x2 aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[0])));
 #pragma unroll
     for (int c = 0; c < R; ++c) {
         if (c > 0 && args.gains > (uint32_t)(c % 2)) aa = both(bucket_gain(args.gain_num, __uint_as_float(mb[c])));
-        encode_group8<BITS, MODE, DITH>(x + 4 * c, p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0, aa, args, out[c]);
+        if (c >= kAhead) dither(c);
+        encode_group8<BITS, MODE>(x + 4 * c, delta[c], aa, args, out[c]);
     }
     if (args.early_read == 0u) grid_dependency_launch_next();
     else if (args.early_store == 0u) grid_dependency_wait();
