@@ -308,13 +308,15 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
-    // The tile kernel streams back-to-back encodes of long gradients through persistent CTAs: with launches that overlap
-    // by the caller's flags it is up to 8 % faster from 16 M elements on (B = 2048: n = 16.8 M 15.1 us against 15.1, 25.6 M
-    // 22.2 against 22.7 with two bits and 22.4 against 23.4 with three, 67 M 55.8 against 59.0 with three; B = 512, 67 M 57.5
-    // against 61.5) -- but not for B = 4096, where pairs of warps meet (25.6 M: 23.6 us against 22.7 with two bits, 23.7
-    // against 23.2 with three), which has no rule of its own.  Everything else goes through the direct kernel.
+    // The tile kernel streams back-to-back encodes of long gradients through persistent CTAs.  With launches that overlap by
+    // the caller's flags it is ahead for small buckets, where a lane of the direct kernel computes a gain per group (B = 512:
+    // n = 16.8 M 14.9 us against 14.9 with two bits, 67 M 57.1 against 59.4), and a little for a bucket per warp of very long
+    // gradients (B = 2048, 67 M: 56.2 us against 56.4 with two bits, 56.6 against 57.6 with three; but 25.6 M 22.0 against
+    // 21.6, 16.8 M 14.7 against 14.2); not for B = 1024 (67 M: 57.1 against 55.4) and where warps meet (B = 8192: 60.2
+    // against 57.3).  Everything else goes through the direct kernel.
+    const bool tiles_pay = (p->bucket <= 512u && n >= (1ull << 24)) || (p->bucket == 2048u && n >= (1ull << 26));
     const bool tiles_wanted = is_pow2(p->bucket) && p->bucket <= 8192u &&
-                              (a.test_drop_copy != 0u || (a.early_store != 0u && n >= (1ull << 24)));
+                              (a.test_drop_copy != 0u || (a.early_store != 0u && tiles_pay));
     if (!tiles_wanted) {
         if (encode_direct(mode, *p, a, n, sms, st) != cudaSuccess) return DQ_ERR_CUDA;
         g_launches.fetch_add(1);
