@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <limits>
 #include <mutex>
 #include <utility>
 
@@ -45,25 +46,22 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 
 void fill_philox(dq::PhiloxStream& ps, uint64_t seed, uint32_t worker, uint64_t step)
 {
-    uint32_t k0 = (uint32_t)(seed & 0xFFFFFFFFull), k1 = (uint32_t)(seed >> 32);
-    for (int r = 0; r < 10; ++r) {
-        ps.rk[r][0] = k0;
-        ps.rk[r][1] = k1;
-        k0 += dq::kPhiloxW0;
-        k1 += dq::kPhiloxW1;
+    uint32_t k[10][2] = {{(uint32_t)(seed & 0xFFFFFFFFull), (uint32_t)(seed >> 32)}};
+    for (int r = 1; r < 10; ++r) {
+        k[r][0] = k[r - 1][0] + dq::kPhiloxW0;
+        k[r][1] = k[r - 1][1] + dq::kPhiloxW1;
     }
-    ps.c1 = worker;
-    ps.c2 = (uint32_t)(step & 0xFFFFFFFFull);
-    ps.c3 = (uint32_t)(step >> 32);
+    const uint32_t c1 = worker, c2 = (uint32_t)(step & 0xFFFFFFFFull), c3 = (uint32_t)(step >> 32);
     // the block-independent parts of rounds 0..2 (see PhiloxStream)
-    const uint64_t p1 = (uint64_t)dq::kPhiloxM1 * (uint64_t)ps.c2;
-    const uint32_t u0 = (uint32_t)(p1 >> 32) ^ ps.c1 ^ ps.rk[0][0];
-    const uint32_t u1 = (uint32_t)p1;
+    const uint64_t p1 = (uint64_t)dq::kPhiloxM1 * (uint64_t)c2;
+    const uint32_t u0 = (uint32_t)(p1 >> 32) ^ c1 ^ k[0][0];
     const uint64_t p0 = (uint64_t)dq::kPhiloxM0 * (uint64_t)u0;
-    ps.v0 = ps.c3 ^ ps.rk[0][1];
-    ps.v1 = u1 ^ ps.rk[1][0];
-    ps.v2 = (uint32_t)(p0 >> 32) ^ ps.rk[1][1];
-    ps.v3 = (uint32_t)p0 ^ ps.rk[2][1];
+    ps.v0 = c3 ^ k[0][1];
+    ps.v1 = (uint32_t)p1 ^ k[1][0];
+    ps.v2 = (uint32_t)(p0 >> 32) ^ k[1][1];
+    ps.v3 = (uint32_t)p0 ^ k[2][1];
+    ps.k2 = k[2][0];
+    std::memcpy(ps.rk, k + 3, sizeof(ps.rk));
 }
 
 int device_sm_count()
@@ -171,12 +169,14 @@ cudaError_t launch_encode(int mode, uint32_t bits, bool dither16, const CUtensor
     }
 }
 
-dq::f32x2 twice(float v)
+uint32_t bits_of(float v)
 {
     uint32_t u;
     std::memcpy(&u, &v, sizeof(u));
-    return ((dq::f32x2)u << 32) | u;
+    return u;
 }
+
+dq::f32x2 twice(float v) { return ((dq::f32x2)bits_of(v) << 32) | bits_of(v); }
 
 cudaError_t launch_direct(int mode, uint32_t bits, bool dither16, int R, const dq::DirectArgs& a, uint32_t grid,
                           uint32_t threads, cudaStream_t st)
@@ -394,6 +394,31 @@ int decode_group_size(uint64_t n, uint32_t W, bool reads_side, bool usual, int s
     return 32;
 }
 
+// The constants of a worker that depend on the form its routine works in (see DecForm).  Returns the largest scale that the
+// form takes.
+float set_decode_form(dq::DecWorker& d, uint32_t kind, int bits, int dith)
+{
+    const int form = dq::dec_form(kind, bits, dith), shift = dq::dec_shift(kind, bits, dith);
+    const float u = 1.0f / (float)(1u << shift);
+    if (form == dq::kFormJoined && dith == 16)
+        d.offset = twice(((float)((1u << bits) - 1u) - d.s + dq::kD16Offset) * u);          // J = (2^bits - 1 - k) 2^16 + h
+    else if (form == dq::kFormJoined)
+        d.offset = twice(-(d.s + dq::kD32Offset));                                          // J = k 2^22 + (2^22 - 1 - j)
+    else
+        d.offset = twice(-(4194304.0f + d.s - 1.5f));
+    if (kind != dq::kDecDqsg) {
+        d.neg_K = twice(-d.K * u);
+        if (form == dq::kFormTiny) d.neg_K_code = twice(-d.K * 0x1p-125f / (float)(1u << bits));
+        d.inv_K = twice(1.0f / d.K / u);
+        d.A *= u;
+    }
+    if (shift == 0) return std::numeric_limits<float>::infinity();
+    // kappa / s / u and alpha kappa / M1 / u below 2^127, alpha M1 u / kappa normal
+    if (kind == dq::kDecDqsg) return 0x1p119f;
+    const float most = std::fmin(d.M1 / d.alpha * 0x1p-6f, d.A);
+    return most >= 1.0f ? 0x1p120f : most * 0x1p120f;
+}
+
 dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t step, const float* side_info,
                         float* out_avg, uint32_t* status_word, bool allow_nested, cudaStream_t st,
                         bool running = false, bool half_dithered = false, uint64_t first_element = 0u,
@@ -403,6 +428,7 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     static thread_local dq::DecodeArgs a;    // ~13 KB: keep it off the stack; the first W entries of a.w are filled
     std::memset(static_cast<dq::DecodeHead*>(&a), 0, sizeof(dq::DecodeHead));
     bool any_nested = false;
+    float kappa_most = std::numeric_limits<float>::infinity();
     for (uint32_t w = 0; w < W; ++w) {
         const dq_msg& m = msgs[w];
         uint32_t L = 0;
@@ -422,20 +448,17 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
         if (m.kind == DQ_KIND_DQSG) {
             kind = dq::kDecDqsg;
             d.s = (float)(L - 1u) / 2.0f;
-            d.neg_c = twice(-(4194304.0f + d.s - 1.5f));
             d.step_mul = is_pow2(L - 1u) && L >= 3u ? 2.0f / (float)(L - 1u) : (L == 2u ? 2.0f : 0.0f);
         } else {
             any_nested = true;
             if (is_pow2(m.p.coarse_K)) kind = (alpha == 1.0f) ? dq::kDecNdqsgPow2 : dq::kDecNdqsgPow2Shrink;
             else kind = (alpha == 1.0f) ? dq::kDecNdqsgAnyK : dq::kDecNdqsgAnyKShrink;
-            d.neg_c = twice(-(4194304.0f - 1.5f));
             d.A = alpha * m.p.fine_M;
             d.M1 = m.p.fine_M;
             d.alpha = alpha;
             const float a2 = alpha * alpha;
             d.one_m_alpha2 = 1.0f - a2;
-            d.neg_K = twice(-(float)m.p.coarse_K);
-            d.inv_K = twice(1.0f / (float)m.p.coarse_K);
+            d.K = (float)m.p.coarse_K;
             d.step_mul = float_is_pow2(m.p.fine_M) ? 1.0f / m.p.fine_M : 0.0f;
             if (running) {
                 if (w == 0u) return DQ_ERR_INVALID_ARG;      // nothing decoded yet to serve as side information
@@ -443,6 +466,8 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
             }
         }
         d.variant = kind * 8u + m.p.bits - 1u;
+        kappa_most = std::fmin(kappa_most, set_decode_form(d, kind, (int)m.p.bits,
+                                                           half_dithered ? 0 : m.p.dither_bits == 16u ? 16 : 32));
     }
     // runs of equal variants (one routine per run, see decode_workers)
     for (uint32_t w = W; w-- > 0u;)
@@ -472,6 +497,9 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     a.has_side = reads_side ? 1u : 0u;
     a.out_align32 = (reinterpret_cast<uintptr_t>(out_avg) & 31u) == 0u ? 1u : 0u;
     a.half_bias_bits = 0x4A800000u;
+    a.low22 = 0x003FFFFFu;
+    // (no limit: above the pattern of any NaN)
+    a.kappa_limit = std::isinf(kappa_most) ? 0xFFFFFFFFu : bits_of(kappa_most);
     a.neg_zero = twice(-0.0f);
     a.magic = twice(dq::kMagic);
     a.neg_magic = twice(-dq::kMagic);

@@ -31,20 +31,23 @@ enum DecKind : uint32_t {
 struct DecWorker {
     const uint32_t* packed;   // } addresses of the (virtual) whole-gradient buffers, see DecodeArgs
     const float* scale;       // }
+    // Pairs of equal values (one 64-bit load each), for the form in which the routine works (DecForm; u = 2^-shift):
+    f32x2 offset;         // joined: see there; biased: minus (DQSG: 4194304 + s - 1.5, NDQSG: 4194304 - 1.5)
+    f32x2 neg_K;          // -K u
+    f32x2 neg_K_code;     // -K in units of the tiny code
+    f32x2 inv_K;          // 1/K rounded to nearest (exact when K is a power of two), over u
     PhiloxStream ps;
     uint32_t variant;     // DecKind * 8 + bits - 1: one jump selects the routine
     uint32_t group_end;   // index after the last worker of the run of equal variants that this worker belongs to
+    float step_mul;       // DQSG: 1/s, NDQSG: 1/M1, when that divisor is a power of two (the division is then an
+                          // exact multiplication); 0 otherwise
     float s;              // DQSG (L-1)/2
-    f32x2 neg_c;          // } pairs of equal values (one 64-bit load each): minus (DQSG: 4194304 + s - 1.5,
-    f32x2 neg_K;          // } NDQSG: 4194304 - 1.5; see unpack_half_biased), -K, and 1/K rounded to nearest (exact
-    f32x2 inv_K;          // } when K is a power of two)
-    float A;              // NDQSG alpha * M1
+    float A;              // NDQSG alpha * M1 * u
     float M1;
     float alpha;
     float one_m_alpha2;   // 1 - alpha*alpha
     float rcp_count;      // running-mean mode: 1 / (number of workers before this one)
-    float step_mul;       // DQSG: 1/s, NDQSG: 1/M1, when that divisor is a power of two (the division is then an
-                          // exact multiplication); 0 otherwise
+    float K;
 };
 
 struct DecodeHead {
@@ -65,6 +68,8 @@ struct DecodeHead {
     uint32_t has_side;        // the side information vector is read
     uint32_t out_align32;     // out is 32-byte aligned: whole groups leave in 32-byte stores
     uint32_t half_bias_bits;  // 0x4A800000 (bit pattern of 2^22), passed in so that it lives in a register
+    uint32_t low22;           // 2^22 - 1, likewise
+    uint32_t kappa_limit;     // bit pattern of the largest scale that the scaled forms of these messages take (see DecForm)
     float Wf;
     f32x2 neg_zero;           // -0.0 twice (see f32x2)           } constants that would otherwise be assembled from
     f32x2 magic, neg_magic;   // +-1.5 * 2^23 twice               } immediates again and again
@@ -105,8 +110,55 @@ constexpr int pair_set(int dqsg_bits, int ndqsg_bits) { return 16 * dqsg_bits + 
 // kernels: what a worker costs per lane (scale, gain, constants, loop: about 65 instructions) is spread over the most
 // elements.  96 registers are 3 % faster for a given side information vector but 2 to 8 % slower otherwise (the compiler
 // then loads a worker's constants lane by lane), 128 registers 7 % slower; the kernel with all routines wants 96.
-// E = 16 and 8 take 64 registers (32 warps).
-constexpr int dec_ctas_per_sm(int E, int set) { return E == 32 ? (set == kSetAll ? 5 : 6) : 8; }
+// E = 16 and 8 take 64 registers (32 warps), but for 72 where all routines in groups of 8 would not fit 64 (W = 8,
+// n = 266,010: 5.65 us with a spill, 5.45 without).
+constexpr int dec_ctas_per_sm(int E, int set) { return E == 32 ? (set == kSetAll ? 5 : 6) : (E == 8 && set == kSetAll) ? 7 : 8; }
+
+// How a routine forms k - s - delta (DQSG) and m - delta, q - delta (NDQSG) from the code and the random bits.  All forms
+// round the same real numbers once, so they give the same bits; they differ in the number of packed instructions.
+//   biased:  X = k - s + 1.5 from the float 2^22 + k, f = delta + 1.5 from the random bits, X - f.
+//   joined:  code and random bits side by side in one mantissa, one multiply-add for both.  The join is an integer below
+//            2^24, read as a (subnormal or small) float; with the 16-bit stream always possible (up to seven bits), with
+//            the 32-bit stream where 22 + bits <= 24 and (NDQSG) m - delta is representable, so that q - delta follows
+//            from it by another multiply-add.
+//   tiny:    NDQSG up to four bits: the code in bits 23.. downwards of a float is an exact multiple of 2^-149, so that
+//            m - delta and q - delta are one multiply-add each and no bias has to be taken off.
+// The values of the last two forms are smaller than the real ones by 2^shift, because a multiply-add cannot scale by more than
+// 2^127; gain and 1/K carry the factor, and groups with a scale where that could overflow or lose bits (kappa_limit, far
+// above any gradient) are decoded again by decode_group_plain.
+enum DecForm : int { kFormBiased = 0, kFormJoined = 1, kFormTiny = 2 };
+
+__host__ __device__ constexpr int dec_form(uint32_t kind, int bits, int dith)
+{
+    if (dith == 16) return bits <= 7 ? kFormJoined : kFormBiased;
+    if (dith == 32 && kind == kDecDqsg) return bits <= 2 ? kFormJoined : kFormBiased;
+    if (dith == 32) return bits == 1 ? kFormJoined : bits <= 4 ? kFormTiny : kFormBiased;
+    return kFormBiased;
+}
+
+__host__ __device__ constexpr int dec_shift(uint32_t kind, int bits, int dith)
+{
+    const int form = dec_form(kind, bits, dith);
+    return form == kFormTiny ? bits - 2 : (form == kFormJoined && dith == 16) ? 6 : 0;
+}
+
+__host__ __device__ constexpr float pow2f(int e)
+{
+    float v = 1.0f;
+    for (; e > 0; --e) v *= 2.0f;
+    for (; e < 0; ++e) v *= 0.5f;
+    return v;
+}
+
+// BITS bits of the stream from bit `start` on (a compile-time constant after unrolling) and what follows them.
+template <int NF>
+__device__ __forceinline__ uint32_t stream_from(const uint32_t (&f)[NF], int start, int bits)
+{
+    const int wi = start >> 5, sh = start & 31;
+    if (sh == 0) return f[wi];
+    if (sh + bits <= 32) return f[wi] >> sh;
+    return __funnelshift_r(f[wi], f[(wi + 1) % NF], sh);
+}
 
 // Code of element `idx` of a group as the float 2^22 + code: the bit pattern of 2^22 with the code in mantissa
 // bits 1.. (floats in [2^22, 2^23) step by 1/2).  Subtracting a constant then gives code - c exactly.
@@ -124,6 +176,61 @@ __device__ __forceinline__ float unpack_half_biased(const uint32_t (&f)[NF], int
         v = __funnelshift_r(f[wi], f[(wi + 1) % NF], sh - 1);
     }
     return __uint_as_float((v & mask2) | bias_bits);          // one logic op: (v & immediate) | register
+}
+
+// 16-bit stream, joined form: the complement of the code above the half-word.  Codes that share a shift are masked
+// together, and one byte permutation takes the two bytes of the half-word, the code's byte, and zeros (the copies of that
+// byte's clear top bit).
+template <int BITS, int NF>
+__device__ __forceinline__ float join16(const uint32_t (&f)[NF], int idx, uint32_t word, int high)
+{
+    constexpr uint32_t mask = (1u << BITS) - 1u;
+    uint32_t v;
+    int byte;
+    if constexpr (8 % BITS == 0) {
+        const int bit = idx * BITS;
+        v = ~(f[bit >> 5] >> (bit & 7)) & (mask * 0x01010101u);
+        byte = (bit >> 3) & 3;
+    } else if constexpr (BITS == 3 || BITS == 6) {            // codes 24 bits apart
+        constexpr int step = 24 / BITS;
+        const int first = idx / (2 * step) * (2 * step) + idx % step;
+        v = ~stream_from(f, first * BITS, (NF * 32 - first * BITS >= 24 + BITS) ? 24 + BITS : BITS) & (mask * 0x01000001u);
+        byte = idx % (2 * step) >= step ? 3 : 0;
+    } else {
+        v = ~stream_from(f, idx * BITS, BITS) & mask;
+        byte = 0;
+    }
+    const uint32_t b = 4u + (uint32_t)byte;
+    uint32_t d;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(word), "r"(v), "r"((high ? 0x32u : 0x10u) | (b << 8) | ((b | 8u) << 12)));
+    return __uint_as_float(d);
+}
+
+// 32-bit stream, joined form: the code above the complement of the 22 random bits.
+template <int BITS, int NF>
+__device__ __forceinline__ float join32(const uint32_t (&f)[NF], int idx, uint32_t word, uint32_t low22)
+{
+    const uint32_t v = __funnelshift_r(word, f[(idx * BITS) >> 5] >> ((idx * BITS) & 31), 10);
+    return __uint_as_float((v & ((1u << (22 + BITS)) - 1u)) ^ low22);      // one logic op: (v & immediate) ^ register
+}
+
+// The code in the BITS bits below bit 24 (one bit: below bit 23).
+template <int BITS, int NF>
+__device__ __forceinline__ float tiny_code(const uint32_t (&f)[NF], int idx)
+{
+    constexpr uint32_t mask = (1u << BITS) - 1u;
+    const int bit = idx * BITS;
+    if constexpr (8 % BITS == 0) {
+        const int up = 8 - BITS - (bit & 7);                  // to the top of its byte
+        const uint32_t v = (up >= 0 ? f[bit >> 5] << up : f[bit >> 5] >> -up) & ((mask << (8 - BITS)) * 0x01010101u);
+        return __uint_as_float(__byte_perm(v, 0u, 0x4044u | (uint32_t)(((bit >> 3) & 3) << 8)));
+    } else {
+        const int sh = (bit & 31) - (24 - BITS), wi = bit >> 5;
+        const uint32_t v = (bit & 31) + BITS > 32 ? __funnelshift_r(f[wi], f[(wi + 1) % NF], sh)
+                           : sh >= 0              ? f[wi] >> sh
+                                                  : f[wi] << -sh;
+        return __uint_as_float(v & (mask << (24 - BITS)));
+    }
 }
 
 constexpr int gcd_of(int a, int b) { return b == 0 ? a : gcd_of(b, a % b); }
@@ -148,6 +255,12 @@ struct Field {
             for (int j = 0; j < kLoads; ++j) w[j] = (wi + j < num_words) ? __ldg(p + j) : 0u;
             return;
         }
+        load_from(p);
+    }
+
+    // (p: the word that holds the field's first bit; every word that a field can touch is there)
+    __device__ __forceinline__ void load_from(const uint32_t* p)
+    {
         if constexpr (kAlign == 32 && kLoads % 4 == 0) {
 #pragma unroll
             for (int j = 0; j < kLoads; j += 4) {
@@ -187,9 +300,56 @@ struct DecLane {
     bool careful;
 };
 
+// Decodes one group and stores its mean, element by element and with nothing scaled: for groups with a scale near the end of
+// the fp32 range (kappa_limit).  (It stores its results
+// itself: an array in local memory for them cost every call of the kernel, n = 266,610, W = 8 6.5 us instead of 6.3.)
+template <int DITH, int SIDE, int E, typename Args>
+__device__ __noinline__ void decode_group_plain(const Args& args, uint32_t group, uint32_t bucket)
+{
+#pragma unroll 1
+    for (uint32_t e = 0; e < (uint32_t)E; ++e) {
+        const uint64_t i = (uint64_t)group * (uint32_t)E + e;
+        if (i >= args.n) return;
+        float acc = 0.0f, y = (SIDE == kSideGiven && args.has_side != 0u) ? __ldg(args.side + i) : 0.0f;
+#pragma unroll 1
+        for (uint32_t w = 0; w < args.W; ++w) {
+            const DecWorker& wk = args.w[w];
+            const uint32_t bits = (wk.variant & 7u) + 1u, kind = wk.variant >> 3;
+            const uint64_t bit = i * bits;
+            const uint32_t sh = (uint32_t)bit & 31u;
+            uint32_t code = __ldg(wk.packed + (bit >> 5)) >> sh;
+            if (sh + bits > 32u) code |= __ldg(wk.packed + (bit >> 5) + 1u) << (32u - sh);
+            const float k = (float)(code & ((1u << bits) - 1u)), kappa = __ldg(wk.scale + bucket);
+            const uint64_t p = (uint64_t)kPhiloxM0 * (uint32_t)(i / (DITH == 16 ? 8u : 4u));
+            const uint32_t hi[1] = {(uint32_t)(p >> 32)}, lo[1] = {(uint32_t)p};
+            uint32_t rnd[1][4];
+            philox4x32_10_after_first<1>(hi, lo, wk.ps, rnd);
+            const uint32_t at = (uint32_t)i & (DITH == 16 ? 7u : 3u), which = DITH == 16 ? at >> 1 : at;
+            const uint32_t word = which == 0u ? rnd[0][0] : which == 1u ? rnd[0][1] : which == 2u ? rnd[0][2] : rnd[0][3];
+            const float delta = DITH == 16 ? __fmaf_rn((float)((word >> (16u * (at & 1u))) & 0xFFFFu), 0x1p-16f, -kD16Offset)
+                                           : __fmaf_rn((float)(word >> 10), 0x1p-22f, -kD32Offset);
+            float gt;
+            if (kind == kDecDqsg) {
+                gt = __fmul_rn(__fdiv_rn(kappa, wk.s), __fsub_rn(__fsub_rn(k, wk.s), delta));
+            } else {
+                const float a = (kappa >= 0x1p-100f) ? __fdiv_rn(__fmul_rn(wk.alpha, wk.M1), kappa) : 0.0f;
+                const float c = __fdiv_rn(__fmul_rn(wk.alpha, kappa), wk.M1);
+                if (SIDE == kSideRunning) y = __fmul_rn(acc, wk.rcp_count);
+                const float r = __fmaf_rn(-y, a, __fsub_rn(k, delta));
+                const float d = __fsub_rn(__fmaf_rn(-wk.K, rintf(__fdiv_rn(r, wk.K)), k), delta);
+                gt = wk.alpha == 1.0f ? __fmul_rn(c, d) : __fmaf_rn(c, d, __fmul_rn(wk.one_m_alpha2, y));
+            }
+            acc = __fadd_rn(acc, gt);
+            if (SIDE == kSideFirst && w == 0u) y = acc;
+        }
+        if (args.W > 1u) acc = (args.invW != 0.0f) ? __fmul_rn(acc, args.invW) : __fdiv_rn(acc, args.Wf);
+        args.out[i] = acc;
+    }
+}
+
 // The contributions of the workers [w, w_end), a run of equal variants: the same routine for each, so the jump on the
 // variant is taken once per run and not once per worker (Algorithm 2's groups P1 and P2 are two runs).
-//   DQSG:  g~ = (kappa/s) ((k - s) - delta); (k - s + 1.5) - f rounds once to the same value.
+//   DQSG:  g~ = (kappa/s) ((k - s) - delta)
 //   NDQSG: r = (m - delta) - y a;  jj = rint(r / K);  q1^ = m - K jj;  g~ = beta (q1^ - delta) [+ (1-alpha^2) y]
 // AHEAD: the packed words are requested one worker ahead (see kWordsAhead).
 //
@@ -205,6 +365,7 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
     constexpr bool RUN = SIDE == kSideRunning;
     constexpr bool ANY_K = KIND == kDecNdqsgAnyK || KIND == kDecNdqsgAnyKShrink;
     constexpr bool SHRINK = KIND == kDecNdqsgPow2Shrink || KIND == kDecNdqsgAnyKShrink;
+    constexpr int FORM = dec_form(KIND, BITS, DITH), SHIFT = dec_shift(KIND, BITS, DITH);
     constexpr int EPB = (DITH == 16) ? 8 : 4;       // elements per Philox block
     constexpr int N = E / EPB;                      // blocks of the group
     constexpr int P = N < 2 ? N : 2;                // blocks in flight
@@ -240,6 +401,8 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
                 }
                 const float kappa = ln.kappa_next;
                 if (w + 1u < args.W) ln.kappa_next = __ldg(args.w[w + 1u].scale + ln.bucket);
+                const uint32_t kb = __float_as_uint(kappa) & 0x7FFFFFFFu;
+                ln.kappa_bits_max = (kb > ln.kappa_bits_max) ? kb : ln.kappa_bits_max;
                 // kappa / s and alpha kappa / M1: a division by a power of two is an exact multiplication
                 float c;
                 if constexpr (KIND == kDecDqsg) {
@@ -249,9 +412,8 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
                     const float ak = __fmul_rn(wk.alpha, kappa);
                     c = (wk.step_mul != 0.0f) ? __fmul_rn(ak, wk.step_mul) : __fdiv_rn(ak, wk.M1);        // beta
                 }
+                if constexpr (SHIFT != 0) c = __fmul_rn(c, pow2f(SHIFT));
                 cc = both(c);
-                const uint32_t kb = __float_as_uint(kappa) & 0x7FFFFFFFu;
-                ln.kappa_bits_max = (kb > ln.kappa_bits_max) ? kb : ln.kappa_bits_max;
             }
 #pragma unroll
             for (int qq = 0; qq < P * EPB / 4; ++qq) {      // four elements at a time (one 16-byte slot of y)
@@ -266,21 +428,35 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
                 for (int e = 0; e < 2; ++e) {
                     const int t = 4 * q + 2 * e;                           // element of the group
                     const int tr = 4 * qq + 2 * e;                         // ... of the blocks in rnd
-                    f32x2 nf;                                              // -f, f = delta + 1.5
-                    if constexpr (DITH == 0) nf = both(-1.5f);
-                    else if constexpr (DITH == 16) nf = fma2(dither_bits2<16>(rnd, tr), both(-kTwo125), both(-kF16Offset));
-                    else nf = fma2(dither_bits2<32>(rnd, tr), both(-kTwo127), both(-kF32Offset));
-                    const f32x2 X = add2(pack2(unpack_half_biased<BITS>(f, t, args.half_bias_bits),
-                                               unpack_half_biased<BITS>(f, t + 1, args.half_bias_bits)), wk.neg_c);
+                    // x = u (k - s - delta) or u (m - delta); biased: X and nf with x = X + nf; tiny: code and nf
+                    f32x2 x, X = 0ull, nf = 0ull;
+                    if constexpr (FORM == kFormJoined && DITH == 16) {
+                        const uint32_t word = rnd[tr >> 3][(tr & 7) >> 1];
+                        x = fma2(pack2(join16<BITS>(f, t, word, 0), join16<BITS>(f, t + 1, word, 1)), both(-kTwo127), wk.offset);
+                    } else if constexpr (FORM == kFormJoined) {
+                        x = fma2(pack2(join32<BITS>(f, t, rnd[tr >> 2][tr & 3], args.low22),
+                                          join32<BITS>(f, t + 1, rnd[tr >> 2][(tr & 3) + 1], args.low22)),
+                                 both(kTwo127), wk.offset);
+                    } else if constexpr (FORM == kFormTiny) {
+                        nf = fma2(dither_bits2<32>(rnd, tr), both(-kTwo127 * pow2f(-SHIFT)), both(kD32Offset * pow2f(-SHIFT)));
+                        X = pack2(tiny_code<BITS>(f, t), tiny_code<BITS>(f, t + 1));
+                        x = fma2(X, both(kTwo127), nf);
+                    } else {
+                        if constexpr (DITH == 0) nf = both(-1.5f);
+                        else if constexpr (DITH == 16) nf = fma2(dither_bits2<16>(rnd, tr), both(-kTwo125), both(-kF16Offset));
+                        else nf = fma2(dither_bits2<32>(rnd, tr), both(-kTwo127), both(-kF32Offset));
+                        X = add2(pack2(unpack_half_biased<BITS>(f, t, args.half_bias_bits),
+                                       unpack_half_biased<BITS>(f, t + 1, args.half_bias_bits)), wk.offset);
+                        x = add2(X, nf);
+                    }
                     f32x2 gt;
                     if constexpr (KIND == kDecDqsg) {
-                        gt = fma2(cc, add2(X, nf), nz);                    // c ((k - s) - delta)
+                        gt = fma2(cc, x, nz);                              // c ((k - s) - delta)
                     } else {
                         // side information: the given vector, the reconstruction of message 0, or (Algorithm 2 as
                         // written) the mean of the reconstructions accumulated so far
                         const f32x2 yy = RUN ? fma2(acc[t >> 1], both(wk.rcp_count), nz) : y[e];
-                        const f32x2 r1 = add2(X, nf);                      // m - delta
-                        const f32x2 r = fma2(yy, na, r1);
+                        const f32x2 r = fma2(yy, na, x);
                         f32x2 jj;
                         if constexpr (ANY_K) {
                             // r / K rounded to nearest from the correctly rounded 1/K: one residual correction leaves
@@ -293,8 +469,11 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
                             // K is a power of two: r * (1/K) is exact, so one rounding gives rint(r / K)
                             jj = add2(fma2(r, wk.inv_K, args.magic), args.neg_magic);
                         }
-                        const f32x2 d = add2(fma2(wk.neg_K, jj, X), nf);   // q1^ - delta  (q1^ + 1.5 is exact)
-                        gt = fma2(cc, d, SHRINK ? fma2(both(wk.one_m_alpha2), yy, nz) : nz);
+                        f32x2 d;                                           // u (q1^ - delta)
+                        if constexpr (FORM == kFormJoined) d = fma2(wk.neg_K, jj, x);
+                        else if constexpr (FORM == kFormTiny) d = fma2(fma2(wk.neg_K_code, jj, X), both(kTwo127), nf);
+                        else d = add2(fma2(wk.neg_K, jj, X), nf);          // (q1^ + 1.5 is exact)
+                        gt = SHRINK ? fma2(cc, d, fma2(both(wk.one_m_alpha2), yy, nz)) : fma2(cc, d, nz);
                     }
                     acc[t >> 1] = add2(acc[t >> 1], gt);
                 }
@@ -372,16 +551,17 @@ __device__ __forceinline__ void store8(float* p, const f32x2 (&v)[4], bool align
 // ---------------------------------------------------------------------------------------------------
 // The decode kernel: one group of E elements per lane.
 // ---------------------------------------------------------------------------------------------------
-template <int DITH, int SIDE, int E, int SET, int MAXW>
-__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(E, SET))
-decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
-{
-    // per lane: E / 4 slots of side information, then the first Philox products (two blocks per slot)
-    constexpr int N = (DITH == 16) ? E / 8 : E / 4;
-    constexpr int kSlots = E / 4 + (DITH != 0 && N > 1 ? N / 2 : 0);
-    __shared__ __align__(16) float4 slots[kSlots][kDecThreads];
+// Shared memory, per lane: E / 4 slots of side information, then the first Philox products (two blocks per slot).
+template <int DITH, int E>
+constexpr int kDecBlocks = (DITH == 16) ? E / 8 : E / 4;
+template <int DITH, int E>
+constexpr int kDecSlots = E / 4 + (DITH != 0 && kDecBlocks<DITH, E> > 1 ? kDecBlocks<DITH, E> / 2 : 0);
 
-    const uint64_t local = (uint64_t)blockIdx.x * (uint32_t)kDecThreads + threadIdx.x;
+// The kernel's work, for the lane's group `local`.
+template <int DITH, int SIDE, int E, int SET, typename Args>
+__device__ __forceinline__ void decode_group(const Args& args, float4 (*slots)[kDecThreads], uint64_t local)
+{
+    constexpr int N = kDecBlocks<DITH, E>;
     // Lanes past the end either leave (there is no barrier below), or repeat the last group and store nothing: then the
     // control flow stays uniform for the compiler and a worker's constants take the uniform data path, which gains 1 to 2 %
     // with long chains per lane and loses as much in the shorter ones.
@@ -443,7 +623,6 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
 #pragma unroll
     for (int e = 0; e < E / 2; ++e) acc[e] = 0ull;
     decode_workers<DITH, SIDE, E, SET>(args, ln, acc);
-
     // The next kernel may become resident when every CTA of this one is about to store.  Let in right after the wait, its
     // CTAs would take the slots that this kernel leaves free, and what does not fit would be placed when these end,
     // several CTAs on one SM and none on others, as soon as a grid takes more than half the slots (W = 8: n = 1.3 M 20.3 us
@@ -465,7 +644,9 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
     }
     float* o = args.out + i0;
     if (kClamp && !live) return;
-    if (whole) {
+    if (DITH != 0 && ln.kappa_bits_max > args.kappa_limit) {
+        decode_group_plain<DITH, SIDE, E>(args, ln.group, ln.bucket);
+    } else if (whole) {
 #pragma unroll
         for (int k = 0; k < E / 8; ++k) {
             const f32x2 v[4] = {acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]};
@@ -481,6 +662,14 @@ decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
         }
     }
     if (args.status != nullptr && ln.kappa_bits_max >= 0x7F800000u) atomicOr(args.status, 0x1u);
+}
+
+template <int DITH, int SIDE, int E, int SET, int MAXW>
+__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(E, SET))
+decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
+{
+    __shared__ __align__(16) float4 slots[kDecSlots<DITH, E>][kDecThreads];
+    decode_group<DITH, SIDE, E, SET>(args, slots, (uint64_t)blockIdx.x * (uint32_t)kDecThreads + threadIdx.x);
 }
 
 }  // namespace dq

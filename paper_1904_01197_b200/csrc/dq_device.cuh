@@ -18,15 +18,16 @@ constexpr uint32_t kPhiloxM1 = 0xCD9E8D57u;
 constexpr uint32_t kPhiloxW0 = 0x9E3779B9u;
 constexpr uint32_t kPhiloxW1 = 0xBB67AE85u;
 
+// Only counter word 0 differs between the blocks of a (seed, worker, step) stream, so parts of rounds 0..2 are the same for
+// all of them; the host folds them into four words.  (No word more than is read: in a short kernel every line of parameters
+// is a cache miss that the first warps wait for.)
 struct PhiloxStream {
-    uint32_t rk[10][2];   // round keys
-    uint32_t c1, c2, c3;  // counter words 1..3: worker, lo32(step), hi32(step)
-    // Only counter word 0 differs between blocks, so parts of rounds 0..2 are the same for every block of a
-    // (seed, worker, step) stream; the host folds them into four words:
-    uint32_t v0;          // c3 ^ rk[0][1]
-    uint32_t v1;          // lo(M1*c2) ^ rk[1][0]
-    uint32_t v2;          // hi(M0*u0) ^ rk[1][1],  u0 = hi(M1*c2) ^ c1 ^ rk[0][0]
-    uint32_t v3;          // lo(M0*u0) ^ rk[2][1]
+    uint32_t v0;          // c3 ^ k[0][1]
+    uint32_t v1;          // lo(M1*c2) ^ k[1][0]
+    uint32_t v2;          // hi(M0*u0) ^ k[1][1],  u0 = hi(M1*c2) ^ c1 ^ k[0][0]
+    uint32_t v3;          // lo(M0*u0) ^ k[2][1]
+    uint32_t k2;          // k[2][0]
+    uint32_t rk[7][2];    // k[3..9]: keys of the rounds after
 };
 
 // M0 * j for j = 0..7: the blocks of a row have consecutive counters base + j, and M0 * (base + j) is
@@ -54,7 +55,7 @@ __device__ __forceinline__ void philox4x32_10_after_first(const uint32_t (&p0hi)
     for (int j = 0; j < N; ++j) {
         const uint64_t p0 = (uint64_t)kPhiloxM0 * (uint64_t)c0[j];
         const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint64_t)c2[j];
-        c0[j] = (uint32_t)(p1 >> 32) ^ c1[j] ^ ps.rk[2][0];
+        c0[j] = (uint32_t)(p1 >> 32) ^ c1[j] ^ ps.k2;
         c1[j] = (uint32_t)p1;
         c2[j] = (uint32_t)(p0 >> 32) ^ ps.v3;
         c3[j] = (uint32_t)p0;
@@ -65,9 +66,9 @@ __device__ __forceinline__ void philox4x32_10_after_first(const uint32_t (&p0hi)
         for (int j = 0; j < N; ++j) {
             const uint64_t p0 = (uint64_t)kPhiloxM0 * (uint64_t)c0[j];
             const uint64_t p1 = (uint64_t)kPhiloxM1 * (uint64_t)c2[j];
-            c0[j] = (uint32_t)(p1 >> 32) ^ c1[j] ^ ps.rk[r][0];
+            c0[j] = (uint32_t)(p1 >> 32) ^ c1[j] ^ ps.rk[r - 3][0];
             c1[j] = (uint32_t)p1;
-            c2[j] = (uint32_t)(p0 >> 32) ^ c3[j] ^ ps.rk[r][1];
+            c2[j] = (uint32_t)(p0 >> 32) ^ c3[j] ^ ps.rk[r - 3][1];
             c3[j] = (uint32_t)p0;
         }
     }

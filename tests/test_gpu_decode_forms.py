@@ -1,0 +1,60 @@
+"""The forms in which the decoder joins code and dither (by kind, code width and dither stream), bit for bit against the
+oracle, at every group size, with scales from subnormal numbers to near the end of the fp32 range: beyond kappa_limit a
+group is decoded by the plain routine."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+from dq_testlib import gpu_encode, gpu_msg, oracle_msg, words_np  # noqa: E402
+from dq_workloads.generators import DQSG, NDQSG, WorkerSpec  # noqa: E402
+from test_gpu_parity import dq, oracle  # noqa: E402,F401
+
+# factors of consecutive buckets: subnormal and tiny scales, ordinary ones, ones around the limits 2^114 to 2^120 and above
+FACTORS = np.array([1.0, 1e-40, 1e-34, 0.0, 1.0, 1e30, 3e34, 2e35, 1e36, 4e36, 1.0, 1.5e37], np.float32)
+BUCKET = 1248                                # (not a power of two, and buckets begin inside a warp's groups)
+
+
+@pytest.mark.parametrize("n,few", [(12 * BUCKET + 77, True), (12 * BUCKET + 77, False), (1300001, True), (8000007, True)],
+                         ids=["8", "8 many", "16", "32"])
+@pytest.mark.parametrize("dither,widths", [(32, (1, 2, 3, 4)), (16, (1, 2, 3, 4, 5, 6, 7, 8))])
+def test_forms_over_the_range_of_scales(dq, oracle, n, few, dither, widths):
+    step = 9
+    rng = np.random.default_rng(n + dither)
+    nb = -(-n // BUCKET)
+    common = rng.standard_normal(n).astype(np.float32)
+    near = common + 0.05 * rng.standard_normal(n).astype(np.float32)
+    for bits in widths if few else widths[1:3]:
+        for K, M1, alpha in ((1 << bits, 2.0, 1.0), ((1 << bits) - 1 if bits > 1 else 2, 0.01, 0.75)):
+            nested = 2 if few else 8
+            # (no overflow in the sum: a step of the coarser quantizer is 75 scales)
+            most = np.float32(2e35 if M1 < 1.0 else 1.5e37 if few else 4e36)
+            factor = np.repeat(np.minimum(np.resize(FACTORS, nb), most), BUCKET)[:n]
+            side = common * factor
+            g_dev = torch.from_numpy(near * factor).cuda()
+            specs = [WorkerSpec(DQSG, bits, 0, 0, 0.0, 1.0, 11, dither),
+                     *[WorkerSpec(NDQSG, bits, 0, K, M1, alpha, 12 + w, dither) for w in range(nested)]]
+            gmsgs, sent = [], []
+            for w, sp in enumerate(specs):
+                pk, sc = gpu_encode(dq, torch, g_dev, sp, w, step, BUCKET)
+                gmsgs.append(gpu_msg(dq, pk, sc, sp, w, BUCKET))
+                sent.append((words_np(pk), sc.cpu().numpy()))
+            outs = {"one": dq.dqsg_decode_aggregate(gmsgs[:1], n, step)[:n].cpu().numpy(),
+                    "dqsg": dq.dqsg_decode_aggregate([gmsgs[0]] * 2, n, step)[:n].cpu().numpy(),
+                    "vector": dq.ndqsg_decode_aggregate(gmsgs, n, step, torch.from_numpy(side).cuda())[:n].cpu().numpy(),
+                    "first": dq.ndqsg_decode_aggregate_side_first(gmsgs, n, step)[:n].cpu().numpy(),
+                    "running": dq.ndqsg_decode_aggregate_running(gmsgs, n, step)[:n].cpu().numpy()}
+            span = len(FACTORS)
+            for b0 in sorted({0, max(0, nb - span)}):
+                lo, hi = b0 * BUCKET, min(n, (b0 + span) * BUCKET)
+                omsgs = [oracle_msg(oracle, pk[lo * bits // 32:-(-hi * bits // 32)], sc[b0:b0 + span], sp, w, BUCKET)
+                         for w, ((pk, sc), sp) in enumerate(zip(sent, specs))]
+                y0 = oracle.decode_aggregate(omsgs[:1], hi - lo, step, i0=lo)
+                want = {"one": y0, "dqsg": oracle.decode_aggregate([omsgs[0]] * 2, hi - lo, step, i0=lo),
+                        "vector": oracle.decode_aggregate(omsgs, hi - lo, step, side_info=side[lo:hi], i0=lo),
+                        "first": oracle.decode_aggregate(omsgs, hi - lo, step, side_info=y0, i0=lo),
+                        "running": oracle.decode_aggregate(omsgs, hi - lo, step, running=True, i0=lo)}
+                for k, ref in want.items():
+                    assert np.array_equal(outs[k][lo:hi].view(np.uint32), ref.view(np.uint32)), (k, bits, K, lo)
