@@ -100,10 +100,12 @@ inline void set_bucket_division(DecodeHead& a)
 constexpr int kDecThreads = 128;
 // Which variants a kernel holds.  With all forty routines in one kernel the compiler's register allocation and its
 // choice between uniform and per-lane loads of a worker's constants cost every routine 5 to 12 %, so the usual variants
-// (DQSG, and NDQSG with a power-of-two K and no shrinkage, up to 4 bits) have kernels of their own, and for long
-// gradients every pair of one DQSG and one NDQSG width has (W = 16, 3 bits, n = 124.4 M: 1973 us with all, 1933 with the
-// usual ones, 1782 with the pair; W = 8, 2 bits, n = 25.6 M: 217, 210 and 197).
-constexpr int kSetAll = 0, kSetUsual = 1;
+// (DQSG, and NDQSG with a power-of-two K and no shrinkage, up to 4 bits) and the odd ones (the same with another K, the
+// paper's K = 3 among them) have kernels of their own, and for long gradients every pair of one DQSG and one NDQSG width has
+// (W = 16, 3 bits, n = 124.4 M: 1973 us with all, 1933 with the usual ones, 1782 with the pair; W = 8, 2 bits, n = 25.6 M:
+// 217, 210 and 197; running mean, W = 8, K = 3, n = 266,010 5.65 us with all, 5.26 with the odd ones; 2.4 M 22.3 and 20.9;
+// but 11.7 M, in groups of 32, 93.3 and 95.1).
+constexpr int kSetAll = 0, kSetUsual = 1, kSetOdd = 2;
 constexpr int pair_set(int dqsg_bits, int ndqsg_bits) { return 16 * dqsg_bits + ndqsg_bits; }
 
 // Resident CTAs per SM that the register budget is set for.  E = 32 takes 80 registers (24 warps per SM) in the pair
@@ -491,6 +493,11 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
 }
 
 inline bool is_usual_variant(uint32_t variant) { return (variant >> 3) <= kDecNdqsgPow2 && (variant & 7u) < 4u; }
+// (one bit has no K but two)
+inline bool is_odd_variant(uint32_t variant)
+{
+    return ((variant >> 3) == kDecDqsg || (variant >> 3) == kDecNdqsgAnyK) && (variant & 7u) < 4u;
+}
 
 // All W workers, run by run; dispatch on (kind, bits) with one jump per run.
 template <int DITH, int SIDE, int E, int SET, typename Args>
@@ -515,6 +522,12 @@ __device__ __forceinline__ void decode_workers(const Args& args, DecLane& ln, f3
                 DQ_DEC_KIND(kDecNdqsgPow2Shrink)
                 DQ_DEC_KIND(kDecNdqsgAnyK)
                 DQ_DEC_KIND(kDecNdqsgAnyKShrink)
+                default: break;
+            }
+        } else if constexpr (SET == kSetOdd) {
+            switch (args.w[w].variant) {
+                DQ_DEC_LOW(kDecDqsg)
+                DQ_DEC_CASE(kDecNdqsgAnyK, 2) DQ_DEC_CASE(kDecNdqsgAnyK, 3) DQ_DEC_CASE(kDecNdqsgAnyK, 4)
                 default: break;
             }
         } else if constexpr (SET == kSetUsual) {
@@ -565,7 +578,7 @@ __device__ __forceinline__ void decode_group(const Args& args, float4 (*slots)[k
     // Lanes past the end either leave (there is no barrier below), or repeat the last group and store nothing: then the
     // control flow stays uniform for the compiler and a worker's constants take the uniform data path, which gains 1 to 2 %
     // with long chains per lane and loses as much in the shorter ones.
-    constexpr bool kClamp = E == 32 || (E == 16 && SET <= kSetUsual);
+    constexpr bool kClamp = E == 32 || (E == 16 && SET <= kSetOdd);
     const bool live = local < args.num_groups;
     if constexpr (!kClamp) {
         if (!live) return;

@@ -43,6 +43,8 @@ cudaError_t launch_groups_of(const DecodeArgs& a, cudaStream_t st)
 {
     const uint32_t grid = (uint32_t)((a.num_groups + kDecThreads - 1u) / kDecThreads);
     bool usual = true, one_pair = true;
+    bool odd = true;
+    for (uint32_t w = 0; w < a.W; ++w) odd = odd && is_odd_variant(a.w[w].variant);
     int width[2] = {0, 0};              // code widths of the DQSG and of the NDQSG messages
     for (uint32_t w = 0; w < a.W; ++w) {
         const uint32_t v = a.w[w].variant;
@@ -71,8 +73,12 @@ cudaError_t launch_groups_of(const DecodeArgs& a, cudaStream_t st)
             static_cast<DecodeHead&>(few) = a;
             std::memcpy(few.w, a.w, a.W * sizeof(DecWorker));
             return usual ? launch_set<E, kSetUsual, kDecFewWorkers>(few, grid, st)
+                   : odd ? launch_set<E, kSetOdd, kDecFewWorkers>(few, grid, st)
                          : launch_set<E, kSetAll, kDecFewWorkers>(few, grid, st);
         }
+    }
+    if constexpr (E < 32) {
+        if (!usual && odd) return launch_set<E, kSetOdd>(a, grid, st);
     }
     return usual ? launch_set<E, kSetUsual>(a, grid, st) : launch_set<E, kSetAll>(a, grid, st);
 }
