@@ -636,11 +636,6 @@ __device__ __forceinline__ void decode_group(const Args& args, float4 (*slots)[k
 #pragma unroll
     for (int e = 0; e < E / 2; ++e) acc[e] = 0ull;
     decode_workers<DITH, SIDE, E, SET>(args, ln, acc);
-    // The next kernel may become resident when every CTA of this one is about to store.  Let in right after the wait, its
-    // CTAs would take the slots that this kernel leaves free, and what does not fit would be placed when these end,
-    // several CTAs on one SM and none on others, as soon as a grid takes more than half the slots (W = 8: n = 1.3 M 20.3 us
-    // per call, now 14.7; 1.6 M 20.6 and 16.9; 266,610 6.8 and 6.5; from a few waves on there is no difference).
-    grid_dependency_launch_next();
     // the mean (of one message: the message itself)
     if (args.W > 1u) {
         const f32x2 nz = args.neg_zero;
@@ -675,6 +670,12 @@ __device__ __forceinline__ void decode_group(const Args& args, float4 (*slots)[k
         }
     }
     if (args.status != nullptr && ln.kappa_bits_max >= 0x7F800000u) atomicOr(args.status, 0x1u);
+    // The next kernel may become resident when every CTA of this one has stored.  Let in right after the wait, its CTAs would
+    // take the slots that this kernel leaves free, and what does not fit would be placed when these end, several CTAs on one
+    // SM and none on others, as soon as a grid takes more than half the slots (W = 8: n = 1.3 M 20.3 us per call, now 14;
+    // from a few waves on there is no difference).  Let in before the stores, the last CTAs to store still make the placement
+    // uneven (W = 8, n = 266,610: running mean 6.1 us per call, now 5.3; vector 6.3 and 5.6; side from message 0 6.7 and 5.9).
+    grid_dependency_launch_next();
 }
 
 template <int DITH, int SIDE, int E, int SET, int MAXW>
