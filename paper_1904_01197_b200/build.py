@@ -36,6 +36,7 @@ UNITS += [(f"enc_m{m}_d{d}", "dq_encode_inst.cu", [f"-DDQ_INST_MODE={m}", f"-DDQ
           for m in (0, 1, 2, 3) for d in (32, 16)]
 UNITS += [(f"dec_d{d}_r{r}_e{e}", "dq_decode_inst.cu", [f"-DDQ_INST_DITH={d}", f"-DDQ_INST_RUN={r}", f"-DDQ_INST_E={e}"])
           for d, r in ((32, 0), (32, 1), (32, 2), (16, 0), (16, 1), (16, 2), (0, 0)) for e in (32, 16, 8)]
+UNITS += [(f"dec_one_d{d}", "dq_decode_one_inst.cu", [f"-DDQ_INST_DITH={d}"]) for d in (32, 16)]
 
 
 def nvcc_path() -> str:

@@ -81,4 +81,8 @@ DQ_DECLARE_DECODE(32, 2) DQ_DECLARE_DECODE(16, 2)
 DQ_DECLARE_DECODE(0, 0)
 #undef DQ_DECLARE_DECODE
 
+// Decoder of one DQSG message; R = groups of 8 elements per lane, 1 or 4.
+cudaError_t launch_decode_one_d32(const DecodeArgsOf<1>& a, int R, cudaStream_t st);
+cudaError_t launch_decode_one_d16(const DecodeArgsOf<1>& a, int R, cudaStream_t st);
+
 }  // namespace dq
