@@ -6,7 +6,7 @@
 // contiguous, every address but the first is a constant further on, and what a lane costs once is spread over 8 R elements;
 // it requests the codes and scales of all of them, and the generator of the first group hides their latency.
 //
-// What bounds it: instruction issue (18 instructions per element, two thirds of them the generator) and the multiplier pipe.
+// What bounds it: the multiplier pipe (82 %) and instruction issue (21 instructions per element, nine of them the generator).
 // Against the general decoder with 16 elements per lane (28 instructions per element, issue slots 67 % used): n = 25.6 M,
 // 3 bits 30.6 -> 25.2 us; 16-bit stream 28.4 -> 19.5; n = 4 M 6.2 -> 5.1; n = 266,037 1.71 -> 1.30.
 #pragma once

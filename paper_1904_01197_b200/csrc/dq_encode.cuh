@@ -1,5 +1,6 @@
 // Tile encoder: the encode step (see dq_encode_direct.cuh, which serves every other call) for long gradients that are
-// encoded back to back with overlapping launches, in power-of-two buckets up to 8192; and what both encoders share.
+// encoded back to back with overlapping launches, in the bucket sizes where it is ahead (see the dispatch; it can take every
+// power of two up to 8192); and what both encoders share.
 //
 // Work decomposition: a "row" is 32 consecutive elements = one 128-byte line of the gradient and exactly
 // `bits` 32-bit words of the bit stream.  One lane quantizes and packs a whole row, so no lane ever shares a
