@@ -413,8 +413,10 @@ float set_decode_form(dq::DecWorker& d, uint32_t kind, int bits, int dith)
         d.A *= u;
     }
     if (shift == 0) return std::numeric_limits<float>::infinity();
-    // kappa / s / u and alpha kappa / M1 / u below 2^127, alpha M1 u / kappa normal
+    // kappa / s / u and alpha kappa / M1 / u below 2^127, alpha M1 u / kappa normal, and alpha M1 u too: a subnormal number
+    // has lost bits
     if (kind == dq::kDecDqsg) return 0x1p119f;
+    if (d.A < 0x1p-126f) return 0.0f;
     const float most = std::fmin(d.M1 / d.alpha * 0x1p-6f, d.A);
     return most >= 1.0f ? 0x1p120f : most * 0x1p120f;
 }

@@ -58,3 +58,20 @@ def test_forms_over_the_range_of_scales(dq, oracle, n, few, dither, widths):
                         "running": oracle.decode_aggregate(omsgs, hi - lo, step, running=True, i0=lo)}
                 for k, ref in want.items():
                     assert np.array_equal(outs[k][lo:hi].view(np.uint32), ref.view(np.uint32)), (k, bits, K, lo)
+
+
+@pytest.mark.parametrize("exponent", [-119, -121, -125, -127, -140])
+@pytest.mark.parametrize("dither,bits", [(32, 3), (32, 4), (16, 1), (16, 2), (16, 7)])
+def test_a_fine_resolution_near_the_end_of_the_fp32_range(dq, oracle, dither, bits, exponent):
+    """alpha M1 close to or among the subnormal numbers: scaled by less than one it would lose bits, and side information a
+    few thousand steps long would be resolved to another coset."""
+    n, step, M1 = 3 * BUCKET + 5, 4, float(np.ldexp(1.37, exponent))
+    rng = np.random.default_rng(bits - exponent)
+    grad = torch.from_numpy(np.float32(2.0 ** -98) * rng.standard_normal(n).astype(np.float32)).cuda()
+    side = np.ldexp(rng.standard_normal(n), -96 - exponent + 12).astype(np.float32)
+    for K, alpha in ((1 << bits, 1.0), (1 << bits, 0.75), ((1 << bits) - 1 if bits > 1 else 2, 1.0)):
+        sp = WorkerSpec(NDQSG, bits, 0, K, M1, alpha, 21, dither)
+        pk, sc = gpu_encode(dq, torch, grad, sp, 2, step, BUCKET)
+        got = dq.ndqsg_decode_aggregate([gpu_msg(dq, pk, sc, sp, 2, BUCKET)], n, step, torch.from_numpy(side).cuda())[:n].cpu().numpy()
+        ref = oracle.decode_aggregate([oracle_msg(oracle, words_np(pk), sc.cpu().numpy(), sp, 2, BUCKET)], n, step, side_info=side)
+        assert np.isfinite(ref).all() and np.array_equal(got.view(np.uint32), ref.view(np.uint32)), (K, alpha)
