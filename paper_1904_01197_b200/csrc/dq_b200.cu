@@ -396,9 +396,11 @@ int decode_group_size(uint64_t n, uint32_t W, bool reads_side, bool usual, int s
 
 // The constants of a worker that depend on the form its routine works in (see DecForm).  Returns the largest scale that the
 // form takes.
-float set_decode_form(dq::DecWorker& d, uint32_t kind, int bits, int dith)
+float set_decode_form(dq::DecWorker& d, int dith, int side, int group)
 {
-    const int form = dq::dec_form(kind, bits, dith), shift = dq::dec_shift(kind, bits, dith);
+    const uint32_t kind = d.variant >> 3;
+    const int bits = (int)(d.variant & 7u) + 1;
+    const int form = dq::dec_form(kind, bits, dith, side, group), shift = dq::dec_shift(kind, bits, dith, side, group);
     const float u = 1.0f / (float)(1u << shift);
     if (form == dq::kFormJoined && dith == 16)
         d.offset = twice(((float)((1u << bits) - 1u) - d.s + dq::kD16Offset) * u);          // J = (2^bits - 1 - k) 2^16 + h
@@ -430,7 +432,6 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     static thread_local dq::DecodeArgs a;    // ~13 KB: keep it off the stack; the first W entries of a.w are filled
     std::memset(static_cast<dq::DecodeHead*>(&a), 0, sizeof(dq::DecodeHead));
     bool any_nested = false;
-    float kappa_most = std::numeric_limits<float>::infinity();
     for (uint32_t w = 0; w < W; ++w) {
         const dq_msg& m = msgs[w];
         uint32_t L = 0;
@@ -468,8 +469,6 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
             }
         }
         d.variant = kind * 8u + m.p.bits - 1u;
-        kappa_most = std::fmin(kappa_most, set_decode_form(d, kind, (int)m.p.bits,
-                                                           half_dithered ? 0 : m.p.dither_bits == 16u ? 16 : 32));
     }
     // runs of equal variants (one routine per run, see decode_workers)
     for (uint32_t w = W; w-- > 0u;)
@@ -500,8 +499,6 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     a.out_align32 = (reinterpret_cast<uintptr_t>(out_avg) & 31u) == 0u ? 1u : 0u;
     a.half_bias_bits = 0x4A800000u;
     a.low22 = 0x003FFFFFu;
-    // (no limit: above the pattern of any NaN)
-    a.kappa_limit = std::isinf(kappa_most) ? 0xFFFFFFFFu : bits_of(kappa_most);
     a.neg_zero = twice(-0.0f);
     a.magic = twice(dq::kMagic);
     a.neg_magic = twice(-dq::kMagic);
@@ -510,30 +507,34 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
     const bool d16 = (msgs[0].p.dither_bits == 16u);
-    if (W == 1u && !half_dithered) {
-        // (a single nested message needs a side information vector and goes the general way)
-        if (msgs[0].kind == DQ_KIND_DQSG) {
-            static thread_local dq::DecodeArgsOf<1> one;
-            static_cast<dq::DecodeHead&>(one) = a;
-            one.w[0] = a.w[0];
-            one.num_groups = (n + 7u) / 8u;
-            // up to one wave of one-group lanes the shortest chain wins (n = 266,037 1.25 us with one group, 1.86 with four;
-            // 0.9 M 2.03 and 2.34; 1.2 M 2.40 and 2.34; 2.4 M 3.66 and 3.26)
-            const int R = n <= (uint64_t)sms * 1024u * 8u ? 1 : 4;
-            const cudaError_t e = d16 ? dq::launch_decode_one_d16(one, R, st) : dq::launch_decode_one_d32(one, R, st);
-            if (e != cudaSuccess) return DQ_ERR_CUDA;
-            g_launches.fetch_add(1);
-            return DQ_OK;
-        }
-    }
+    // (a single nested message needs a side information vector and goes the general way)
+    const bool one_message = W == 1u && !half_dithered && !any_nested;
     bool usual = true;
     for (uint32_t w = 0; w < W; ++w) usual = usual && dq::is_usual_variant(a.w[w].variant);
-    const int E = decode_group_size(n, W, reads_side, usual, sms);
+    const int E = one_message ? 8 : decode_group_size(n, W, reads_side, usual, sms);
     a.num_groups = (n + (uint32_t)E - 1u) / (uint32_t)E;
+    const int side = from_first ? dq::kSideFirst : (running && any_nested) ? dq::kSideRunning : dq::kSideGiven;
+    float kappa_most = std::numeric_limits<float>::infinity();
+    for (uint32_t w = 0; w < W; ++w)
+        kappa_most = std::fmin(kappa_most, set_decode_form(a.w[w], half_dithered ? 0 : d16 ? 16 : 32, side, E));
+    // (no limit: above the pattern of any NaN)
+    a.kappa_limit = std::isinf(kappa_most) ? 0xFFFFFFFFu : bits_of(kappa_most);
+    if (one_message) {
+        static thread_local dq::DecodeArgsOf<1> one;
+        static_cast<dq::DecodeHead&>(one) = a;
+        one.w[0] = a.w[0];
+        // up to one wave of one-group lanes the shortest chain wins (n = 266,037 1.25 us with one group, 1.86 with four;
+        // 0.9 M 2.03 and 2.34; 1.2 M 2.40 and 2.34; 2.4 M 3.66 and 3.26)
+        const int R = n <= (uint64_t)sms * 1024u * 8u ? 1 : 4;
+        const cudaError_t e = d16 ? dq::launch_decode_one_d16(one, R, st) : dq::launch_decode_one_d32(one, R, st);
+        if (e != cudaSuccess) return DQ_ERR_CUDA;
+        g_launches.fetch_add(1);
+        return DQ_OK;
+    }
     cudaError_t le;
     if (half_dithered) le = dq::launch_decode_d0_r0(a, E, st);
-    else if (running && any_nested) le = d16 ? dq::launch_decode_d16_r1(a, E, st) : dq::launch_decode_d32_r1(a, E, st);
-    else if (from_first) le = d16 ? dq::launch_decode_d16_r2(a, E, st) : dq::launch_decode_d32_r2(a, E, st);
+    else if (side == dq::kSideRunning) le = d16 ? dq::launch_decode_d16_r1(a, E, st) : dq::launch_decode_d32_r1(a, E, st);
+    else if (side == dq::kSideFirst) le = d16 ? dq::launch_decode_d16_r2(a, E, st) : dq::launch_decode_d32_r2(a, E, st);
     else le = d16 ? dq::launch_decode_d16_r0(a, E, st) : dq::launch_decode_d32_r0(a, E, st);
     if (le != cudaSuccess) return DQ_ERR_CUDA;
     g_launches.fetch_add(1);

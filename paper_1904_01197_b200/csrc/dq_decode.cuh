@@ -122,7 +122,10 @@ constexpr int dec_ctas_per_sm(int E, int set) { return E == 32 ? (set == kSetAll
 //   joined:  code and random bits side by side in one mantissa, one multiply-add for both.  The join is an integer below
 //            2^24, read as a (subnormal or small) float; with the 16-bit stream always possible (up to seven bits), with
 //            the 32-bit stream where 22 + bits <= 24 and (NDQSG) m - delta is representable, so that q - delta follows
-//            from it by another multiply-add.
+//            from it by another multiply-add.  Not in groups of 32 for DQSG with the 32-bit stream, where the biased form is
+//            ahead in its own routines (W = 8, 2 bits, n = 25.6 M: joined 166.5 us, biased 158.6; in groups of 8, 266,610
+//            4.45 and 4.56) and in the others of their kernel (side information from message 0, six bits, 11.7 M: 99.6 and
+//            92.1), nor for one bit against the running mean (W = 2, DQSG 2 bits, 25.6 M: 52.5 and 51.1).
 //   tiny:    NDQSG up to four bits: the code in bits 23.. downwards of a float is an exact multiple of 2^-149, so that
 //            m - delta and q - delta are one multiply-add each and no bias has to be taken off.
 // The values of the last two forms are smaller than the real ones by 2^shift, because a multiply-add cannot scale by more than
@@ -130,17 +133,18 @@ constexpr int dec_ctas_per_sm(int E, int set) { return E == 32 ? (set == kSetAll
 // above any gradient) are decoded again by decode_group_plain.
 enum DecForm : int { kFormBiased = 0, kFormJoined = 1, kFormTiny = 2 };
 
-__host__ __device__ constexpr int dec_form(uint32_t kind, int bits, int dith)
+__host__ __device__ constexpr int dec_form(uint32_t kind, int bits, int dith, int side, int group)
 {
     if (dith == 16) return bits <= 7 ? kFormJoined : kFormBiased;
-    if (dith == 32 && kind == kDecDqsg) return bits <= 2 ? kFormJoined : kFormBiased;
-    if (dith == 32) return bits == 1 ? kFormJoined : bits <= 4 ? kFormTiny : kFormBiased;
+    if (dith == 32 && kind == kDecDqsg) return bits <= 2 && group < 32 ? kFormJoined : kFormBiased;
+    if (dith == 32 && bits == 1) return side == kSideRunning && group == 32 ? kFormBiased : kFormJoined;
+    if (dith == 32) return bits <= 4 ? kFormTiny : kFormBiased;
     return kFormBiased;
 }
 
-__host__ __device__ constexpr int dec_shift(uint32_t kind, int bits, int dith)
+__host__ __device__ constexpr int dec_shift(uint32_t kind, int bits, int dith, int side, int group)
 {
-    const int form = dec_form(kind, bits, dith);
+    const int form = dec_form(kind, bits, dith, side, group);
     return form == kFormTiny ? bits - 2 : (form == kFormJoined && dith == 16) ? 6 : 0;
 }
 
@@ -367,7 +371,7 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
     constexpr bool RUN = SIDE == kSideRunning;
     constexpr bool ANY_K = KIND == kDecNdqsgAnyK || KIND == kDecNdqsgAnyKShrink;
     constexpr bool SHRINK = KIND == kDecNdqsgPow2Shrink || KIND == kDecNdqsgAnyKShrink;
-    constexpr int FORM = dec_form(KIND, BITS, DITH), SHIFT = dec_shift(KIND, BITS, DITH);
+    constexpr int FORM = dec_form(KIND, BITS, DITH, SIDE, E), SHIFT = dec_shift(KIND, BITS, DITH, SIDE, E);
     constexpr int EPB = (DITH == 16) ? 8 : 4;       // elements per Philox block
     constexpr int N = E / EPB;                      // blocks of the group
     constexpr int P = N < 2 ? N : 2;                // blocks in flight
