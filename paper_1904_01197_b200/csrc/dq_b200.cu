@@ -388,9 +388,10 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 int decode_group_size(uint64_t n, uint32_t W, bool reads_side, bool usual, int sms)
 {
     const uint64_t lanes = (uint64_t)sms * dq::kDecThreads;
-    if (n <= 8u * lanes * dq::dec_ctas_per_sm(8, dq::kSetUsual)) return 8;
-    if (!usual && W >= 8u && n > 16u * lanes * dq::dec_ctas_per_sm(16, dq::kSetAll)) return 32;
-    if (W <= (reads_side ? 2u : 1u) || 2u * n < 5u * 32u * lanes * dq::dec_ctas_per_sm(32, dq::kSetAll)) return 16;
+    const uint64_t wave8 = 8u * lanes * 8u, wave16 = 16u * lanes * 8u, wave32 = 32u * lanes * 5u;
+    if (n <= wave8) return 8;
+    if (!usual && W >= 8u && n > wave16) return 32;
+    if (W <= (reads_side ? 2u : 1u) || 2u * n < 5u * wave32) return 16;
     return 32;
 }
 
@@ -532,10 +533,10 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
         return DQ_OK;
     }
     cudaError_t le;
-    if (half_dithered) le = dq::launch_decode_d0_r0(a, E, st);
-    else if (side == dq::kSideRunning) le = d16 ? dq::launch_decode_d16_r1(a, E, st) : dq::launch_decode_d32_r1(a, E, st);
-    else if (side == dq::kSideFirst) le = d16 ? dq::launch_decode_d16_r2(a, E, st) : dq::launch_decode_d32_r2(a, E, st);
-    else le = d16 ? dq::launch_decode_d16_r0(a, E, st) : dq::launch_decode_d32_r0(a, E, st);
+    if (half_dithered) le = dq::launch_decode_d0_r0(a, E, sms, st);
+    else if (side == dq::kSideRunning) le = d16 ? dq::launch_decode_d16_r1(a, E, sms, st) : dq::launch_decode_d32_r1(a, E, sms, st);
+    else if (side == dq::kSideFirst) le = d16 ? dq::launch_decode_d16_r2(a, E, sms, st) : dq::launch_decode_d32_r2(a, E, sms, st);
+    else le = d16 ? dq::launch_decode_d16_r0(a, E, sms, st) : dq::launch_decode_d32_r0(a, E, sms, st);
     if (le != cudaSuccess) return DQ_ERR_CUDA;
     g_launches.fetch_add(1);
     return DQ_OK;

@@ -105,16 +105,24 @@ constexpr int kDecThreads = 128;
 // (W = 16, 3 bits, n = 124.4 M: 1973 us with all, 1933 with the usual ones, 1782 with the pair; W = 8, 2 bits, n = 25.6 M:
 // 217, 210 and 197; running mean, W = 8, K = 3, n = 266,010 5.65 us with all, 5.26 with the odd ones; 2.4 M 22.3 and 20.9;
 // but 11.7 M, in groups of 32, 93.3 and 95.1).
-constexpr int kSetAll = 0, kSetUsual = 1, kSetOdd = 2;
+constexpr int kSetAll = 0, kSetUsual = 1, kSetOdd = 2, kSetAllFull = 3;      // (kSetAllFull: see dec_ctas_per_sm)
 constexpr int pair_set(int dqsg_bits, int ndqsg_bits) { return 16 * dqsg_bits + ndqsg_bits; }
 
 // Resident CTAs per SM that the register budget is set for.  E = 32 takes 80 registers (24 warps per SM) in the pair
 // kernels: what a worker costs per lane (scale, gain, constants, loop: about 65 instructions) is spread over the most
 // elements.  96 registers are 3 % faster for a given side information vector but 2 to 8 % slower otherwise (the compiler
 // then loads a worker's constants lane by lane), 128 registers 7 % slower; the kernel with all routines wants 96.
-// E = 16 and 8 take 64 registers (32 warps), but for 72 where all routines in groups of 8 would not fit 64 (W = 8,
-// n = 266,010: 5.65 us with a spill, 5.45 without).
-constexpr int dec_ctas_per_sm(int E, int set) { return E == 32 ? (set == kSetAll ? 5 : 6) : (E == 8 && set == kSetAll) ? 7 : 8; }
+// E = 16 and 8 take 64 registers (32 warps), but for 72 (28 warps) where all routines in one kernel spill at 64 and are faster
+// without (E = 16, 32-bit stream: running mean, W = 8, 8 and 3 bits, n = 1.7 M 18.0 us with 64, 17.4 with 72; E = 8, 16-bit
+// stream, W = 16, up to 1 M: 64 is 3 to 6 % slower; but E = 8, 32-bit stream, DQSG and a vector: W = 4, 5 bits, n = 1.2 M 7.1 us
+// with 64, 8.3 with 72, W = 16, 128,073 8.7 and 11.0).  A grid that is one wave of eight CTAs per SM and would be two of seven
+// takes the same routines at 64 (kSetAllFull: W = 2, n = 1.2 M, 16-bit stream and a vector 4.4 us, with 72 registers 5.1).
+constexpr int dec_ctas_per_sm(int dith, int side, int E, int set)
+{
+    if (E == 32) return set == kSetAll ? 5 : 6;
+    if (set != kSetAll || dith == 0) return 8;
+    return (E == 16 ? dith == 32 : dith == 16 || side != kSideGiven) ? 7 : 8;
+}
 
 // How a routine forms k - s - delta (DQSG) and m - delta, q - delta (NDQSG) from the code and the random bits.  All forms
 // round the same real numbers once, so they give the same bits; they differ in the number of packed instructions.
@@ -519,7 +527,7 @@ __device__ __forceinline__ void decode_workers(const Args& args, DecLane& ln, f3
 #pragma unroll 1
     for (uint32_t w = 0; w < args.W;) {
         const uint32_t w_end = args.w[w].group_end;
-        if constexpr (SET == kSetAll) {
+        if constexpr (SET == kSetAll || SET == kSetAllFull) {
             switch (args.w[w].variant) {
                 DQ_DEC_KIND(kDecDqsg)
                 DQ_DEC_KIND(kDecNdqsgPow2)
@@ -683,7 +691,7 @@ __device__ __forceinline__ void decode_group(const Args& args, float4 (*slots)[k
 }
 
 template <int DITH, int SIDE, int E, int SET, int MAXW>
-__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(E, SET))
+__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(DITH, SIDE, E, SET))
 decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
 {
     __shared__ __align__(16) float4 slots[kDecSlots<DITH, E>][kDecThreads];

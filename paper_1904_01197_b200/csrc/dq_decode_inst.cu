@@ -23,6 +23,18 @@ cudaError_t launch_set(const DecodeArgsOf<MAXW>& a, uint32_t grid, cudaStream_t 
                              st, 1u, a);
 }
 
+// All routines.  One wave of CTAs must stay one: where the kernel's registers allow seven CTAs per SM and the grid is a wave of
+// eight, it takes the one that is held to eight.
+template <int E, int MAXW>
+cudaError_t launch_all(const DecodeArgsOf<MAXW>& a, uint32_t grid, int sms, cudaStream_t st)
+{
+    constexpr uint32_t fits = dec_ctas_per_sm(DQ_INST_DITH, DQ_INST_RUN, E, kSetAll);
+    if constexpr (E < 32 && fits < 8u) {
+        if (grid > fits * (uint32_t)sms && grid <= 8u * (uint32_t)sms) return launch_set<E, kSetAllFull>(a, grid, st);
+    }
+    return launch_set<E, kSetAll>(a, grid, st);
+}
+
 template <int E, int A>
 cudaError_t launch_pair(int b, const DecodeArgs& a, uint32_t grid, cudaStream_t st)
 {
@@ -39,7 +51,7 @@ cudaError_t launch_pair(int b, const DecodeArgs& a, uint32_t grid, cudaStream_t 
 }
 
 template <int E>
-cudaError_t launch_groups_of(const DecodeArgs& a, cudaStream_t st)
+cudaError_t launch_groups_of(const DecodeArgs& a, int sms, cudaStream_t st)
 {
     const uint32_t grid = (uint32_t)((a.num_groups + kDecThreads - 1u) / kDecThreads);
     bool usual = true, one_pair = true;
@@ -74,20 +86,20 @@ cudaError_t launch_groups_of(const DecodeArgs& a, cudaStream_t st)
             std::memcpy(few.w, a.w, a.W * sizeof(DecWorker));
             return usual ? launch_set<E, kSetUsual, kDecFewWorkers>(few, grid, st)
                    : odd ? launch_set<E, kSetOdd, kDecFewWorkers>(few, grid, st)
-                         : launch_set<E, kSetAll, kDecFewWorkers>(few, grid, st);
+                         : launch_all<E>(few, grid, sms, st);
         }
     }
     if constexpr (E < 32) {
         if (!usual && odd) return launch_set<E, kSetOdd>(a, grid, st);
     }
-    return usual ? launch_set<E, kSetUsual>(a, grid, st) : launch_set<E, kSetAll>(a, grid, st);
+    return usual ? launch_set<E, kSetUsual>(a, grid, st) : launch_all<E>(a, grid, sms, st);
 }
 
 }  // namespace
 
-cudaError_t DQ_NAME(DQ_INST_DITH, DQ_INST_RUN, DQ_INST_E)(const DecodeArgs& a, cudaStream_t st)
+cudaError_t DQ_NAME(DQ_INST_DITH, DQ_INST_RUN, DQ_INST_E)(const DecodeArgs& a, int sms, cudaStream_t st)
 {
-    return launch_groups_of<DQ_INST_E>(a, st);
+    return launch_groups_of<DQ_INST_E>(a, sms, st);
 }
 
 }  // namespace dq

@@ -65,16 +65,16 @@ DQ_DECLARE_DIRECT(0, 16) DQ_DECLARE_DIRECT(1, 16) DQ_DECLARE_DIRECT(2, 16) DQ_DE
 
 // Decoder: dith = 32, 16 or 0 (no dither at the receiver); run = DecSide (0 given vector or none, 1 running mean,
 // 2 reconstruction of message 0).
-// group_size: elements per lane, 32, 16 or 8; the grid follows from a.num_groups.
+// group_size: elements per lane, 32, 16 or 8; the grid follows from a.num_groups.  sms: the device's SMs.
 #define DQ_DECLARE_DECODE(DITH, RUN)                                                                               \
-    cudaError_t launch_decode_d##DITH##_r##RUN##_e32(const DecodeArgs& a, cudaStream_t st);                        \
-    cudaError_t launch_decode_d##DITH##_r##RUN##_e16(const DecodeArgs& a, cudaStream_t st);                        \
-    cudaError_t launch_decode_d##DITH##_r##RUN##_e8(const DecodeArgs& a, cudaStream_t st);                         \
-    inline cudaError_t launch_decode_d##DITH##_r##RUN(const DecodeArgs& a, int group_size, cudaStream_t st)        \
+    cudaError_t launch_decode_d##DITH##_r##RUN##_e32(const DecodeArgs& a, int sms, cudaStream_t st);               \
+    cudaError_t launch_decode_d##DITH##_r##RUN##_e16(const DecodeArgs& a, int sms, cudaStream_t st);               \
+    cudaError_t launch_decode_d##DITH##_r##RUN##_e8(const DecodeArgs& a, int sms, cudaStream_t st);                \
+    inline cudaError_t launch_decode_d##DITH##_r##RUN(const DecodeArgs& a, int group_size, int sms, cudaStream_t st) \
     {                                                                                                              \
-        return group_size == 32   ? launch_decode_d##DITH##_r##RUN##_e32(a, st)                                    \
-               : group_size == 16 ? launch_decode_d##DITH##_r##RUN##_e16(a, st)                                    \
-                                  : launch_decode_d##DITH##_r##RUN##_e8(a, st);                                    \
+        return group_size == 32   ? launch_decode_d##DITH##_r##RUN##_e32(a, sms, st)                               \
+               : group_size == 16 ? launch_decode_d##DITH##_r##RUN##_e16(a, sms, st)                               \
+                                  : launch_decode_d##DITH##_r##RUN##_e8(a, sms, st);                               \
     }
 DQ_DECLARE_DECODE(32, 0) DQ_DECLARE_DECODE(32, 1) DQ_DECLARE_DECODE(16, 0) DQ_DECLARE_DECODE(16, 1)
 DQ_DECLARE_DECODE(32, 2) DQ_DECLARE_DECODE(16, 2)
