@@ -524,9 +524,10 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
         static thread_local dq::DecodeArgsOf<1> one;
         static_cast<dq::DecodeHead&>(one) = a;
         one.w[0] = a.w[0];
-        // up to one wave of one-group lanes the shortest chain wins (n = 266,037 1.25 us with one group, 1.86 with four;
-        // 0.9 M 2.03 and 2.34; 1.2 M 2.40 and 2.34; 2.4 M 3.66 and 3.26)
-        const int R = n <= (uint64_t)sms * 1024u * 8u ? 1 : 4;
+        // up to one wave of one-group lanes the shortest chain wins, with the 32-bit stream to a quarter more (calls in a
+        // stream, 3 bits: n = 266,037 1.25 us with one group, 1.86 with four; 1.3 M 2.75 and 3.06; 1.5 M 3.02 and 3.12; 1.7 M
+        // 3.28 and 3.07; 2.4 M 3.99 and 3.69; 16-bit stream: 1.25 M 2.56 and 2.51; 1.7 M 3.06 and 2.60)
+        const int R = n <= (uint64_t)sms * 1024u * (d16 ? 8u : 10u) ? 1 : 4;
         const cudaError_t e = d16 ? dq::launch_decode_one_d16(one, R, st) : dq::launch_decode_one_d32(one, R, st);
         if (e != cudaSuccess) return DQ_ERR_CUDA;
         g_launches.fetch_add(1);
