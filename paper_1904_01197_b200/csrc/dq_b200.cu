@@ -384,13 +384,17 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 // warps to hide it (n = 25.6 M: W = 1 30.6 us with 16, 34.0 with 32; W = 2 with a vector 62.6 and 67.4, without 56.9 and
 // 51.9).  In the kernel with all routines, whose routines are longer, 32 pays from one wave of 16-element lanes on if there
 // are eight messages (`usual` false; six bits, W = 8: n = 2.4 M 24.1 us with 16, 24.2 with 32; 3 M 29.2 and 26.1; 4.2 M
-// 39.4 and 35.0; W = 32, 4.2 M 151 and 133; but W = 3 and a vector, 4.2 M 19.5 and 22.5).
+// 39.4 and 35.0; W = 32, 4.2 M 151 and 133; but W = 3 and a vector, 4.2 M 19.5 and 22.5).  From 48 messages on, whose parameters
+// do not stay in the caches between a warp's steps, 32 pays from 1.33 waves of 16-element lanes on (W = 64, 32-bit stream, one
+// nested bit: running mean 3.3 M 228 and 200 us, 4.2 M 296 and 234; first 243 and 203; two bits, 4.2 M: running 248 and 236, vector
+// 245 and 239; but W = 64, 2.5 M, two bits: 161 and 167).
 int decode_group_size(uint64_t n, uint32_t W, bool reads_side, bool usual, int sms)
 {
     const uint64_t lanes = (uint64_t)sms * dq::kDecThreads;
     const uint64_t wave8 = 8u * lanes * 8u, wave16 = 16u * lanes * 8u, wave32 = 32u * lanes * 5u;
     if (n <= wave8) return 8;
     if (!usual && W >= 8u && n > wave16) return 32;
+    if (W >= 48u && 3u * n > 4u * wave16) return 32;
     if (W <= (reads_side ? 2u : 1u) || 2u * n < 5u * wave32) return 16;
     return 32;
 }

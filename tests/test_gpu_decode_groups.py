@@ -54,3 +54,30 @@ def test_group_sizes_at_their_edges(dq, oracle, edge, bits, K, alpha, dither, bu
                 "running": oracle.decode_aggregate(omsgs, hi - lo, step, running=True, i0=lo)}
         for k, ref in want.items():
             assert np.array_equal(outs[k][lo:hi].view(np.uint32), ref.view(np.uint32)), (k, lo)
+
+
+@pytest.mark.parametrize("workers,over", [(47, 33), (48, 0), (48, 33)])
+@pytest.mark.parametrize("bits,dither", [(1, 32), (2, 16)])
+def test_many_messages_take_long_groups_sooner(dq, oracle, workers, over, bits, dither):
+    n, step, bucket = 4 * _edges()["16 last of all routines"] // 3 + over, 6, 992
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    side = 0.01 * torch.randn(n, device="cuda", generator=gen)
+    specs = [WorkerSpec(DQSG, bits, 0, 0, 0.0, 1.0, 11, dither),
+             *[WorkerSpec(NDQSG, bits, 0, 1 << bits, float(1 << bits), 1.0, 12 + w, dither) for w in range(workers - 1)]]
+    gmsgs, sent = [], []
+    for w, sp in enumerate(specs):
+        pk, sc = gpu_encode(dq, torch, side + 0.0005 * torch.randn(n, device="cuda", generator=gen), sp, w, step, bucket)
+        gmsgs.append(gpu_msg(dq, pk, sc, sp, w, bucket))
+        sent.append((pk, sc))
+    outs = {"first": dq.ndqsg_decode_aggregate_side_first(gmsgs, n, step)[:n].cpu().numpy(),
+            "running": dq.ndqsg_decode_aggregate_running(gmsgs, n, step)[:n].cpu().numpy()}
+    nb = -(-n // bucket)
+    for b0 in (0, nb - 3):
+        lo, hi = b0 * bucket, min(n, (b0 + 3) * bucket)
+        omsgs = [oracle_msg(oracle, words_np(pk[lo * bits // 32:-(-hi * bits // 32)]), sc[b0:b0 + 3].cpu().numpy(), sp, w, bucket)
+                 for w, ((pk, sc), sp) in enumerate(zip(sent, specs))]
+        y0 = oracle.decode_aggregate(omsgs[:1], hi - lo, step, i0=lo)
+        want = {"first": oracle.decode_aggregate(omsgs, hi - lo, step, side_info=y0, i0=lo),
+                "running": oracle.decode_aggregate(omsgs, hi - lo, step, running=True, i0=lo)}
+        for k, ref in want.items():
+            assert np.array_equal(outs[k][lo:hi].view(np.uint32), ref.view(np.uint32)), (k, lo)
