@@ -156,6 +156,15 @@ __host__ __device__ constexpr int dec_shift(uint32_t kind, int bits, int dith, i
     return form == kFormTiny ? bits - 2 : (form == kFormJoined && dith == 16) ? 6 : 0;
 }
 
+// Whether a kernel calls decode_group_plain.  Not where none of its routines is scaled: against a vector the call costs registers
+// there (the pair of 3 and 2 bits spills 52 bytes with it; W = 8, n = 25.6 M 0.4 % slower).  Against message 0 and the running
+// mean the compiler's allocation comes out better with the call, although it is never taken (the same pair 2 % faster).
+__host__ __device__ constexpr bool may_be_plain(int set, int dith, int side, int group)
+{
+    return dith != 0 && (side != kSideGiven || set <= kSetAllFull || dec_shift(kDecDqsg, set / 16, dith, side, group) != 0 ||
+                         dec_shift(kDecNdqsgPow2, set % 16, dith, side, group) != 0);
+}
+
 __host__ __device__ constexpr float pow2f(int e)
 {
     float v = 1.0f;
@@ -664,7 +673,7 @@ __device__ __forceinline__ void decode_group(const Args& args, float4 (*slots)[k
     }
     float* o = args.out + i0;
     if (kClamp && !live) return;
-    if (DITH != 0 && ln.kappa_bits_max > args.kappa_limit) {
+    if (may_be_plain(SET, DITH, SIDE, E) && ln.kappa_bits_max > args.kappa_limit) {
         decode_group_plain<DITH, SIDE, E>(args, ln.group, ln.bucket);
     } else if (whole) {
 #pragma unroll

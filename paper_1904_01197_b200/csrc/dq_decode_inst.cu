@@ -55,8 +55,6 @@ cudaError_t launch_groups_of(const DecodeArgs& a, int sms, cudaStream_t st)
 {
     const uint32_t grid = (uint32_t)((a.num_groups + kDecThreads - 1u) / kDecThreads);
     bool usual = true, one_pair = true;
-    bool odd = true;
-    for (uint32_t w = 0; w < a.W; ++w) odd = odd && is_odd_variant(a.w[w].variant);
     int width[2] = {0, 0};              // code widths of the DQSG and of the NDQSG messages
     for (uint32_t w = 0; w < a.W; ++w) {
         const uint32_t v = a.w[w].variant;
@@ -67,7 +65,7 @@ cudaError_t launch_groups_of(const DecodeArgs& a, int sms, cudaStream_t st)
         have = (int)(v & 7u) + 1;
     }
     if constexpr (E >= 16) {
-        // (not for one or two messages in groups of 16: W = 1, n = 25.6 M 31.8 us with the usual set, 33.9 with the pair)
+        // (not for one or two messages in groups of 16)
         if (usual && one_pair && (a.W > 2u || E == 32)) {
             if (width[0] == 0) width[0] = width[1];
             if (width[1] == 0) width[1] = width[0];
@@ -78,19 +76,23 @@ cudaError_t launch_groups_of(const DecodeArgs& a, int sms, cudaStream_t st)
                 default: return launch_pair<E, 4>(width[1], a, grid, st);
             }
         }
-    } else {
+    }
+    bool odd = DQ_INST_DITH != 0 && !usual;       // (the receiver without the dither takes DQSG messages only: usual or wide)
+    for (uint32_t w = 0; w < a.W; ++w) odd = odd && is_odd_variant(a.w[w].variant);
+    if constexpr (E == 8) {
         // short gradients: the launch itself counts
         if (a.W <= (uint32_t)kDecFewWorkers) {
             DecodeArgsOf<kDecFewWorkers> few;
             static_cast<DecodeHead&>(few) = a;
             std::memcpy(few.w, a.w, a.W * sizeof(DecWorker));
-            return usual ? launch_set<E, kSetUsual, kDecFewWorkers>(few, grid, st)
-                   : odd ? launch_set<E, kSetOdd, kDecFewWorkers>(few, grid, st)
-                         : launch_all<E>(few, grid, sms, st);
+            if constexpr (DQ_INST_DITH != 0) {
+                if (odd) return launch_set<E, kSetOdd, kDecFewWorkers>(few, grid, st);
+            }
+            return usual ? launch_set<E, kSetUsual, kDecFewWorkers>(few, grid, st) : launch_all<E>(few, grid, sms, st);
         }
     }
-    if constexpr (E < 32) {
-        if (!usual && odd) return launch_set<E, kSetOdd>(a, grid, st);
+    if constexpr (E < 32 && DQ_INST_DITH != 0) {
+        if (odd) return launch_set<E, kSetOdd>(a, grid, st);
     }
     return usual ? launch_set<E, kSetUsual>(a, grid, st) : launch_all<E>(a, grid, sms, st);
 }
