@@ -178,18 +178,18 @@ uint32_t bits_of(float v)
 
 dq::f32x2 twice(float v) { return ((dq::f32x2)bits_of(v) << 32) | bits_of(v); }
 
-cudaError_t launch_direct(int mode, uint32_t bits, bool dither16, int R, const dq::DirectArgs& a, uint32_t grid,
+cudaError_t launch_direct(int mode, uint32_t bits, bool dither16, int R, int kind, const dq::DirectArgs& a, uint32_t grid,
                           uint32_t threads, cudaStream_t st)
 {
     switch (mode * 2 + (dither16 ? 1 : 0)) {
-        case 0: return dq::launch_direct_m0_d32(bits, R, a, grid, threads, st);
-        case 1: return dq::launch_direct_m0_d16(bits, R, a, grid, threads, st);
-        case 2: return dq::launch_direct_m1_d32(bits, R, a, grid, threads, st);
-        case 3: return dq::launch_direct_m1_d16(bits, R, a, grid, threads, st);
-        case 4: return dq::launch_direct_m2_d32(bits, R, a, grid, threads, st);
-        case 5: return dq::launch_direct_m2_d16(bits, R, a, grid, threads, st);
-        case 6: return dq::launch_direct_m3_d32(bits, R, a, grid, threads, st);
-        default: return dq::launch_direct_m3_d16(bits, R, a, grid, threads, st);
+        case 0: return dq::launch_direct_m0_d32(bits, R, kind, a, grid, threads, st);
+        case 1: return dq::launch_direct_m0_d16(bits, R, kind, a, grid, threads, st);
+        case 2: return dq::launch_direct_m1_d32(bits, R, kind, a, grid, threads, st);
+        case 3: return dq::launch_direct_m1_d16(bits, R, kind, a, grid, threads, st);
+        case 4: return dq::launch_direct_m2_d32(bits, R, kind, a, grid, threads, st);
+        case 5: return dq::launch_direct_m2_d16(bits, R, kind, a, grid, threads, st);
+        case 6: return dq::launch_direct_m3_d32(bits, R, kind, a, grid, threads, st);
+        default: return dq::launch_direct_m3_d16(bits, R, kind, a, grid, threads, st);
     }
 }
 
@@ -248,7 +248,25 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     // (with early_read one cluster more: see the kernel)
     const uint64_t grid = ((dq_num_buckets(n, p.bucket) + shape.buckets - 1u) / shape.buckets + (a.early_read ? 1u : 0u)) *
                           shape.cluster;
-    return launch_direct(mode, p.bits, p.dither_bits == 16u, R, a, (uint32_t)grid, shape.threads, st);
+    // More resident CTAs instead of more dithers ahead (times of calls in a stream, ahead and dense):
+    //   - where they make one wave of two: n = 4.2 M, B = 4096, 2 bits, flagged 5.4 and 4.6 us; 3.7 M, B = 1504, K = 15 8.5 and
+    //     6.5; one-group lanes in CTAs of 656 to 768 threads, of which the ahead kernels run one to an SM: 1.2 M, B = 12288,
+    //     4 bits 5.1 and 3.7;
+    //   - where the CTAs of a cluster, which must find room together, wait for one another's maxima: B = 65536, 16-bit stream,
+    //     3.3 M 4.9 and 4.1, 11.7 M 13.3 and 12.0; B = 8224, K = 3, 11.7 M 19.5 and 18.3; but between 1.25 and 1.5 of the ahead
+    //     kernels' waves these are 5 % faster;
+    //   - past two waves where the buckets of a window share warps: B = 1504 and 2080 4 to 5 %.
+    // Else the dithers ahead win: 11.7 M, B = 2048, 2 bits 12.5 and 12.6; B = 4096, 1 bit, 16-bit stream 10.2 and 10.8; 2.4 M
+    // 3 to 5 %.
+    auto slots = [&](int kind) { return (uint64_t)sms * (65536u / (dq::direct_registers(R, kind) * shape.threads)); };
+    const uint64_t ahead = slots(dq::kDirectAhead), fits = slots(dq::kDirectDense);
+    const bool cluster = shape.cluster > 1u;
+    const bool dense = shape.threads <= (R == 1 ? dq::kDenseMaxThreads<1> : dq::kDenseMaxThreads<4>) &&
+                       ((grid <= fits && (grid > ahead || (R == 4 && cluster && 4u * grid > 3u * ahead))) ||
+                        (R == 4 && cluster && 2u * grid > 3u * ahead) ||
+                        (R == 4 && a.reduce == dq::kAnywhere && 4u * grid > 9u * ahead));
+    return launch_direct(mode, p.bits, p.dither_bits == 16u, R, dense ? dq::kDirectDense : dq::kDirectAhead, a, (uint32_t)grid,
+                         shape.threads, st);
 }
 
 dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t seed, uint32_t worker,

@@ -26,13 +26,20 @@ namespace dq {
 template <int R> constexpr int kDirectMaxThreads = R == 1 ? 1024 : 256;
 template <int R> constexpr int kDirectMaxCluster = 65536 / (8 * R * kDirectMaxThreads<R>);
 
+// The kernels come in two kinds.  kDirectAhead makes most dithers before the first use of the elements and takes 80 registers
+// (R = 1: 48); kDirectDense makes two at most and is held to 64 (40), for more resident CTAs where the shape leaves the GPU
+// waiting for latency or for a second wave: see the dispatch.
+enum DirectKind : int { kDirectAhead = 0, kDirectDense = 1 };
+template <int R> constexpr uint32_t kDenseMaxThreads = R == 1 ? 768 : 256;
+constexpr uint32_t direct_registers(int R, int kind) { return R == 1 ? (kind == kDirectAhead ? 48 : 40) : kind == kDirectAhead ? 80 : 64; }
+
 // Groups of a lane whose dither is made before the first use of its elements.  With none, a CTA computes nothing while it
 // waits for memory, and then for the maxima of its other warps (n = 11.7 M, B = 2048, 2 bits: 14.1 us with none, 13.4 with one,
 // 13.1 two, 12.7 three, 12.8 four; 25.6 M: 25.4, 24.5, 24.1, 23.7, 23.7; B = 8192: 27.2, 25.6, 25.0, 24.3, 24.3; n = 124.4 M,
 // 3 bits: 112.2, 109.4, 109.0, 107.8, 108.3).  All four fit beside the elements with the 16-bit stream (25.6 M: 19.7 us
-// with none, 18.8 three, 18.4 four).  Two groups per Philox pass instead of one: no difference (23.8).  One-group lanes:
-// n = 1.66 M, B = 16384, K = 3 5.0 us without, 4.7 with it; 2.4 M 4.06 and 3.8.
-template <int R, int DITH> constexpr int kDitherAhead = R == 1 ? 1 : DITH == 16 ? 4 : 3;
+// with none, 18.8 three, 18.4 four).  Two groups per Philox pass instead of one: no difference (23.8).  In the dense kernels two
+// fit beside the elements but for 8 bytes (4.2 M, B = 4096, 2 bits, flagged 4.61 us; with one 4.6, none 4.8).
+template <int R, int DITH, int KIND> constexpr int kDitherAhead = R == 1 ? 1 : KIND == kDirectDense ? 2 : DITH == 16 ? 4 : 3;
 
 // How the lanes' maxima meet in a bucket's scale.  Where a bucket is a power-of-two number of chunks the warp needs
 // neither a barrier nor a gain (a division) per chunk: n = 25.6 M, 2 bits: bucket 1024 28.8 -> 26.5 us, 512 29.0 -> 28.0,
@@ -189,8 +196,9 @@ __device__ __forceinline__ uint32_t cluster_max(uint32_t mine, uint32_t part, ui
     return m;
 }
 
-template <int BITS, int MODE, int DITH, int R>
-__global__ void __launch_bounds__(kDirectMaxThreads<R>, R == 1 ? 1 : 3)
+template <int BITS, int MODE, int DITH, int R, int KIND>
+__global__ void __launch_bounds__(KIND == kDirectDense ? kDenseMaxThreads<R> : kDirectMaxThreads<R>,
+                                  R == 1 ? (KIND == kDirectDense ? 2 : 1) : (KIND == kDirectDense ? 4 : 3))
 encode_direct_kernel(const __grid_constant__ DirectArgs args)
 {
     constexpr int NW = (BITS + 3) / 4;
@@ -227,7 +235,7 @@ encode_direct_kernel(const __grid_constant__ DirectArgs args)
     // M0 k + M0 j), which are cheaper than wide multiplies on the pipe that bounds the kernel
     const uint64_t p0 = (uint64_t)kPhiloxM0 * ((args.first_group + group) * kBlocks);
     // The dither does not depend on the gradient: the dithers of kAhead groups are made while the elements are on their way.
-    constexpr int kAhead = kDitherAhead<R, DITH>;
+    constexpr int kAhead = kDitherAhead<R, DITH, KIND>;
     f32x2 delta[R][4];
     auto dither = [&](int c) { dither_group8<DITH>(p0 + (uint64_t)(32u * c * kBlocks) * kPhiloxM0, args, delta[c]); };
     // (a value that is used here is not computed further down)

@@ -30,10 +30,12 @@ cudaError_t launch_one(const CUtensorMap& map, const EncodeArgs& a, uint32_t gri
 }
 
 template <int BITS>
-cudaError_t launch_direct_one(int R, const DirectArgs& a, uint32_t grid, uint32_t threads, cudaStream_t st)
+cudaError_t launch_direct_one(int R, int kind, const DirectArgs& a, uint32_t grid, uint32_t threads, cudaStream_t st)
 {
-    auto k = R == 1 ? encode_direct_kernel<BITS, DQ_INST_MODE, DQ_INST_DITH, 1>
-                    : encode_direct_kernel<BITS, DQ_INST_MODE, DQ_INST_DITH, 4>;
+    auto k = kind == kDirectDense ? (R == 1 ? encode_direct_kernel<BITS, DQ_INST_MODE, DQ_INST_DITH, 1, kDirectDense>
+                                            : encode_direct_kernel<BITS, DQ_INST_MODE, DQ_INST_DITH, 4, kDirectDense>)
+                                  : (R == 1 ? encode_direct_kernel<BITS, DQ_INST_MODE, DQ_INST_DITH, 1, kDirectAhead>
+                                            : encode_direct_kernel<BITS, DQ_INST_MODE, DQ_INST_DITH, 4, kDirectAhead>);
     return launch_overlapped(k, grid, threads, 0, st, a.cluster, a);
 }
 
@@ -60,18 +62,18 @@ cudaError_t DQ_NAME(DQ_INST_MODE, DQ_INST_DITH)(uint32_t bits, const CUtensorMap
 #define DQ_DNAME2(M, D) launch_direct_m##M##_d##D
 #define DQ_DNAME(M, D) DQ_DNAME2(M, D)
 
-cudaError_t DQ_DNAME(DQ_INST_MODE, DQ_INST_DITH)(uint32_t bits, int R, const DirectArgs& a, uint32_t grid,
+cudaError_t DQ_DNAME(DQ_INST_MODE, DQ_INST_DITH)(uint32_t bits, int R, int kind, const DirectArgs& a, uint32_t grid,
                                                   uint32_t threads, cudaStream_t st)
 {
     switch (bits) {
-        case 1: return launch_direct_one<1>(R, a, grid, threads, st);
-        case 2: return launch_direct_one<2>(R, a, grid, threads, st);
-        case 3: return launch_direct_one<3>(R, a, grid, threads, st);
-        case 4: return launch_direct_one<4>(R, a, grid, threads, st);
-        case 5: return launch_direct_one<5>(R, a, grid, threads, st);
-        case 6: return launch_direct_one<6>(R, a, grid, threads, st);
-        case 7: return launch_direct_one<7>(R, a, grid, threads, st);
-        default: return launch_direct_one<8>(R, a, grid, threads, st);
+        case 1: return launch_direct_one<1>(R, kind, a, grid, threads, st);
+        case 2: return launch_direct_one<2>(R, kind, a, grid, threads, st);
+        case 3: return launch_direct_one<3>(R, kind, a, grid, threads, st);
+        case 4: return launch_direct_one<4>(R, kind, a, grid, threads, st);
+        case 5: return launch_direct_one<5>(R, kind, a, grid, threads, st);
+        case 6: return launch_direct_one<6>(R, kind, a, grid, threads, st);
+        case 7: return launch_direct_one<7>(R, kind, a, grid, threads, st);
+        default: return launch_direct_one<8>(R, kind, a, grid, threads, st);
     }
 }
 

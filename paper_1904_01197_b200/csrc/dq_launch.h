@@ -55,10 +55,10 @@ DQ_DECLARE_ENCODE(0, 32) DQ_DECLARE_ENCODE(1, 32) DQ_DECLARE_ENCODE(2, 32) DQ_DE
 DQ_DECLARE_ENCODE(0, 16) DQ_DECLARE_ENCODE(1, 16) DQ_DECLARE_ENCODE(2, 16) DQ_DECLARE_ENCODE(3, 16)
 #undef DQ_DECLARE_ENCODE
 
-// The same for the direct encoder; R = groups per lane, 1 or 4.
+// The same for the direct encoder; R = groups per lane, 1 or 4; kind = DirectKind.
 #define DQ_DECLARE_DIRECT(MODE, DITH)                                                                              \
-    cudaError_t launch_direct_m##MODE##_d##DITH(uint32_t bits, int R, const DirectArgs& a, uint32_t grid,          \
-                                                uint32_t threads, cudaStream_t st);
+    cudaError_t launch_direct_m##MODE##_d##DITH(uint32_t bits, int R, int kind, const DirectArgs& a,               \
+                                                uint32_t grid, uint32_t threads, cudaStream_t st);
 DQ_DECLARE_DIRECT(0, 32) DQ_DECLARE_DIRECT(1, 32) DQ_DECLARE_DIRECT(2, 32) DQ_DECLARE_DIRECT(3, 32)
 DQ_DECLARE_DIRECT(0, 16) DQ_DECLARE_DIRECT(1, 16) DQ_DECLARE_DIRECT(2, 16) DQ_DECLARE_DIRECT(3, 16)
 #undef DQ_DECLARE_DIRECT

@@ -1,6 +1,7 @@
 """The direct encoder where its shapes change: buckets within a chunk, a warp, a CTA and a cluster, bucket sizes that
-leave idle lanes, the length at which a lane takes four groups instead of one, ragged ends, gradients that are 16- but
-not 32-byte aligned, and the launch flags -- bit for bit against the oracle."""
+leave idle lanes, the length at which a lane takes four groups instead of one, the grids that take the kernels with fewer
+registers, ragged ends, gradients that are 16- but not 32-byte aligned, and the launch flags -- bit for bit against the
+oracle."""
 import numpy as np
 import pytest
 
@@ -65,3 +66,33 @@ def test_overlapping_launches_give_the_bits_of_plain_ones(dq, oracle, n, bucket)
     assert torch.equal(avg, ref)
     for (pk, sc), (pk0, sc0) in zip(over, plain):
         assert torch.equal(pk, pk0) and torch.equal(sc, sc0)
+
+
+KERNELS = [(m, b, d) for m in ("dqsg", "pow2", "mask", "any") for b in range(1, 9) for d in (32, 16)
+           if not (b == 1 and m in ("mask", "any"))]
+
+
+@pytest.mark.parametrize("k", range(len(KERNELS)))
+def test_grids_that_take_the_dense_kernels(dq, oracle, k):
+    """One wave of CTAs with 64 (one group per lane: 40) registers that would be two with 80 (48), buckets in clusters, and
+    more waves of windows whose buckets share warps."""
+    mode, bits, dither = KERNELS[k]
+    sms = _one_group_limit() // 8192
+    K = {"dqsg": 0, "pow2": 1 << bits, "mask": 1 << (bits - 1), "any": (1 << bits) - 1}[mode]
+    sp = WorkerSpec(NDQSG if K else DQSG, bits, 0, K, 1.5 * K, 0.9 if K else 1.0, 33, dither)
+    flags = dq.DQ_FLAG_INPUT_READY | dq.DQ_FLAG_OUTPUT_FREE if k % 2 else 0
+    encode = dq.ndqsg_encode if K else dq.dqsg_encode
+    for n, bucket in ((6 * sms * 4096 + 4099, 2048), (8192 * sms - 77, 12288), (sms * 10 * 2080 * 4 + 1, 2080),
+                      (51 * 65536 + 31, 65536)):
+        g = 0.01 * torch.randn(n, device="cuda", generator=torch.Generator(device="cuda").manual_seed(n))
+        p = dq.binding.make_params(bucket, bits, sp.levels, sp.coarse_K, sp.fine_M, sp.alpha, dither, flags)
+        out = dq.binding.alloc_message(n, p)
+        torch.cuda.synchronize()
+        pk, sc = encode(g, sp.seed, 4, 3, p, *out)
+        nb = -(-n // bucket)
+        span = max(1, 8192 // bucket)
+        for b0 in sorted({0, nb // 2, nb - span}):
+            lo, hi = b0 * bucket, min(n, (b0 + span) * bucket)
+            opk, osc = oracle_encode(oracle, g[lo:hi].cpu().numpy(), sp, 4, 3, bucket, i0=lo, threads=8)
+            assert np.array_equal(words_np(pk)[lo * bits // 32:lo * bits // 32 + opk.size], opk), (n, lo)
+            assert np.array_equal(sc[b0:b0 + osc.size].cpu().numpy().view(np.uint32), osc.view(np.uint32)), (n, lo)
