@@ -269,6 +269,30 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
                          shape.threads, st);
 }
 
+// The tile kernel streams back-to-back encodes of long gradients, whose launches overlap by the caller's flags, through
+// persistent CTAs, a row of 32 elements per lane.  From 16 M elements on it is ahead of the direct kernel (times of calls in a
+// stream, tile and direct)
+//   - in small buckets, where a lane of the direct kernel computes a gain per group: B = 128, 16.8 M, 2 bits 17.0 and 18.1 us,
+//     67 M 57.6 and 65.3; B = 256 2 to 8 %; B = 512 only from 33 M on (16.8 M 16.0 and 15.7, 67 M, 3 bits 61.9 and 65.7);
+//   - where a direct lane's codes leave as single bytes and the tile kernel's as words, at seven bits (B = 8192, 16.8 M, 16-bit
+//     stream 15.5 and 19.6, 67 M 49.0 and 78.7; B = 2048, 25.6 M 20.7 and 23.8; B = 4096, 16.8 M 14.9 and 16.1) and, B = 8192, at
+//     five and six (67 M, 5 bits 46.9 and 52.6, 6 bits 49.8 and 51.5);
+//   - in very long gradients in buckets of 1024 and 2048: B = 2048, 124 M, 2 bits 108 and 115, 3 bits 117 and 126; 67 M, 3 bits
+//     57.3 and 58.7; B = 1024, 124 M, 3 bits 112 and 115, 67 M, 2 bits, 16-bit stream 42.5 and 41.1.
+// Not elsewhere: B = 4096, 25.6 M 7 % slower, B = 1024 and 8192, 16.8 M 7 to 12 %.
+bool tile_encoder_pays(uint64_t n, uint32_t bucket, uint32_t bits)
+{
+    if (n < (1ull << 24)) return false;
+    if (bucket <= 256u || bits == 7u) return true;
+    switch (bucket) {
+        case 512u: return n >= (1ull << 25);
+        case 1024u: return n >= 3ull * (1ull << 25);
+        case 2048u: return n >= (1ull << 26);
+        case 8192u: return (bits == 5u || bits == 6u) && n >= 3ull * (1ull << 23);
+        default: return false;
+    }
+}
+
 dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t seed, uint32_t worker,
                         uint64_t step, const dq_params* p, uint32_t* out_packed, float* out_scale,
                         cudaStream_t st, uint64_t first_element = 0u)
@@ -326,15 +350,8 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 
     const int sms = device_sm_count();
     if (sms <= 0) return DQ_ERR_CUDA;
-    // The tile kernel streams back-to-back encodes of long gradients through persistent CTAs.  With launches that overlap by
-    // the caller's flags it is ahead for small buckets, where a lane of the direct kernel computes a gain per group (B = 512:
-    // n = 16.8 M 14.9 us against 14.9 with two bits, 67 M 57.1 against 59.4), and a little for a bucket per warp of very long
-    // gradients (B = 2048, 67 M: 56.2 us against 56.4 with two bits, 56.6 against 57.6 with three; but 25.6 M 22.0 against
-    // 21.6, 16.8 M 14.7 against 14.2); not for B = 1024 (67 M: 57.1 against 55.4) and where warps meet (B = 8192: 60.2
-    // against 57.3).  Everything else goes through the direct kernel.
-    const bool tiles_pay = (p->bucket <= 512u && n >= (1ull << 24)) || (p->bucket == 2048u && n >= (1ull << 26));
     const bool tiles_wanted = is_pow2(p->bucket) && p->bucket <= 8192u &&
-                              (a.test_drop_copy != 0u || (a.early_store != 0u && tiles_pay));
+                              (a.test_drop_copy != 0u || (a.early_store != 0u && tile_encoder_pays(n, p->bucket, p->bits)));
     if (!tiles_wanted) {
         if (encode_direct(mode, *p, a, n, sms, st) != cudaSuccess) return DQ_ERR_CUDA;
         g_launches.fetch_add(1);

@@ -1,5 +1,5 @@
-"""The tile encoder, which takes encodes of 2^24 elements and more that overlap by the launch flags (power-of-two buckets
-up to 8192): every mode, dither stream and code width, every bucket size, whole and ragged ends, bucket ranges and graph
+"""The tile encoder, which takes long encodes that overlap by the launch flags in the lengths, power-of-two buckets and widths
+of first_length: every mode, dither stream and code width, every bucket size, whole and ragged ends, bucket ranges and graph
 capture.  The whole message against the unflagged call (the direct encoder's kernels), its ends and middle against the
 oracle, bit for bit."""
 import numpy as np
@@ -13,8 +13,19 @@ from dq_testlib import oracle_encode, words_np  # noqa: E402
 from dq_workloads.generators import DQSG, NDQSG, WorkerSpec  # noqa: E402
 from test_gpu_parity import dq, oracle  # noqa: E402,F401
 
-FIRST = 1 << 24                           # shortest gradient that the tile encoder takes
 BUCKETS = [32, 64, 128, 256, 512, 1024, 2048, 4096, 8192]
+
+
+def first_length(bucket, bits):
+    """The shortest gradient that the tile encoder takes, None where it takes none."""
+    if bucket <= 256 or bits == 7:
+        return 1 << 24
+    if bucket == 8192:
+        return 3 << 23 if bits in (5, 6) else None
+    return {512: 1 << 25, 1024: 3 << 25, 2048: 1 << 26}.get(bucket)
+
+
+WIDEST = 3 << 25
 
 
 def _spec(mode, bits, dither):
@@ -31,7 +42,29 @@ KERNELS = [(m, b, d) for m in ("dqsg", "pow2", "mask", "any") for b in range(1, 
 @pytest.fixture(scope="module")
 def gradient():
     gen = torch.Generator(device="cuda").manual_seed(77)
-    return 0.01 * torch.randn(FIRST + 10 * 8192, device="cuda", generator=gen)
+    return 0.01 * torch.randn(WIDEST + 10 * 8192, device="cuda", generator=gen)
+
+
+def _takes_tiles(dq, g, spec, bucket):
+    """Whether a flagged encode of `g` launches the tile encoder, the one with dynamic shared memory: from a captured graph."""
+    from cuda.bindings import driver
+    p = dq.binding.make_params(bucket, spec.bits, spec.levels, spec.coarse_K, spec.fine_M, spec.alpha, spec.dither_bits,
+                               dq.DQ_FLAG_INPUT_READY | dq.DQ_FLAG_OUTPUT_FREE)
+    out = dq.binding.alloc_message(g.numel(), p)
+    encode = dq.dqsg_encode if spec.kind == DQSG else dq.ndqsg_encode
+    encode(g, 1, 0, 0, p, *out)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        encode(g, 1, 0, 0, p, *out)
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    err, _, count = driver.cuGraphGetNodes(raw, 0)
+    assert int(err) == 0 and count == 1
+    err, nodes, _ = driver.cuGraphGetNodes(raw, 1)
+    assert int(err) == 0
+    err, params = driver.cuGraphKernelNodeGetParams(nodes[0])
+    assert int(err) == 0
+    return params.sharedMemBytes > 0
 
 
 def _check(dq, oracle, g, spec, bucket, first=0, step=(1 << 33) + 6, worker=5):
@@ -57,31 +90,38 @@ def _check(dq, oracle, g, spec, bucket, first=0, step=(1 << 33) + 6, worker=5):
 @pytest.mark.parametrize("k", range(len(KERNELS)))
 def test_every_kernel(dq, oracle, gradient, k):
     mode, bits, dither = KERNELS[k]
-    for bucket in (BUCKETS[k % 6], BUCKETS[6 + k % 3]):                # one within a warp's unit, one in two halves
-        _check(dq, oracle, gradient[:FIRST + 12_345], _spec(mode, bits, dither), bucket)
+    large = [b for b in BUCKETS[4:] if first_length(b, bits)]
+    for bucket in (BUCKETS[k % 4], large[k % len(large)], 2048):       # within a warp's unit; in two halves
+        _check(dq, oracle, gradient[:first_length(bucket, bits) + 12_345], _spec(mode, bits, dither), bucket)
 
 
 @pytest.mark.parametrize("bucket", BUCKETS)
 @pytest.mark.parametrize("more", [0, 1, 31, 33, 8192, 9 * 8192 + 8191])
 def test_ends(dq, oracle, gradient, bucket, more):
-    _check(dq, oracle, gradient[:FIRST + more], _spec("dqsg", 3, 32), bucket)
-    _check(dq, oracle, gradient[:FIRST + more], _spec("any", 2, 16), bucket)
+    n = (1 << 24) + more
+    for mode, bits, dither in (("dqsg", 3, 32), ("any", 2, 16)) if bucket <= 256 else (("dqsg", 7, 32), ("any", 7, 16)):
+        _check(dq, oracle, gradient[:n], _spec(mode, bits, dither), bucket)
 
 
 def test_a_bucket_range(dq, oracle, gradient):
-    for bucket in (512, 4096):
-        _check(dq, oracle, gradient[:FIRST + 77], _spec("pow2", 3, 32), bucket, first=bucket * 1_000_001)
+    for bucket, bits in ((256, 3), (4096, 7)):
+        _check(dq, oracle, gradient[:(1 << 24) + 77], _spec("pow2", bits, 32), bucket, first=bucket * 1_000_001)
 
 
-def test_the_shortest_gradient_of_the_tile_encoder_and_the_longest_of_the_other(dq, oracle, gradient):
-    for n in (FIRST - 1, FIRST):
-        _check(dq, oracle, gradient[:n], _spec("dqsg", 2, 32), 2048)
+@pytest.mark.parametrize("bucket", BUCKETS)
+def test_the_shortest_gradients_of_the_tile_encoder_and_the_longest_of_the_other(dq, oracle, gradient, bucket):
+    for bits in (2, 6, 7, 8):
+        first, spec = first_length(bucket, bits), _spec("dqsg", bits, 32)
+        for n in (WIDEST,) if first is None else (first - 1, first):
+            assert _takes_tiles(dq, gradient[:n], spec, bucket) == (first is not None and n >= first), (bits, n)
+            _check(dq, oracle, gradient[:n], spec, bucket)
 
 
-def test_a_captured_sequence_replays_bit_identically(dq, gradient):
+@pytest.mark.parametrize("bucket,bits", [(256, 2), (2048, 7)])
+def test_a_captured_sequence_replays_bit_identically(dq, gradient, bucket, bits):
     flags = dq.DQ_FLAG_INPUT_READY | dq.DQ_FLAG_OUTPUT_FREE
-    n = FIRST + 4321
-    p = dq.binding.make_params(2048, 2, 0, 4, 2.0, 1.0, 32, flags)
+    n = first_length(bucket, bits) + 4321
+    p = dq.binding.make_params(bucket, bits, 0, 1 << bits, 2.0, 1.0, 32, flags)
     grads = [gradient[:n], -gradient[:n], 0.5 * gradient[:n]]
     bufs = [dq.binding.alloc_message(n, p) for _ in grads]
 
@@ -111,16 +151,26 @@ def test_a_captured_sequence_replays_bit_identically(dq, gradient):
 
 @pytest.mark.parametrize("mode,bits,dither", [("mask", 8, 32), ("any", 8, 16), ("any", 8, 32), ("dqsg", 8, 32), ("mask", 7, 16),
                                               ("pow2", 8, 16), ("any", 5, 32), ("dqsg", 3, 16)])
-@pytest.mark.parametrize("bucket", [1024, 2048, 8192])
+@pytest.mark.parametrize("bucket", [128, 1024, 2048])
 def test_many_launches_give_the_same_bits(dq, gradient, mode, bits, dither, bucket):
+    _many_launches(dq, gradient, mode, bits, dither, bucket)
+
+
+@pytest.mark.parametrize("mode,bits,dither", [("mask", 7, 16), ("any", 7, 32), ("dqsg", 7, 32), ("any", 5, 32), ("pow2", 6, 16)])
+def test_many_launches_in_buckets_of_several_warps_give_the_same_bits(dq, gradient, mode, bits, dither):
+    _many_launches(dq, gradient, mode, bits, dither, 8192)
+
+
+def _many_launches(dq, gradient, mode, bits, dither, bucket):
     """A row must be in registers before its stage takes the next copy: where it was not, one launch in a few hundred had
     codes of the wrong elements at the ends of some rows."""
-    sp, g = _spec(mode, bits, dither), gradient[:FIRST]
+    n = first_length(bucket, bits)
+    sp, g = _spec(mode, bits, dither), gradient[:n]
     encode = dq.dqsg_encode if sp.kind == DQSG else dq.ndqsg_encode
     make = lambda f: dq.binding.make_params(bucket, bits, sp.levels, sp.coarse_K, sp.fine_M, sp.alpha, dither, f)  # noqa: E731
     want = encode(g, 3, 1, 2, make(0))
     p = make(dq.DQ_FLAG_INPUT_READY | dq.DQ_FLAG_OUTPUT_FREE)
-    out = dq.binding.alloc_message(FIRST, p)
+    out = dq.binding.alloc_message(n, p)
     wrong = torch.zeros((), dtype=torch.int64, device="cuda")
     for _ in range(1000):
         encode(g, 3, 1, 2, p, *out)

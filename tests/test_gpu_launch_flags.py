@@ -9,9 +9,9 @@ torch = pytest.importorskip("torch")
 
 from test_gpu_parity import dq  # noqa: E402,F401
 
-# around one CTA per SM of either kernel, one and several waves, a cluster per bucket, and the tile encoder
+# around one CTA per SM, one and several waves, a cluster per bucket, long gradients, and the tile encoder
 SHAPES = [(65_536, 512), (70_001, 32), (266_610, 1024), (300_000, 65536), (1_100_000, 2048), (1_663_370, 16384),
-          (4_194_304, 4096), (17_000_000, 2048)]
+          (4_194_304, 4096), (17_000_000, 2048), (17_000_000, 256)]
 ROUNDS = 6
 
 
