@@ -436,11 +436,11 @@ int decode_group_size(uint64_t n, uint32_t W, bool reads_side, bool usual, int s
 
 // The constants of a worker that depend on the form its routine works in (see DecForm).  Returns the largest scale that the
 // form takes.
-float set_decode_form(dq::DecWorker& d, int dith, int side, int group)
+float set_decode_form(dq::DecWorker& d, int dith, int group)
 {
     const uint32_t kind = d.variant >> 3;
     const int bits = (int)(d.variant & 7u) + 1;
-    const int form = dq::dec_form(kind, bits, dith, side, group), shift = dq::dec_shift(kind, bits, dith, side, group);
+    const int form = dq::dec_form(kind, bits, dith, group), shift = dq::dec_shift(kind, bits, dith, group);
     const float u = 1.0f / (float)(1u << shift);
     if (form == dq::kFormJoined && dith == 16)
         d.offset = twice(((float)((1u << bits) - 1u) - d.s + dq::kD16Offset) * u);          // J = (2^bits - 1 - k) 2^16 + h
@@ -556,7 +556,7 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
     const int side = from_first ? dq::kSideFirst : (running && any_nested) ? dq::kSideRunning : dq::kSideGiven;
     float kappa_most = std::numeric_limits<float>::infinity();
     for (uint32_t w = 0; w < W; ++w)
-        kappa_most = std::fmin(kappa_most, set_decode_form(a.w[w], half_dithered ? 0 : d16 ? 16 : 32, side, E));
+        kappa_most = std::fmin(kappa_most, set_decode_form(a.w[w], half_dithered ? 0 : d16 ? 16 : 32, E));
     // (no limit: above the pattern of any NaN)
     a.kappa_limit = std::isinf(kappa_most) ? 0xFFFFFFFFu : bits_of(kappa_most);
     if (one_message) {

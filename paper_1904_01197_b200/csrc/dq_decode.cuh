@@ -114,14 +114,14 @@ constexpr int pair_set(int dqsg_bits, int ndqsg_bits) { return 16 * dqsg_bits + 
 // then loads a worker's constants lane by lane), 128 registers 7 % slower; the kernel with all routines wants 96.
 // E = 16 and 8 take 64 registers (32 warps), but for 72 (28 warps) where all routines in one kernel spill at 64 and are faster
 // without (E = 16, 32-bit stream: running mean, W = 8, 8 and 3 bits, n = 1.7 M 18.0 us with 64, 17.4 with 72; E = 8, 16-bit
-// stream, W = 16, up to 1 M: 64 is 3 to 6 % slower; but E = 8, 32-bit stream, DQSG and a vector: W = 4, 5 bits, n = 1.2 M 7.1 us
-// with 64, 8.3 with 72, W = 16, 128,073 8.7 and 11.0).  A grid that is one wave of eight CTAs per SM and would be two of seven
-// takes the same routines at 64 (kSetAllFull: W = 2, n = 1.2 M, 16-bit stream and a vector 4.4 us, with 72 registers 5.1).
-constexpr int dec_ctas_per_sm(int dith, int side, int E, int set)
+// stream, W = 16, up to 1 M: 64 is 3 to 6 % slower).  The same routines at 64 (kSetAllFull) serve a grid that is one wave of
+// eight CTAs per SM and would be two of seven (W = 2, n = 1.2 M, 16-bit stream and a vector 4.4 us, with 72 registers 5.1), and
+// messages of 5 to 7 bits against a vector or none in groups of 8 (32-bit stream, W = 16, 5 bits, n = 128,073 8.7 us and 11.0;
+// but 8 bits, 266,610 9.5 and 8.9).
+constexpr int dec_ctas_per_sm(int dith, int E, int set)
 {
     if (E == 32) return set == kSetAll ? 5 : 6;
-    if (set != kSetAll || dith == 0) return 8;
-    return (E == 16 ? dith == 32 : dith == 16 || side != kSideGiven) ? 7 : 8;
+    return set == kSetAll && (E == 16 ? dith == 32 : dith != 0) ? 7 : 8;
 }
 
 // How a routine forms k - s - delta (DQSG) and m - delta, q - delta (NDQSG) from the code and the random bits.  All forms
@@ -133,7 +133,7 @@ constexpr int dec_ctas_per_sm(int dith, int side, int E, int set)
 //            from it by another multiply-add.  Not in groups of 32 for DQSG with the 32-bit stream, where the biased form is
 //            ahead in its own routines (W = 8, 2 bits, n = 25.6 M: joined 166.5 us, biased 158.6; in groups of 8, 266,610
 //            4.45 and 4.56) and in the others of their kernel (side information from message 0, six bits, 11.7 M: 99.6 and
-//            92.1), nor for one bit against the running mean (W = 2, DQSG 2 bits, 25.6 M: 52.5 and 51.1).
+//            92.1).
 //   tiny:    NDQSG up to four bits: the code in bits 23.. downwards of a float is an exact multiple of 2^-149, so that
 //            m - delta and q - delta are one multiply-add each and no bias has to be taken off.
 // The values of the last two forms are smaller than the real ones by 2^shift, because a multiply-add cannot scale by more than
@@ -141,18 +141,17 @@ constexpr int dec_ctas_per_sm(int dith, int side, int E, int set)
 // above any gradient) are decoded again by decode_group_plain.
 enum DecForm : int { kFormBiased = 0, kFormJoined = 1, kFormTiny = 2 };
 
-__host__ __device__ constexpr int dec_form(uint32_t kind, int bits, int dith, int side, int group)
+__host__ __device__ constexpr int dec_form(uint32_t kind, int bits, int dith, int group)
 {
     if (dith == 16) return bits <= 7 ? kFormJoined : kFormBiased;
     if (dith == 32 && kind == kDecDqsg) return bits <= 2 && group < 32 ? kFormJoined : kFormBiased;
-    if (dith == 32 && bits == 1) return side == kSideRunning && group == 32 ? kFormBiased : kFormJoined;
-    if (dith == 32) return bits <= 4 ? kFormTiny : kFormBiased;
+    if (dith == 32) return bits == 1 ? kFormJoined : bits <= 4 ? kFormTiny : kFormBiased;
     return kFormBiased;
 }
 
-__host__ __device__ constexpr int dec_shift(uint32_t kind, int bits, int dith, int side, int group)
+__host__ __device__ constexpr int dec_shift(uint32_t kind, int bits, int dith, int group)
 {
-    const int form = dec_form(kind, bits, dith, side, group);
+    const int form = dec_form(kind, bits, dith, group);
     return form == kFormTiny ? bits - 2 : (form == kFormJoined && dith == 16) ? 6 : 0;
 }
 
@@ -161,8 +160,8 @@ __host__ __device__ constexpr int dec_shift(uint32_t kind, int bits, int dith, i
 // mean the compiler's allocation comes out better with the call, although it is never taken (the same pair 2 % faster).
 __host__ __device__ constexpr bool may_be_plain(int set, int dith, int side, int group)
 {
-    return dith != 0 && (side != kSideGiven || set <= kSetAllFull || dec_shift(kDecDqsg, set / 16, dith, side, group) != 0 ||
-                         dec_shift(kDecNdqsgPow2, set % 16, dith, side, group) != 0);
+    return dith != 0 && (side != kSideGiven || set <= kSetAllFull || dec_shift(kDecDqsg, set / 16, dith, group) != 0 ||
+                         dec_shift(kDecNdqsgPow2, set % 16, dith, group) != 0);
 }
 
 __host__ __device__ constexpr float pow2f(int e)
@@ -388,7 +387,7 @@ __device__ __forceinline__ void decode_run(const Args& args, uint32_t w, uint32_
     constexpr bool RUN = SIDE == kSideRunning;
     constexpr bool ANY_K = KIND == kDecNdqsgAnyK || KIND == kDecNdqsgAnyKShrink;
     constexpr bool SHRINK = KIND == kDecNdqsgPow2Shrink || KIND == kDecNdqsgAnyKShrink;
-    constexpr int FORM = dec_form(KIND, BITS, DITH, SIDE, E), SHIFT = dec_shift(KIND, BITS, DITH, SIDE, E);
+    constexpr int FORM = dec_form(KIND, BITS, DITH, E), SHIFT = dec_shift(KIND, BITS, DITH, E);
     constexpr int EPB = (DITH == 16) ? 8 : 4;       // elements per Philox block
     constexpr int N = E / EPB;                      // blocks of the group
     constexpr int P = N < 2 ? N : 2;                // blocks in flight
@@ -700,7 +699,7 @@ __device__ __forceinline__ void decode_group(const Args& args, float4 (*slots)[k
 }
 
 template <int DITH, int SIDE, int E, int SET, int MAXW>
-__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(DITH, SIDE, E, SET))
+__global__ void __launch_bounds__(kDecThreads, dec_ctas_per_sm(DITH, E, SET))
 decode_aggregate_kernel(const __grid_constant__ DecodeArgsOf<MAXW> args)
 {
     __shared__ __align__(16) float4 slots[kDecSlots<DITH, E>][kDecThreads];

@@ -23,14 +23,17 @@ cudaError_t launch_set(const DecodeArgsOf<MAXW>& a, uint32_t grid, cudaStream_t 
                              st, 1u, a);
 }
 
-// All routines.  One wave of CTAs must stay one: where the kernel's registers allow seven CTAs per SM and the grid is a wave of
-// eight, it takes the one that is held to eight.
+// All routines: with the registers that they want, or held to eight CTAs per SM (see dec_ctas_per_sm).
 template <int E, int MAXW>
 cudaError_t launch_all(const DecodeArgsOf<MAXW>& a, uint32_t grid, int sms, cudaStream_t st)
 {
-    constexpr uint32_t fits = dec_ctas_per_sm(DQ_INST_DITH, DQ_INST_RUN, E, kSetAll);
+    constexpr uint32_t fits = dec_ctas_per_sm(DQ_INST_DITH, E, kSetAll);
     if constexpr (E < 32 && fits < 8u) {
-        if (grid > fits * (uint32_t)sms && grid <= 8u * (uint32_t)sms) return launch_set<E, kSetAllFull>(a, grid, st);
+        bool full = grid > fits * (uint32_t)sms && grid <= 8u * (uint32_t)sms;
+        if constexpr (E == 8 && DQ_INST_DITH == 32 && DQ_INST_RUN == kSideGiven) {
+            for (uint32_t w = 0; w < a.W; ++w) full = full || ((a.w[w].variant & 7u) >= 4u && (a.w[w].variant & 7u) < 7u);
+        }
+        if (full) return launch_set<E, kSetAllFull>(a, grid, st);
     }
     return launch_set<E, kSetAll>(a, grid, st);
 }

@@ -28,7 +28,7 @@ template <int DITH, int BITS, int R, bool WHOLE>
 __device__ __forceinline__ void decode_one_chunk(const DecodeArgsOf<1>& args, uint32_t group, uint32_t last)
 {
     constexpr int N = (DITH == 16) ? 1 : 2;                    // Philox blocks of a group
-    constexpr int FORM = dec_form(kDecDqsg, BITS, DITH, kSideGiven, 8), SHIFT = dec_shift(kDecDqsg, BITS, DITH, kSideGiven, 8);
+    constexpr int FORM = dec_form(kDecDqsg, BITS, DITH, 8), SHIFT = dec_shift(kDecDqsg, BITS, DITH, 8);
     const DecWorker& wk = args.w[0];
     using F = Field<BITS, 8>;
     auto bucket_of = [&](uint32_t g) {
