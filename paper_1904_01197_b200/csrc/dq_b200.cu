@@ -251,20 +251,28 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     // More resident CTAs instead of more dithers ahead (times of calls in a stream, ahead and dense):
     //   - where they make one wave of two: n = 4.2 M, B = 4096, 2 bits, flagged 5.4 and 4.6 us; 3.7 M, B = 1504, K = 15 8.5 and
     //     6.5; one-group lanes in CTAs of 656 to 768 threads, of which the ahead kernels run one to an SM: 1.2 M, B = 12288,
-    //     4 bits 5.1 and 3.7;
-    //   - where the CTAs of a cluster, which must find room together, wait for one another's maxima: B = 65536, 16-bit stream,
-    //     3.3 M 4.9 and 4.1, 11.7 M 13.3 and 12.0; B = 8224, K = 3, 11.7 M 19.5 and 18.3; but between 1.25 and 1.5 of the ahead
-    //     kernels' waves these are 5 % faster;
-    //   - past two waves where the buckets of a window share warps: B = 1504 and 2080 4 to 5 %.
+    //     4 bits 5.1 and 3.7.  (Clusters of four and eight CTAs, which must find room together, do not fill every slot: B = 65536,
+    //     16-bit stream, 3.3 M, 0.94 of the slots 4.9 and 4.1; but 0.82 of them 4 % slower.  Where the buckets of a window share
+    //     warps the second wave has to hold a sixteenth of the CTAs, but for flagged calls: B = 1504, 3.6 M 7.5 and 8.0);
+    //   - from 1.75 waves on where the CTAs of a cluster wait for one another's maxima: B = 65536, 16-bit stream, 11.7 M 13.3 and
+    //     12.0; B = 8224, K = 3, 11.7 M 19.5 and 18.3; but 6 M, B = 65536, 2 bits, 1.66 waves 9.7 and 10.2;
+    //   - where the buckets of a window share warps, from four waves on 3 to 5 %, from 2.25 on flagged or with codes that are
+    //     stored in many bytes (B = 1504, 11.7 M, 7 bits, 16-bit stream 23.7 and 21.9, but 3 bits 17.8 and 18.4).
     // Else the dithers ahead win: 11.7 M, B = 2048, 2 bits 12.5 and 12.6; B = 4096, 1 bit, 16-bit stream 10.2 and 10.8; 2.4 M
     // 3 to 5 %.
     auto slots = [&](int kind) { return (uint64_t)sms * (65536u / (dq::direct_registers(R, kind) * shape.threads)); };
     const uint64_t ahead = slots(dq::kDirectAhead), fits = slots(dq::kDirectDense);
-    const bool cluster = shape.cluster > 1u;
-    const bool dense = shape.threads <= (R == 1 ? dq::kDenseMaxThreads<1> : dq::kDenseMaxThreads<4>) &&
-                       ((grid <= fits && (grid > ahead || (R == 4 && cluster && 4u * grid > 3u * ahead))) ||
-                        (R == 4 && cluster && 2u * grid > 3u * ahead) ||
-                        (R == 4 && a.reduce == dq::kAnywhere && 4u * grid > 9u * ahead));
+    const bool shared = R == 4 && a.reduce == dq::kAnywhere;
+    const uint64_t full = R == 1                               ? ahead
+                          : shape.cluster == 8u                ? ahead * 7u / 8u
+                          : shape.cluster == 4u                ? ahead * 15u / 16u
+                          : (shared && a.early_read == 0u)     ? ahead * 17u / 16u
+                                                               : ahead;
+    bool dense = grid > full && grid <= fits;
+    if (R == 4 && shape.cluster > 1u) dense = dense || 4u * grid > 7u * ahead;
+    if (shared)
+        dense = dense || grid > 4u * ahead || (4u * grid > 9u * ahead && (a.early_read != 0u || p.bits >= 5u));
+    dense = dense && shape.threads <= (R == 1 ? dq::kDenseMaxThreads<1> : dq::kDenseMaxThreads<4>);
     return launch_direct(mode, p.bits, p.dither_bits == 16u, R, dense ? dq::kDirectDense : dq::kDirectAhead, a, (uint32_t)grid,
                          shape.threads, st);
 }
