@@ -68,9 +68,10 @@ cudaError_t launch_groups_of(const DecodeArgs& a, int sms, cudaStream_t st)
         have = (int)(v & 7u) + 1;
     }
     if constexpr (E >= 16) {
-        // (not for one message in groups of 16, where it is 4 % faster or 2 % slower, nor two DQSG messages of the 16-bit stream:
-        // n = 1.3 M 4 % slower, 4.2 M 1 %; two others 0 to 7 % faster.  The receiver without the dither was not measured.)
-        const bool two_gain = DQ_INST_DITH == 32 || (DQ_INST_DITH == 16 && width[1] != 0);
+        // (not for one message in groups of 16, where it is 4 % faster or 2 % slower; two messages against message 0 or the running
+        // mean and two DQSG messages of the 32-bit stream take 1 to 7 % less, two DQSG messages of the 16-bit stream up to 4 % more,
+        // a vector 2 % less to 4 % more)
+        const bool two_gain = DQ_INST_RUN != kSideGiven || (DQ_INST_DITH == 32 && width[1] == 0);
         if (usual && one_pair && (E == 32 || a.W > 2u || (a.W == 2u && two_gain))) {
             if (width[0] == 0) width[0] = width[1];
             if (width[1] == 0) width[1] = width[0];
