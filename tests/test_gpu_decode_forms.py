@@ -1,5 +1,5 @@
-"""The forms in which the decoder joins code and dither (by kind, code width and dither stream), bit for bit against the
-oracle, at every group size, with scales from subnormal numbers to near the end of the fp32 range: beyond kappa_limit a
+"""The forms in which the decoder joins code and dither (by kind, code width, dither stream and group size), bit for bit
+against the oracle, at every group size, with scales from subnormal numbers to near the end of the fp32 range: beyond kappa_limit a
 group is decoded by the plain routine."""
 import numpy as np
 import pytest
@@ -17,17 +17,24 @@ FACTORS = np.array([1.0, 1e-40, 1e-34, 0.0, 1.0, 1e30, 3e34, 2e35, 1e36, 4e36, 1
 BUCKET = 1248                                # (not a power of two, and buckets begin inside a warp's groups)
 
 
-@pytest.mark.parametrize("n,few", [(12 * BUCKET + 77, True), (12 * BUCKET + 77, False), (1300001, True), (8000007, True)],
-                         ids=["8", "8 many", "16", "32"])
+def _length(group):
+    """A length that the decoder takes in groups of `group` elements per lane."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+    return {8: 12 * BUCKET + 77, 16: sms * 128 * 8 * 8 + 1, 32: sms * 128 * 32 * 5 * 5 // 2 + 1}[group]
+
+
+@pytest.mark.parametrize("group,few", [(8, True), (8, False), (16, True), (16, False), (32, True)],
+                         ids=["8", "8 many", "16", "16 many", "32"])
 @pytest.mark.parametrize("dither,widths", [(32, (1, 2, 3, 4)), (16, (1, 2, 3, 4, 5, 6, 7, 8))])
-def test_forms_over_the_range_of_scales(dq, oracle, n, few, dither, widths):
-    step = 9
+def test_forms_over_the_range_of_scales(dq, oracle, group, few, dither, widths):
+    n, step = _length(group), 9
     rng = np.random.default_rng(n + dither)
     nb = -(-n // BUCKET)
     common = rng.standard_normal(n).astype(np.float32)
     near = common + 0.05 * rng.standard_normal(n).astype(np.float32)
     for bits in widths if few else widths[1:3]:
-        for K, M1, alpha in ((1 << bits, 2.0, 1.0), ((1 << bits) - 1 if bits > 1 else 2, 0.01, 0.75)):
+        odd_K = (1 << bits) - 1 if bits > 1 else 2
+        for K, M1, alpha in ((1 << bits, 2.0, 1.0), (odd_K, 0.01, 0.75), (odd_K, 2.0, 1.0), (1 << bits, 2.0, 0.75)):
             nested = 2 if few else 8
             # (no overflow in the sum: a step of the coarser quantizer is 75 scales)
             most = np.float32(2e35 if M1 < 1.0 else 1.5e37 if few else 4e36)
@@ -72,6 +79,8 @@ def test_a_fine_resolution_near_the_end_of_the_fp32_range(dq, oracle, dither, bi
     for K, alpha in ((1 << bits, 1.0), (1 << bits, 0.75), ((1 << bits) - 1 if bits > 1 else 2, 1.0)):
         sp = WorkerSpec(NDQSG, bits, 0, K, M1, alpha, 21, dither)
         pk, sc = gpu_encode(dq, torch, grad, sp, 2, step, BUCKET)
-        got = dq.ndqsg_decode_aggregate([gpu_msg(dq, pk, sc, sp, 2, BUCKET)], n, step, torch.from_numpy(side).cuda())[:n].cpu().numpy()
-        ref = oracle.decode_aggregate([oracle_msg(oracle, words_np(pk), sc.cpu().numpy(), sp, 2, BUCKET)], n, step, side_info=side)
+        msg = gpu_msg(dq, pk, sc, sp, 2, BUCKET)
+        got = dq.ndqsg_decode_aggregate([msg], n, step, torch.from_numpy(side).cuda())[:n].cpu().numpy()
+        omsg = oracle_msg(oracle, words_np(pk), sc.cpu().numpy(), sp, 2, BUCKET)
+        ref = oracle.decode_aggregate([omsg], n, step, side_info=side)
         assert np.isfinite(ref).all() and np.array_equal(got.view(np.uint32), ref.view(np.uint32)), (K, alpha)

@@ -18,17 +18,19 @@ def _edges():
     wave8 = sms * 128 * 8 * 8                    # longest call of 8-element lanes
     two_and_a_half32 = sms * 128 * 32 * 5 * 5 // 2
     return {"8 last": wave8, "16 first": wave8 + 1, "16 last": two_and_a_half32 - 1, "32 first": two_and_a_half32 + 9,
-            "16 last of all routines": 2 * wave8, "32 first of all routines": 2 * wave8 + 33}
+            "16 last of all routines": 2 * wave8, "32 first of all routines": 2 * wave8 + 33,
+            "8 last, many": wave8, "8 in seven CTAs, many": wave8 // 8 * 7}
 
 
 @pytest.mark.parametrize("edge", ["8 last", "16 first", "16 last", "32 first", "16 last of all routines",
-                                  "32 first of all routines"])
-@pytest.mark.parametrize("bits,K,alpha,dither,bucket", [(1, 2, 1.0, 32, 96), (3, 8, 1.0, 16, 2048), (5, 21, 0.75, 32, 1248),
+                                  "32 first of all routines", "8 last, many", "8 in seven CTAs, many"])
+@pytest.mark.parametrize("bits,K,alpha,dither,bucket", [(1, 2, 1.0, 32, 96), (3, 8, 1.0, 16, 2048), (2, 3, 1.0, 32, 1024),
+                                                        (2, 3, 1.0, 16, 992), (5, 21, 0.75, 32, 1248),
                                                         (7, 100, 1.0, 16, 32), (8, 128, 0.5, 32, 65536)])
 def test_group_sizes_at_their_edges(dq, oracle, edge, bits, K, alpha, dither, bucket):
     n, step = _edges()[edge], 5
     rng = np.random.default_rng(bits)
-    nested = 7 if "all routines" in edge else 2
+    nested = 7 if "all routines" in edge else 9 if "many" in edge else 2
     specs = [WorkerSpec(DQSG, bits, 0, 0, 0.0, 1.0, 11, dither),
              *[WorkerSpec(NDQSG, bits, 0, K, float(K), alpha, 12 + w, dither) for w in range(nested)]]
     side = (0.01 * rng.standard_normal(n)).astype(np.float32)
