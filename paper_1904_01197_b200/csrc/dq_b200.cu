@@ -206,8 +206,9 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     a.num_groups = (uint32_t)((n + 31u) / 32u * 4u);
     a.whole_groups = (uint32_t)(n / 8u);
     // Up to one wave of one-group lanes (1.2 M elements on 148 SMs) the GPU is not full and the shortest chain per lane
-    // wins (B = 2048: n = 266,610 1.8 us with one group, 2.4 with four; 1.2 M 2.7 and 3.1).  Past it large buckets want four at
-    // once (B = 16384: 1.3 M 6.3 and 4.7 us), small ones from 2 M on (B = 2048: 1.3 M 3.0 and 3.6, 2.4 M 4.4 and 4.2).
+    // wins (B = 2048: n = 266,610 1.6 us with one group, 2.7 with four; 1.2 M 2.5 and 2.8).  Past it large buckets want four at
+    // once (B = 16384: 1.3 M 5.9 and 4.3 us), small ones from 1.7 M on (B = 2048: 1.3 M 2.8 and 3.2, 1.7 M 3.4 and 3.3, 2.4 M
+    // 4.6 and 4.2).
     const int R = n <= (uint64_t)sms * 1024u * 8u ? 1 : 4;
     const uint32_t gpb = p.bucket / 8u;
     const dq::DirectShape shape = dq::direct_shape(gpb, R);
@@ -241,9 +242,9 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     a.off = e.off;
     a.ps = e.ps;
     // A grid of up to two waves lets the next kernel in late: beside it, the CTAs of the next one would be placed unevenly
-    // (see the decoder; n = 2.4 M, B = 2048: 5.5 us per call, late 4.2; 1.9 M, B = 16384: 5.6 and 4.7; 1.2 M, B = 2048: 3.4
-    // and 2.7).  With more waves it does not matter and the early launch hides a little more (11.7 M: 13.8 us, late 14.0), and
-    // so it does where clusters of one-group lanes leave the GPU half empty (0.6 M, B = 16384: 3.65 us, late 3.86).
+    // (see the decoder; n = 2.4 M, B = 2048: 4.9 us per call, late 4.2; 1.9 M, B = 16384: 5.1 and 4.4; 1.2 M, B = 2048: 2.8
+    // and 2.5).  With more waves it does not matter and the early launch hides a little more (11.7 M: 13.3 us, late 13.4), and
+    // so it does where clusters of one-group lanes leave the GPU half empty (0.6 M, B = 16384: 3.31 us, late 3.36).
     a.late_launch = (R == 4 ? n <= (uint64_t)sms * 768u * 32u * 2u : shape.cluster == 1u) ? 1u : 0u;
     // (with early_read one cluster more: see the kernel)
     const uint64_t grid = ((dq_num_buckets(n, p.bucket) + shape.buckets - 1u) / shape.buckets + (a.early_read ? 1u : 0u)) *
@@ -419,18 +420,17 @@ dq_status encode_common(dq_kind kind, const float* grad, uint64_t n, uint64_t se
 }
 
 // Elements per lane of the decoder.  Up to one wave of 8-element lanes (1.2 M elements on 148 SMs) the GPU is not
-// full and the shortest chain per lane wins (W = 8: n = 266,610 6.5 us with 8, 8.0 with 16, 9.9 with 32).  Beyond it 16 and
-// then 32 elements amortise what a worker costs per lane.  32 pays from about two and a half of its own waves, a little
-// before or after with the side information (W = 8: first 3.3 M +5 %, 4.2 M -2 %, 7.4 M -2 %; running mean 0, -6, -5 %; a vector
-// +14, +5, +4 %; two widths of nested messages and the running mean +9, +3, +3 %; W = 4 and 2, 7.6 M -4 %; W = 8, 11.7 M
-// -5 %), and not for one worker, or two and a side information vector, where memory latency matters more and 16 has more
-// warps to hide it (n = 25.6 M: W = 1 30.6 us with 16, 34.0 with 32; W = 2 with a vector 62.6 and 67.4, without 56.9 and
-// 51.9).  In the kernel with all routines, whose routines are longer, 32 pays from one wave of 16-element lanes on if there
-// are eight messages (`usual` false; six bits, W = 8: n = 2.4 M 24.1 us with 16, 24.2 with 32; 3 M 29.2 and 26.1; 4.2 M
-// 39.4 and 35.0; W = 32, 4.2 M 151 and 133; but W = 3 and a vector, 4.2 M 19.5 and 22.5).  From 48 messages on, whose parameters
-// do not stay in the caches between a warp's steps, 32 pays from 1.33 waves of 16-element lanes on (W = 64, 32-bit stream, one
-// nested bit: running mean 3.3 M 228 and 200 us, 4.2 M 296 and 234; first 243 and 203; two bits, 4.2 M: running 248 and 236, vector
-// 245 and 239; but W = 64, 2.5 M, two bits: 161 and 167).
+// full and the shortest chain per lane wins (W = 8, running mean: n = 266,610 5.3 us with 8, 6.7 with 16, 9.1 with 32).  Beyond
+// it 16 and then 32 elements amortise what a worker costs per lane.  32 pays from about two and a half of its own waves, a
+// little before or after with the side information (W = 8: first 3.3 M +2 %, 4.2 M -5 %, 7.4 M -4 %; running mean +1, -5, -4 %;
+// a vector +10, +2, +1 %; 7.6 M W = 4 -5 %, W = 2 0 %; W = 8, 11.7 M -7 %), and not for one nested message, or two messages and
+// a vector, where memory latency matters more and 16 has more warps to hide it (n = 25.6 M: W = 1 45.5 us with 16, 55.6 with
+// 32; W = 2 with a vector 62.9 and 69.3, without 51.3 and 48.1).  (One DQSG message has a kernel of its own.)  In the kernel with
+// all routines, whose routines are longer, 32 pays from one wave of 16-element lanes on if there are eight messages (`usual`
+// false; six bits, W = 8: n = 2.4 M 23.5 us with 16, 23.0 with 32; 3 M 28.3 and 26.3; 4.2 M 38.3 and 35.2; W = 32, 4.2 M 147
+// and 134; but W = 3 and a vector, 4.2 M 18.9 and 22.9).  From 48 messages on, whose parameters do not stay in the caches between
+// a warp's steps, 32 pays from 1.33 waves of 16-element lanes on (W = 64, one nested bit: running mean 3.3 M 228 and 200 us, 4.2 M
+// 296 and 234; first 3.3 M 243 and 203; two bits, running mean 4.2 M 249 and 235, but 2.5 M 162 and 167).
 int decode_group_size(uint64_t n, uint32_t W, bool reads_side, bool usual, int sms)
 {
     const uint64_t lanes = (uint64_t)sms * dq::kDecThreads;
@@ -477,7 +477,7 @@ dq_status decode_common(const dq_msg* msgs, uint32_t W, uint64_t n, uint64_t ste
                         bool side_first = false)
 {
     if (!msgs || W == 0u || W > DQ_MAX_WORKERS) return DQ_ERR_INVALID_ARG;
-    static thread_local dq::DecodeArgs a;    // ~13 KB: keep it off the stack; the first W entries of a.w are filled
+    static thread_local dq::DecodeArgs a;    // ~11 KB: keep it off the stack; the first W entries of a.w are filled
     std::memset(static_cast<dq::DecodeHead*>(&a), 0, sizeof(dq::DecodeHead));
     bool any_nested = false;
     for (uint32_t w = 0; w < W; ++w) {

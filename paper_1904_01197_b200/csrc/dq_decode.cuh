@@ -76,7 +76,7 @@ struct DecodeHead {
     float invW;               // 1/W when W is a power of two, else 0
 };
 
-// Kernel parameters for up to MAXW workers.  A launch copies all of them: 0.8 us more for 64 workers (13 KB) than for 8,
+// Kernel parameters for up to MAXW workers.  A launch copies all of them: 0.8 us more for 64 workers (11 KB) than for 8,
 // which counts for short gradients (kDecFewWorkers).
 template <int MAXW>
 struct DecodeArgsOf : DecodeHead {
@@ -99,12 +99,12 @@ inline void set_bucket_division(DecodeHead& a)
 
 constexpr int kDecThreads = 128;
 // Which variants a kernel holds.  With all forty routines in one kernel the compiler's register allocation and its
-// choice between uniform and per-lane loads of a worker's constants cost every routine 5 to 12 %, so the usual variants
+// choice between uniform and per-lane loads of a worker's constants cost routines up to 5 %, so the usual variants
 // (DQSG, and NDQSG with a power-of-two K and no shrinkage, up to 4 bits) and the odd ones (the same with another K, the
 // paper's K = 3 among them) have kernels of their own, and for long gradients every pair of one DQSG and one NDQSG width has
-// (W = 16, 3 bits, n = 124.4 M: 1973 us with all, 1933 with the usual ones, 1782 with the pair; W = 8, 2 bits, n = 25.6 M:
-// 217, 210 and 197; running mean, W = 8, K = 3, n = 266,010 5.65 us with all, 5.26 with the odd ones; 2.4 M 22.3 and 20.9;
-// but 11.7 M, in groups of 32, 93.3 and 95.1).
+// (n = 25.6 M, W = 16, 3 bits and a vector 362 us with all, 375 with the usual ones, 348 with the pair; W = 8, 3 and 2 bits, side
+// information from message 0 181, 181 and 179; running mean, W = 8, K = 3, n = 266,010 5.6 us with all, 5.4 with the odd ones,
+// 2.4 M 22.6 and 21.8; but 11.7 M, in groups of 32, 91.5 and 92.3).
 constexpr int kSetAll = 0, kSetUsual = 1, kSetOdd = 2, kSetAllFull = 3;      // (kSetAllFull: see dec_ctas_per_sm)
 constexpr int pair_set(int dqsg_bits, int ndqsg_bits) { return 16 * dqsg_bits + ndqsg_bits; }
 
@@ -692,9 +692,9 @@ __device__ __forceinline__ void decode_group(const Args& args, float4 (*slots)[k
     if (args.status != nullptr && ln.kappa_bits_max >= 0x7F800000u) atomicOr(args.status, 0x1u);
     // The next kernel may become resident when every CTA of this one has stored.  Let in right after the wait, its CTAs would
     // take the slots that this kernel leaves free, and what does not fit would be placed when these end, several CTAs on one
-    // SM and none on others, as soon as a grid takes more than half the slots (W = 8: n = 1.3 M 20.3 us per call, now 14;
-    // from a few waves on there is no difference).  Let in before the stores, the last CTAs to store still make the placement
-    // uneven (W = 8, n = 266,610: running mean 6.1 us per call, now 5.3; vector 6.3 and 5.6; side from message 0 6.7 and 5.9).
+    // SM and none on others, as soon as a grid takes more than half the slots (W = 8 and a vector: n = 1.3 M 19.7 us per call,
+    // here 14.3; 266,610 5.9 and 5.5; from a few waves on there is no difference).  Let in before the stores, the last CTAs to
+    // store still make the placement uneven (W = 8, n = 266,610: running mean 5.6 us per call, here 5.3; vector 5.9 and 5.5).
     grid_dependency_launch_next();
 }
 

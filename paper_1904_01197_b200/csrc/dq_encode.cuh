@@ -1,6 +1,6 @@
 // Tile encoder: the encode step (see dq_encode_direct.cuh, which serves every other call) for long gradients that are
-// encoded back to back with overlapping launches, in the bucket sizes where it is ahead (see the dispatch; it can take every
-// power of two up to 8192); and what both encoders share.
+// encoded back to back with overlapping launches, in the bucket sizes and code widths where it is ahead (see
+// tile_encoder_pays; any power of two up to 8192); and what both encoders share.
 //
 // Work decomposition: a "row" is 32 consecutive elements = one 128-byte line of the gradient and exactly
 // `bits` 32-bit words of the bit stream.  One lane quantizes and packs a whole row, so no lane ever shares a
@@ -22,9 +22,8 @@
 // buckets of up to 4096 elements one per warp, larger ones one per CTA (a sweep for the maximum, then a second, cached
 // sweep that quantizes).
 //
-// What bounds it: the multiplier pipe and instruction issue, as in the direct encoder.  On packed fp32 pairs and with
-// the clamp in one instruction the overlapped encode of n = 25.6 M, B = 2048 takes 22.2 us (2 bits, before 22.6) and 22.4 us
-// (3 bits, before 25.5).
+// What bounds it: the multiplier pipe and instruction issue, as in the direct encoder.  Overlapped encodes of two bits in
+// buckets of 128 take 17.0 us at n = 16.8 M and 57.6 at 67 M (the direct encoder 18.1 and 65.3).
 #pragma once
 
 #include "dq_device.cuh"

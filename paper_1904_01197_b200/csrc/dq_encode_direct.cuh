@@ -31,14 +31,18 @@ template <int R> constexpr int kDirectMaxCluster = 65536 / (8 * R * kDirectMaxTh
 // waiting for latency or for a second wave: see the dispatch.
 enum DirectKind : int { kDirectAhead = 0, kDirectDense = 1 };
 template <int R> constexpr uint32_t kDenseMaxThreads = R == 1 ? 768 : 256;
-constexpr uint32_t direct_registers(int R, int kind) { return R == 1 ? (kind == kDirectAhead ? 48 : 40) : kind == kDirectAhead ? 80 : 64; }
+constexpr uint32_t direct_registers(int R, int kind)
+{
+    return R == 1 ? (kind == kDirectAhead ? 48u : 40u) : kind == kDirectAhead ? 80u : 64u;
+}
 
 // Groups of a lane whose dither is made before the first use of its elements.  With none, a CTA computes nothing while it
 // waits for memory, and then for the maxima of its other warps (n = 11.7 M, B = 2048, 2 bits: 14.1 us with none, 13.4 with one,
 // 13.1 two, 12.7 three, 12.8 four; 25.6 M: 25.4, 24.5, 24.1, 23.7, 23.7; B = 8192: 27.2, 25.6, 25.0, 24.3, 24.3; n = 124.4 M,
 // 3 bits: 112.2, 109.4, 109.0, 107.8, 108.3).  All four fit beside the elements with the 16-bit stream (25.6 M: 19.7 us
 // with none, 18.8 three, 18.4 four).  Two groups per Philox pass instead of one: no difference (23.8).  In the dense kernels two
-// fit beside the elements but for 8 bytes (4.2 M, B = 4096, 2 bits, flagged 4.61 us; with one 4.6, none 4.8).
+// fit beside the elements but for 8 bytes; a draw of 490 encodes with four groups per lane takes 1.03 of the time with none, 1.006
+// with one.  One-group lanes: n = 1.2 M, B = 2048 2.65 us with none, 2.50 with its one; 0.6 M, B = 16384 3.53 and 3.28.
 template <int R, int DITH, int KIND> constexpr int kDitherAhead = R == 1 ? 1 : KIND == kDirectDense ? 2 : DITH == 16 ? 4 : 3;
 
 // How the lanes' maxima meet in a bucket's scale.  Where a bucket is a power-of-two number of chunks the warp needs
