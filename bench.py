@@ -37,12 +37,17 @@ L2_BYTES = 126 * 1024 * 1024
 HBM_NOMINAL_GBS = 8000.0
 SM_COUNT, ISSUE_PER_SM_CLK, LANES = 148, 4, 32           # issue ceiling: SMs x schedulers x lanes x clock
 # Algorithmic lane-instructions of the method itself, in scalar operations (the kernels do the fp32 part on
-# packed pairs and execute 21 per (element, worker) and 20 per element, profiles/counters_*.md): a quarter of a
-# Philox block per dither value (4.5 wide multiplies + 4.75 three-input XORs), the dither conversion (2), and
-# for the fused decode unpacking (3) plus 5 (DQSG) to 9 (NDQSG) fp32 operations per (element, worker), about 10
-# per element for the mean and the stores; for the encode 24 per element with the scale reduction and the
-# packing.
+# packed pairs and execute fewer, profiles/counters_*.md): a quarter of a Philox block per dither value (4.5 wide
+# multiplies + 4.75 three-input XORs; an eighth with the 16-bit stream), the dither conversion (2), and for the
+# fused decode unpacking (3) plus 5 (DQSG) to 9 (NDQSG) fp32 operations per (element, worker), about 10 per
+# element for the mean and the stores; for the encode 24 per element with the scale reduction and the packing.
 DEC_INSTR_PER_ELEM_WORKER, DEC_INSTR_PER_ELEM, ENC_INSTR_PER_ELEM = 22.0, 10.0, 24.0
+
+
+def instr_per_elem(count_32bit_stream, dither_bits):
+    return count_32bit_stream - (9.25 / 2 if dither_bits == 16 else 0.0)
+
+
 FLAG_INPUT_READY, FLAG_OUTPUT_FREE = 1, 2
 
 
@@ -306,6 +311,7 @@ def kernel_timings(st: GpuState, hbm_peak, sm_max_mhz):
     for key, w in seen.items():
         s = cfg.workers[w]
         by = encode_bytes(dq, n, s, cfg.bucket)
+        enc_instr = instr_per_elem(ENC_INSTR_PER_ELEM, s.dither_bits)
         name = f"encode_{'dqsg' if s.kind == st.DQSG else 'ndqsg'}_b{s.bits}"
         # rotating inputs AND outputs: consecutive launches share nothing, as the overlapped variant requires
         outs = [dq.binding.alloc_message(n, st.params[w], st.dev) for _ in range(rot)]
@@ -318,8 +324,7 @@ def kernel_timings(st: GpuState, hbm_peak, sm_max_mhz):
                 "frac_hbm": by / ms / 1e6 / hbm_peak, "rotating_buffers": rot,
                 "launch_flags": ("DQ_FLAG_INPUT_READY|DQ_FLAG_OUTPUT_FREE: back-to-back launches overlap"
                                  if variant else "none: each launch waits for the previous one"),
-                "alu_tinstr_s": ENC_INSTR_PER_ELEM * n / ms / 1e9,
-                "frac_alu": ENC_INSTR_PER_ELEM * n / ms * 1e3 / alu_peak,
+                "alu_tinstr_s": enc_instr * n / ms / 1e9, "frac_alu": enc_instr * n / ms * 1e3 / alu_peak,
                 "traffic": counters.get(f"{cfg.name}.{name}.dram_bytes") if s.dither_bits == 32 else None}
         del outs
     # decode: rotate over message sets / side / out copies so that nothing is L2-resident
@@ -385,7 +390,7 @@ def kernel_timings(st: GpuState, hbm_peak, sm_max_mhz):
                          "frac_hbm": by_t / ms_t / 1e6 / hbm_peak,
                          "container_bits_per_element": 8 * dq.ternary_bytes(n) / n}
     elem_workers = n * cfg.W
-    alg_instr = DEC_INSTR_PER_ELEM_WORKER * elem_workers + DEC_INSTR_PER_ELEM * n
+    alg_instr = instr_per_elem(DEC_INSTR_PER_ELEM_WORKER, cfg.workers[0].dither_bits) * elem_workers + DEC_INSTR_PER_ELEM * n
     res["decode_aggregate"] = {"ms": ms, "bytes": per_set, "gbs": per_set / ms / 1e6, "gelem_s": n / ms / 1e6,
                                "frac_hbm": per_set / ms / 1e6 / hbm_peak,
                                "gelem_worker_s": elem_workers / ms / 1e6, "rotating_buffers": sets,
@@ -724,9 +729,9 @@ def main():
             # decode: bound by instruction issue; algorithmic lane-instructions against the issue ceiling, and the
             # multiplier pipe beside it (a 32x32->64 multiply holds it for four cycles, 4.5 of them per dither value)
             alu_peak = SM_COUNT * ISSUE_PER_SM_CLK * LANES * sm_max_mhz * 1e6
-            alg_instr = DEC_INSTR_PER_ELEM_WORKER * cfg.n * cfg.W + DEC_INSTR_PER_ELEM * cfg.n
-            cyc_per_unit = SM_COUNT * ISSUE_PER_SM_CLK * LANES * sm_max_mhz * 1e6 / (kd["gelem_worker_s"] * 1e9)
             dith = cfg.workers[0].dither_bits
+            alg_instr = instr_per_elem(DEC_INSTR_PER_ELEM_WORKER, dith) * cfg.n * cfg.W + DEC_INSTR_PER_ELEM * cfg.n
+            cyc_per_unit = SM_COUNT * ISSUE_PER_SM_CLK * LANES * sm_max_mhz * 1e6 / (kd["gelem_worker_s"] * 1e9)
             wide_per_unit = 18.0 / (4 if dith == 32 else 8)
             roofline_decode = {"kernel": dec_name, "bound": "alu", "achieved": alg_instr / kd["ms"] / 1e9,
                                "peak": alu_peak / 1e12, "unit": "Tlane-instr/s",
