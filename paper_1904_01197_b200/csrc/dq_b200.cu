@@ -254,7 +254,8 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
     //     6.5; one-group lanes in CTAs of 656 to 768 threads, of which the ahead kernels run one to an SM: 1.2 M, B = 12288,
     //     4 bits 5.1 and 3.7.  (Clusters of four and eight CTAs, which must find room together, do not fill every slot: B = 65536,
     //     16-bit stream, 3.3 M, 0.94 of the slots 4.9 and 4.1; but 0.82 of them 4 % slower.  Where the buckets of a window share
-    //     warps the second wave has to hold a sixteenth of the CTAs, but for flagged calls: B = 1504, 3.6 M 7.5 and 8.0);
+    //     warps the second wave has to hold a sixteenth of the CTAs, but for flagged calls: B = 1504, 3.6 M 7.5 and 8.0.  Not the
+    //     16-bit stream unflagged, whose four dithers ahead hide more: B = 4096, 4.4 M from HBM 5.1 and 5.4);
     //   - from 1.75 waves on where the CTAs of a cluster wait for one another's maxima: B = 65536, 16-bit stream, 11.7 M 13.3 and
     //     12.0; B = 8224, K = 3, 11.7 M 19.5 and 18.3; but 6 M, B = 65536, 2 bits, 1.66 waves 9.7 and 10.2;
     //   - where the buckets of a window share warps, from four waves on 3 to 5 %, from 2.25 on flagged or with codes that are
@@ -269,7 +270,8 @@ cudaError_t encode_direct(int mode, const dq_params& p, const dq::EncodeArgs& e,
                           : shape.cluster == 4u                ? ahead * 15u / 16u
                           : (shared && a.early_read == 0u)     ? ahead * 17u / 16u
                                                                : ahead;
-    bool dense = grid > full && grid <= fits;
+    bool dense = grid > full && grid <= fits &&
+                 (R == 1 || shape.cluster > 1u || shared || a.early_read != 0u || p.dither_bits != 16u);
     if (R == 4 && shape.cluster > 1u) dense = dense || 4u * grid > 7u * ahead;
     if (shared)
         dense = dense || grid > 4u * ahead || (4u * grid > 9u * ahead && (a.early_read != 0u || p.bits >= 5u));
