@@ -68,10 +68,10 @@ cudaError_t launch_groups_of(const DecodeArgs& a, int sms, cudaStream_t st)
         have = (int)(v & 7u) + 1;
     }
     if constexpr (E >= 16) {
-        // (not for one message in groups of 16, where it is 4 % faster or 2 % slower; two messages against message 0 or the running
-        // mean and two DQSG messages of the 32-bit stream take 1 to 7 % less, two DQSG messages of the 16-bit stream up to 4 % more,
-        // a vector 2 % less to 4 % more)
-        const bool two_gain = DQ_INST_RUN != kSideGiven || (DQ_INST_DITH == 32 && width[1] == 0);
+        // (not for one message in groups of 16, where it is 4 % faster or 2 % slower; two messages of the 32-bit stream against
+        // message 0, the running mean or nothing take 1 to 5 % less, against a vector 2 % less to 3 % more; of the 16-bit stream
+        // up to 13 % more with messages from HBM: running mean, 3 and 2 bits, n = 1.7 M 4.7 and 5.3 us)
+        const bool two_gain = DQ_INST_DITH == 32 && (DQ_INST_RUN != kSideGiven || width[1] == 0);
         if (usual && one_pair && (E == 32 || a.W > 2u || (a.W == 2u && two_gain))) {
             if (width[0] == 0) width[0] = width[1];
             if (width[1] == 0) width[1] = width[0];
